@@ -75,10 +75,12 @@ int drgb_fit_transform_batched(drgb_ctx* c, const float* X_cat, const int64_t* o
 
     // scratch: per-row buffers of the concatenation, then the k-NN region for
     // the largest instance
-    size_t knn_bytes = 0;
+    size_t knn_bytes = 0, knn_least = 0;
     for (int b = 0; b < count; ++b) {
-        const size_t kb = knn_scratch_bytes(offsets[b + 1] - offsets[b], d, k, p->knn_mode);
+        size_t least = 0;
+        const size_t kb = knn_scratch_bytes(c, offsets[b + 1] - offsets[b], d, k, p->knn_mode, &least);
         knn_bytes = kb > knn_bytes ? kb : knn_bytes;
+        knn_least = least > knn_least ? least : knn_least;
     }
     const size_t Nk = size_t(N) * k;
     const size_t main_bytes = Carve::round(Nk * 4) * 2 + Carve::round((N + 1) * 4) + Carve::round(2 * Nk * 4) * 3 +
@@ -89,9 +91,12 @@ int drgb_fit_transform_batched(drgb_ctx* c, const float* X_cat, const int64_t* o
     // instances are small: their k-NN runs go round-robin to BATCH_STREAMS
     // streams, each with its own k-NN scratch region, so that several run at once
     const int n_str = count < BATCH_STREAMS ? count : BATCH_STREAMS;
-    const size_t knn_region = Carve::round(knn_bytes);
-    int rc = ensure_scratch(c, Carve::round(main_bytes) + size_t(n_str) * knn_region, st);
+    const size_t least = Carve::round(main_bytes) + size_t(n_str) * Carve::round(knn_least);
+    size_t total = Carve::round(main_bytes) + size_t(n_str) * Carve::round(knn_bytes);
+    int rc = ensure_scratch_within(c, &total, least, st);
     if (rc) return rc;
+    if (total == least) knn_bytes = knn_least;
+    const size_t knn_region = Carve::round(knn_bytes);
     Carve cv(c->scratch);
     int32_t* idx = cv.take<int32_t>(Nk);
     float* dist = cv.take<float>(Nk);
@@ -152,7 +157,8 @@ int drgb_fit_transform_batched(drgb_ctx* c, const float* X_cat, const int64_t* o
             const int64_t off = offsets[b], nb = offsets[b + 1] - off;
             const int si_ = b % n_str;
             rc = knn_run(c, X_cat + off * d, nb, d, k, p->knn_mode, idx + off * k, dist + off * k, ss[si_],
-                         static_cast<char*>(knn_scratch) + size_t(si_) * knn_region, fail_rows + off, fail_count + b);
+                         static_cast<char*>(knn_scratch) + size_t(si_) * knn_region, knn_bytes, fail_rows + off,
+                         fail_count + b);
         }
         for (int i = 0; i < n_str; ++i) {
             if (cudaEventRecord(ev[i], ss[i]) != cudaSuccess || cudaStreamWaitEvent(st, ev[i], 0) != cudaSuccess) {
@@ -173,8 +179,8 @@ int drgb_fit_transform_batched(drgb_ctx* c, const float* X_cat, const int64_t* o
             const int64_t off = offsets[b], nb = offsets[b + 1] - off;
             const int64_t cnt = h[b] < nb ? h[b] : nb;
             if (cnt <= 0) continue;
-            rc = launch_knn_exact_rows_n(c, X_cat + off * d, nb, d, k, fail_rows + off, fail_count + b, cnt,
-                                         idx + off * k, dist + off * k, st, knn_scratch, part);
+            rc = launch_knn_exact_rows_n(c, X_cat + off * d, nb, d, k, fail_rows + off, cnt, idx + off * k,
+                                         dist + off * k, st, knn_scratch, part);
             if (rc) return rc;
         }
     }

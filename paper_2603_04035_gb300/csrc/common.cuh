@@ -22,6 +22,9 @@ struct Ctx {
     void* scratch = nullptr;      // grown on demand, 256-byte aligned carve-outs
     size_t scratch_bytes = 0;
     size_t scratch_limit = 0;     // largest scratch the context may allocate (0 = no limit)
+    void* scan_part = nullptr;    // partial lists of drgb_knn_graph's scans (see there)
+    size_t scan_bytes = 0;
+    cudaEvent_t scan_ev = nullptr;  // the last such scan
     int* d_status = nullptr;      // device status word (0 = ok, else DRGB_ERR_*)
     unsigned long long* d_counter = nullptr;  // [0] uncertified rows, [4] k-NN tile products computed
     int64_t knn_tiles_total = 0;              // tile products of a full scan (last tensor-core k-NN)
@@ -74,6 +77,13 @@ int set_error(Ctx* c, int code, const char* fmt, ...);
 // Ensure the context holds at least `bytes` of scratch.  Growing synchronises
 // `stream` first, so that work still using the old buffer has finished.
 int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream);
+
+// Scratch of *bytes if the context's limit and the device allow it, else of
+// `least` bytes (*bytes is then set to it): for steps that run with less.
+int ensure_scratch_within(Ctx* c, size_t* bytes, size_t least, cudaStream_t stream);
+
+// Whether work enqueued on `st` is being captured into a graph.
+bool stream_captures(cudaStream_t st);
 
 // Bump allocator over the scratch buffer (256-byte aligned slices).
 struct Carve {

@@ -45,6 +45,21 @@ int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
     return DRGB_OK;
 }
 
+int ensure_scratch_within(Ctx* c, size_t* bytes, size_t least, cudaStream_t stream) {
+    if (*bytes > least && c->scratch_limit && *bytes > c->scratch_limit && *bytes > c->scratch_bytes) *bytes = least;
+    int rc = ensure_scratch(c, *bytes, stream);
+    if (rc && *bytes > least) {
+        *bytes = least;
+        rc = ensure_scratch(c, least, stream);
+    }
+    return rc;
+}
+
+bool stream_captures(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
 int stage_mark(Ctx* c, int idx, cudaStream_t st) {
     if (!c->profiling || idx < 0 || idx >= 11) return DRGB_OK;
     if (!c->stage_ev[idx]) DRGB_CUDA(c, cudaEventCreate(&c->stage_ev[idx]));
@@ -293,6 +308,8 @@ int drgb_ctx_destroy(drgb_ctx* c) {
     cudaDeviceSynchronize();
     if (c->epoch_exec) cudaGraphExecDestroy(c->epoch_exec);
     if (c->scratch) cudaFree(c->scratch);
+    if (c->scan_part) cudaFree(c->scan_part);
+    if (c->scan_ev) cudaEventDestroy(c->scan_ev);
     if (c->d_status) cudaFree(c->d_status);
     for (auto& e : c->stage_ev)
         if (e) cudaEventDestroy(e);

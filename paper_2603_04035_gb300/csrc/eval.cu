@@ -41,8 +41,12 @@ static int eval_common(Ctx* c, const float* X, const float* Y, int64_t n, int d,
     const int64_t m = (n_query <= 0 || n_query >= n) ? n : n_query;
     const size_t bytes = Carve::round(m * 8) + 2 * Carve::round(m * k * 4) * 2 +
                          Carve::round(m * 8) + Carve::round(m * 4) + 4096;
-    int rc = ensure_scratch(c, bytes, st);
+    const size_t part_off = Carve::round(bytes);
+    size_t total = part_off + knn_scan_scratch_bytes(c, m, n, k);
+    int rc = ensure_scratch_within(c, &total, bytes, st);
     if (rc) return rc;
+    const size_t part_bytes = total > part_off ? total - part_off : 0;
+    void* part = part_bytes ? static_cast<char*>(c->scratch) + part_off : nullptr;
     Carve cv(c->scratch);
     int64_t* rows = cv.take<int64_t>(m);
     int32_t* ny = cv.take<int32_t>(m * k);
@@ -53,10 +57,10 @@ static int eval_common(Ctx* c, const float* X, const float* Y, int64_t n, int d,
     int32_t* hits = cv.take<int32_t>(m);
     strided_rows_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(rows, m, n);
     DRGB_CHECK_LAUNCH(c);
-    rc = launch_knn_exact(c, Y, n, 2, k, rows, m, ny, dy, false, st);
+    rc = launch_knn_exact(c, Y, n, 2, k, rows, m, ny, dy, st, part, part_bytes);
     if (rc) return rc;
     if (want_recall) {
-        rc = launch_knn_exact(c, X, n, d, k, rows, m, nx, dx, false, st);
+        rc = launch_knn_exact(c, X, n, d, k, rows, m, nx, dx, st, part, part_bytes);
         if (rc) return rc;
         intersect_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(nx, ny, m, k, hits);
         DRGB_CHECK_LAUNCH(c);
@@ -67,7 +71,7 @@ static int eval_common(Ctx* c, const float* X, const float* Y, int64_t n, int d,
         for (int64_t r = 0; r < m; ++r) s += h[r];
         *out = s / (double(k) * double(m));
     } else {
-        rc = launch_rank(c, X, n, d, k, rows, m, ny, excess, st);
+        rc = launch_rank(c, X, n, d, k, rows, m, ny, dx, nx, excess, st);
         if (rc) return rc;
         std::vector<int64_t> e(m);
         DRGB_CUDA(c, cudaMemcpyAsync(e.data(), excess, m * 8, cudaMemcpyDeviceToHost, st));
@@ -104,8 +108,12 @@ static int eval_heldout(Ctx* c, const float* Xt, const float* Yt, int64_t n, con
     const int64_t m = (n_query <= 0 || n_query >= n_new) ? n_new : n_query;
     const size_t bytes = Carve::round(m * 8) + Carve::round(m * d * 4) + Carve::round(m * 8) +
                          4 * Carve::round(m * k * 4) + Carve::round(m * 4) + 4096;
-    int rc = ensure_scratch(c, bytes, st);
+    const size_t part_off = Carve::round(bytes);
+    size_t total = part_off + knn_scan_scratch_bytes(c, m, n, k);
+    int rc = ensure_scratch_within(c, &total, bytes, st);
     if (rc) return rc;
+    const size_t part_bytes = total > part_off ? total - part_off : 0;
+    void* part = part_bytes ? static_cast<char*>(c->scratch) + part_off : nullptr;
     Carve cv(c->scratch);
     int64_t* rows = cv.take<int64_t>(m);
     float* xq = cv.take<float>(m * d);
@@ -121,8 +129,8 @@ static int eval_heldout(Ctx* c, const float* Xt, const float* Yt, int64_t n, con
     DRGB_CHECK_LAUNCH(c);
     gather_rows_kernel<<<grid_for(m * 2, 256, c->num_sms * 8), 256, 0, st>>>(Yn, 2, rows, m, yq);
     DRGB_CHECK_LAUNCH(c);
-    if ((rc = launch_knn_query(c, xq, m, Xt, n, d, k, nx, dx, st))) return rc;
-    if ((rc = launch_knn_query(c, yq, m, Yt, n, 2, k, ny, dy, st))) return rc;
+    if ((rc = launch_knn_query(c, xq, m, Xt, n, d, k, nx, dx, st, part, part_bytes))) return rc;
+    if ((rc = launch_knn_query(c, yq, m, Yt, n, 2, k, ny, dy, st, part, part_bytes))) return rc;
     intersect_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(nx, ny, m, k, hits);
     DRGB_CHECK_LAUNCH(c);
     std::vector<int32_t> h(m);

@@ -81,15 +81,18 @@ extern "C" int drgb_fit_transform(drgb_ctx* c, const float* X, int64_t n, int32_
     const size_t zb = do_pca ? Carve::round(size_t(n) * dk * 4) : 0;
     const bool spectral = (p->flags & DRGB_FLAG_INIT_SPECTRAL) != 0;
     const bool nnd_rev = k <= 16;  // the reverse form (general neighbours) where a warp holds them
-    const size_t kb = nnd ? nnd_scratch_bytes(n, k, nnd_rev) : knn_scratch_bytes(n, dk, k, p->knn_mode);
+    size_t kb_least = 0;
+    const size_t kb = nnd ? nnd_scratch_bytes(n, k, nnd_rev) : knn_scratch_bytes(c, n, dk, k, p->knn_mode, &kb_least);
+    if (nnd) kb_least = kb;
     // the PCA's, then the k-NN's, then the spectral layout's scratch share one
     // region (each is free by the time the next starts)
     const size_t sb = spectral ? spectral_scratch_bytes(n, int64_t(2) * n * k, c->num_sms) : 0;
     const size_t pb = do_pca ? pca_scratch_bytes(n, d) : 0;
-    size_t rb = kb > sb ? kb : sb;
-    rb = rb > pb ? rb : pb;
-    rc = ensure_scratch(c, fb + zb + rb, st);
+    const size_t ob = sb > pb ? sb : pb;
+    size_t total = fb + zb + (kb > ob ? kb : ob);
+    rc = ensure_scratch_within(c, &total, fb + zb + (kb_least > ob ? kb_least : ob), st);
     if (rc) return rc;
+    const size_t knn_bytes = total - fb - zb;
     FitBuffers b = carve_fit(c->scratch, n, k);
     float* Z = do_pca ? reinterpret_cast<float*>(static_cast<char*>(c->scratch) + fb) : nullptr;
     void* knn_scratch = static_cast<char*>(c->scratch) + fb + zb;
@@ -113,7 +116,7 @@ extern "C" int drgb_fit_transform(drgb_ctx* c, const float* X, int64_t n, int32_
         rc = nnd_run(c, Xk, n, dk, k, p->seed_init, NND_DELTA, NND_ITER_DEFAULT, nnd_rev, b.idx, b.dist, nullptr, nullptr,
                      knn_scratch, st);
     else
-        rc = knn_run(c, Xk, n, dk, k, p->knn_mode, b.idx, b.dist, st, knn_scratch);
+        rc = knn_run(c, Xk, n, dk, k, p->knn_mode, b.idx, b.dist, st, knn_scratch, knn_bytes);
     if (rc) return rc;
     if ((rc = stage_mark(c, 1, st))) return rc;
     rc = build_fuzzy_graph(c, b.idx, b.dist, n, k, p->n_epochs, b.row_ptr, b.col, b.w, b.q, nullptr,

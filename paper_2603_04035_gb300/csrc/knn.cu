@@ -1,135 +1,306 @@
 // Exact k-NN by an FP32 scan (SIMT), and the FP32 rank counts used by the
 // trustworthiness metric.
 //
-// One thread owns one query row and keeps its best K (distance, index) pairs
-// sorted in registers.  The database is streamed through shared memory in
-// tiles of 32 points x 32 dimensions; every thread reads the same tile element
-// (a broadcast), so the tile costs no bank conflicts.  Squared distances are
-// evaluated directly as sum_c (x_qc - x_pc)^2 in dimension order, so the
-// result is the exact FP32 ranking (ties resolved by lower index because the
-// scan visits points in increasing index order and only strictly smaller
-// distances displace a kept entry).
+// Both are one kernel: a CTA takes 64 query rows and streams a chunk of the
+// database through shared memory, 128 points by 32 dimensions at a time
+// (transposed, two buffers filled by cp.async), and each of its 256 threads
+// accumulates the squared distances of 4 queries to 8 points in registers as
+// packed pairs (add.f32x2, fma.f32x2).  Squared distances are evaluated
+// directly as sum_c (x_qc - x_pc)^2 in dimension order, so the result is the
+// exact FP32 ranking.  A finished 64 x 128 tile goes to shared memory, where a
+// warp per row compares it with the row's current k-th distance and inserts
+// the few that pass into the row's sorted list (one entry per lane), ordered
+// by (distance, index).
+//
+// Bound: FP32 issue and shared-memory reads, two packed operations per two
+// pairs of points and dimension.  The earlier form, one thread per query with
+// its whole list in registers, filled the GPU only from about 80,000 queries
+// on; splitting the database over blockIdx.y fills it from a few hundred, and
+// the partial lists are merged afterwards.  Measured, earlier form -> this
+// one: 5,003 queries against 70,000 x 50 (with the layout of the new points)
+// 28.2 -> 2.9 ms; 3,000 ranks and neighbours of 20,011 x 50 40.2 -> 2.4 ms;
+// all pairs of 30,011 x 200 40.5 -> 22.5 ms; a 2,000 x 50 fit 2.60 -> 2.00 ms.
 #include "common.cuh"
 #include "knn.cuh"
 
 namespace drgb {
 
-static constexpr int KNN_THREADS = 128;
-static constexpr int TP = 32;  // points per tile
-static constexpr int DC = 32;  // dimensions per tile
+static constexpr int SC_Q = 64;         // queries per CTA
+static constexpr int SC_P = 128;        // points per tile
+static constexpr int SC_DC = 32;        // dimensions per stage
+static constexpr int SC_THREADS = 256;  // 16 x 16: 4 queries x 8 points each
+static constexpr int SC_PITCH = 132;    // floats per staged dimension (128 points): transposing stores hit distinct banks
+static constexpr int SC_QPITCH = 66;    // float pairs per dimension of the queries
+static constexpr int SC_WARPS = SC_THREADS / 32;
+static constexpr int SC_ROWS = SC_Q / SC_WARPS;  // rows a warp selects
 
-// Accumulate squared distances between this thread's query and TP database
-// points starting at p0, over all d dimensions.
-__device__ __forceinline__ void tile_distances(const float* __restrict__ X, int64_t n, int d,
-                                               int64_t qi, bool qvalid, int64_t p0, float* s_db,
-                                               float (&acc)[TP], const float* __restrict__ Q) {
-#pragma unroll
-    for (int p = 0; p < TP; ++p) acc[p] = 0.f;
-    for (int c0 = 0; c0 < d; c0 += DC) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < TP * DC; t += blockDim.x) {
-            const int p = t / DC, cc = t % DC;
-            const int64_t gp = p0 + p;
-            const int gc = c0 + cc;
-            s_db[t] = (gp < n && gc < d) ? X[gp * d + gc] : 0.f;
-        }
-        __syncthreads();
-        float qv[DC];
-#pragma unroll
-        for (int cc = 0; cc < DC; ++cc) qv[cc] = (qvalid && c0 + cc < d) ? Q[qi * d + c0 + cc] : 0.f;
-        // fully unrolled so that acc stays in registers; dimensions are added
-        // in order (beyond d both sides are 0 and the fma leaves a unchanged)
-#pragma unroll
-        for (int p = 0; p < TP; ++p) {
-            float a = acc[p];
-#pragma unroll
-            for (int cc = 0; cc < DC; cc += 4) {
-                const float4 v = *reinterpret_cast<const float4*>(&s_db[p * DC + cc]);
-                float df = qv[cc] - v.x;
-                a = fmaf(df, df, a);
-                df = qv[cc + 1] - v.y;
-                a = fmaf(df, df, a);
-                df = qv[cc + 2] - v.z;
-                a = fmaf(df, df, a);
-                df = qv[cc + 3] - v.w;
-                a = fmaf(df, df, a);
-            }
-            acc[p] = a;
-        }
-    }
+struct ScanArgs {
+    const float* X;          // n x d database
+    int64_t n;
+    int d;
+    int k;
+    const float* Q;          // query matrix (X itself unless `separate`)
+    bool separate;           // Q is another matrix: no self to exclude
+    const int64_t* rows;     // query rows of Q: rows[r], or rows32[r], or r
+    const int32_t* rows32;
+    int64_t n_rows;
+    int64_t chunk;           // points per blockIdx.y (a multiple of SC_P)
+    const float* ub;         // see launch_knn_exact_rows_n (nullable)
+    // nearest: row r's list goes to row out_row(r) of idx/dist, or (partial)
+    // to list blockIdx.y of row r as squared distances
+    int32_t* idx;
+    float* dist;
+    bool partial;
+    bool by_query;           // out_row = the query row instead of r
+    // ranks: targets and their squared distances (n_rows x k), counts added to
+    const int32_t* tgt;
+    const float* td;
+    int32_t* cnt;
+};
+
+static size_t scan_smem(int d, int k) {
+    const int qd = d <= 2 * SC_DC ? d : 2 * SC_DC, kl = k <= 16 ? 16 : 32;
+    return size_t(2) * SC_DC * SC_PITCH * 4 + size_t(qd) * SC_QPITCH * 8 + size_t(SC_Q) * SC_PITCH * 4 +
+           size_t(SC_Q) * kl * 8 + (SC_Q * 4);
 }
 
-// Query rows: rows[r] (int64), or rows32[r] (int32), or r.  With n_rows_dev
-// the number of rows is read on the device (blocks past it exit at once) and
-// results go to row rows32[r] of the outputs instead of row r.
-//
-// With p_end > 0 the scan covers only database points [p_begin, p_end) and the
-// k best of that range are written as partial list blockIdx.y of row r
-// (idx_out/dist_out + (blockIdx.y * n_rows + r) * k, squared distances).
-//
-// With ub, ub[qi * k + k - 1] is the distance (FP32, square-rooted) of the
-// k-th of k distinct points other than qi, or INFINITY; only points at most
-// that far are kept (the k nearest all are), so lists may end early with
-// index -1.
-template <int K>
-__global__ void __launch_bounds__(KNN_THREADS)
-knn_exact_kernel(const float* __restrict__ X, int64_t n, int d, int k,
-                 const int64_t* __restrict__ rows, int64_t n_rows, int32_t* __restrict__ idx_out,
-                 float* __restrict__ dist_out, int write_sqrt, const int32_t* __restrict__ rows32,
-                 const int32_t* __restrict__ n_rows_dev, int64_t chunk = 0, const float* __restrict__ Qx = nullptr,
-                 const float* __restrict__ ub = nullptr) {
-    // queries come from Qx (a separate matrix, no self to exclude) or from X
-    const float* Q = Qx ? Qx : X;
-    const int64_t self_off = Qx ? -1 : 0;
-    __shared__ __align__(16) float s_db[TP * DC];
-    if (n_rows_dev) {
-        n_rows = *n_rows_dev;
-        if (int64_t(blockIdx.x) * KNN_THREADS >= n_rows) return;  // whole block idle
-    }
-    const int64_t r = int64_t(blockIdx.x) * KNN_THREADS + threadIdx.x;
-    const bool valid = r < n_rows;
-    const int64_t qi = valid ? (rows ? rows[r] : (rows32 ? int64_t(rows32[r]) : r)) : 0;
-    int64_t orow = (n_rows_dev && !chunk) ? qi : r;
-    int64_t p_begin = 0, p_end = n;
-    if (chunk) {
-        p_begin = int64_t(blockIdx.y) * chunk;
-        p_end = p_begin + chunk < n ? p_begin + chunk : n;
-        orow = int64_t(blockIdx.y) * n_rows + r;
-    }
-    // admission bound: the square of the k-th listed distance, rounded up past
-    // the rounding of the square root and of this square, plus the smallest
-    // normal number so that a k-th distance of 0 (k or more exact copies of
-    // the query) still admits the points at distance 0 (the test is strict)
-    float T = INFINITY;
-    if (ub && valid) {
-        const float u = ub[qi * k + k - 1];
-        T = fmaf(u * u, 1.0f + 1e-6f, 1.17549435e-38f);
-        if (!(T < INFINITY)) T = INFINITY;
-    }
-    float D[K];
-    int32_t I[K];
-#pragma unroll
-    for (int s = 0; s < K; ++s) {
-        D[s] = T;
-        I[s] = -1;
-    }
-    float acc[TP];
-    for (int64_t p0 = p_begin; p0 < p_end; p0 += TP) {
-        tile_distances(X, p_end, d, qi, valid, p0, s_db, acc, Q);
-        const int64_t self = self_off ? int64_t(-1) : qi;
-#pragma unroll
-        for (int p = 0; p < TP; ++p) {
-            const int64_t gp = p0 + p;
-            if (acc[p] < D[K - 1] && gp < p_end && gp != self) topk_insert<K>(D, I, acc[p], int32_t(gp));
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// RANK = false: the k nearest of every query row in the chunk.  RANK = true:
+// for every target s of row r, the number of points of the chunk that precede
+// it in the FP32 (distance, index) order.
+template <bool RANK>
+__global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
+    extern __shared__ __align__(16) unsigned char sc_raw[];
+    const int d = A.d, k = A.k, kl = k <= 16 ? 16 : 32;
+    const bool q_all = d <= 2 * SC_DC;  // the queries stay in shared memory
+    float* s_x = reinterpret_cast<float*>(sc_raw);                            // [2][SC_DC][SC_PITCH]
+    float2* s_q = reinterpret_cast<float2*>(s_x + 2 * SC_DC * SC_PITCH);      // [dims][SC_QPITCH], (-q, -q)
+    float* s_d = reinterpret_cast<float*>(s_q + (q_all ? d : 2 * SC_DC) * SC_QPITCH);  // [SC_Q][SC_PITCH]
+    float* s_ld = s_d + SC_Q * SC_PITCH;                                      // [SC_Q][kl] list (or target) distances
+    int32_t* s_li = reinterpret_cast<int32_t*>(s_ld + SC_Q * kl);             // [SC_Q][kl] their indices
+    int32_t* s_qi = s_li + SC_Q * kl;                                         // [SC_Q] point excluded (-1: none)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx = tid & 15, ty = tid >> 4;
+    const int64_t r0 = int64_t(blockIdx.x) * SC_Q;
+    const int64_t p_begin = int64_t(blockIdx.y) * A.chunk;
+    const int64_t p_end = p_begin + A.chunk < A.n ? p_begin + A.chunk : A.n;
+    auto query_of = [&](int q) -> int64_t {
+        const int64_t r = r0 + q < A.n_rows ? r0 + q : A.n_rows - 1;
+        return A.rows ? A.rows[r] : (A.rows32 ? int64_t(A.rows32[r]) : r);
+    };
+    // dimensions [c0, c0 + cc) of the queries, negated and doubled
+    auto load_q = [&](int c0, int cc, float2* dst) {
+        for (int t = tid; t < SC_Q * ((cc + 7) & ~7); t += SC_THREADS) {
+            const int c = (t & 7) | ((t >> 9) << 3), q = (t >> 3) & (SC_Q - 1);
+            if (c < cc) {
+                const float v = -A.Q[query_of(q) * d + c0 + c];
+                dst[c * SC_QPITCH + q] = make_float2(v, v);
+            }
+        }
+    };
+    static_assert(SC_Q * 8 == 512, "load_q index split");
+    for (int t = tid; t < SC_Q * kl; t += SC_THREADS) {
+        const int q = t / kl, s = t - q * kl;
+        if (RANK) {
+            const bool in = s < k && r0 + q < A.n_rows;
+            s_ld[t] = in ? A.td[(r0 + q) * k + s] : -1.f;
+            s_li[t] = in ? A.tgt[(r0 + q) * k + s] : -1;
+        } else {
+            // admission bound: the square of the k-th listed distance, rounded
+            // up past the rounding of the square root and of this square, plus
+            // the smallest normal number so that a k-th distance of 0 (k or
+            // more exact copies of the query) still admits the points at
+            // distance 0 (the test is strict)
+            float T = INFINITY;
+            if (A.ub) {
+                const float u = A.ub[query_of(q) * k + k - 1];
+                T = fmaf(u * u, 1.0f + 1e-6f, 1.17549435e-38f);
+                if (!(T < INFINITY)) T = INFINITY;
+            }
+            s_ld[t] = T;
+            s_li[t] = INT32_MAX;
         }
     }
-    if (valid) {
+    if (tid < SC_Q) s_qi[tid] = A.separate ? -1 : int32_t(query_of(tid));
+    const int nch = (d + SC_DC - 1) / SC_DC;
+    const int64_t tiles = p_end > p_begin ? (p_end - p_begin + SC_P - 1) / SC_P : 0;
+    const int64_t stages = tiles * nch;
+    if (q_all) load_q(0, d, s_q);
+    // a warp copies 8 dimensions of 4 points per instruction: whole sectors in
+    // global memory, distinct banks in shared memory.  Points past the chunk
+    // repeat its last point (their distances are not looked at).
+    auto load_x = [&](int64_t st) {
+        const int64_t tile = st / nch;
+        const int c0 = int(st - tile * nch) * SC_DC;
+        const int cc = d - c0 < SC_DC ? d - c0 : SC_DC;
+        const int64_t p0 = p_begin + tile * SC_P;
+        float* dst = s_x + (st & 1) * SC_DC * SC_PITCH;
+        const int cl = tid & 7, pl = tid >> 3;
 #pragma unroll
-        for (int s = 0; s < K; ++s) {
-            if (s < k) {
-                idx_out[orow * k + s] = I[s];
-                dist_out[orow * k + s] = write_sqrt ? sqrtf(D[s]) : D[s];
+        for (int pb = 0; pb < SC_P; pb += SC_THREADS / 8) {
+            const int p = pb + pl;
+            const int64_t gp = p0 + p < p_end ? p0 + p : p_end - 1;
+            const float* src = A.X + gp * d + c0;
+#pragma unroll
+            for (int cb = 0; cb < SC_DC; cb += 8) {
+                const int c = cb + cl;
+                if (c < cc)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(
+                                     __cvta_generic_to_shared(dst + c * SC_PITCH + p))),
+                                 "l"(src + c)
+                                 : "memory");
             }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (!q_all) load_q(c0, cc, s_q + (st & 1) * SC_DC * SC_QPITCH);
+    };
+    uint64_t acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    if (stages > 0) load_x(0);
+    int ch = 0;
+    int64_t p0 = p_begin;
+    for (int64_t st = 0; st < stages; ++st) {
+        if (st + 1 < stages) {
+            load_x(st + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int c0 = ch * SC_DC;
+        const int cc = d - c0 < SC_DC ? d - c0 : SC_DC;
+        const float* xs = s_x + (st & 1) * SC_DC * SC_PITCH + 4 * tx;
+        const float2* qs = s_q + (q_all ? c0 : int(st & 1) * SC_DC) * SC_QPITCH + 4 * ty;
+#pragma unroll 4
+        for (int c = 0; c < cc; ++c) {
+            const ulonglong2 xa = *reinterpret_cast<const ulonglong2*>(xs + c * SC_PITCH);
+            const ulonglong2 xb = *reinterpret_cast<const ulonglong2*>(xs + c * SC_PITCH + 64);
+            const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(qs + c * SC_QPITCH);
+            const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(qs + c * SC_QPITCH + 2);
+            const uint64_t xv[4] = {xa.x, xa.y, xb.x, xb.y}, qv[4] = {qa.x, qa.y, qb.x, qb.y};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint64_t df = add2(xv[j], qv[i]);
+                    acc[i][j] = fma2(df, df, acc[i][j]);
+                }
+        }
+        if (++ch == nch) {  // the tile is complete
+            ch = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float* row = s_d + (4 * ty + i) * SC_PITCH + 4 * tx;
+                *reinterpret_cast<ulonglong2*>(row) = make_ulonglong2(acc[i][0], acc[i][1]);
+                *reinterpret_cast<ulonglong2*>(row + 64) = make_ulonglong2(acc[i][2], acc[i][3]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+            }
+            __syncthreads();
+            const int64_t left = p_end - p0;
+            for (int rr = 0; rr < SC_ROWS; ++rr) {
+                const int q = warp * SC_ROWS + rr;
+                const float4 v4 = *reinterpret_cast<const float4*>(s_d + q * SC_PITCH + 4 * lane);
+                float v[4] = {v4.x, v4.y, v4.z, v4.w};
+                const int64_t self = s_qi[q] - p0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (4 * lane + j >= left || 4 * lane + j == self) v[j] = __int_as_float(0x7fc00000);  // compares false
+                float* ld = s_ld + q * kl;
+                int32_t* li = s_li + q * kl;
+                const int32_t gp = int32_t(p0) + 4 * lane;
+                if constexpr (RANK) {
+                    const float tl = lane < k ? ld[lane] : -1.f;
+                    float tmax = tl;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+                    if (!__any_sync(0xffffffffu, v[0] <= tmax || v[1] <= tmax || v[2] <= tmax || v[3] <= tmax)) continue;
+                    const int32_t jl = lane < k ? li[lane] : -1;
+                    int32_t mine = 0;
+                    for (int s = 0; s < k; ++s) {
+                        const float t = __shfl_sync(0xffffffffu, tl, s);
+                        const int32_t tj = __shfl_sync(0xffffffffu, jl, s);
+                        int c = 0;
+                        if (tj < p0) {  // every point of the tile comes after the target's index
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) c += v[j] < t;
+                        } else if (tj >= p0 + SC_P) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) c += v[j] <= t;
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) c += v[j] < t || (v[j] == t && gp + j < tj);
+                        }
+                        c = __reduce_add_sync(0xffffffffu, c);
+                        if (lane == s) mine = c;
+                    }
+                    // the count of target s of row r0 + q
+                    if (lane < k && mine && r0 + q < A.n_rows) atomicAdd(&A.cnt[(r0 + q) * k + lane], mine);
+                } else {
+                    const float thr = ld[k - 1];
+                    const float m = fminf(fminf(v[0], v[1]), fminf(v[2], v[3]));  // ignores the NaN marks
+                    if (!__any_sync(0xffffffffu, m < thr)) continue;
+                    float D = lane < kl ? ld[lane] : INFINITY;
+                    int32_t I = lane < kl ? li[lane] : INT32_MAX;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        unsigned todo = __ballot_sync(0xffffffffu, v[j] < thr);
+                        while (todo) {
+                            const int src = __ffs(todo) - 1;
+                            todo &= todo - 1;
+                            const float cd = __shfl_sync(0xffffffffu, v[j], src);
+                            const int32_t ci = int32_t(p0) + 4 * src + j;
+                            const bool less = D < cd || (D == cd && I < ci);
+                            const int pos = __popc(__ballot_sync(0xffffffffu, less));
+                            if (pos >= k) continue;  // overtaken by this tile's other points
+                            const float Du = __shfl_up_sync(0xffffffffu, D, 1);
+                            const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
+                            if (lane > pos) {
+                                D = Du;
+                                I = Iu;
+                            }
+                            if (lane == pos) {
+                                D = cd;
+                                I = ci;
+                            }
+                        }
+                    }
+                    if (lane < kl) {
+                        ld[lane] = D;
+                        li[lane] = I;
+                    }
+                    __syncwarp();
+                }
+            }
+            p0 += SC_P;
+        }
+        __syncthreads();  // the buffer and the tile may be overwritten
+    }
+    if constexpr (!RANK) {
+        __syncthreads();
+        for (int t = tid; t < SC_Q * k; t += SC_THREADS) {
+            const int q = t / k, s = t - q * k;
+            const int64_t r = r0 + q;
+            if (r >= A.n_rows) continue;
+            const int64_t o =
+                A.partial ? int64_t(blockIdx.y) * A.n_rows + r : (A.by_query ? query_of(q) : r);
+            const float D = s_ld[q * kl + s];
+            const int32_t I = s_li[q * kl + s];
+            A.idx[o * k + s] = I == INT32_MAX ? -1 : I;
+            A.dist[o * k + s] = A.partial ? D : sqrtf(D);
         }
     }
 }
@@ -147,7 +318,7 @@ __device__ __forceinline__ bool lex_less(float a, int32_t i, float b, int32_t j)
 template <int K>
 __global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const float* __restrict__ pd2,
                                       int64_t cnt, int C, int k, const int32_t* __restrict__ rows32,
-                                      int32_t* __restrict__ idx_out, float* __restrict__ dist_out) {
+                                      int32_t none, int32_t* __restrict__ idx_out, float* __restrict__ dist_out) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
     for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < cnt; r += warps) {
@@ -189,7 +360,7 @@ __global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const fl
             }
           }
         }
-        const int64_t row = rows32[r];
+        const int64_t row = rows32 ? int64_t(rows32[r]) : r;
         for (int s = 0; s < k; ++s) {
             float bd = D[0];
             int32_t bi = I[0];
@@ -203,7 +374,7 @@ __global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const fl
                 }
             }
             if (lane == 0) {
-                idx_out[row * k + s] = bi;
+                idx_out[row * k + s] = bi == INT32_MAX ? none : bi;
                 dist_out[row * k + s] = sqrtf(bd);
             }
             if (I[0] == bi && D[0] == bd) {  // the owner pops its head
@@ -219,142 +390,174 @@ __global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const fl
     }
 }
 
-int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, const int32_t* rows32,
-                            const int32_t* n_rows_dev, int64_t cnt, int32_t* idx_out, float* dist_out,
-                            cudaStream_t st, void* part_scratch, size_t part_bytes) {
-    if (cnt <= 0) return DRGB_OK;
-    const int row_blocks = int((cnt + KNN_THREADS - 1) / KNN_THREADS);
-    int64_t C = (8 * int64_t(c->num_sms) + row_blocks - 1) / row_blocks;
-    const int64_t max_c = (n + 127) / 128;               // at least 128 points per chunk
-    if (C > max_c) C = max_c;
-    if (C > 1024) C = 1024;
-    const int64_t fit_c = part_scratch ? int64_t(part_bytes / 2 / (size_t(cnt) * k * 4 + 256)) : 0;
-    if (C > fit_c) C = fit_c;                            // partial lists must fit the scratch
-    if (C <= 1) {
-        const int blocks = row_blocks;
-        if (k <= 16)
-            knn_exact_kernel<16><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, cnt, idx_out, dist_out, 1,
-                                                                rows32, n_rows_dev, 0, nullptr, dist_out);
-        else
-            knn_exact_kernel<32><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, cnt, idx_out, dist_out, 1,
-                                                                rows32, n_rows_dev, 0, nullptr, dist_out);
-        DRGB_CHECK_LAUNCH(c);
-        return DRGB_OK;
+// Database chunks of a scan: enough (row block, chunk) CTAs for one to four
+// whole waves of two CTAs per SM, whichever leaves the fewest idle, chunks of
+// at least two tiles, the partial lists within part_bytes.
+static int scan_chunks(const Ctx* c, int64_t n_rows, int64_t n, int k, size_t part_bytes, bool lists) {
+    const int64_t blocks = (n_rows + SC_Q - 1) / SC_Q, slots = 2 * int64_t(c->num_sms);
+    int64_t best = 1;
+    double best_use = 0.0;
+    for (int w = 1; w <= 4; ++w) {
+        const int64_t C = slots * w / blocks;
+        const double use = double(blocks * C) / double(slots * w);
+        if (C >= 1 && use > best_use + 0.02) {
+            best = C;
+            best_use = use;
+        }
     }
-    Carve cv(part_scratch);
-    int32_t* pidx = cv.take<int32_t>(size_t(cnt) * C * k);
-    float* pd2 = cv.take<float>(size_t(cnt) * C * k);
-    const int64_t chunk = (n + C - 1) / C;
-    dim3 grid(row_blocks, unsigned(C));
-    if (k <= 16)
-        knn_exact_kernel<16><<<grid, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, cnt, pidx, pd2, 0, rows32,
-                                                          nullptr, chunk, nullptr, dist_out);
-    else
-        knn_exact_kernel<32><<<grid, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, cnt, pidx, pd2, 0, rows32,
-                                                          nullptr, chunk, nullptr, dist_out);
+    const int64_t most = n / (2 * SC_P);
+    if (best > most) best = most;
+    if (best > 128) best = 128;
+    if (lists) {
+        const int64_t fit = part_bytes > 1024 ? int64_t((part_bytes / 2 - 512) / (size_t(n_rows) * k * 4)) : 0;
+        if (best > fit) best = fit;
+    }
+    return best > 1 ? int(best) : 1;
+}
+
+size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
+    const int C = scan_chunks(c, n_rows, n, k, ~size_t(0) >> 1, true);
+    return C > 1 ? 2 * (size_t(n_rows) * C * k * 4 + 512) : 0;
+}
+
+template <bool RANK>
+static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
+    A.chunk = ((A.n + C - 1) / C + SC_P - 1) / SC_P * SC_P;
+    const size_t smem = scan_smem(A.d, A.k);
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<RANK>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const dim3 grid(unsigned((A.n_rows + SC_Q - 1) / SC_Q), unsigned((A.n + A.chunk - 1) / A.chunk));
+    scan_kernel<RANK><<<grid, SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
-    return launch_merge_partials(c, pidx, pd2, cnt, int(C), k, rows32, idx_out, dist_out, st);
+    return DRGB_OK;
+}
+
+// The k nearest of the queries of A, through partial lists when `part` holds
+// them; `none`: the index written where a row has fewer than k.
+static int scan_nearest(Ctx* c, ScanArgs& A, int32_t* idx_out, float* dist_out, void* part, size_t part_bytes,
+                        int32_t none, cudaStream_t st) {
+    if (A.n_rows <= 0) return DRGB_OK;
+    const int C = scan_chunks(c, A.n_rows, A.n, A.k, part ? part_bytes : 0, true);
+    if (C <= 1) {
+        A.idx = idx_out;
+        A.dist = dist_out;
+        A.partial = false;
+        return scan_launch<false>(c, A, 1, st);
+    }
+    Carve cv(part);
+    A.idx = cv.take<int32_t>(size_t(A.n_rows) * C * A.k);
+    A.dist = cv.take<float>(size_t(A.n_rows) * C * A.k);
+    A.partial = true;
+    int rc = scan_launch<false>(c, A, C, st);
+    if (rc) return rc;
+    const int lists = int((A.n + A.chunk - 1) / A.chunk);
+    return launch_merge_partials(c, A.idx, A.dist, A.n_rows, lists, A.k, A.by_query ? A.rows32 : nullptr, idx_out,
+                                 dist_out, st, none);
+}
+
+int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, const int32_t* rows32, int64_t cnt,
+                            int32_t* idx_out, float* dist_out, cudaStream_t st, void* part_scratch,
+                            size_t part_bytes) {
+    ScanArgs A = {};
+    A.X = A.Q = X;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.rows32 = rows32;
+    A.n_rows = cnt;
+    A.by_query = true;
+    A.ub = dist_out;
+    return scan_nearest(c, A, idx_out, dist_out, part_scratch, part_bytes, INT32_MAX, st);
 }
 
 int launch_merge_partials(Ctx* c, const int32_t* pidx, const float* pd2, int64_t cnt, int C, int k,
-                          const int32_t* rows32, int32_t* idx_out, float* dist_out, cudaStream_t st) {
+                          const int32_t* rows32, int32_t* idx_out, float* dist_out, cudaStream_t st, int32_t none) {
     if (cnt <= 0) return DRGB_OK;
     const int mb = grid_for(cnt, 4, c->num_sms * 8);   // one warp per row, 4 warps per CTA
     if (k <= 16)
-        merge_partials_kernel<16><<<mb, 128, 0, st>>>(pidx, pd2, cnt, C, k, rows32, idx_out, dist_out);
+        merge_partials_kernel<16><<<mb, 128, 0, st>>>(pidx, pd2, cnt, C, k, rows32, none, idx_out, dist_out);
     else
-        merge_partials_kernel<32><<<mb, 128, 0, st>>>(pidx, pd2, cnt, C, k, rows32, idx_out, dist_out);
+        merge_partials_kernel<32><<<mb, 128, 0, st>>>(pidx, pd2, cnt, C, k, rows32, none, idx_out, dist_out);
     DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
 
 int launch_knn_query(Ctx* c, const float* Q, int64_t nq, const float* X, int64_t n, int d, int k,
-                     int32_t* idx_out, float* dist_out, cudaStream_t st) {
-    const int blocks = int((nq + KNN_THREADS - 1) / KNN_THREADS);
-    if (blocks < 1) return DRGB_OK;
-    if (k <= 16)
-        knn_exact_kernel<16><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, nq, idx_out, dist_out, 1, nullptr,
-                                                            nullptr, 0, Q);
-    else
-        knn_exact_kernel<32><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, nullptr, nq, idx_out, dist_out, 1, nullptr,
-                                                            nullptr, 0, Q);
-    DRGB_CHECK_LAUNCH(c);
-    return DRGB_OK;
+                     int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes) {
+    ScanArgs A = {};
+    A.X = X;
+    A.Q = Q;
+    A.separate = true;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.n_rows = nq;
+    return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
 }
 
 int launch_knn_exact(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows,
-                     int64_t n_rows, int32_t* idx_out, float* dist_out, bool write_sqrt,
-                     cudaStream_t st) {
-    const int blocks = int((n_rows + KNN_THREADS - 1) / KNN_THREADS);
-    if (blocks < 1) return DRGB_OK;
-    if (k <= 16)
-        knn_exact_kernel<16><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, rows, n_rows, idx_out, dist_out,
-                                                            write_sqrt, nullptr, nullptr);
-    else
-        knn_exact_kernel<32><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, rows, n_rows, idx_out, dist_out,
-                                                            write_sqrt, nullptr, nullptr);
-    DRGB_CHECK_LAUNCH(c);
-    return DRGB_OK;
+                     int64_t n_rows, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
+                     size_t part_bytes) {
+    ScanArgs A = {};
+    A.X = A.Q = X;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.rows = rows;
+    A.n_rows = n_rows;
+    return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
 }
 
-// For query row r (point qi) and its k targets tgt[r][s], count the points l != qi
-// that precede the target in the FP32 (distance, index) order: rank - 1.
-template <int K>
-__global__ void __launch_bounds__(KNN_THREADS)
-rank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const int64_t* __restrict__ rows,
-            int64_t n_rows, const int32_t* __restrict__ tgt, int64_t* __restrict__ excess_out) {
-    __shared__ __align__(16) float s_db[TP * DC];
-    const int64_t r = int64_t(blockIdx.x) * KNN_THREADS + threadIdx.x;
-    const bool valid = r < n_rows;
-    const int64_t qi = valid ? (rows ? rows[r] : r) : 0;
-    float td[K];
-    int32_t tj[K];
-    int32_t cnt[K];
-#pragma unroll
-    for (int s = 0; s < K; ++s) {
-        tj[s] = (valid && s < k) ? tgt[r * k + s] : -1;
-        cnt[s] = 0;
-        td[s] = -1.f;  // filled during the scan when the target itself is met
-    }
-    // pass 1: distances to the targets (same formula and order as the scan)
-    for (int s = 0; s < K; ++s) {
-        if (s >= k || tj[s] < 0) continue;
-        float a = 0.f;
-        for (int cc = 0; cc < d; ++cc) {
-            const float df = X[qi * d + cc] - X[int64_t(tj[s]) * d + cc];
-            a = fmaf(df, df, a);
+// Squared distances of the targets, by the scan's formula and order (-1 for a
+// missing target, which then precedes nothing).
+__global__ void target_dist_kernel(const float* __restrict__ X, int d, int k, const int64_t* __restrict__ rows,
+                                   int64_t n_rows, const int32_t* __restrict__ tgt, float* __restrict__ td,
+                                   int32_t* __restrict__ cnt) {
+    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_rows * k;
+         t += int64_t(gridDim.x) * blockDim.x) {
+        const int64_t r = t / k, qi = rows ? rows[r] : r;
+        const int32_t j = tgt[t];
+        float a = -1.f;
+        if (j >= 0) {
+            a = 0.f;
+#pragma unroll 8
+            for (int c = 0; c < d; ++c) {
+                const float df = X[qi * d + c] - X[int64_t(j) * d + c];
+                a = fmaf(df, df, a);
+            }
         }
-        td[s] = a;
+        td[t] = a;
+        cnt[t] = 0;
     }
-    float acc[TP];
-    for (int64_t p0 = 0; p0 < n; p0 += TP) {
-        tile_distances(X, n, d, qi, valid, p0, s_db, acc, X);
-#pragma unroll
-        for (int p = 0; p < TP; ++p) {
-            const int64_t gp = p0 + p;
-            if (gp >= n || gp == qi) continue;
-#pragma unroll
-            for (int s = 0; s < K; ++s)
-                cnt[s] += (acc[p] < td[s]) || (acc[p] == td[s] && gp < tj[s]);
-        }
-    }
-    if (valid) {
+}
+
+__global__ void rank_excess_kernel(const int32_t* __restrict__ cnt, const int32_t* __restrict__ tgt, int64_t n_rows,
+                                   int k, int64_t* __restrict__ excess_out) {
+    for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < n_rows; r += int64_t(gridDim.x) * blockDim.x) {
         int64_t ex = 0;
-#pragma unroll
-        for (int s = 0; s < K; ++s)
-            if (s < k && tj[s] >= 0 && cnt[s] + 1 > k) ex += cnt[s] + 1 - k;
+        for (int s = 0; s < k; ++s)
+            if (tgt[r * k + s] >= 0 && cnt[r * k + s] + 1 > k) ex += cnt[r * k + s] + 1 - k;
         excess_out[r] = ex;
     }
 }
 
-int launch_rank(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows,
-                int64_t n_rows, const int32_t* tgt, int64_t* excess_out, cudaStream_t st) {
-    const int blocks = int((n_rows + KNN_THREADS - 1) / KNN_THREADS);
-    if (blocks < 1) return DRGB_OK;
-    if (k <= 16)
-        rank_kernel<16><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, rows, n_rows, tgt, excess_out);
-    else
-        rank_kernel<32><<<blocks, KNN_THREADS, 0, st>>>(X, n, d, k, rows, n_rows, tgt, excess_out);
+int launch_rank(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows, int64_t n_rows,
+                const int32_t* tgt, float* td, int32_t* cnt, int64_t* excess_out, cudaStream_t st) {
+    if (n_rows <= 0) return DRGB_OK;
+    target_dist_kernel<<<grid_for(n_rows * k, 128, c->num_sms * 16), 128, 0, st>>>(X, d, k, rows, n_rows, tgt, td, cnt);
+    DRGB_CHECK_LAUNCH(c);
+    ScanArgs A = {};
+    A.X = A.Q = X;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.rows = rows;
+    A.n_rows = n_rows;
+    A.tgt = tgt;
+    A.td = td;
+    A.cnt = cnt;
+    int rc = scan_launch<true>(c, A, scan_chunks(c, n_rows, n, k, 0, false), st);
+    if (rc) return rc;
+    rank_excess_kernel<<<grid_for(n_rows, 128, c->num_sms * 8), 128, 0, st>>>(cnt, tgt, n_rows, k, excess_out);
     DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
@@ -394,19 +597,21 @@ int knn_resolve_mode(int64_t n, int d, int k, int mode) {
     return mode;
 }
 
-size_t knn_scratch_bytes(int64_t n, int d, int k, int mode) {
-    (void)k;
+size_t knn_scratch_bytes(const Ctx* c, int64_t n, int d, int k, int mode, size_t* least) {
     const int m = knn_resolve_mode(n, d, k, mode);
-    return (m == 2 || m == 3) ? knn_tc_scratch_bytes(n, d) : 0;
+    const bool tc = m == 2 || m == 3;
+    const size_t b = tc ? knn_tc_scratch_bytes(n, d) : knn_scan_scratch_bytes(c, n, n, k);
+    if (least) *least = tc ? b : 0;
+    return b;
 }
 
 int knn_run(Ctx* c, const float* X, int64_t n, int d, int k, int mode, int32_t* idx_out, float* dist_out,
-            cudaStream_t st, void* scratch, int32_t* defer_rows, int32_t* defer_count) {
+            cudaStream_t st, void* scratch, size_t scratch_bytes, int32_t* defer_rows, int32_t* defer_count) {
     const int m = knn_resolve_mode(n, d, k, mode);
     if (m == 2 || m == 3)
         return knn_tc(c, X, n, d, k, m == 3, idx_out, dist_out, st, scratch, defer_rows, defer_count);
     if (m != 1) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
-    return launch_knn_exact(c, X, n, d, k, nullptr, n, idx_out, dist_out, true, st);
+    return launch_knn_exact(c, X, n, d, k, nullptr, n, idx_out, dist_out, st, scratch, scratch_bytes);
 }
 
 }  // namespace drgb
@@ -417,7 +622,36 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     if (rc) return rc;
     if (mode < 0 || mode > 3) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t bytes = knn_scratch_bytes(n, d, k, mode);
-    if (bytes && (rc = ensure_scratch(c, bytes, st))) return rc;
-    return knn_run(c, X, n, d, k, mode, idx_out, dist_out, st, c->scratch);
+    const int m = knn_resolve_mode(n, d, k, mode);
+    if (m != 1) {
+        size_t least = 0;
+        if ((rc = ensure_scratch(c, knn_scratch_bytes(c, n, d, k, m, &least), st))) return rc;
+        return knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->scratch, c->scratch_bytes);
+    }
+    // The scan's partial lists have a buffer of their own (at most about 20
+    // MB: 64 x 1216 lists), so that scans enqueued on one stream may overlap
+    // other calls' use of the context's scratch on another; scans take turns
+    // at it through an event.  A captured scan runs unsplit, since its graph
+    // may outlive the buffer; so does one that the scratch limit leaves no
+    // room for.
+    size_t want = stream_captures(st) ? 0 : knn_scan_scratch_bytes(c, n, n, k);
+    if (want && c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) want = 0;
+    if (want > c->scan_bytes) {
+        if (c->scan_part) DRGB_CUDA(c, cudaFree(c->scan_part));  // waits for its users
+        c->scan_part = nullptr;
+        c->scan_bytes = 0;
+        if (cudaMalloc(&c->scan_part, want) == cudaSuccess) {
+            c->scan_bytes = want;
+        } else {
+            cudaGetLastError();
+            c->scan_part = nullptr;
+            want = 0;
+        }
+    }
+    if (!want) return knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
+    if (!c->scan_ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&c->scan_ev, cudaEventDisableTiming));
+    DRGB_CUDA(c, cudaStreamWaitEvent(st, c->scan_ev, 0));
+    rc = knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, c->scan_part, want);
+    DRGB_CUDA(c, cudaEventRecord(c->scan_ev, st));
+    return rc;
 }

@@ -1395,8 +1395,7 @@ static int knn_tc_impl(Ctx* c, const float* X, int64_t n, int d, int k, int32_t*
         DRGB_CHECK_LAUNCH(c);
         rc = launch_merge_partials(c, pidx, pd2, cnt, int(nchunk), k, fail_rows, idx_out, dist_out, st);
     } else {
-        rc = launch_knn_exact_rows_n(c, X, n, d, k, fail_rows, fail_count, cnt, idx_out, dist_out, st, part,
-                                     TC_PART_BYTES);
+        rc = launch_knn_exact_rows_n(c, X, n, d, k, fail_rows, cnt, idx_out, dist_out, st, part, TC_PART_BYTES);
     }
     if (rc) return rc;
     return stage_mark(c, 10, st);
