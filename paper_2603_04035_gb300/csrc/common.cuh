@@ -22,9 +22,9 @@ struct Ctx {
     void* scratch = nullptr;      // grown on demand, 256-byte aligned carve-outs
     size_t scratch_bytes = 0;
     size_t scratch_limit = 0;     // largest scratch the context may allocate (0 = no limit)
-    void* scan_part = nullptr;    // partial lists of drgb_knn_graph's scans (see there)
-    size_t scan_bytes = 0;
-    cudaEvent_t scan_ev = nullptr;  // the last such scan
+    void* knn_buf = nullptr;      // buffer of drgb_knn_graph's scans and wide products (see there)
+    size_t knn_buf_bytes = 0;
+    cudaEvent_t knn_ev = nullptr;  // its last use
     int* d_status = nullptr;      // device status word (0 = ok, else DRGB_ERR_*)
     unsigned long long* d_counter = nullptr;  // [0] uncertified rows, [4] k-NN tile products computed
     int64_t knn_tiles_total = 0;              // tile products of a full scan (last tensor-core k-NN)

@@ -308,8 +308,8 @@ int drgb_ctx_destroy(drgb_ctx* c) {
     cudaDeviceSynchronize();
     if (c->epoch_exec) cudaGraphExecDestroy(c->epoch_exec);
     if (c->scratch) cudaFree(c->scratch);
-    if (c->scan_part) cudaFree(c->scan_part);
-    if (c->scan_ev) cudaEventDestroy(c->scan_ev);
+    if (c->knn_buf) cudaFree(c->knn_buf);
+    if (c->knn_ev) cudaEventDestroy(c->knn_ev);
     if (c->d_status) cudaFree(c->d_status);
     for (auto& e : c->stage_ev)
         if (e) cudaEventDestroy(e);

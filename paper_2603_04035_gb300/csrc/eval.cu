@@ -42,7 +42,8 @@ static int eval_common(Ctx* c, const float* X, const float* Y, int64_t n, int d,
     const size_t bytes = Carve::round(m * 8) + 2 * Carve::round(m * k * 4) * 2 +
                          Carve::round(m * 8) + Carve::round(m * 4) + 4096;
     const size_t part_off = Carve::round(bytes);
-    size_t total = part_off + knn_scan_scratch_bytes(c, m, n, k);
+    const size_t px = knn_queries_scratch_bytes(c, m, n, d, k), py = knn_queries_scratch_bytes(c, m, n, 2, k);
+    size_t total = part_off + (px > py ? px : py);
     int rc = ensure_scratch_within(c, &total, bytes, st);
     if (rc) return rc;
     const size_t part_bytes = total > part_off ? total - part_off : 0;
@@ -57,10 +58,10 @@ static int eval_common(Ctx* c, const float* X, const float* Y, int64_t n, int d,
     int32_t* hits = cv.take<int32_t>(m);
     strided_rows_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(rows, m, n);
     DRGB_CHECK_LAUNCH(c);
-    rc = launch_knn_exact(c, Y, n, 2, k, rows, m, ny, dy, st, part, part_bytes);
+    rc = knn_queries(c, Y, m, false, rows, Y, n, 2, k, ny, dy, st, part, part_bytes);
     if (rc) return rc;
     if (want_recall) {
-        rc = launch_knn_exact(c, X, n, d, k, rows, m, nx, dx, st, part, part_bytes);
+        rc = knn_queries(c, X, m, false, rows, X, n, d, k, nx, dx, st, part, part_bytes);
         if (rc) return rc;
         intersect_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(nx, ny, m, k, hits);
         DRGB_CHECK_LAUNCH(c);
@@ -109,7 +110,8 @@ static int eval_heldout(Ctx* c, const float* Xt, const float* Yt, int64_t n, con
     const size_t bytes = Carve::round(m * 8) + Carve::round(m * d * 4) + Carve::round(m * 8) +
                          4 * Carve::round(m * k * 4) + Carve::round(m * 4) + 4096;
     const size_t part_off = Carve::round(bytes);
-    size_t total = part_off + knn_scan_scratch_bytes(c, m, n, k);
+    const size_t px = knn_queries_scratch_bytes(c, m, n, d, k), py = knn_queries_scratch_bytes(c, m, n, 2, k);
+    size_t total = part_off + (px > py ? px : py);
     int rc = ensure_scratch_within(c, &total, bytes, st);
     if (rc) return rc;
     const size_t part_bytes = total > part_off ? total - part_off : 0;
@@ -129,8 +131,8 @@ static int eval_heldout(Ctx* c, const float* Xt, const float* Yt, int64_t n, con
     DRGB_CHECK_LAUNCH(c);
     gather_rows_kernel<<<grid_for(m * 2, 256, c->num_sms * 8), 256, 0, st>>>(Yn, 2, rows, m, yq);
     DRGB_CHECK_LAUNCH(c);
-    if ((rc = launch_knn_query(c, xq, m, Xt, n, d, k, nx, dx, st, part, part_bytes))) return rc;
-    if ((rc = launch_knn_query(c, yq, m, Yt, n, 2, k, ny, dy, st, part, part_bytes))) return rc;
+    if ((rc = knn_queries(c, xq, m, true, nullptr, Xt, n, d, k, nx, dx, st, part, part_bytes))) return rc;
+    if ((rc = knn_queries(c, yq, m, true, nullptr, Yt, n, 2, k, ny, dy, st, part, part_bytes))) return rc;
     intersect_kernel<<<grid_for(m, 256, c->num_sms * 8), 256, 0, st>>>(nx, ny, m, k, hits);
     DRGB_CHECK_LAUNCH(c);
     std::vector<int32_t> h(m);

@@ -41,17 +41,16 @@ struct ScanArgs {
     int k;
     const float* Q;          // query matrix (X itself unless `separate`)
     bool separate;           // Q is another matrix: no self to exclude
-    const int64_t* rows;     // query rows of Q: rows[r], or rows32[r], or r
-    const int32_t* rows32;
+    const int32_t* list;     // queries scanned: list[r], or r
+    const int64_t* rows;     // query p is row rows[p] of Q, or row p
     int64_t n_rows;
     int64_t chunk;           // points per blockIdx.y (a multiple of SC_P)
     const float* ub;         // see launch_knn_exact_rows_n (nullable)
-    // nearest: row r's list goes to row out_row(r) of idx/dist, or (partial)
-    // to list blockIdx.y of row r as squared distances
+    // nearest: the list of query p goes to row p of idx/dist, or (partial) to
+    // list blockIdx.y of r as squared distances
     int32_t* idx;
     float* dist;
     bool partial;
-    bool by_query;           // out_row = the query row instead of r
     // ranks: targets and their squared distances (n_rows x k), counts added to
     const int32_t* tgt;
     const float* td;
@@ -94,9 +93,13 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     const int64_t r0 = int64_t(blockIdx.x) * SC_Q;
     const int64_t p_begin = int64_t(blockIdx.y) * A.chunk;
     const int64_t p_end = p_begin + A.chunk < A.n ? p_begin + A.chunk : A.n;
-    auto query_of = [&](int q) -> int64_t {
+    auto place_of = [&](int q) -> int64_t {
         const int64_t r = r0 + q < A.n_rows ? r0 + q : A.n_rows - 1;
-        return A.rows ? A.rows[r] : (A.rows32 ? int64_t(A.rows32[r]) : r);
+        return A.list ? int64_t(A.list[r]) : r;
+    };
+    auto query_of = [&](int q) -> int64_t {
+        const int64_t p = place_of(q);
+        return A.rows ? A.rows[p] : p;
     };
     // dimensions [c0, c0 + cc) of the queries, negated and doubled
     auto load_q = [&](int c0, int cc, float2* dst) {
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
             // distance 0 (the test is strict)
             float T = INFINITY;
             if (A.ub) {
-                const float u = A.ub[query_of(q) * k + k - 1];
+                const float u = A.ub[place_of(q) * k + k - 1];
                 T = fmaf(u * u, 1.0f + 1e-6f, 1.17549435e-38f);
                 if (!(T < INFINITY)) T = INFINITY;
             }
@@ -295,8 +298,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
             const int q = t / k, s = t - q * k;
             const int64_t r = r0 + q;
             if (r >= A.n_rows) continue;
-            const int64_t o =
-                A.partial ? int64_t(blockIdx.y) * A.n_rows + r : (A.by_query ? query_of(q) : r);
+            const int64_t o = A.partial ? int64_t(blockIdx.y) * A.n_rows + r : place_of(q);
             const float D = s_ld[q * kl + s];
             const int32_t I = s_li[q * kl + s];
             A.idx[o * k + s] = I == INT32_MAX ? -1 : I;
@@ -450,7 +452,7 @@ static int scan_nearest(Ctx* c, ScanArgs& A, int32_t* idx_out, float* dist_out, 
     int rc = scan_launch<false>(c, A, C, st);
     if (rc) return rc;
     const int lists = int((A.n + A.chunk - 1) / A.chunk);
-    return launch_merge_partials(c, A.idx, A.dist, A.n_rows, lists, A.k, A.by_query ? A.rows32 : nullptr, idx_out,
+    return launch_merge_partials(c, A.idx, A.dist, A.n_rows, lists, A.k, A.list, idx_out,
                                  dist_out, st, none);
 }
 
@@ -462,11 +464,27 @@ int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, con
     A.n = n;
     A.d = d;
     A.k = k;
-    A.rows32 = rows32;
+    A.list = rows32;
     A.n_rows = cnt;
-    A.by_query = true;
     A.ub = dist_out;
     return scan_nearest(c, A, idx_out, dist_out, part_scratch, part_bytes, INT32_MAX, st);
+}
+
+int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t* rows, const float* X, int64_t n,
+                            int d, int k, const int32_t* list, int64_t cnt, int32_t* idx_out, float* dist_out,
+                            cudaStream_t st, void* part, size_t part_bytes) {
+    ScanArgs A = {};
+    A.X = X;
+    A.Q = Q;
+    A.separate = separate;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.list = list;
+    A.rows = rows;
+    A.n_rows = cnt;
+    A.ub = dist_out;
+    return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
 }
 
 int launch_merge_partials(Ctx* c, const int32_t* pidx, const float* pd2, int64_t cnt, int C, int k,
@@ -481,30 +499,30 @@ int launch_merge_partials(Ctx* c, const int32_t* pidx, const float* pd2, int64_t
     return DRGB_OK;
 }
 
-int launch_knn_query(Ctx* c, const float* Q, int64_t nq, const float* X, int64_t n, int d, int k,
-                     int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes) {
+int launch_knn_scan(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
+                    int d, int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes) {
     ScanArgs A = {};
     A.X = X;
     A.Q = Q;
-    A.separate = true;
-    A.n = n;
-    A.d = d;
-    A.k = k;
-    A.n_rows = nq;
-    return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
-}
-
-int launch_knn_exact(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows,
-                     int64_t n_rows, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
-                     size_t part_bytes) {
-    ScanArgs A = {};
-    A.X = A.Q = X;
+    A.separate = separate;
     A.n = n;
     A.d = d;
     A.k = k;
     A.rows = rows;
-    A.n_rows = n_rows;
+    A.n_rows = nq;
     return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
+}
+
+size_t knn_queries_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d, int k) {
+    return knn_wide_preferred(nq, n, d, k) ? knn_wide_scratch_bytes(c, nq, n, d) : knn_scan_scratch_bytes(c, nq, n, k);
+}
+
+int knn_queries(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
+                int d, int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* scratch,
+                size_t scratch_bytes) {
+    if (knn_wide_preferred(nq, n, d, k) && scratch && scratch_bytes >= knn_wide_scratch_bytes(c, nq, n, d))
+        return knn_wide(c, Q, nq, separate, rows, X, n, d, k, idx_out, dist_out, st, scratch);
+    return launch_knn_scan(c, Q, nq, separate, rows, X, n, d, k, idx_out, dist_out, st, scratch, scratch_bytes);
 }
 
 // Squared distances of the targets, by the scan's formula and order (-1 for a
@@ -593,14 +611,16 @@ using namespace drgb;
 namespace drgb {
 
 int knn_resolve_mode(int64_t n, int d, int k, int mode) {
-    if (mode == 0) return knn_tc_preferred(n, d, k) ? 3 : 1;
-    return mode;
+    if (mode != 0) return mode;
+    if (knn_tc_preferred(n, d, k)) return 3;
+    return knn_wide_preferred(n, n, d, k) ? KNN_WIDE : 1;
 }
 
 size_t knn_scratch_bytes(const Ctx* c, int64_t n, int d, int k, int mode, size_t* least) {
     const int m = knn_resolve_mode(n, d, k, mode);
     const bool tc = m == 2 || m == 3;
-    const size_t b = tc ? knn_tc_scratch_bytes(n, d) : knn_scan_scratch_bytes(c, n, n, k);
+    const size_t b = tc ? knn_tc_scratch_bytes(n, d)
+                        : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
     if (least) *least = tc ? b : 0;
     return b;
 }
@@ -610,8 +630,10 @@ int knn_run(Ctx* c, const float* X, int64_t n, int d, int k, int mode, int32_t* 
     const int m = knn_resolve_mode(n, d, k, mode);
     if (m == 2 || m == 3)
         return knn_tc(c, X, n, d, k, m == 3, idx_out, dist_out, st, scratch, defer_rows, defer_count);
-    if (m != 1) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
-    return launch_knn_exact(c, X, n, d, k, nullptr, n, idx_out, dist_out, st, scratch, scratch_bytes);
+    if (m == KNN_WIDE && scratch && scratch_bytes >= knn_wide_scratch_bytes(c, n, n, d))
+        return knn_wide(c, X, n, false, nullptr, X, n, d, k, idx_out, dist_out, st, scratch, defer_rows, defer_count);
+    if (m != 1 && m != KNN_WIDE) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
+    return launch_knn_scan(c, X, n, false, nullptr, X, n, d, k, idx_out, dist_out, st, scratch, scratch_bytes);
 }
 
 }  // namespace drgb
@@ -623,35 +645,34 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     if (mode < 0 || mode > 3) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int m = knn_resolve_mode(n, d, k, mode);
-    if (m != 1) {
-        size_t least = 0;
-        if ((rc = ensure_scratch(c, knn_scratch_bytes(c, n, d, k, m, &least), st))) return rc;
+    if (m == 2 || m == 3) {
+        if ((rc = ensure_scratch(c, knn_scratch_bytes(c, n, d, k, m, nullptr), st))) return rc;
         return knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->scratch, c->scratch_bytes);
     }
-    // The scan's partial lists have a buffer of their own (at most about 20
-    // MB: 64 x 1216 lists), so that scans enqueued on one stream may overlap
-    // other calls' use of the context's scratch on another; scans take turns
-    // at it through an event.  A captured scan runs unsplit, since its graph
-    // may outlive the buffer; so does one that the scratch limit leaves no
-    // room for.
-    size_t want = stream_captures(st) ? 0 : knn_scan_scratch_bytes(c, n, n, k);
+    // The other forms can do without scratch, and what they want is a buffer
+    // of its own, so that one enqueued on one stream may overlap other calls'
+    // use of the context's scratch on another; they take turns at it through
+    // an event.  A captured call scans unsplit (its graph may outlive the
+    // buffer, and the wide form reads a count back); so does one that the
+    // scratch limit or the device leaves no room for.
+    size_t want = stream_captures(st) ? 0 : knn_scratch_bytes(c, n, d, k, m, nullptr);
     if (want && c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) want = 0;
-    if (want > c->scan_bytes) {
-        if (c->scan_part) DRGB_CUDA(c, cudaFree(c->scan_part));  // waits for its users
-        c->scan_part = nullptr;
-        c->scan_bytes = 0;
-        if (cudaMalloc(&c->scan_part, want) == cudaSuccess) {
-            c->scan_bytes = want;
+    if (want > c->knn_buf_bytes) {
+        if (c->knn_buf) DRGB_CUDA(c, cudaFree(c->knn_buf));  // waits for its users
+        c->knn_buf = nullptr;
+        c->knn_buf_bytes = 0;
+        if (cudaMalloc(&c->knn_buf, want) == cudaSuccess) {
+            c->knn_buf_bytes = want;
         } else {
             cudaGetLastError();
-            c->scan_part = nullptr;
+            c->knn_buf = nullptr;
             want = 0;
         }
     }
     if (!want) return knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
-    if (!c->scan_ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&c->scan_ev, cudaEventDisableTiming));
-    DRGB_CUDA(c, cudaStreamWaitEvent(st, c->scan_ev, 0));
-    rc = knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, c->scan_part, want);
-    DRGB_CUDA(c, cudaEventRecord(c->scan_ev, st));
+    if (!c->knn_ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&c->knn_ev, cudaEventDisableTiming));
+    DRGB_CUDA(c, cudaStreamWaitEvent(st, c->knn_ev, 0));
+    rc = knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->knn_buf, want);
+    DRGB_CUDA(c, cudaEventRecord(c->knn_ev, st));
     return rc;
 }

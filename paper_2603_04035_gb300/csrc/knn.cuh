@@ -23,13 +23,13 @@ __device__ __forceinline__ void topk_insert(float (&D)[K], int32_t (&I)[K], floa
 
 int check_knn_args(Ctx* c, const float* X, int64_t n, int d, int k, const void* idx_out,
                    const void* dist_out);
-// Exact FP32 scan for the given query rows (rows == nullptr: rows 0..n_rows-1).
+// Exact FP32 k-NN scan: query p is row rows[p] (null: p) of Q; `separate`: Q is
+// another matrix than X, so no row is excluded as the query itself.
 // This and the other scans split the database into chunks when `part` (part_bytes
 // of scratch, knn_scan_scratch_bytes for the preferred split) holds the partial
 // lists, and take it whole when it is null or too small; the results are the same.
-int launch_knn_exact(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows,
-                     int64_t n_rows, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
-                     size_t part_bytes);
+int launch_knn_scan(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
+                    int d, int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes);
 size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k);
 // Exact FP32 scan of the rows listed in rows32[0 .. cnt).  On entry each listed
 // row of idx_out/dist_out must already hold k
@@ -40,6 +40,10 @@ size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k);
 int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, const int32_t* rows32, int64_t cnt,
                             int32_t* idx_out, float* dist_out, cudaStream_t st, void* part_scratch,
                             size_t part_bytes);
+// The same for the queries list[0 .. cnt) of a query set (as for knn_wide).
+int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t* rows, const float* X, int64_t n,
+                            int d, int k, const int32_t* list, int64_t cnt, int32_t* idx_out, float* dist_out,
+                            cudaStream_t st, void* part, size_t part_bytes);
 // Merge C partial k-lists per listed row: list l of row r at
 // (l * cnt + r) * k in pidx/pd2 (squared distances, ascending by (distance,
 // index), ended early by index -1); the k best by (distance, index) go to
@@ -48,9 +52,6 @@ int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, con
 int launch_merge_partials(Ctx* c, const int32_t* pidx, const float* pd2, int64_t cnt, int C, int k,
                           const int32_t* rows32, int32_t* idx_out, float* dist_out, cudaStream_t st,
                           int32_t none = INT32_MAX);
-// Exact FP32 k-NN of the nq rows of Q among the n rows of X (no self exclusion).
-int launch_knn_query(Ctx* c, const float* Q, int64_t nq, const float* X, int64_t n, int d, int k,
-                     int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes);
 // Per query row: sum over its k targets of max(0, rank_X - k); td, cnt: n_rows x k scratch.
 int launch_rank(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* rows, int64_t n_rows,
                 const int32_t* tgt, float* td, int32_t* cnt, int64_t* excess_out, cudaStream_t st);
@@ -69,6 +70,19 @@ int knn_tc(Ctx* c, const float* X, int64_t n, int d, int k, bool f16, int32_t* i
 // Bytes of scratch a deferred re-scan may use for its partial lists.
 size_t knn_rescan_part_bytes();
 
+// The same for larger problems on the tensor cores (knn_wide.cu).
+// Synchronises `st` once (the count of uncertified queries) unless it is
+// deferred to the caller (as for knn_tc).  `scratch` holds knn_wide_scratch_bytes.
+bool knn_wide_preferred(int64_t nq, int64_t n, int d, int k);
+size_t knn_wide_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d);
+int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n, int d,
+             int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* scratch, int32_t* defer_rows = nullptr,
+             int32_t* defer_count = nullptr);
+// Whichever of the two is preferred and has its scratch.
+size_t knn_queries_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d, int k);
+int knn_queries(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
+                int d, int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* scratch, size_t scratch_bytes);
+
 // Spatial order for the tensor-core k-NN (knn_order.cu): K cells from
 // farthest-point pivots; perm[p] = point at position p (p < n), cell c holds
 // positions [cell_beg[c], cell_beg[c+1]) inside the sphere (centre[c], radius[c]).
@@ -80,6 +94,7 @@ int knn_order(Ctx* c, const float* X, int64_t n, int d, int K, int32_t* perm, in
 // k-NN graph with the mode resolved (0 = auto).  `scratch` holds scratch_bytes;
 // knn_scratch_bytes gives what the mode wants and in *least what it cannot do
 // without (0 for the scans, which then run unsplit).
+static constexpr int KNN_WIDE = 5;  // knn_wide (auto mode only)
 int knn_resolve_mode(int64_t n, int d, int k, int mode);
 size_t knn_scratch_bytes(const Ctx* c, int64_t n, int d, int k, int mode, size_t* least);
 // defer_rows/defer_count: as for knn_tc (the exact-scan modes leave no

@@ -41,6 +41,7 @@
 
 #include "common.cuh"
 #include "knn.cuh"
+#include "knn_select.cuh"
 #include "tc_ptx.cuh"
 
 namespace drgb {
@@ -49,15 +50,10 @@ static constexpr int TC_BM = 128;
 static constexpr int TC_BN = 256;
 static constexpr int TC_K = 64;
 static constexpr int TC_STAGES = 3;
-static constexpr int TC_KP = 32;                 // candidates kept per row
-static constexpr int TC_EPI_WARPS = 8;
 static constexpr int TC_THREADS = 64 + TC_EPI_WARPS * 32;
 static constexpr int TC_A_BYTES = TC_BM * TC_K * 2;   // 16 KiB
 static constexpr int TC_B_BYTES = TC_BN * TC_K * 2;   // 32 KiB
 static constexpr int TC_TMEM_COLS = 512;               // two 256-column accumulators
-static constexpr int TC_QCAP = 32;                     // per-thread candidate queue slots (one chunk)
-static constexpr size_t TC_QUEUE_BYTES = size_t(TC_EPI_WARPS) * 32 * TC_QCAP * 8;
-static constexpr int TC_NQ = 4;                       // list quantiles a column half publishes
 static constexpr size_t TC_THR_BYTES = size_t(2) * TC_BM * TC_NQ * 4;   // per (column half, row) quantiles
 static constexpr int TC_CELLS = 128;                   // most cells a schedule may hold
 static constexpr int TC_GROUPS = 4;                    // row groups (runs of one cell) bounded separately
@@ -69,77 +65,7 @@ static constexpr size_t TC_SCHED_BYTES =
 static constexpr size_t TC_SMEM =
     1024 + TC_A_BYTES + TC_STAGES * TC_B_BYTES + 256 + TC_QUEUE_BYTES + TC_THR_BYTES + TC_SCHED_BYTES;
 
-// Compare-exchange of (value, index) pairs i < l: afterwards the pair at i is
-// the smaller (asc) or the larger (!asc) of the two values.
-__device__ __forceinline__ void cas(float& vi, int32_t& ii, float& vl, int32_t& il, bool asc) {
-    const bool sw = asc ? (vl < vi) : (vi < vl);
-    const float a = vi, b = vl;
-    const int32_t x = ii, y = il;
-    vi = sw ? b : a;
-    vl = sw ? a : b;
-    ii = sw ? y : x;
-    il = sw ? x : y;
-}
-
-// Bitonic merge of a bitonic sequence of N (power of two) into ascending order.
-template <int N>
-__device__ __forceinline__ void bitonic_merge_asc(float (&v)[N], int32_t (&ix)[N]) {
-#pragma unroll
-    for (int j = N / 2; j > 0; j >>= 1) {
-#pragma unroll
-        for (int i = 0; i < N; ++i)
-            if ((i & j) == 0) cas(v[i], ix[i], v[i + j], ix[i + j], true);
-    }
-}
-
-// Bitonic sort of N (power of two) into ascending order.
-template <int N>
-__device__ __forceinline__ void bitonic_sort_asc(float (&v)[N], int32_t (&ix)[N]) {
-#pragma unroll
-    for (int k = 2; k <= N; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                const int l = i ^ j;
-                if (l > i) cas(v[i], ix[i], v[l], ix[l], (i & k) == 0);
-            }
-        }
-    }
-}
-
-// Three-input minimum (sm_100 and later).
-__device__ __forceinline__ float min3f(float a, float b, float c) {
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 // ------------------------------------------------------------------ A1: staging
-typedef uint16_t op16;  // raw 16-bit operand (BF16 or FP16 bits)
-
-template <bool F16>
-__device__ __forceinline__ op16 to_op(float v) {
-    if constexpr (F16) return __half_as_ushort(__float2half_rn(v));
-    else return __bfloat16_as_ushort(__float2bfloat16_rn(v));
-}
-template <bool F16>
-__device__ __forceinline__ float from_op(op16 b) {
-    if constexpr (F16) return __half2float(__ushort_as_half(b));
-    else return __bfloat162float(__ushort_as_bfloat16(b));
-}
-
-// Power-of-two operand scale: FP16 maps max |x - mean| to at most 2^10.
-template <bool F16>
-__device__ __forceinline__ float operand_scale(const unsigned int* maxbits) {
-    if constexpr (!F16) return 1.0f;
-    const float amax = __uint_as_float(maxbits[2]);
-    if (!(amax > 0.f)) return 1.0f;
-    int e;
-    frexpf(amax, &e);                      // amax < 2^e
-    return ldexpf(1.0f, e - 10);
-}
-
 // Column statistics of X (d <= 64) for the operand staging.  Block b sums,
 // and takes the minimum and maximum of, every column over its range of rows
 // (a warp per row, lanes on dimensions (lane, lane + 32)) into partial[b]; the
@@ -743,60 +669,16 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             s_ua[row] = ua;
             s_uc[row] = uc;
         }
-        // Candidates below the row's threshold are appended to this thread's
-        // queue (slot s at q[s * 256 + tid], conflict-free).  The threshold
-        // is a bound on the row's 32nd-best value over both column halves:
-        // each half publishes the 8th, 16th, 24th and 32nd values of its
-        // sorted list, and for b in {0, 8, 16, 24, 32} the 32 - b smallest of
-        // this half's list together with the b smallest of the other's are 32
-        // distinct columns, so max(own[31 - b], other's b-th) bounds the
-        // row's 32nd-best; the threshold is the smallest of the five.  A value
-        // at or above it cannot be among the row's 32 best.  A stale (larger)
-        // published value still bounds correctly, since a list only improves.
-        // When a chunk would overflow any lane's queue, all lanes merge their
-        // queues into their lists in lockstep: the queue (padded with +inf)
-        // is sorted by a bitonic network, the 32 smallest of list and queue
-        // are selected by pairing the list's upper half with the reversed
-        // queue, and a bitonic merge restores the order.
         const int qb = e * 32 + lane;
         volatile float* q_mine = s_thr + (half * TC_BM + row) * TC_NQ;
         volatile float* q_other = s_thr + ((1 - half) * TC_BM + row) * TC_NQ;
 #pragma unroll
         for (int j = 0; j < TC_NQ; ++j) q_mine[j] = INFINITY;
         asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI_WARPS * 32) : "memory");
-        // the row's threshold from this half's list and the other's quantiles
-        auto row_bound = [&]() {
-            const float o8 = q_other[0], o16 = q_other[1], o24 = q_other[2], o32 = q_other[3];
-            float t = fminf(L[TC_KP - 1], o32);
-            t = fminf(t, fmaxf(L[23], o8));
-            t = fminf(t, fmaxf(L[15], o16));
-            t = fminf(t, fmaxf(L[7], o24));
-            return t;
-        };
+        auto row_bound = [&]() { return list_bound(L, q_other); };
         int qn = 0;
         auto flush = [&]() {
-            float qv[TC_QCAP];
-            int32_t qi[TC_QCAP];
-#pragma unroll
-            for (int s = 0; s < TC_QCAP; ++s) {
-                const int2 c = s < qn ? q[s * (TC_EPI_WARPS * 32) + qb] : make_int2(__float_as_int(INFINITY), -1);
-                qv[s] = __int_as_float(c.x);
-                qi[s] = c.y;
-            }
-            bitonic_sort_asc<TC_QCAP>(qv, qi);
-            // the 32 smallest of L and Q: min(L[s], Q[31 - s]) is bitonic
-#pragma unroll
-            for (int s = 0; s < TC_KP; ++s) {
-                const bool take = qv[TC_KP - 1 - s] < L[s];
-                L[s] = take ? qv[TC_KP - 1 - s] : L[s];
-                I[s] = take ? qi[TC_KP - 1 - s] : I[s];
-            }
-            bitonic_merge_asc<TC_KP>(L, I);
-            qn = 0;
-            q_mine[0] = L[7];
-            q_mine[1] = L[15];
-            q_mine[2] = L[23];
-            q_mine[3] = L[TC_KP - 1];
+            list_merge(L, I, qn, q, qb, q_mine);
             const float thr = row_bound();
             if (g_row >= 0 && thr < INFINITY)
                 s_U[row] = (sqrtf(fmaxf(s_ua[row] + thr * s_misc[2], 0.f)) + s_uc[row]) * (1.0f + 1e-5f);
@@ -818,53 +700,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             if (tile < 0) break;
             const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * TC_BN + half * 128);
             const int32_t j0 = tile * TC_BN + half * 128;
-            // the row's threshold, with the other half's quantiles read once
-            // per tile (stale, larger, values still bound correctly)
-            float thr_t = row_bound();
-#pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-                float v[32];
-                __syncwarp();
-                tmem_ld32(tbase + c * 32, v);
-                float thr = thr_t;
-                float gm[4];
-#pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    gm[g] = min3f(min3f(v[8 * g], v[8 * g + 1], v[8 * g + 2]),
-                                  min3f(v[8 * g + 3], v[8 * g + 4], v[8 * g + 5]), fminf(v[8 * g + 6], v[8 * g + 7]));
-                const float m = fminf(min3f(gm[0], gm[1], gm[2]), gm[3]);
-                if (__any_sync(0xffffffffu, m < thr)) {
-                    // room for this chunk's candidates: a bound from the groups
-                    // first, the exact count only when the bound overflows
-                    const int ub = 8 * ((gm[0] < thr) + (gm[1] < thr) + (gm[2] < thr) + (gm[3] < thr));
-                    if (__any_sync(0xffffffffu, qn + ub > TC_QCAP)) {
-                        int cnt = 0;
-#pragma unroll
-                        for (int u = 0; u < 32; ++u) cnt += v[u] < thr ? 1 : 0;
-                        if (__any_sync(0xffffffffu, qn + cnt > TC_QCAP)) {
-                            // the chunk is read again after the merge, which
-                            // keeps its 32 values out of registers meanwhile
-                            flush();
-                            __syncwarp();
-                            tmem_ld32(tbase + c * 32, v);
-                            thr = thr_t = row_bound();
-                        }
-                    }
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if (__any_sync(0xffffffffu, gm[g] < thr)) {
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                if (v[8 * g + u] < thr) {
-                                    q[qn * (TC_EPI_WARPS * 32) + qb] =
-                                        make_int2(__float_as_int(v[8 * g + u]), j0 + c * 32 + 8 * g + u);
-                                    ++qn;
-                                }
-                            }
-                        }
-                    }
-                }
-            }
+            select_tile(tbase, j0, qn, q, qb, row_bound, flush);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);

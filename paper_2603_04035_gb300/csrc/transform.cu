@@ -64,7 +64,7 @@ extern "C" int drgb_transform(drgb_ctx* c, const float* X_train, const float* Y_
     const size_t least = 4 * Carve::round(nk * 4) + Carve::round(nk * 4) + Carve::round((n_new + 1) * 4) +
                          2 * Carve::round(size_t(N) * 8) + Carve::round(epoch_scratch_bytes(N, int64_t(nk), 0)) + 4096;
     const size_t part_off = Carve::round(least);
-    size_t total = part_off + knn_scan_scratch_bytes(c, n_new, n_train, k);
+    size_t total = part_off + knn_queries_scratch_bytes(c, n_new, n_train, d, k);
     int rc = ensure_scratch_within(c, &total, least, st);
     if (rc) return rc;
     const size_t part_bytes = total > part_off ? total - part_off : 0;
@@ -83,8 +83,8 @@ extern "C" int drgb_transform(drgb_ctx* c, const float* X_train, const float* Y_
 
     float a = 0.f, b = 0.f;
     if ((rc = drgb_find_ab(p->spread, p->min_dist, &a, &b))) return set_error(c, rc, "bad spread/min_dist");
-    if ((rc = launch_knn_query(c, X_new, n_new, X_train, n_train, d, k, idx, dist, st, part, part_bytes)))
-        return rc;
+    rc = knn_queries(c, X_new, n_new, true, nullptr, X_train, n_train, d, k, idx, dist, st, part, part_bytes);
+    if (rc) return rc;
     if ((rc = launch_directed_weights(c, idx, dist, n_new, k, n_train, w_dir, out_col, out_w, st))) return rc;
     DRGB_CUDA(c, cudaMemcpyAsync(Ya, Y_train, size_t(n_train) * 8, cudaMemcpyDeviceToDevice, st));
     DRGB_CUDA(c, cudaMemcpyAsync(Yb, Y_train, size_t(n_train) * 8, cudaMemcpyDeviceToDevice, st));
