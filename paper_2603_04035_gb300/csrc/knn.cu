@@ -612,22 +612,28 @@ namespace drgb {
 
 int knn_resolve_mode(int64_t n, int d, int k, int mode) {
     if (mode != 0) return mode;
-    if (knn_tc_preferred(n, d, k)) return 3;
+    // The cell-ordered product (knn_tc) spends about 150 us on the order and
+    // its bounds, and wins from about 14,000 rows on (10 clusters in 50
+    // dimensions; wide / cells: 4,096 rows 126 / 234 us, 8,000 175 / 256,
+    // 16,000 295 / 287, 30,000 786 / 429; 100 clusters: 297 / 434 at 16,000,
+    // 1,237 / 1,176 at 40,000).
+    if (knn_tc_preferred(n, d, k) && (n > 14000 || !knn_wide_preferred(n, n, d, k))) return 3;
     return knn_wide_preferred(n, n, d, k) ? KNN_WIDE : 1;
 }
 
 size_t knn_scratch_bytes(const Ctx* c, int64_t n, int d, int k, int mode, size_t* least) {
     const int m = knn_resolve_mode(n, d, k, mode);
-    const bool tc = m == 2 || m == 3;
-    const size_t b = tc ? knn_tc_scratch_bytes(n, d)
-                        : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
-    if (least) *least = tc ? b : 0;
-    return b;
+    const bool cells = m == 2 || m == 3 || (m == KNN_WIDE && knn_tc_preferred(n, d, k));
+    const size_t tb = cells ? knn_tc_scratch_bytes(n, d) : 0;
+    const size_t b = m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : (m == 1 ? knn_scan_scratch_bytes(c, n, n, k) : 0);
+    if (least) *least = tb;
+    return b > tb ? b : tb;
 }
 
 int knn_run(Ctx* c, const float* X, int64_t n, int d, int k, int mode, int32_t* idx_out, float* dist_out,
             cudaStream_t st, void* scratch, size_t scratch_bytes, int32_t* defer_rows, int32_t* defer_count) {
-    const int m = knn_resolve_mode(n, d, k, mode);
+    int m = knn_resolve_mode(n, d, k, mode);
+    if (m == KNN_WIDE && knn_tc_preferred(n, d, k) && scratch_bytes < knn_wide_scratch_bytes(c, n, n, d)) m = 3;
     if (m == 2 || m == 3)
         return knn_tc(c, X, n, d, k, m == 3, idx_out, dist_out, st, scratch, defer_rows, defer_count);
     if (m == KNN_WIDE && scratch && scratch_bytes >= knn_wide_scratch_bytes(c, n, n, d))
@@ -645,8 +651,9 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     if (mode < 0 || mode > 3) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int m = knn_resolve_mode(n, d, k, mode);
-    if (m == 2 || m == 3) {
-        if ((rc = ensure_scratch(c, knn_scratch_bytes(c, n, d, k, m, nullptr), st))) return rc;
+    if (m == 2 || m == 3 || (m == KNN_WIDE && knn_tc_preferred(n, d, k))) {
+        size_t least = 0, bytes = knn_scratch_bytes(c, n, d, k, m, &least);
+        if ((rc = ensure_scratch_within(c, &bytes, least, st))) return rc;
         return knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->scratch, c->scratch_bytes);
     }
     // The other forms can do without scratch, and what they want is a buffer

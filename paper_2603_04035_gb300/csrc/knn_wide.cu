@@ -184,6 +184,7 @@ struct WideParams {
     float* cand_s;
     int64_t nq_pad;
     int* status;
+    unsigned long long* tiles_done;  // += tiles this CTA multiplies (null: not counted)
 };
 
 __global__ void __launch_bounds__(WD_THREADS, 1)
@@ -231,6 +232,7 @@ knn_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 
     if (warp == 0) {
         if (lane == 0) {
+            if (P.tiles_done) atomicAdd(P.tiles_done, static_cast<unsigned long long>(nt));
             const int steps = nt * P.kch;
             int u = 0;
             for (int t = 0; t < nt && u >= 0; ++t) {
@@ -515,8 +517,13 @@ size_t knn_wide_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d) {
            8192;
 }
 
+// Against the FP32 scan (the line lies where they cross, measured for a graph of
+// X on itself): 1.5e8 pairs x dimensions, 1,100 x 50 144 and 144 us, 2,000 x 50
+// 113 and 168 us, 4,096 x 50 126 and 427 us, 2,000 x 784 (some rows re-scanned)
+// 493 and 682 us.  Rows of fewer than 16 dimensions are often denser than the
+// operands' rounding, and would mostly be re-scanned.
 bool knn_wide_preferred(int64_t nq, int64_t n, int d, int k) {
-    return d >= 16 && d <= WD_MAX_D && k < TC_KP && n >= 1024 && double(nq) * double(n) * d >= 3e9;
+    return d >= 16 && d <= WD_MAX_D && k < TC_KP && n >= 1024 && double(nq) * double(n) * d >= 1.5e8;
 }
 
 int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n, int d,
@@ -537,6 +544,9 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     int32_t* fail_rows = cv.take<int32_t>(nq);
     void* part = cv.take<char>(WD_PART_BYTES);
 
+    const bool graph = !separate && !rows;  // a graph of X on itself: the context's k-NN counters report it
+    int rc;
+    if ((rc = stage_mark(c, 8, st))) return rc;
     DRGB_CUDA(c, cudaMemsetAsync(maxbits, 0, 64, st));
     DRGB_CUDA(c, cudaMemsetAsync(fail_count, 0, 64, st));
     const int blocks = WD_STAT_BLOCKS + (separate ? WD_STAT_QBLOCKS : 0);
@@ -551,7 +561,6 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
                                                                                   maxbits, XA, norm, resid);
     DRGB_CHECK_LAUNCH(c);
     CUtensorMap mA, mB;
-    int rc;
     if ((rc = make_map_k64(c, &mA, XA, w.nq_pad, w.K, WD_BM, true))) return rc;
     if ((rc = make_map_k64(c, &mB, XB, w.n_pad, w.K, WD_BN, true))) return rc;
     DRGB_CUDA(c, cudaFuncSetAttribute(knn_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(WD_SMEM)));
@@ -564,8 +573,16 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     P.cand_s = cand_s;
     P.nq_pad = w.nq_pad;
     P.status = c->d_status;
+    P.tiles_done = nullptr;
+    if (graph) {
+        P.tiles_done = c->d_counter + 4;
+        c->knn_tiles_total = (w.nq_pad / WD_BM) * w.n_tiles;
+        DRGB_CUDA(c, cudaMemsetAsync(c->d_counter + 4, 0, 8, st));
+    }
+    if ((rc = stage_mark(c, 6, st))) return rc;
     knn_wide_kernel<<<dim3(unsigned(w.nq_pad / WD_BM), w.splits), WD_THREADS, WD_SMEM, st>>>(mA, mB, P);
     DRGB_CHECK_LAUNCH(c);
+    if ((rc = stage_mark(c, 7, st))) return rc;
     // |s - s~| for K columns: a K = 16 step adds 16 exact products and the
     // accumulator, each aligned with an error below an FP32 unit (2^-23) of the
     // largest magnitude, which is at most n_j + 2 |x_i| |x_j| <= 2 (n_i + n_max):
@@ -575,13 +592,16 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
         X, n, d, k, Q, separate, rows, nq, w.nq_pad, w.splits, cand_idx, cand_s, norm, resid, maxbits, eps_rel,
         idx_out, dist_out, defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count);
     DRGB_CHECK_LAUNCH(c);
+    if ((rc = stage_mark(c, 9, st))) return rc;
     if (defer_rows) return DRGB_OK;  // the caller re-scans them
+    if (graph) DRGB_CUDA(c, cudaMemcpyAsync(c->d_counter, fail_count, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     int32_t cnt = 0;
     DRGB_CUDA(c, cudaMemcpyAsync(&cnt, fail_count, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     DRGB_CUDA(c, cudaStreamSynchronize(st));
-    if (cnt <= 0) return DRGB_OK;
-    return launch_knn_exact_listed(c, Q, separate, rows, X, n, d, k, fail_rows, cnt, idx_out, dist_out, st, part,
-                                   WD_PART_BYTES);
+    if (cnt > 0 && (rc = launch_knn_exact_listed(c, Q, separate, rows, X, n, d, k, fail_rows, cnt, idx_out, dist_out,
+                                                 st, part, WD_PART_BYTES)))
+        return rc;
+    return stage_mark(c, 10, st);
 }
 
 }  // namespace drgb

@@ -28,7 +28,8 @@ def _points(torch, n, d, seed, kind):
 # 1022: the scan); n ragged against the 128-query block and 256-row tile
 @pytest.mark.parametrize("kind", ["clusters", "ties"])
 @pytest.mark.parametrize("n,d,k", [(7001, 62, 15), (6913, 125, 1), (4000, 253, 31), (4097, 254, 16), (2050, 784, 15),
-                                   (1800, 1021, 10), (1800, 1022, 10), (5000, 200, 32)])
+                                   (1800, 1021, 10), (1800, 1022, 10), (5000, 200, 32), (1733, 50, 15), (4096, 16, 15),
+                                   (13999, 61, 15)])
 def test_wide_graph_equals_scan(drgb, n, d, k, kind):
     import torch
     X = _points(torch, n, d, n + d, kind)
