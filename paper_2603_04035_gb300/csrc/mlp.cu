@@ -16,13 +16,17 @@
 // rows per edge, M = B R rows):
 //   sample     edges proportional to w (integer rejection on q) + negatives
 //   gather     X rows -> Xb (M x 64) and Xb^T (64 x M), BF16
-//   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16, + transposed)
+//   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16, H1 also
+//              transposed) ; GELU'(pre_l) (FP32, blocked)
 //   head       z = H2 W3^T + b3 ; loss and dL/dz per edge
 //   L3 back    dpre2 = (dz W3) . GELU'(pre2) ; dW3, db3, db2 partial sums
-//   dW2        dpre2^T H1     (split-K, FP32 partials)
+//   dW2        dpre2^T H1     (split-K, FP32 partials; beside dH1 and dW1)
 //   dH1        dpre1 = (dpre2 W2) . GELU'(pre1)
-//   dW1        dpre1^T Xb     (split-K)
-//   reduce     gradient vector (fixed summation order) ; Adam ; BF16 copies
+//   dW1        dpre1^T Xb     (split-K) ; db1 partial sums
+//   update     gradient (fixed summation order), Adam, BF16 copies
+//
+// Sums over the batch run in a fixed order: over the rows of chunks of 512 in
+// order, then over the chunks (or K splits) in order.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -56,46 +60,62 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // ------------------------------------------------------------------ tensor-core GEMM
+// 128 x 128 (or 64) tiles, two CTAs per SM: the epilogue (bias, GELU and its
+// derivative: about 60 instructions an element) is the larger part, and 16
+// epilogue warps an SM hide its latency (4 warps on one CTA per SM, with
+// 128 x 256 tiles: 41-52 us for 28,672 rows; now 12-17).
 static constexpr int G_BM = 128;
-static constexpr int G_STAGES = 4;
-static constexpr int G_THREADS = 192;  // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+static constexpr int G_EPI_WARPS = 8;  // two per TMEM lane quarter, one per column half
+static constexpr int G_THREADS = 64 + G_EPI_WARPS * 32;  // warp 0 TMA, warp 1 MMA
 enum { EPI_GELU = 0, EPI_GELU_GRAD = 1, EPI_F32 = 2 };
+
+// Blocked FP32 layout of an M x N matrix that only epilogues (and kernels of
+// the same tiling) exchange: 128 x 32 blocks, within a block float4 columns of
+// 128 rows, so that a warp's accesses are 512 contiguous bytes.
+__host__ __device__ __forceinline__ int64_t blocked_at(int64_t row, int col, int N) {
+    return ((row >> 7) * (N >> 5) + (col >> 5)) * 4096 + (int64_t((col & 31) >> 2) * 128 + (row & 127)) * 4 + (col & 3);
+}
 
 struct GemmArgs {
     int M, N, K;          // M, N multiples of 128 / BN; K multiple of 64
     int kb_per_split;     // 64-wide K blocks per split (grid z)
     const float* bias;    // EPI_GELU: [N]
-    float* pre;           // EPI_GELU: out [M][N] (nullable); EPI_GELU_GRAD: in [M][N]
+    float* dgelu;         // GELU'(pre), blocked: EPI_GELU out (nullable), EPI_GELU_GRAD in
     bf16* out;            // [M][N] (nullable)
     bf16* out_t;          // [N][M] transposed (nullable)
-    float* out_f32;       // EPI_F32: [splits][M][N]; EPI_GELU_GRAD: FP32 copy [M][N] (nullable)
+    float* out_f32;       // EPI_F32: [splits][M][N]; EPI_GELU_GRAD: blocked FP32 copy (nullable)
     int* status;
 };
 
 template <int BN>
 struct GemmSmem {
+    static constexpr int STAGES = BN == 128 ? 3 : 4;
     static constexpr int A_BYTES = G_BM * 64 * 2;
     static constexpr int B_BYTES = BN * 64 * 2;
-    static constexpr size_t TOTAL = 1024 + size_t(G_STAGES) * (A_BYTES + B_BYTES) + 256;
+    static constexpr size_t TOTAL = 1024 + size_t(STAGES) * (A_BYTES + B_BYTES) + 256 + BN * 4;
 };
+static constexpr int G_PITCH = 36;  // floats per row of a warp's 32 x 32 transposing tile (16-byte rows)
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(G_THREADS, 1)
+__global__ void __launch_bounds__(G_THREADS, 2)
 mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs G) {
     using SM = GemmSmem<BN>;
+    constexpr int STAGES = SM::STAGES;
+    static_assert(STAGES * (SM::A_BYTES + SM::B_BYTES) >= G_EPI_WARPS * 32 * G_PITCH * 4, "epilogue tiles fit the ring");
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned (swizzled operand tiles); an offset from the shared
     // array, so that every pointer below stays a known shared-memory address
     uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* sA = base;
-    uint8_t* sB = base + G_STAGES * SM::A_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + G_STAGES * SM::B_BYTES);
+    uint8_t* sB = base + STAGES * SM::A_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + STAGES * SM::B_BYTES);
     uint64_t* full = bars;
-    uint64_t* empty = bars + G_STAGES;
-    uint64_t* acc_full = bars + 2 * G_STAGES;
+    uint64_t* empty = bars + STAGES;
+    uint64_t* acc_full = bars + 2 * STAGES;
     uint64_t* mma_done = acc_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    float* s_bias = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * G_BM, n0 = blockIdx.y * BN;
@@ -104,7 +124,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (nkb > G.kb_per_split) nkb = G.kb_per_split;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < G_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -114,6 +134,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (EPI == EPI_GELU && threadIdx.x >= 64 && threadIdx.x < 64 + BN) s_bias[threadIdx.x - 64] = G.bias[n0 + threadIdx.x - 64];
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(BN) : "memory");
@@ -128,16 +149,16 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (lane == 0) {
             int kb = 0;
             for (; kb < nkb; ++kb) {
-                const int s = kb % G_STAGES;
-                if (kb >= G_STAGES && !mbar_wait(&empty[s], ((kb / G_STAGES) & 1) ^ 1, abort_flag, G.status)) break;
+                const int s = kb % STAGES;
+                if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) & 1) ^ 1, abort_flag, G.status)) break;
                 mbar_expect_tx(&full[s], SM::A_BYTES + SM::B_BYTES);
                 tma_load_2d(sA + s * SM::A_BYTES, &tmA, (kb0 + kb) * 64, m0, &full[s]);
                 tma_load_2d(sB + s * SM::B_BYTES, &tmB, (kb0 + kb) * 64, n0, &full[s]);
             }
             if (kb < nkb) {  // aborted: let issued loads land before exit
-                for (int u = (kb > G_STAGES ? kb - G_STAGES : 0); u < kb; ++u) {
+                for (int u = (kb > STAGES ? kb - STAGES : 0); u < kb; ++u) {
                     const unsigned long long t0 = global_timer();
-                    while (!mbar_try(&full[u % G_STAGES], (u / G_STAGES) & 1) && global_timer() - t0 < 100000000ull) {
+                    while (!mbar_try(&full[u % STAGES], (u / STAGES) & 1) && global_timer() - t0 < 100000000ull) {
                     }
                 }
             }
@@ -146,8 +167,8 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (lane == 0) {
             const uint32_t idesc = idesc_f16kind(G_BM, BN, false);
             for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % G_STAGES;
-                if (!mbar_wait(&full[s], (kb / G_STAGES) & 1, abort_flag, G.status)) break;
+                const int s = kb % STAGES;
+                if (!mbar_wait(&full[s], (kb / STAGES) & 1, abort_flag, G.status)) break;
                 tc_fence_after();
                 const uint64_t ad = sdesc_sw128(smem_u32(sA + s * SM::A_BYTES));
                 const uint64_t bd = sdesc_sw128(smem_u32(sB + s * SM::B_BYTES));
@@ -162,62 +183,91 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             }
         }
     } else {
-        const int quarter = warp & 3;
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
         const int row = quarter * 32 + lane;
         const int64_t gr = m0 + row;
+        // once the accumulator is complete the operand ring is free: each warp
+        // transposes its 32 x 32 pieces through its own part of it
+        float* tile = reinterpret_cast<float*>(base) + (warp - 2) * 32 * G_PITCH;
         const bool ok = mbar_wait(acc_full, 0, abort_flag, G.status) && nkb > 0;
         tc_fence_after();
         if (ok) {
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
+            for (int c = half * (BN / 64); c < (half + 1) * (BN / 64); ++c) {
                 float v[32];
                 __syncwarp();
                 tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(c * 32), v);
                 const int gc0 = n0 + c * 32;
                 if (EPI == EPI_F32) {
-                    float* o = G.out_f32 + (int64_t(blockIdx.z) * G.M + gr) * G.N + gc0;
 #pragma unroll
-                    for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                    for (int i = 0; i < 32; i += 4)
+                        *reinterpret_cast<float4*>(tile + lane * G_PITCH + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                    __syncwarp();
+                    float* o = G.out_f32 + (int64_t(blockIdx.z) * G.M + m0 + quarter * 32) * G.N + gc0;
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {  // four rows of 128 bytes an instruction
+                        const int r = it * 4 + (lane >> 3), i = 4 * (lane & 7);
+                        *reinterpret_cast<float4*>(o + int64_t(r) * G.N + i) =
+                            *reinterpret_cast<const float4*>(tile + r * G_PITCH + i);
+                    }
                 } else {
+                    float* bl = nullptr;  // this lane's float4 column of the blocked matrices
+                    const int64_t bo = blocked_at(gr, gc0, G.N);
                     if (EPI == EPI_GELU) {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] += G.bias[gc0 + i];
-                        if (G.pre) {
-                            float* o = G.pre + gr * G.N + gc0;
-#pragma unroll
-                            for (int i = 0; i < 32; i += 4)
-                                *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = gelu(v[i]);
-                    } else {  // EPI_GELU_GRAD
-                        const float* p = G.pre + gr * G.N + gc0;
+                        if (G.dgelu) bl = G.dgelu + bo;
 #pragma unroll
                         for (int i = 0; i < 32; i += 4) {
-                            const float4 x = *reinterpret_cast<const float4*>(p + i);
-                            v[i] *= gelu_grad(x.x);
-                            v[i + 1] *= gelu_grad(x.y);
-                            v[i + 2] *= gelu_grad(x.z);
-                            v[i + 3] *= gelu_grad(x.w);
+                            const float4 b4 = *reinterpret_cast<const float4*>(s_bias + c * 32 + i);
+                            v[i] += b4.x;
+                            v[i + 1] += b4.y;
+                            v[i + 2] += b4.z;
+                            v[i + 3] += b4.w;
+                            if (bl)
+                                *reinterpret_cast<float4*>(bl + i * 128) = make_float4(
+                                    gelu_grad(v[i]), gelu_grad(v[i + 1]), gelu_grad(v[i + 2]), gelu_grad(v[i + 3]));
+                            v[i] = gelu(v[i]);
+                            v[i + 1] = gelu(v[i + 1]);
+                            v[i + 2] = gelu(v[i + 2]);
+                            v[i + 3] = gelu(v[i + 3]);
+                        }
+                    } else {  // EPI_GELU_GRAD
+                        const float* p = G.dgelu + bo;
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
+                            const float4 x = *reinterpret_cast<const float4*>(p + i * 128);
+                            v[i] *= x.x;
+                            v[i + 1] *= x.y;
+                            v[i + 2] *= x.z;
+                            v[i + 3] *= x.w;
                         }
                         if (G.out_f32) {
-                            float* o = G.out_f32 + gr * G.N + gc0;
+                            bl = G.out_f32 + bo;
 #pragma unroll
                             for (int i = 0; i < 32; i += 4)
-                                *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                                *reinterpret_cast<float4*>(bl + i * 128) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
                         }
                     }
                     if (G.out) {
-                        uint32_t packed[16];
+                        uint32_t* wt = reinterpret_cast<uint32_t*>(tile);  // rows of 20 words: 16-byte reads and writes
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                            packed[i] = *reinterpret_cast<const uint32_t*>(&h2);
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t packed[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[8 * i + 2 * j], v[8 * i + 2 * j + 1]);
+                                packed[j] = *reinterpret_cast<const uint32_t*>(&h2);
+                            }
+                            *reinterpret_cast<uint4*>(wt + lane * 20 + 4 * i) =
+                                make_uint4(packed[0], packed[1], packed[2], packed[3]);
                         }
-                        uint4* o = reinterpret_cast<uint4*>(G.out + gr * G.N + gc0);
+                        __syncwarp();
+                        bf16* o = G.out + (int64_t(m0) + quarter * 32) * G.N + gc0;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            o[i] = make_uint4(packed[4 * i], packed[4 * i + 1], packed[4 * i + 2], packed[4 * i + 3]);
+                        for (int it = 0; it < 4; ++it) {  // eight rows of 64 bytes an instruction
+                            const int r = it * 8 + (lane >> 2), i = lane & 3;
+                            *reinterpret_cast<uint4*>(o + int64_t(r) * G.N + 8 * i) =
+                                *reinterpret_cast<const uint4*>(wt + r * 20 + 4 * i);
+                        }
                     }
                     if (G.out_t) {
 #pragma unroll
@@ -274,8 +324,8 @@ static int gemm_attr(Ctx* c) {
 // Opt the GEMM instantiations into their shared-memory size (before any capture).
 static int gemm_prepare(Ctx* c) {
     int rc;
-    if ((rc = gemm_attr<256, EPI_GELU>(c)) || (rc = gemm_attr<256, EPI_GELU_GRAD>(c)) ||
-        (rc = gemm_attr<256, EPI_F32>(c)) || (rc = gemm_attr<64, EPI_F32>(c)))
+    if ((rc = gemm_attr<128, EPI_GELU>(c)) || (rc = gemm_attr<128, EPI_GELU_GRAD>(c)) ||
+        (rc = gemm_attr<128, EPI_F32>(c)) || (rc = gemm_attr<64, EPI_F32>(c)))
         return rc;
     return DRGB_OK;
 }
@@ -288,9 +338,9 @@ static int gemm_launch_t(Ctx* c, const Gemm& G, cudaStream_t st) {
 }
 
 static int gemm_launch(Ctx* c, const Gemm& G, cudaStream_t st) {
-    if (G.bn == 256 && G.epi == EPI_GELU) return gemm_launch_t<256, EPI_GELU>(c, G, st);
-    if (G.bn == 256 && G.epi == EPI_GELU_GRAD) return gemm_launch_t<256, EPI_GELU_GRAD>(c, G, st);
-    if (G.bn == 256 && G.epi == EPI_F32) return gemm_launch_t<256, EPI_F32>(c, G, st);
+    if (G.bn == 128 && G.epi == EPI_GELU) return gemm_launch_t<128, EPI_GELU>(c, G, st);
+    if (G.bn == 128 && G.epi == EPI_GELU_GRAD) return gemm_launch_t<128, EPI_GELU_GRAD>(c, G, st);
+    if (G.bn == 128 && G.epi == EPI_F32) return gemm_launch_t<128, EPI_F32>(c, G, st);
     if (G.bn == 64 && G.epi == EPI_F32) return gemm_launch_t<64, EPI_F32>(c, G, st);
     return set_error(c, DRGB_ERR_INVALID, "mlp gemm: unsupported tile");
 }
@@ -300,11 +350,11 @@ static int gemm_launch(Ctx* c, const Gemm& G, cudaStream_t st) {
 int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, int splits, float* partials,
                    int* splits_used, cudaStream_t st) {
     Gemm G;
-    const int bn = (N % 256 == 0) ? 256 : 64;
+    const int bn = (N % 128 == 0) ? 128 : 64;
     int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, EPI_F32, splits);
     if (rc) return rc;
     G.g.out_f32 = partials;
-    if ((rc = bn == 256 ? gemm_attr<256, EPI_F32>(c) : gemm_attr<64, EPI_F32>(c))) return rc;
+    if ((rc = bn == 128 ? gemm_attr<128, EPI_F32>(c) : gemm_attr<64, EPI_F32>(c))) return rc;
     if (splits_used) *splits_used = int(G.grid.z);
     return gemm_launch(c, G, st);
 }
@@ -317,16 +367,23 @@ struct MlpWeights {          // BF16 working copies of the master weights
     float* W3f;              // [2][256]    BF16-rounded values in FP32
 };
 
-__global__ void mlp_cast_kernel(const float* __restrict__ P, MlpWeights W) {
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < MLP_H * MLP_H;
-         t += int64_t(gridDim.x) * blockDim.x) {
-        const int o = int(t / MLP_H), i = int(t % MLP_H);
-        const bf16 v = __float2bfloat16_rn(P[OFF_W2 + t]);
+// Working copies of master weight p.
+__device__ __forceinline__ void mlp_cast_one(float w, int64_t p, const MlpWeights& W) {
+    if (p < OFF_B1) {
+        W.W1b[p] = __float2bfloat16_rn(w);
+    } else if (p >= OFF_W2 && p < OFF_B2) {
+        const int t = int(p - OFF_W2), o = t / MLP_H, i = t % MLP_H;
+        const bf16 v = __float2bfloat16_rn(w);
         W.W2b[t] = v;
-        W.W2tb[int64_t(i) * MLP_H + o] = v;
-        if (t < MLP_H * MLP_IN) W.W1b[t] = __float2bfloat16_rn(P[OFF_W1 + t]);
-        if (t < MLP_OUT * MLP_H) W.W3f[t] = __bfloat162float(__float2bfloat16_rn(P[OFF_W3 + t]));
+        W.W2tb[i * MLP_H + o] = v;
+    } else if (p >= OFF_W3 && p < OFF_B3) {
+        W.W3f[p - OFF_W3] = __bfloat162float(__float2bfloat16_rn(w));
     }
+}
+
+__global__ void mlp_cast_kernel(const float* __restrict__ P, MlpWeights W) {
+    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < MLP_P; p += int64_t(gridDim.x) * blockDim.x)
+        mlp_cast_one(P[p], p, W);
 }
 
 // Edge sampling proportional to w: try uniform entries e, accept when the
@@ -334,7 +391,7 @@ __global__ void mlp_cast_kernel(const float* __restrict__ P, MlpWeights W) {
 __global__ void mlp_sample_kernel(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                                   const uint32_t* __restrict__ q, int64_t n, int64_t nnz, int B, int neg,
                                   const uint32_t* __restrict__ step_dev, uint32_t k0, uint32_t k1,
-                                  int32_t* __restrict__ rows) {
+                                  const int32_t* __restrict__ row_of, int32_t* __restrict__ rows) {
     const int R = 2 + neg;
     const uint32_t step = *step_dev;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < B; s += gridDim.x * blockDim.x) {
@@ -344,7 +401,13 @@ __global__ void mlp_sample_kernel(const int32_t* __restrict__ rp, const int32_t*
             e = __umulhi(u.x, uint32_t(nnz));
             if ((u.y >> 8) < q[e]) break;
         }
-        int64_t lo = 0, hi = n - 1;  // head row: last i with rp[i] <= e
+        // head row: from the table when there is one (a search is 17 dependent
+        // loads at 70,000 rows), else the last i with rp[i] <= e
+        int64_t lo = row_of ? row_of[e] : -1, hi = lo;
+        if (lo < 0) {
+            lo = 0;
+            hi = n - 1;
+        }
         while (lo < hi) {
             const int64_t mid = (lo + hi + 1) >> 1;
             if (rp[mid] <= int32_t(e)) lo = mid; else hi = mid - 1;
@@ -356,6 +419,15 @@ __global__ void mlp_sample_kernel(const int32_t* __restrict__ rp, const int32_t*
             const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
             rows[int64_t(s) * R + 2 + t] = int32_t(__umulhi(w4[t & 3], uint32_t(n)));
         }
+    }
+}
+
+// Head row of every CSR entry (entries that no row covers keep -1).
+__global__ void mlp_heads_kernel(const int32_t* __restrict__ rp, int64_t n, int64_t nnz, int32_t* __restrict__ row_of) {
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+        const int32_t b = rp[i], e = rp[i + 1];
+        if (b < 0 || e > nnz) continue;
+        for (int32_t t = b; t < e; ++t) row_of[t] = int32_t(i);
     }
 }
 
@@ -380,25 +452,46 @@ __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int3
         }
 }
 
-// z = H2 W3^T + b3: one warp per row.
-__global__ void mlp_head_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
-                                const float* __restrict__ P, int M, float* __restrict__ z) {
+// z = H2 W3^T + b3: one warp per row, lanes on columns lane + 32 i; four rows'
+// loads are in flight together.
+static constexpr int HEAD_ROWS = 4;
+
+__global__ void __launch_bounds__(256) mlp_head_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
+                                                       const float* __restrict__ P, int M, float* __restrict__ z) {
     const int lane = threadIdx.x & 31;
-    for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < M;
-         r += (int64_t(gridDim.x) * blockDim.x) >> 5) {
-        float s0 = 0.f, s1 = 0.f;
-        for (int cc = lane; cc < MLP_H; cc += 32) {
-            const float h = __bfloat162float(H2[r * MLP_H + cc]);
-            s0 = fmaf(h, W3f[cc], s0);
-            s1 = fmaf(h, W3f[MLP_H + cc], s1);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        }
-        if (lane == 0) {
-            z[2 * r] = s0 + P[OFF_B3];
-            z[2 * r + 1] = s1 + P[OFF_B3 + 1];
+    float w0[MLP_H / 32], w1[MLP_H / 32];
+#pragma unroll
+    for (int i = 0; i < MLP_H / 32; ++i) {
+        w0[i] = W3f[lane + 32 * i];
+        w1[i] = W3f[MLP_H + lane + 32 * i];
+    }
+    const float b0 = P[OFF_B3], b1 = P[OFF_B3 + 1];
+    const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    // M is a multiple of 128, so groups of HEAD_ROWS rows are whole
+    for (int64_t r0 = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * HEAD_ROWS; r0 < M; r0 += warps * HEAD_ROWS) {
+        bf16 h[HEAD_ROWS][MLP_H / 32];
+#pragma unroll
+        for (int u = 0; u < HEAD_ROWS; ++u)
+#pragma unroll
+            for (int i = 0; i < MLP_H / 32; ++i) h[u][i] = H2[(r0 + u) * MLP_H + lane + 32 * i];
+#pragma unroll
+        for (int u = 0; u < HEAD_ROWS; ++u) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < MLP_H / 32; ++i) {
+                const float x = __bfloat162float(h[u][i]);
+                s0 = fmaf(x, w0[i], s0);
+                s1 = fmaf(x, w1[i], s1);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            }
+            if (lane == 0) {
+                z[2 * (r0 + u)] = s0 + b0;
+                z[2 * (r0 + u) + 1] = s1 + b1;
+            }
         }
     }
 }
@@ -449,54 +542,110 @@ __global__ void mlp_loss_kernel(const float* __restrict__ z, const int32_t* __re
     }
 }
 
-// dpre2 = (dz W3) . GELU'(pre2): BF16 row-major and transposed (32 x 32 tiles).
-__global__ void mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f,
-                                  const float* __restrict__ pre2, int M, bf16* __restrict__ D, bf16* __restrict__ Dt,
-                                  float* __restrict__ Df) {
-    __shared__ bf16 tile[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    for (int ty = threadIdx.y; ty < 32; ty += blockDim.y) {
-        const int64_t r = r0 + ty;
-        const int cc = c0 + threadIdx.x;
-        const float g = dz[2 * r] * W3f[cc] + dz[2 * r + 1] * W3f[MLP_H + cc];
-        const float v = g * gelu_grad(pre2[r * MLP_H + cc]);
-        Df[r * MLP_H + cc] = v;
-        const bf16 bv = __float2bfloat16_rn(v);
-        D[r * MLP_H + cc] = bv;
-        tile[ty][threadIdx.x] = bv;
-    }
-    __syncthreads();
-    for (int ty = threadIdx.y; ty < 32; ty += blockDim.y) {
-        const int cc = c0 + ty;
-        Dt[int64_t(cc) * M + r0 + threadIdx.x] = tile[threadIdx.x][ty];
-    }
-}
+// One CTA takes a chunk of MLP_CHUNK rows and 32 columns.  The sums over a
+// chunk's rows run in row order, one column a lane, from shared memory: their
+// chains of 512 additions take about 2 us when no load sits inside them (56
+// CTAs of 256 columns reading each row from L2 took 140 us for dW3, 40 us for
+// a bias gradient).
+static constexpr int MLP_CHUNK = 512;
+static constexpr int MC_THREADS = 256;
+static constexpr int MC_PITCH = MLP_CHUNK * 4 + 4;  // floats per float4 column: lanes of a row hit distinct banks
 
-// Column sums of an FP32 [M x C] matrix over row chunks: part[blk][c].
-__global__ void mlp_colsum_kernel(const float* __restrict__ A, int M, int C, int chunk, float* __restrict__ part) {
-    for (int cc = threadIdx.x; cc < C; cc += blockDim.x) {
-        float s = 0.f;
-        const int r_end = (blockIdx.x + 1) * chunk < M ? (blockIdx.x + 1) * chunk : M;
-        for (int r = blockIdx.x * chunk; r < r_end; ++r) s += A[int64_t(r) * C + cc];
-        part[int64_t(blockIdx.x) * C + cc] = s;
-    }
-}
+// dpre2 = (dz W3) . GELU'(pre2) (BF16 row-major and transposed) and, over the
+// chunk, db2 = sum dpre2, dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
+static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 64 + MLP_CHUNK * 8;
 
-// dW3[o][c] = sum_r dz[r][o] H2[r][c] and db3[o] = sum_r dz[r][o] over row chunks.
-__global__ void mlp_w3grad_kernel(const float* __restrict__ dz, const bf16* __restrict__ H2, int M, int chunk,
-                                  float* __restrict__ part) {
-    const int r_end = (blockIdx.x + 1) * chunk < M ? (blockIdx.x + 1) * chunk : M;
-    for (int t = threadIdx.x; t < 2 * MLP_H + 2; t += blockDim.x) {
-        float s = 0.f;
-        if (t < 2 * MLP_H) {
-            const int o = t / MLP_H, cc = t % MLP_H;
-            for (int r = blockIdx.x * chunk; r < r_end; ++r)
-                s += dz[2 * int64_t(r) + o] * __bfloat162float(H2[int64_t(r) * MLP_H + cc]);
-        } else {
-            const int o = t - 2 * MLP_H;
-            for (int r = blockIdx.x * chunk; r < r_end; ++r) s += dz[2 * int64_t(r) + o];
+__global__ void __launch_bounds__(MC_THREADS, 2)
+mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2,
+                  const bf16* __restrict__ H2, int M, bf16* __restrict__ D, bf16* __restrict__ Dt,
+                  float* __restrict__ pb2, float* __restrict__ pw3) {
+    extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]: dpre2, float4 columns
+    bf16* s_h = reinterpret_cast<bf16*>(s_v + 8 * MC_PITCH);       // [MLP_CHUNK][32]: H2
+    float2* s_z = reinterpret_cast<float2*>(s_h + MLP_CHUNK * 32);  // [MLP_CHUNK]: dz
+    const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
+    const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
+    for (int t = tid; t < rows * 4; t += MC_THREADS) {
+        const int r = t >> 2, i = t & 3;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s_h + r * 32 + 8 * i)),
+                     "l"(H2 + int64_t(r0 + r) * MLP_H + c0 + 8 * i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int r = tid; r < rows; r += MC_THREADS) {
+        const float2 dz2 = *reinterpret_cast<const float2*>(dz + 2 * int64_t(r0 + r));
+        s_z[r] = dz2;
+        const float* p = dgelu2 + blocked_at(r0 + r, c0, MLP_H);
+        float4 x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float4*>(p + i * 512);
+        uint32_t packed[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float v[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int cc = c0 + 4 * i + j;
+                const float g = dz2.x * W3f[cc] + dz2.y * W3f[MLP_H + cc];
+                v[j] = g * v[j];
+                Dt[int64_t(cc) * M + r0 + r] = __float2bfloat16_rn(v[j]);
+            }
+            *reinterpret_cast<float4*>(s_v + i * MC_PITCH + 4 * r) = make_float4(v[0], v[1], v[2], v[3]);
+            const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+            packed[2 * i] = *reinterpret_cast<const uint32_t*>(&a);
+            packed[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&b);
         }
-        part[int64_t(blockIdx.x) * (2 * MLP_H + 2) + t] = s;
+        uint4* o = reinterpret_cast<uint4*>(D + int64_t(r0 + r) * MLP_H + c0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = make_uint4(packed[4 * i], packed[4 * i + 1], packed[4 * i + 2], packed[4 * i + 3]);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const int warp = tid >> 5, lane = tid & 31;
+    if (warp == 0) {
+        const float* col = s_v + (lane >> 2) * MC_PITCH + (lane & 3);
+        float s = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) s += col[4 * r];
+        pb2[int64_t(blockIdx.x) * MLP_H + c0 + lane] = s;
+    } else if (warp <= 2) {
+        const int o = warp - 1;
+        const float* zo = reinterpret_cast<const float*>(s_z) + o;
+        float s = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) s += zo[2 * r] * __bfloat162float(s_h[r * 32 + lane]);
+        pw3[int64_t(blockIdx.x) * (2 * MLP_H + 2) + o * MLP_H + c0 + lane] = s;
+    } else if (warp == 3 && c0 == 0 && lane < 2) {
+        const float* zo = reinterpret_cast<const float*>(s_z) + lane;
+        float s = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) s += zo[2 * r];
+        pw3[int64_t(blockIdx.x) * (2 * MLP_H + 2) + 2 * MLP_H + lane] = s;
+    }
+}
+
+// Column sums of a blocked FP32 M x MLP_H matrix over the chunk's rows.
+static constexpr size_t CS_SMEM = size_t(8) * MC_PITCH * 4;
+
+__global__ void __launch_bounds__(MC_THREADS, 3)
+mlp_colsum_kernel(const float* __restrict__ A, int M, float* __restrict__ part) {
+    extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]
+    const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
+    const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
+    for (int r = tid; r < rows; r += MC_THREADS) {
+        const float* p = A + blocked_at(r0 + r, c0, MLP_H);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s_v + i * MC_PITCH + 4 * r)),
+                         "l"(p + i * 512) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (tid < 32) {
+        const float* col = s_v + (tid >> 2) * MC_PITCH + (tid & 3);
+        float s = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) s += col[4 * r];
+        part[int64_t(blockIdx.x) * MLP_H + c0 + tid] = s;
     }
 }
 
@@ -515,24 +664,61 @@ struct GradParts {
     int B;
 };
 
-// Gradient vector from the partial sums (each summed in a fixed order) and
-// the batch loss.
-__global__ void mlp_reduce_kernel(GradParts g, float* __restrict__ grad, float* __restrict__ loss_out,
-                                  const uint32_t* __restrict__ step_dev) {
+template <class F>
+__device__ __forceinline__ float sum_splits(int count, F&& at) {
+    float s = 0.f;
+    for (int z0 = 0; z0 < count; z0 += 8) {  // eight loads in flight, added in order
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = z0 + u < count ? at(z0 + u) : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (z0 + u < count) s += v[u];
+    }
+    return s;
+}
+
+// Adam's state and step (adam_m null: the gradient alone).
+struct AdamArgs {
+    float* P;
+    float* m;
+    float* v;
+    float lr, b1, b2, eps;
+    MlpWeights W;
+};
+
+// Gradient vector from the partial sums (each summed in a fixed order), the
+// batch loss, and with `ADAM` the update of the FP32 master weights
+// (bias-corrected step t = *step + 1) and their BF16 copies.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) mlp_update_kernel(GradParts g, AdamArgs A, float* __restrict__ grad,
+                                                         float* __restrict__ loss_out,
+                                                         const uint32_t* __restrict__ step_dev) {
+    const uint32_t step = *step_dev;
+    float c1 = 1.f, c2 = 1.f;
+    if (ADAM) {
+        const float t = float(step + 1);
+        c1 = 1.0f - powf(A.b1, t);
+        c2 = 1.0f - powf(A.b2, t);
+    }
     for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < MLP_P; p += int64_t(gridDim.x) * blockDim.x) {
-        float s = 0.f;
-        if (p < OFF_B1) {
-            for (int z = 0; z < g.s1; ++z) s += g.dW1[int64_t(z) * MLP_H * MLP_IN + p];
-        } else if (p < OFF_W2) {
-            for (int z = 0; z < g.n1; ++z) s += g.db1[int64_t(z) * MLP_H + (p - OFF_B1)];
-        } else if (p < OFF_B2) {
-            for (int z = 0; z < g.s2; ++z) s += g.dW2[int64_t(z) * MLP_H * MLP_H + (p - OFF_W2)];
-        } else if (p < OFF_W3) {
-            for (int z = 0; z < g.n2; ++z) s += g.db2[int64_t(z) * MLP_H + (p - OFF_B2)];
-        } else {
-            for (int z = 0; z < g.n3; ++z) s += g.w3[int64_t(z) * (2 * MLP_H + 2) + (p - OFF_W3)];
-        }
+        float s;
+        if (p < OFF_B1) s = sum_splits(g.s1, [&](int z) { return g.dW1[int64_t(z) * MLP_H * MLP_IN + p]; });
+        else if (p < OFF_W2) s = sum_splits(g.n1, [&](int z) { return g.db1[int64_t(z) * MLP_H + (p - OFF_B1)]; });
+        else if (p < OFF_B2) s = sum_splits(g.s2, [&](int z) { return g.dW2[int64_t(z) * MLP_H * MLP_H + (p - OFF_W2)]; });
+        else if (p < OFF_W3) s = sum_splits(g.n2, [&](int z) { return g.db2[int64_t(z) * MLP_H + (p - OFF_B2)]; });
+        else s = sum_splits(g.n3, [&](int z) { return g.w3[int64_t(z) * (2 * MLP_H + 2) + (p - OFF_W3)]; });
         grad[p] = s;
+        if (ADAM) {
+            const float mm = A.b1 * A.m[p] + (1.0f - A.b1) * s;
+            const float vv = A.b2 * A.v[p] + (1.0f - A.b2) * s * s;
+            A.m[p] = mm;
+            A.v[p] = vv;
+            float w = A.P[p];
+            w -= A.lr * (mm / c1) / (sqrtf(vv / c2) + A.eps);
+            A.P[p] = w;
+            mlp_cast_one(w, p, A.W);
+        }
     }
     if (blockIdx.x == 0 && loss_out) {
         __shared__ float red[256];
@@ -544,24 +730,7 @@ __global__ void mlp_reduce_kernel(GradParts g, float* __restrict__ grad, float* 
             if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
             __syncthreads();
         }
-        if (threadIdx.x == 0) loss_out[step_dev ? *step_dev : 0] = red[0];
-    }
-}
-
-// Adam on the FP32 master weights (bias-corrected step t = *step + 1), then
-// the step counter advances.
-__global__ void mlp_adam_kernel(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                                const float* __restrict__ grad, float lr, float b1, float b2, float eps,
-                                uint32_t* __restrict__ step_dev) {
-    const float t = float(*step_dev + 1);
-    const float c1 = 1.0f - powf(b1, t), c2 = 1.0f - powf(b2, t);
-    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < MLP_P; p += int64_t(gridDim.x) * blockDim.x) {
-        const float g = grad[p];
-        const float mm = b1 * m[p] + (1.0f - b1) * g;
-        const float vv = b2 * v[p] + (1.0f - b2) * g * g;
-        m[p] = mm;
-        v[p] = vv;
-        P[p] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+        if (threadIdx.x == 0) loss_out[step] = red[0];
     }
 }
 
@@ -582,11 +751,18 @@ __global__ void mlp_init_kernel(float* __restrict__ P, int d, uint32_t k0, uint3
 }
 
 // ------------------------------------------------------------------ host: one forward/backward
+// Opt the chunk kernels into their shared-memory sizes (before any capture).
+static int chunk_prepare(Ctx* c) {
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_l3back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(L3_SMEM)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_colsum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(CS_SMEM)));
+    return DRGB_OK;
+}
+
 struct MlpBuffers {
     int M;                       // rows of the batch (padded to 128)
     int32_t* rows;
-    bf16 *Xb, *Xbt, *H1b, *H1bt, *H2b, *H2bt, *D2b, *D2bt, *D1b, *D1bt;
-    float *pre1, *pre2, *z, *dz, *D2f, *D1f, *loss_part;
+    bf16 *Xb, *Xbt, *H1b, *H1bt, *H2b, *D2b, *D2bt, *D1b, *D1bt;
+    float *dg1, *dg2, *z, *dz, *D1f, *loss_part;
     float *pW2, *pW1, *pb1, *pb2, *pw3;
     float* grad;
     MlpWeights W;
@@ -595,15 +771,13 @@ struct MlpBuffers {
 };
 
 static constexpr int MLP_SPLITS = 32;
-static constexpr int MLP_CHUNK = 512;
-
 static size_t mlp_batch_bytes(int M) {
     const size_t m = size_t(M);
     const int nch = int((m + MLP_CHUNK - 1) / MLP_CHUNK);
     size_t b = Carve::round(m * 4);                                   // rows
     b += 2 * Carve::round(m * MLP_IN * 2);                            // Xb, Xbt
-    b += 8 * Carve::round(m * MLP_H * 2);                             // H1b, H1bt, H2b, H2bt, D2b, D2bt, D1b, D1bt
-    b += 4 * Carve::round(m * MLP_H * 4);                             // pre1, pre2, D2f, D1f
+    b += 7 * Carve::round(m * MLP_H * 2);                             // H1b, H1bt, H2b, D2b, D2bt, D1b, D1bt
+    b += 3 * Carve::round(m * MLP_H * 4);                             // dg1, dg2, D1f
     b += 2 * Carve::round(m * 2 * 4) + Carve::round(m * 4);           // z, dz, loss_part
     b += Carve::round(size_t(MLP_SPLITS) * MLP_H * MLP_H * 4);        // pW2
     b += Carve::round(size_t(MLP_SPLITS) * MLP_H * MLP_IN * 4);       // pW1
@@ -628,14 +802,12 @@ static MlpBuffers mlp_carve(void* base, int M) {
     b.H1b = cv.take<bf16>(m * MLP_H);
     b.H1bt = cv.take<bf16>(m * MLP_H);
     b.H2b = cv.take<bf16>(m * MLP_H);
-    b.H2bt = cv.take<bf16>(m * MLP_H);
     b.D2b = cv.take<bf16>(m * MLP_H);
     b.D2bt = cv.take<bf16>(m * MLP_H);
     b.D1b = cv.take<bf16>(m * MLP_H);
     b.D1bt = cv.take<bf16>(m * MLP_H);
-    b.pre1 = cv.take<float>(m * MLP_H);
-    b.pre2 = cv.take<float>(m * MLP_H);
-    b.D2f = cv.take<float>(m * MLP_H);
+    b.dg1 = cv.take<float>(m * MLP_H);
+    b.dg2 = cv.take<float>(m * MLP_H);
     b.D1f = cv.take<float>(m * MLP_H);
     b.z = cv.take<float>(m * 2);
     b.dz = cv.take<float>(m * 2);
@@ -654,57 +826,64 @@ static MlpBuffers mlp_carve(void* base, int M) {
     return b;
 }
 
+// A second branch of the step: with a stream, work forks off `st` and joins
+// it again through the events; without one it runs in line.
+struct MlpFork {
+    cudaStream_t side = nullptr;
+    cudaEvent_t forked = nullptr, joined = nullptr;
+};
+
 // Forward + backward of the batch whose rows are already gathered (Xb, Xbt)
 // with B edges of R rows; leaves the gradient in b.grad and the loss in
-// loss_out[*step] (if given).
+// loss_out[*step] (if given), and with `adam` updates the weights.
 static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, float a, float bb,
-                       float* loss_out, cudaStream_t st) {
+                       float* loss_out, const AdamArgs* adam, const MlpFork& fork, cudaStream_t st) {
     const int M = b.M;
     int rc;
     Gemm F1, F2, DW2, DH1, DW1;
-    if ((rc = gemm_setup(c, F1, b.Xb, b.W.W1b, M, MLP_H, MLP_IN, 256, EPI_GELU, 1))) return rc;
+    if ((rc = gemm_setup(c, F1, b.Xb, b.W.W1b, M, MLP_H, MLP_IN, 128, EPI_GELU, 1))) return rc;
     F1.g.bias = P + OFF_B1;
-    F1.g.pre = b.pre1;
+    F1.g.dgelu = b.dg1;
     F1.g.out = b.H1b;
     F1.g.out_t = b.H1bt;
-    if ((rc = gemm_setup(c, F2, b.H1b, b.W.W2b, M, MLP_H, MLP_H, 256, EPI_GELU, 1))) return rc;
+    if ((rc = gemm_setup(c, F2, b.H1b, b.W.W2b, M, MLP_H, MLP_H, 128, EPI_GELU, 1))) return rc;
     F2.g.bias = P + OFF_B2;
-    F2.g.pre = b.pre2;
+    F2.g.dgelu = b.dg2;
     F2.g.out = b.H2b;
-    F2.g.out_t = b.H2bt;
     if ((rc = gemm_launch(c, F1, st))) return rc;
     if ((rc = gemm_launch(c, F2, st))) return rc;
-    mlp_head_kernel<<<grid_for(int64_t(M) * 32, 256, c->num_sms * 16), 256, 0, st>>>(b.H2b, b.W.W3f, P, M, b.z);
+    mlp_head_kernel<<<grid_for(M / HEAD_ROWS, 8, c->num_sms * 8), 256, 0, st>>>(b.H2b, b.W.W3f, P, M, b.z);
     DRGB_CHECK_LAUNCH(c);
     if (M > B * (2 + neg))  // padding rows carry no gradient
         DRGB_CUDA(c, cudaMemsetAsync(b.dz + 2 * int64_t(B) * (2 + neg), 0,
                                      (size_t(M) - size_t(B) * (2 + neg)) * 2 * 4, st));
-    mlp_loss_kernel<<<grid_for(B, 128, c->num_sms * 8), 128, 0, st>>>(b.z, b.rows, B, neg, a, bb, b.dz, b.loss_part);
+    mlp_loss_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, st>>>(b.z, b.rows, B, neg, a, bb, b.dz, b.loss_part);
     DRGB_CHECK_LAUNCH(c);
-    mlp_l3back_kernel<<<dim3(M / 32, MLP_H / 32), dim3(32, 8), 0, st>>>(b.dz, b.W.W3f, b.pre2, M, b.D2b, b.D2bt,
-                                                                      b.D2f);
+    const dim3 cgrid(b.n_chunks, MLP_H / 32);
+    mlp_l3back_kernel<<<cgrid, MC_THREADS, L3_SMEM, st>>>(b.dz, b.W.W3f, b.dg2, b.H2b, M, b.D2b, b.D2bt, b.pb2, b.pw3);
     DRGB_CHECK_LAUNCH(c);
-    mlp_w3grad_kernel<<<b.n_chunks, 256, 0, st>>>(b.dz, b.H2b, M, MLP_CHUNK, b.pw3);
-    DRGB_CHECK_LAUNCH(c);
-    mlp_colsum_kernel<<<b.n_chunks, 256, 0, st>>>(b.D2f, M, MLP_H, MLP_CHUNK, b.pb2);
-    DRGB_CHECK_LAUNCH(c);
-    // dW2 = dpre2^T H1 (K = M, split)
-    if ((rc = gemm_setup(c, DW2, b.D2bt, b.H1bt, MLP_H, MLP_H, M, 256, EPI_F32, MLP_SPLITS))) return rc;
+    // dW2 = dpre2^T H1 (K = M, split), beside dH1 and what follows from it
+    if (fork.side) {
+        DRGB_CUDA(c, cudaEventRecord(fork.forked, st));
+        DRGB_CUDA(c, cudaStreamWaitEvent(fork.side, fork.forked, 0));
+    }
+    if ((rc = gemm_setup(c, DW2, b.D2bt, b.H1bt, MLP_H, MLP_H, M, 128, EPI_F32, MLP_SPLITS))) return rc;
     DW2.g.out_f32 = b.pW2;
-    if ((rc = gemm_launch(c, DW2, st))) return rc;
+    if ((rc = gemm_launch(c, DW2, fork.side ? fork.side : st))) return rc;
+    if (fork.side) DRGB_CUDA(c, cudaEventRecord(fork.joined, fork.side));
     // dpre1 = (dpre2 W2) . GELU'(pre1): A = dpre2 [M x 256(out)], B = W2^T [256(in) x 256(out)]
-    if ((rc = gemm_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H, MLP_H, 256, EPI_GELU_GRAD, 1))) return rc;
-    DH1.g.pre = b.pre1;
-    DH1.g.out = b.D1b;
+    if ((rc = gemm_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H, MLP_H, 128, EPI_GELU_GRAD, 1))) return rc;
+    DH1.g.dgelu = b.dg1;
     DH1.g.out_t = b.D1bt;
     DH1.g.out_f32 = b.D1f;
     if ((rc = gemm_launch(c, DH1, st))) return rc;
-    mlp_colsum_kernel<<<b.n_chunks, 256, 0, st>>>(b.D1f, M, MLP_H, MLP_CHUNK, b.pb1);
+    mlp_colsum_kernel<<<cgrid, MC_THREADS, CS_SMEM, st>>>(b.D1f, M, b.pb1);
     DRGB_CHECK_LAUNCH(c);
     // dW1 = dpre1^T Xb: A = dpre1^T [256 x M], B = Xb^T [64 x M]
     if ((rc = gemm_setup(c, DW1, b.D1bt, b.Xbt, MLP_H, MLP_IN, M, 64, EPI_F32, MLP_SPLITS))) return rc;
     DW1.g.out_f32 = b.pW1;
     if ((rc = gemm_launch(c, DW1, st))) return rc;
+    if (fork.side) DRGB_CUDA(c, cudaStreamWaitEvent(st, fork.joined, 0));
     GradParts gp;
     gp.dW1 = b.pW1;
     gp.s1 = int(DW1.grid.z);
@@ -718,7 +897,9 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     gp.n3 = b.n_chunks;
     gp.loss = b.loss_part;
     gp.B = B;
-    mlp_reduce_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(gp, b.grad, loss_out, b.step);
+    const int ugrid = grid_for(MLP_P, 256, c->num_sms * 4);
+    if (adam) mlp_update_kernel<true><<<ugrid, 256, 0, st>>>(gp, *adam, b.grad, loss_out, b.step);
+    else mlp_update_kernel<false><<<ugrid, 256, 0, st>>>(gp, AdamArgs{}, b.grad, loss_out, b.step);
     DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
@@ -756,7 +937,7 @@ int drgb_mlp_grad(drgb_ctx* c, const float* params, const float* X, int64_t n, i
     if (!params || !X || !rows || !grad_out || n_edges < 1 || neg < 0 || neg > 8 || n < 2)
         return set_error(c, DRGB_ERR_INVALID, "mlp_grad: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if ((rc = gemm_prepare(c))) return rc;
+    if ((rc = gemm_prepare(c)) || (rc = chunk_prepare(c))) return rc;
     const int Mv = n_edges * (2 + neg);
     const int M = round_up(Mv, 128);
     if ((rc = ensure_scratch(c, mlp_batch_bytes(M), st))) return rc;
@@ -764,11 +945,11 @@ int drgb_mlp_grad(drgb_ctx* c, const float* params, const float* X, int64_t n, i
     DRGB_CUDA(c, cudaMemsetAsync(bu.rows, 0, size_t(M) * 4, st));
     DRGB_CUDA(c, cudaMemcpyAsync(bu.rows, rows, size_t(Mv) * 4, cudaMemcpyDeviceToDevice, st));
     DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0, 64, st));
-    mlp_cast_kernel<<<grid_for(MLP_H * MLP_H, 256, c->num_sms * 4), 256, 0, st>>>(params, bu.W);
+    mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, bu.W);
     DRGB_CHECK_LAUNCH(c);
     mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, st>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt);
     DRGB_CHECK_LAUNCH(c);
-    if ((rc = mlp_fwd_bwd(c, bu, params, n_edges, neg, a, b, loss_out, st))) return rc;
+    if ((rc = mlp_fwd_bwd(c, bu, params, n_edges, neg, a, b, loss_out, nullptr, MlpFork{}, st))) return rc;
     DRGB_CUDA(c, cudaMemcpyAsync(grad_out, bu.grad, MLP_P * 4, cudaMemcpyDeviceToDevice, st));
     return drgb_sync(c, stream);
 }
@@ -782,39 +963,58 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
         mp->batch_edges < 1 || mp->neg < 0 || mp->neg > 8 || mp->steps < 0)
         return set_error(c, DRGB_ERR_INVALID, "mlp_train: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if ((rc = gemm_prepare(c))) return rc;
+    if ((rc = gemm_prepare(c)) || (rc = chunk_prepare(c))) return rc;
     const int B = mp->batch_edges, neg = mp->neg, R = 2 + neg;
     const int Mv = B * R;
     const int M = round_up(Mv, 128);
-    if ((rc = ensure_scratch(c, mlp_batch_bytes(M), st))) return rc;
+    // the heads of the CSR entries, if there is room for them beside the batch
+    const size_t least = mlp_batch_bytes(M);
+    size_t bytes = Carve::round(least) + size_t(nnz) * 4;
+    if ((rc = ensure_scratch_within(c, &bytes, least, st))) return rc;
     MlpBuffers bu = mlp_carve(c->scratch, M);
+    int32_t* row_of = bytes > least ? reinterpret_cast<int32_t*>(static_cast<char*>(c->scratch) + Carve::round(least)) : nullptr;
     DRGB_CUDA(c, cudaMemsetAsync(bu.rows, 0, size_t(M) * 4, st));
     DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0, 64, st));
+    if (row_of) {
+        DRGB_CUDA(c, cudaMemsetAsync(row_of, 0xFF, size_t(nnz) * 4, st));
+        mlp_heads_kernel<<<grid_for(n, 256, c->num_sms * 8), 256, 0, st>>>(row_ptr, n, nnz, row_of);
+        DRGB_CHECK_LAUNCH(c);
+    }
+    mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, bu.W);
+    DRGB_CHECK_LAUNCH(c);
     const uint32_t k0 = uint32_t(mp->seed), k1 = uint32_t(mp->seed >> 32);
 
     // capture one step, replay it mp->steps times (the step counter lives on
     // the device, so every replay draws a fresh batch)
-    cudaStream_t cap;
-    DRGB_CUDA(c, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+    cudaStream_t cap = nullptr;
+    MlpFork fork;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    auto release = [&]() {
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+        if (fork.forked) cudaEventDestroy(fork.forked);
+        if (fork.joined) cudaEventDestroy(fork.joined);
+        if (fork.side) cudaStreamDestroy(fork.side);
+        if (cap) cudaStreamDestroy(cap);
+    };
+    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&fork.side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork.forked, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork.joined, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) {
-        cudaStreamDestroy(cap);
+        release();
         return set_error(c, DRGB_ERR_CUDA, "mlp_train: begin capture: %s", cudaGetErrorString(e));
     }
+    const AdamArgs adam{params, adam_m, adam_v, mp->lr, mp->beta1, mp->beta2, mp->eps, bu.W};
     do {
-        mlp_cast_kernel<<<grid_for(MLP_H * MLP_H, 256, c->num_sms * 4), 256, 0, cap>>>(params, bu.W);
-        if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
-        mlp_sample_kernel<<<grid_for(B, 128, c->num_sms * 8), 128, 0, cap>>>(row_ptr, col, q, n, nnz, B, neg, bu.step,
-                                                                            k0, k1, bu.rows);
+        mlp_sample_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, cap>>>(row_ptr, col, q, n, nnz, B, neg, bu.step,
+                                                                          k0, k1, row_of, bu.rows);
         if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
         mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, cap>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt);
         if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
-        if ((rc = mlp_fwd_bwd(c, bu, params, B, neg, a, b, losses, cap))) break;
-        mlp_adam_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, cap>>>(
-            params, adam_m, adam_v, bu.grad, mp->lr, mp->beta1, mp->beta2, mp->eps, bu.step);
-        if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
+        if ((rc = mlp_fwd_bwd(c, bu, params, B, neg, a, b, losses, &adam, fork, cap))) break;
         mlp_step_advance_kernel<<<1, 1, 0, cap>>>(bu.step);
         if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
     } while (0);
@@ -826,9 +1026,7 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
         e = cudaGraphLaunch(exec, st);
         if (e != cudaSuccess) rc = set_error(c, DRGB_ERR_CUDA, "mlp_train: launch: %s", cudaGetErrorString(e));
     }
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-    cudaStreamDestroy(cap);
+    release();
     if (rc) return rc;
     return drgb_sync(c, stream);
 }
@@ -846,7 +1044,7 @@ int drgb_mlp_sample(drgb_ctx* c, const int32_t* row_ptr, const int32_t* col, con
     DRGB_CUDA(c, cudaMemcpyAsync(step_dev, &step, 4, cudaMemcpyHostToDevice, st));
     mlp_sample_kernel<<<grid_for(n_edges, 128, c->num_sms * 8), 128, 0, st>>>(row_ptr, col, q, n, nnz, n_edges, neg,
                                                                              step_dev, uint32_t(seed),
-                                                                             uint32_t(seed >> 32), rows);
+                                                                             uint32_t(seed >> 32), nullptr, rows);
     DRGB_CHECK_LAUNCH(c);
     return drgb_sync(c, stream);
 }
@@ -872,7 +1070,7 @@ int drgb_mlp_embed(drgb_ctx* c, const float* params, const float* X, int64_t n, 
     W.W2tb = cv.take<bf16>(MLP_H * MLP_H);
     W.W1b = cv.take<bf16>(MLP_H * MLP_IN);
     W.W3f = cv.take<float>(2 * MLP_H);
-    mlp_cast_kernel<<<grid_for(MLP_H * MLP_H, 256, c->num_sms * 4), 256, 0, st>>>(params, W);
+    mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, W);
     DRGB_CHECK_LAUNCH(c);
     for (int64_t r0 = 0; r0 < n; r0 += CH) {
         const int mv = int(n - r0 < CH ? n - r0 : CH);
@@ -881,14 +1079,14 @@ int drgb_mlp_embed(drgb_ctx* c, const float* params, const float* X, int64_t n, 
                                                                             nullptr);
         DRGB_CHECK_LAUNCH(c);
         Gemm F1, F2;
-        if ((rc = gemm_setup(c, F1, Xb, W.W1b, M, MLP_H, MLP_IN, 256, EPI_GELU, 1))) return rc;
+        if ((rc = gemm_setup(c, F1, Xb, W.W1b, M, MLP_H, MLP_IN, 128, EPI_GELU, 1))) return rc;
         F1.g.bias = params + OFF_B1;
         F1.g.out = H1;
-        if ((rc = gemm_setup(c, F2, H1, W.W2b, M, MLP_H, MLP_H, 256, EPI_GELU, 1))) return rc;
+        if ((rc = gemm_setup(c, F2, H1, W.W2b, M, MLP_H, MLP_H, 128, EPI_GELU, 1))) return rc;
         F2.g.bias = params + OFF_B2;
         F2.g.out = H2;
         if ((rc = gemm_launch(c, F1, st)) || (rc = gemm_launch(c, F2, st))) return rc;
-        mlp_head_kernel<<<grid_for(int64_t(M) * 32, 256, c->num_sms * 16), 256, 0, st>>>(H2, W.W3f, params, M, z);
+        mlp_head_kernel<<<grid_for(M / HEAD_ROWS, 8, c->num_sms * 8), 256, 0, st>>>(H2, W.W3f, params, M, z);
         DRGB_CHECK_LAUNCH(c);
         DRGB_CUDA(c, cudaMemcpyAsync(Y + 2 * r0, z, size_t(mv) * 8, cudaMemcpyDeviceToDevice, st));
     }
