@@ -32,6 +32,12 @@
 
 namespace drgb {
 
+__device__ __forceinline__ unsigned long long loop_timer() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 __global__ void init_embedding_kernel(float2* __restrict__ Y, int64_t n, float range, uint32_t k0,
                                       uint32_t k1) {
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
@@ -79,8 +85,13 @@ __device__ __forceinline__ float pow_pos(float d, float b) { return hw_ex2(b * h
 static constexpr unsigned FULL = 0xffffffffu;
 
 // Read of one point of Y^(t).  (Read-only-path and L1 evict-last loads were
-// measured and made no difference.)
-__device__ __forceinline__ float2 load_y(const float2* p) { return *p; }
+// measured and made no difference.)  L2: through L2 only, for a kernel that
+// runs several epochs (its L1 may hold an older epoch's line).
+template <bool L2 = false>
+__device__ __forceinline__ float2 load_y(const float2* p) {
+    if constexpr (L2) return __ldcg(p);
+    return *p;
+}
 
 // Instance-local view of a row: rows [off, off + n) with entries from eoff on,
 // negatives drawn under Philox key (k0, k1).  A single instance has off = 0,
@@ -95,8 +106,8 @@ struct RowInst {
 // What changes from one epoch to the next: the positions read and written,
 // the learning rate and the epoch number.
 struct EpochStep {
-    const float2* __restrict__ Y_in;
-    float2* __restrict__ Y_out;
+    const float2* Y_in;
+    float2* Y_out;
     float lr;
     uint32_t t;
 };
@@ -117,9 +128,9 @@ __device__ __forceinline__ U4 negative_words(const EpochArgs& A, const EpochStep
 // for any count up to 64 (A.neg).
 //
 // It is split in two so that a warp can gather one group's points while it
-// computes the previous group's forces: fetch_entry draws the first (up to
-// eight) negatives and issues the loads of Y_i, Y_j and Y_m; entry_math does
-// the arithmetic (and, for more than eight negatives, draws and gathers the
+// computes the previous group's forces: draw_entry draws the first (up to
+// eight) negatives, gather_entry issues the loads of Y_i, Y_j and Y_m, and
+// entry_math does the arithmetic (and, for more than eight negatives, draws and gathers the
 // rest itself).
 //
 // A skipped negative (m = i) is evaluated with Y_m = Y_i: its difference vector
@@ -136,23 +147,30 @@ struct EntryInputs {
     bool ok;
 };
 
+// Which points an entry reads: everything that does not need Y.
+template <int NEG>
+struct EntryPlan {
+    static constexpr int NP = EntryInputs<NEG>::NP;
+    int32_t e, i;      // as in EntryInputs
+    int32_t ii, jj;    // rows of Y_i and Y_j (a valid row for an invalid entry)
+    uint32_t m[NP > 0 ? NP : 1];  // negatives (instance-local; a skipped one names row i)
+    bool ok;
+};
+
 template <int NEG, bool BATCHED>
-__device__ __forceinline__ void fetch_entry(const EpochArgs& A, const EpochStep& S, const RowInst& R, bool valid,
-                                            int32_t e, int32_t j,
-                                            int32_t i, int64_t h_lo, int64_t h_hi, int lane,
-                                            EntryInputs<NEG>& in) {
+__device__ __forceinline__ void draw_entry(const EpochArgs& A, const EpochStep& S, const RowInst& R, bool valid,
+                                           int32_t e, int32_t j, int32_t i, int64_t h_lo, int64_t h_hi, int lane,
+                                           EntryPlan<NEG>& pl) {
     constexpr int NP = EntryInputs<NEG>::NP;
     const int neg = NEG >= 0 ? NEG : A.neg;
-    bool ok = valid && i >= h_lo && i < h_hi && uint64_t(uint32_t(j)) < uint64_t(A.n);
+    const bool ok = valid && i >= h_lo && i < h_hi && uint64_t(uint32_t(j)) < uint64_t(A.n);
     if (valid && !ok) report_status(A.status, DRGB_ERR_INVALID);  // malformed CSR: skip the entry
-    in.ok = ok;
-    in.e = e;
-    in.i = ok ? i : -1 - lane;
-    const int32_t ii = ok ? i : int32_t(h_lo);
-    in.yi = load_y(S.Y_in + ii);
-    in.yj = load_y(S.Y_in + (ok ? j : ii));
-    const uint32_t n32 = R.n, i32 = uint32_t(ii - R.off), e32 = uint32_t(e - R.eoff);
-    const float2* Yb = S.Y_in + R.off;
+    pl.ok = ok;
+    pl.e = e;
+    pl.i = ok ? i : -1 - lane;
+    pl.ii = ok ? i : int32_t(h_lo);
+    pl.jj = ok ? j : pl.ii;
+    const uint32_t n32 = R.n, i32 = uint32_t(pl.ii - R.off), e32 = uint32_t(e - R.eoff);
     U4 r0{0u, 0u, 0u, 0u}, r1{0u, 0u, 0u, 0u};
     if (NP > 0 && neg > 0) r0 = negative_words<BATCHED>(A, S, R, e32, 0u);
     if (NP > 4 && neg > 4) r1 = negative_words<BATCHED>(A, S, R, e32, 1u);
@@ -161,11 +179,24 @@ __device__ __forceinline__ void fetch_entry(const EpochArgs& A, const EpochStep&
     for (int w = 0; w < NP; ++w) {
         const uint32_t m = __umulhi(u[w], n32);  // floor(u n / 2^32)
         const bool take = ok && (NEG >= 0 || w < neg) && (m != i32);
-        in.ym[w] = load_y(Yb + (take ? m : i32));  // a skipped negative reads Y_i
+        pl.m[w] = take ? m : i32;  // a skipped negative reads Y_i
     }
 }
 
-template <int NEG, bool BATCHED>
+template <int NEG, bool L2 = false>
+__device__ __forceinline__ void gather_entry(const EpochStep& S, const RowInst& R, const EntryPlan<NEG>& pl,
+                                             EntryInputs<NEG>& in) {
+    in.ok = pl.ok;
+    in.e = pl.e;
+    in.i = pl.i;
+    in.yi = load_y<L2>(S.Y_in + pl.ii);
+    in.yj = load_y<L2>(S.Y_in + pl.jj);
+    const float2* Yb = S.Y_in + R.off;
+#pragma unroll
+    for (int w = 0; w < EntryInputs<NEG>::NP; ++w) in.ym[w] = load_y<L2>(Yb + pl.m[w]);
+}
+
+template <int NEG, bool BATCHED, bool L2 = false>
 __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep& S, const RowInst& R,
                                              const EntryInputs<NEG>& in, float two_ab, float two_b) {
     constexpr int NP = EntryInputs<NEG>::NP;
@@ -201,7 +232,7 @@ __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep
             for (int w = 0; w < 4; ++w) {
                 const uint32_t m = __umulhi(v[w], n32);
                 const bool ok = (g * 4 + w < neg) && (m != i32);
-                yg[w] = ok ? load_y(Yb + m) : yi;
+                yg[w] = ok ? load_y<L2>(Yb + m) : yi;
             }
 #pragma unroll
             for (int w = 0; w < 4; ++w) repel(yg[w]);
@@ -298,6 +329,7 @@ int epoch_prepare(Ctx* c, const int32_t* rp, int64_t n, int64_t row_begin, int64
     es->win_cap = (nnz_cap + EPOCH_WIN - 1) / EPOCH_WIN + count;
     es->row_of = cv.take<int32_t>(size_t(nnz_cap > 0 ? nnz_cap : 1));
     es->win_row = cv.take<int32_t>(size_t(es->win_cap + 2));
+    es->sync = cv.take<unsigned int>(2);
     DRGB_CUDA(c, cudaMemsetAsync(es->row_of, 0xFF, size_t(nnz_cap > 0 ? nnz_cap : 1) * 4, st));
     const int64_t n_rows = n - row_begin;
     if (n_rows > 0) {
@@ -358,6 +390,28 @@ struct CsrGlobal {
         hv = in ? __ldcs(row_of + e) : -1;
     }
 };
+// The instance that window W belongs to and the rows [h_lo, h_hi) of its heads.
+template <bool BATCHED>
+__device__ __forceinline__ void window_instance(const EpochArgs& A, int32_t W, RowInst& R, int64_t& h_lo, int64_t& h_hi) {
+    R = RowInst{0, A.neg_n ? A.neg_n : uint32_t(A.n), 0, A.k0, A.k1};
+    h_lo = A.row_begin;
+    h_hi = A.n;
+    if (BATCHED) {
+        int lo = 0, hi = A.count - 1;  // the instance whose windows hold W
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (A.win_base[mid] <= W) lo = mid; else hi = mid - 1;
+        }
+        R.off = A.inst_off[lo];
+        R.n = uint32_t(A.inst_off[lo + 1] - R.off);
+        R.eoff = A.inst_eoff[lo];
+        R.k0 = uint32_t(A.inst_seed[lo]);
+        R.k1 = uint32_t(A.inst_seed[lo] >> 32);
+        h_lo = R.off;
+        h_hi = R.off + R.n;
+    }
+}
+
 // One window W of epoch S, by one warp.  No row crosses a window, so the warp
 // writes the final Y' of every row of the window.
 //
@@ -383,22 +437,9 @@ __device__ __forceinline__ void epoch_window(const EpochArgs& A, const EpochStep
     const unsigned lt_mask = (1u << lane) - 1u;
     const int32_t rA = A.win_row[W], rB = A.win_row[W + 1];
     if (rA >= rB) return;  // a long row started in an earlier window covers this one
-    RowInst R{0, A.neg_n ? A.neg_n : uint32_t(A.n), 0, A.k0, A.k1};
-    int64_t h_lo = A.row_begin, h_hi = A.n;  // rows a head may take (the instance's rows)
-    if (BATCHED) {
-        int lo = 0, hi = A.count - 1;  // the instance whose windows hold W
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (A.win_base[mid] <= W) lo = mid; else hi = mid - 1;
-        }
-        R.off = A.inst_off[lo];
-        R.n = uint32_t(A.inst_off[lo + 1] - R.off);
-        R.eoff = A.inst_eoff[lo];
-        R.k0 = uint32_t(A.inst_seed[lo]);
-        R.k1 = uint32_t(A.inst_seed[lo] >> 32);
-        h_lo = R.off;
-        h_hi = R.off + R.n;
-    }
+    RowInst R;
+    int64_t h_lo, h_hi;  // rows a head may take (the instance's rows)
+    window_instance<BATCHED>(A, W, R, h_lo, h_hi);
     if (rA < h_lo || rB > h_hi) {
         if (lane == 0) report_status(A.status, DRGB_ERR_INVALID);
         return;
@@ -408,7 +449,9 @@ __device__ __forceinline__ void epoch_window(const EpochArgs& A, const EpochStep
     auto fetch_group = [&](int p, int cnt, EntryInputs<NEG>& in) {
         const bool v = lane < cnt;
         const int2 ej = v ? act_w[p + lane] : make_int2(es, 0);
-        fetch_entry<NEG, BATCHED>(A, S, R, v, ej.x, ej.y, v ? head_w[p + lane] : -1, h_lo, h_hi, lane, in);
+        EntryPlan<NEG> pl;
+        draw_entry<NEG, BATCHED>(A, S, R, v, ej.x, ej.y, v ? head_w[p + lane] : -1, h_lo, h_hi, lane, pl);
+        gather_entry<NEG>(S, R, pl, in);
     };
     // Forces of a fetched group of `cnt` entries, added by head.
     auto finish_group = [&](const EntryInputs<NEG>& cur, int cnt) {
@@ -582,6 +625,346 @@ __global__ void __launch_bounds__(NW * 32, epoch_warps_per_sm(PIPE) / NW)
                                                       two_ab, two_b);
 }
 
+// ------------------------------------------------------------------ loop of epochs in one launch
+// All epochs [t_begin, t_end) in one cooperative launch, for graphs of few
+// windows: a CTA takes a window (or every gridDim-th one) with all its warps,
+// and the CTAs meet at a barrier after every epoch.
+//
+// Why: with one warp per window and one launch per epoch an epoch of a small
+// graph is one chain of dependent steps (a warp's 16 CSR chunks, five groups of
+// gathers and forces, the next launch) on a few SMs: 8 us for 2,000 rows (15
+// CTAs), 13 us for the anchored epochs of 5,000 new points.  Here the
+// window's entries are tested by all warps at once and every group of 32
+// active entries has its own warp, so the chain is one group; the test of the
+// next epoch's first window runs while the CTA waits at the barrier.
+//
+// Bound: the latency of the barrier and of one group's gathers up to about
+// 5,000 rows (3.2 us an epoch at 2,000), then the windows a CTA takes in turn.
+//
+// The groups and the order of every sum are those of epoch_window: a group's
+// runs that start and end inside it are final, and the first and last run of
+// each group are joined to their neighbours in group order by one thread.
+static constexpr int LOOP_ROUND = 768;  // entries tested per round (a window has about 512)
+static constexpr int LOOP_QCAP = LOOP_ROUND + 32;
+static constexpr int LOOP_LR = 128;     // learning rates computed at a time
+// CTAs of 8 warps while two per SM hold every window, else of 4 warps, which
+// keep more windows in flight (16,000 rows: 9.8 us an epoch with 4 warps and 5
+// CTAs per SM, 11.8 with 8; 6 CTAs per SM spill registers, 13.2 against 11.3
+// at 20,000 rows; CTAs of 2 warps 14.0 against 12.0 at 30,000).
+constexpr int loop_ctas_per_sm(int nw) { return nw == 8 ? 2 : 5; }
+static constexpr int LOOP_WINDOWS = 16;  // windows a CTA may hold
+
+// A CTA's window: its rows, entries and instance.
+struct LoopWindow {
+    int32_t rA, rB, es, ee;
+    RowInst R;
+    int64_t h_lo, h_hi;
+};
+
+struct LoopArgs {
+    float2* buf[2];        // positions of even and odd steps
+    int t_begin, t_end, T;
+    float lr0;
+    unsigned int* arrived;  // barrier counter (0 at the start)
+    int* stop;              // raised by a CTA whose wait ran out (0 at the start)
+};
+
+// The first and the last run of a group.
+struct GroupEnds {
+    int32_t head0, head1;  // their heads (negative: an invalid entry); equal when the group is one run
+    float2 sum0, sum1, y0, y1;
+    bool one;              // the group is one run
+};
+
+template <bool BATCHED, int NEG, int LOOP_WARPS>
+__global__ void __launch_bounds__(LOOP_WARPS * 32, loop_ctas_per_sm(LOOP_WARPS))
+    epoch_loop_kernel(const __grid_constant__ EpochArgs A, const __grid_constant__ LoopArgs P) {
+    constexpr int LOOP_THREADS = LOOP_WARPS * 32;
+    constexpr int LOOP_CHUNKS = LOOP_ROUND / LOOP_THREADS;  // chunks of 32 entries a warp tests per round
+    __shared__ int32_t s_e[LOOP_QCAP];  // active entries
+    __shared__ int s_cnt[LOOP_WARPS];
+    __shared__ GroupEnds s_end[LOOP_QCAP / 32];
+    __shared__ float s_lr[LOOP_LR];
+    __shared__ int32_t s_chead;
+    __shared__ float4 s_carry;
+    __shared__ int s_stop, s_nw;
+    __shared__ LoopWindow s_win[LOOP_WINDOWS];
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const float two_ab = 2.0f * A.a * A.b, two_b = 2.0f * A.b;
+    int32_t nnz = 0, n_win = 0;
+    if (!epoch_extent(A, nnz, n_win)) {
+        if (tid == 0 && blockIdx.x == 0) report_status(A.status, DRGB_ERR_INVALID);
+        return;
+    }
+    if (n_win == 0) {  // no entries at all: every row keeps its position
+        const int last = (P.t_end - P.t_begin) & 1;
+        for (int64_t r = A.row_begin + int64_t(blockIdx.x) * blockDim.x + tid; r < A.n; r += int64_t(gridDim.x) * blockDim.x) {
+            const float2 y = P.buf[0][r];
+            P.buf[last][r] = make_float2(fmaf(P.lr0, 0.f, y.x), fmaf(P.lr0, 0.f, y.y));
+        }
+        return;
+    }
+    const unsigned ctas = unsigned(n_win) < gridDim.x ? unsigned(n_win) : gridDim.x;
+    if (blockIdx.x >= ctas) return;
+    unsigned arrivals = 0;  // epochs this CTA has finished
+    if (tid == 0) {  // this CTA's windows (host: at most LOOP_WINDOWS)
+        s_stop = 0;
+        s_chead = -1;
+        s_carry = make_float4(0.f, 0.f, 0.f, 0.f);
+        int k = 0;
+        for (int32_t W = int32_t(blockIdx.x); W < n_win && k < LOOP_WINDOWS; W += int32_t(ctas)) {
+            LoopWindow d;
+            d.rA = A.win_row[W];
+            d.rB = A.win_row[W + 1];
+            if (d.rA >= d.rB) continue;  // a long row started in an earlier window covers this one
+            window_instance<BATCHED>(A, W, d.R, d.h_lo, d.h_hi);
+            if (d.rA < d.h_lo || d.rB > d.h_hi) {
+                report_status(A.status, DRGB_ERR_INVALID);
+                continue;
+            }
+            d.es = A.row_ptr[d.rA - A.row_begin];
+            d.ee = A.row_ptr[d.rB - A.row_begin];
+            s_win[k++] = d;
+        }
+        s_nw = k;
+    }
+    __syncthreads();
+    const int n_mine = s_nw;
+    // Schedule words of one round of a window, in this thread's registers.
+    // They are loaded a window ahead, when the previous ones have been
+    // compacted; tails and heads are read for the active entries alone.
+    uint32_t qv[LOOP_CHUNKS];
+    auto load_round = [&](int32_t c0, int32_t ee) {
+        const int32_t e0 = c0 + w * (32 * LOOP_CHUNKS) + lane;
+#pragma unroll
+        for (int b = 0; b < LOOP_CHUNKS; ++b) qv[b] = e0 + 32 * b < ee ? A.q[e0 + 32 * b] : 0u;  // 0 never fires
+    };
+    if (n_mine > 0) load_round(s_win[0].es, s_win[0].ee);
+    // every CTA has finished the previous epoch (bounded; false: give up)
+    auto wait_epoch = [&]() -> bool {
+        if (tid == 0 && arrivals) {
+            const unsigned target = arrivals * ctas;
+            const unsigned long long t0 = loop_timer();
+            for (;;) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(P.arrived) : "memory");
+                if (v >= target) break;
+                if (loop_timer() - t0 > 2000000000ull || *static_cast<volatile int*>(P.stop)) {
+                    *static_cast<volatile int*>(P.stop) = 1;
+                    report_status(A.status, DRGB_ERR_TIMEOUT);
+                    s_stop = 1;
+                    break;
+                }
+            }
+        }
+        __syncthreads();
+        return s_stop == 0;
+    };
+    for (int t = P.t_begin; t < P.t_end; ++t) {
+        const int step = t - P.t_begin;
+        if (step % LOOP_LR == 0) {  // learning rates of the next epochs
+            __syncthreads();
+            for (int u = tid; u < LOOP_LR; u += LOOP_THREADS)
+                s_lr[u] = float(double(P.lr0) * (1.0 - double(t + u) / double(P.T)));
+            __syncthreads();
+        }
+        const EpochStep S{P.buf[step & 1], P.buf[(step & 1) ^ 1], s_lr[step % LOOP_LR], uint32_t(t)};
+        bool waited = false;
+        for (int k = 0; k < n_mine; ++k) {
+            const int32_t rA = s_win[k].rA, rB = s_win[k].rB, es = s_win[k].es, ee = s_win[k].ee;
+            const RowInst R = s_win[k].R;
+            const int64_t h_lo = s_win[k].h_lo, h_hi = s_win[k].h_hi;
+            int qn = 0;  // active entries waiting at the front of the list
+            for (int32_t c0 = es; c0 == es || c0 < ee; c0 += LOOP_ROUND) {
+                const int32_t e0 = c0 + w * (32 * LOOP_CHUNKS) + lane;
+                unsigned m[LOOP_CHUNKS];
+                int cnt = 0;
+#pragma unroll
+                for (int b = 0; b < LOOP_CHUNKS; ++b) {
+                    // floor((t+1) q / 2^24) > floor(t q / 2^24)  <=>  (t q mod 2^24) + q >= 2^24
+                    m[b] = __ballot_sync(FULL, qv[b] >= 0x1000000u - ((S.t * qv[b]) & 0xFFFFFFu));
+                    cnt += __popc(m[b]);
+                }
+                if (lane == 0) s_cnt[w] = cnt;
+                __syncthreads();
+                int pos = qn, total = 0;
+#pragma unroll
+                for (int u = 0; u < LOOP_WARPS; ++u) {
+                    const int v = s_cnt[u];
+                    pos += u < w ? v : 0;
+                    total += v;
+                }
+#pragma unroll
+                for (int b = 0; b < LOOP_CHUNKS; ++b) {
+                    if (m[b] >> lane & 1u) {
+                        const int p = pos + __popc(m[b] & lt_mask);
+                        s_e[p] = e0 + 32 * b;
+                    }
+                    pos += __popc(m[b]);
+                }
+                qn += total;
+                const bool last = c0 + LOOP_ROUND >= ee;
+                if (!last) {
+                    load_round(c0 + LOOP_ROUND, ee);
+                } else if (n_mine > 1 || c0 != es) {  // (a lone window of one round stays in registers)
+                    const int kn = k + 1 < n_mine ? k + 1 : 0;
+                    load_round(s_win[kn].es, s_win[kn].ee);
+                }
+                if (c0 == es && tid == 0) s_chead = -1;
+                __syncthreads();
+                const int ng = last ? (qn + 31) / 32 : qn / 32;
+                auto draw = [&](int g, EntryPlan<NEG>& pl) {
+                    const int p = 32 * g + lane;
+                    const bool v = p < qn;
+                    const int32_t e = v ? s_e[p] : es;
+                    draw_entry<NEG, BATCHED>(A, S, R, v, e, v ? A.col[e] : 0, v ? A.row_of[e] : -1, h_lo, h_hi, lane, pl);
+                };
+                EntryPlan<NEG> pl;
+                if (w < ng) draw(w, pl);
+                if (!waited) {  // the first read of Y
+                    if (!wait_epoch()) return;
+                    waited = true;
+                }
+                EntryInputs<NEG> in;
+                if (w < ng) gather_entry<NEG>(S, R, pl, in);
+                if (c0 == es) {
+                    // every row of the window first gets Y + lr * 0; rows with
+                    // active entries are rewritten with their force below
+                    for (int64_t r = rA + tid; r < rB; r += LOOP_THREADS) {
+                        const float2 y = load_y(S.Y_in + r);
+                        S.Y_out[r] = make_float2(fmaf(S.lr, 0.f, y.x), fmaf(S.lr, 0.f, y.y));
+                    }
+                    __syncthreads();
+                }
+                for (int g = w; g < ng; g += LOOP_WARPS) {
+                    if (g != w) {
+                        draw(g, pl);
+                        gather_entry<NEG>(S, R, pl, in);
+                    }
+                    const int gn = qn - 32 * g < 32 ? qn - 32 * g : 32;
+                    float fx = 0.f, fy = 0.f;
+                    if (in.ok) {
+                        const float2 f = entry_math<NEG, BATCHED>(A, S, R, in, two_ab, two_b);
+                        fx = f.x;
+                        fy = f.y;
+                    }
+                    const int32_t i = in.i;
+                    const int32_t i_prev = __shfl_up_sync(FULL, i, 1), i_next = __shfl_down_sync(FULL, i, 1);
+                    const unsigned starts = __ballot_sync(FULL, lane == 0 || i_prev != i);
+                    const int seg0 = 31 - __clz(starts & (FULL >> (31 - lane)));
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const float ox = __shfl_up_sync(FULL, fx, d), oy = __shfl_up_sync(FULL, fy, d);
+                        if (lane - d >= seg0) {
+                            fx = ox + fx;
+                            fy = oy + fy;
+                        }
+                    }
+                    const bool ends = lane == gn - 1 || (lane < gn - 1 && i_next != i);
+                    if (ends && lane < gn - 1 && seg0 > 0 && in.ok)  // inside the group: final
+                        S.Y_out[i] = make_float2(fmaf(S.lr, 0.f + fx, in.yi.x), fmaf(S.lr, 0.f + fy, in.yi.y));
+                    if (ends && seg0 == 0) {
+                        s_end[g].head0 = in.ok ? i : -1;
+                        s_end[g].sum0 = make_float2(fx, fy);
+                        s_end[g].y0 = in.yi;
+                        s_end[g].one = lane == gn - 1;
+                    }
+                    if (lane == gn - 1) {
+                        s_end[g].head1 = in.ok ? i : -1;
+                        s_end[g].sum1 = make_float2(fx, fy);
+                        s_end[g].y1 = in.yi;
+                    }
+                }
+                // entries of an incomplete group go to the front for the next round
+                const int left = qn - 32 * ng > 0 ? qn - 32 * ng : 0;
+                const int32_t le = !last && w == 0 && lane < left ? s_e[32 * ng + lane] : 0;
+                __syncthreads();
+                if (!last && w == 0 && lane < left) s_e[lane] = le;
+                qn = left;
+                if (w == 0) {
+                    auto put = [&](int32_t h, float2 f, float2 y) {
+                        if (h >= 0) S.Y_out[h] = make_float2(fmaf(S.lr, 0.f + f.x, y.x), fmaf(S.lr, 0.f + f.y, y.y));
+                    };
+                    // Lane g joins group g's first run to the run before it
+                    // (the previous group's last, or the carry of the previous
+                    // round).  A group that is one run passes its join on, so
+                    // with one of those before the last group (rare: a row with
+                    // more than 32 active entries) one lane walks the groups.
+                    static_assert(LOOP_QCAP / 32 <= 32, "a lane per group");
+                    GroupEnds E;
+                    E.head0 = E.head1 = -1;
+                    E.one = false;
+                    if (lane < ng) E = s_end[lane];
+                    int32_t chead = s_chead;
+                    float4 cv = s_carry;
+                    if (__any_sync(FULL, lane < ng - 1 && E.one)) {
+                        if (lane == 0) {
+                            for (int g = 0; g < ng; ++g) {
+                                E = s_end[g];
+                                float2 f = E.sum0;
+                                if (chead >= 0 && E.head0 == chead) {
+                                    f.x = cv.x + f.x;
+                                    f.y = cv.y + f.y;
+                                } else {
+                                    put(chead, make_float2(cv.x, cv.y), make_float2(cv.z, cv.w));
+                                }
+                                if (E.one) {
+                                    chead = E.head0;
+                                    cv = make_float4(f.x, f.y, E.y0.x, E.y0.y);
+                                } else {
+                                    put(E.head0, f, E.y0);
+                                    chead = E.head1;
+                                    cv = make_float4(E.sum1.x, E.sum1.y, E.y1.x, E.y1.y);
+                                }
+                            }
+                            if (last) put(chead, make_float2(cv.x, cv.y), make_float2(cv.z, cv.w));
+                            s_chead = chead;
+                            s_carry = cv;
+                        }
+                    } else if (ng > 0) {
+                        const int32_t ph = __shfl_up_sync(FULL, E.head1, 1);
+                        const float4 pv = make_float4(__shfl_up_sync(FULL, E.sum1.x, 1), __shfl_up_sync(FULL, E.sum1.y, 1),
+                                                      __shfl_up_sync(FULL, E.y1.x, 1), __shfl_up_sync(FULL, E.y1.y, 1));
+                        if (lane > 0) {
+                            chead = ph;
+                            cv = pv;
+                        }
+                        if (lane < ng) {
+                            float2 f = E.sum0;
+                            if (chead >= 0 && E.head0 == chead) {
+                                f.x = cv.x + f.x;
+                                f.y = cv.y + f.y;
+                            } else {
+                                put(chead, make_float2(cv.x, cv.y), make_float2(cv.z, cv.w));
+                            }
+                            if (E.one) {  // the last group
+                                E.head1 = E.head0;
+                                E.sum1 = f;
+                                E.y1 = E.y0;
+                            } else {
+                                put(E.head0, f, E.y0);
+                            }
+                            if (lane == ng - 1) {
+                                if (last) put(E.head1, E.sum1, E.y1);
+                                s_chead = E.head1;
+                                s_carry = make_float4(E.sum1.x, E.sum1.y, E.y1.x, E.y1.y);
+                            }
+                        }
+                    } else if (last && lane == 0) {
+                        put(chead, make_float2(cv.x, cv.y), make_float2(cv.z, cv.w));
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        if (!waited && !wait_epoch()) return;  // (a CTA whose windows were all skipped)
+        __syncthreads();
+        ++arrivals;
+        if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(P.arrived) : "memory");
+    }
+}
+
 bool epoch_warps_supported(int warps) { return warps == 4 || warps == 8; }
 
 int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool after_epoch) {
@@ -675,6 +1058,62 @@ static void fill_args(EpochArgs& A, const int32_t* rp, const int32_t* col, const
     A.neg_n = neg_n;
 }
 
+// Windows (by capacity) up to which an epoch loop runs as one cooperative launch
+// (epoch_loop_kernel): microseconds an epoch against the chained launches, 15
+// neighbours: 2,000 rows 3.2 / 9.2, 8,000 5.1 / 13.4, 12,000 6.3 / 15.0, 20,000
+// 11.3 / 15.9, 30,000 12.0 / 17.0, 45,000 16.7 / 18.8, 70,000 24.1 / 20.2.
+static constexpr int64_t LOOP_MAX_WINDOWS_PER_SM = 18;
+static constexpr int LOOP_MAX_EPOCHS = 1000000;  // the barrier counts epochs x CTAs in 32 bits
+
+static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float lr0, int t_begin, int t_end, int T,
+                          unsigned int* sync, cudaStream_t st) {
+    DRGB_CUDA(c, cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned int), st));
+    LoopArgs P;
+    P.buf[0] = Y;
+    P.buf[1] = Y_tmp;
+    P.t_begin = t_begin;
+    P.t_end = t_end;
+    P.T = T;
+    P.lr0 = lr0;
+    P.arrived = sync;
+    P.stop = reinterpret_cast<int*>(sync + 1);
+    philox_round_keys(A.k0, A.k1, A.rk);
+    const bool bat = A.count > 0, n5 = A.neg == 5;
+    auto pick = [&](auto nw) {
+        constexpr int NW = decltype(nw)::value;
+        return bat ? (n5 ? epoch_loop_kernel<true, 5, NW> : epoch_loop_kernel<true, -1, NW>)
+                   : (n5 ? epoch_loop_kernel<false, 5, NW> : epoch_loop_kernel<false, -1, NW>);
+    };
+    const int64_t per = A.win_cap * 5 / 6;  // (about a sixth of the capacity is pruned or merged away)
+    const int nw = per <= int64_t(c->num_sms) * loop_ctas_per_sm(8) ? 8 : 4;
+    auto kernel = nw == 8 ? pick(std::integral_constant<int, 8>{}) : pick(std::integral_constant<int, 4>{});
+    int per_sm = 0;
+    DRGB_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, nw * 32, 0));
+    if (per_sm > loop_ctas_per_sm(nw)) per_sm = loop_ctas_per_sm(nw);
+    // as for the force kernel: shared memory for the resident CTAs, L1 for the rest
+    cudaFuncAttributes fa;
+    DRGB_CUDA(c, cudaFuncGetAttributes(&fa, kernel));
+    const size_t need = size_t(per_sm) * (fa.sharedSizeBytes + 1024);
+    const int pct = int((need * 100 + c->smem_per_sm - 1) / (c->smem_per_sm ? c->smem_per_sm : 1));
+    DRGB_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct < 100 ? pct : 100));
+    const int64_t ctas = grid_for(A.win_cap, 1, c->num_sms * (per_sm > 0 ? per_sm : 1));
+    if (A.win_cap > ctas * LOOP_WINDOWS) return set_error(c, DRGB_ERR_CUDA, "epoch loop: too few CTAs fit the device");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(ctas));
+    cfg.blockDim = dim3(nw * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    DRGB_CUDA(c, cudaLaunchKernelEx(&cfg, kernel, static_cast<const EpochArgs&>(A), static_cast<const LoopArgs&>(P)));
+    DRGB_CHECK_LAUNCH(c);
+    if ((t_end - t_begin) & 1)
+        DRGB_CUDA(c, cudaMemcpyAsync(Y, Y_tmp, size_t(A.n) * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    return DRGB_OK;
+}
+
 // Epochs [t_begin, t_end) of a T-epoch schedule, ping-ponging between Y and
 // Y_tmp; the result is left in Y.  The launches are captured into a CUDA
 // graph (on a private stream) and the graph is launched on `st`.  Building an
@@ -690,6 +1129,12 @@ int run_epochs(Ctx* c, float2* Y, float2* Y_tmp, const int32_t* rp, const int32_
     EpochScratch es;
     int rc = epoch_prepare(c, rp, n, row_begin, nnz_cap, count, inst_off, scratch, &es, st);
     if (rc) return rc;
+    if (t_end - t_begin > 1 && t_end - t_begin <= LOOP_MAX_EPOCHS &&
+        es.win_cap <= LOOP_MAX_WINDOWS_PER_SM * c->num_sms) {
+        EpochArgs A;
+        fill_args(A, rp, col, q, n, a, b, neg, seed, c->d_status, es, count, inst_off, inst_seed, row_begin, neg_n);
+        return run_epoch_loop(c, Y, Y_tmp, A, lr0, t_begin, t_end, T, es.sync, st);
+    }
     cudaStream_t cap;
     DRGB_CUDA(c, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;

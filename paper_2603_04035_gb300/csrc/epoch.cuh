@@ -48,6 +48,7 @@ struct EpochScratch {
     int32_t* win_row = nullptr;
     int32_t* inst_eoff = nullptr;
     int32_t* win_base = nullptr;
+    unsigned int* sync = nullptr;  // barrier words of the one-launch epoch loop
     int64_t nnz_cap = 0;
     int64_t win_cap = 0;
 };
