@@ -79,6 +79,41 @@ __device__ __forceinline__ float hw_lg2(float x) {
     return y;
 }
 
+// a / b as a * (1 / b) for normal b (subnormal operands count as 0).
+__device__ __forceinline__ float hw_div(float a, float b) {
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+
+// Both components of a point in one packed operation.
+__device__ __forceinline__ uint64_t pack2(float2 v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t r) {
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
+    return v;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+// a - b: the product by -1 is exact, so one rounding
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(b)), "l"(pack2(make_float2(-1.f, -1.f))), "l"(pack2(a)));
+    return unpack2(r);
+}
+
 // d^b for d > 0 via the hardware base-2 logarithm and exponential.
 __device__ __forceinline__ float pow_pos(float d, float b) { return hw_ex2(b * hw_lg2(d)); }
 
@@ -201,22 +236,28 @@ __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep
                                              const EntryInputs<NEG>& in, float two_ab, float two_b) {
     constexpr int NP = EntryInputs<NEG>::NP;
     const float2 yi = in.yi;
-    float gx = 0.f, gy = 0.f;
+    float2 g = make_float2(0.f, 0.f);
+    // the clipped step c (dx, dy) added to the sum, both components at once
+    auto add_clipped = [&](float c, float2 df) {
+        const float2 v = mul2(make_float2(c, c), df);
+        g = add2(g, make_float2(clip4(v.x), clip4(v.y)));
+    };
     {
-        const float dx = yi.x - in.yj.x, dy = yi.y - in.yj.y;
-        const float d = fmaf(dx, dx, dy * dy);
-        const float pb = d > 0.f ? pow_pos(d, A.b) : 0.f;
-        const float c = d > 0.f ? __fdividef(-two_ab * pb, d * fmaf(A.a, pb, 1.0f)) : 0.f;
-        gx += clip4(c * dx);
-        gy += clip4(c * dy);
+        const float2 df = sub2(yi, in.yj);
+        const float d = fmaf(df.x, df.x, df.y * df.y);
+        // (below the smallest normal number d^b is 0, and so is the force)
+        const bool far = d >= 1.17549435e-38f;
+        const float pb = far ? pow_pos(d, A.b) : 0.f;
+        const float c = far ? hw_div(-two_ab * pb, d * fmaf(A.a, pb, 1.0f)) : 0.f;
+        add_clipped(c, df);
     }
     auto repel = [&](float2 y) {
-        const float rx = yi.x - y.x, ry = yi.y - y.y;
-        const float dm = fmaf(rx, rx, ry * ry);
-        const float pb = dm > 0.f ? pow_pos(dm, A.b) : 0.f;
-        const float c = __fdividef(two_b, (0.001f + dm) * fmaf(A.a, pb, 1.0f));
-        gx += clip4(c * rx);
-        gy += clip4(c * ry);
+        const float2 df = sub2(yi, y);
+        const float dm = fmaf(df.x, df.x, df.y * df.y);
+        // for b > 0 the hardware's log2 and exp2 give 0^b = 0 by themselves
+        const float pb = (NEG >= 0 || dm > 0.f) ? pow_pos(dm, A.b) : 0.f;
+        const float c = hw_div(two_b, (0.001f + dm) * fmaf(A.a, pb, 1.0f));
+        add_clipped(c, df);
     };
 #pragma unroll
     for (int w = 0; w < NP; ++w) repel(in.ym[w]);
@@ -238,23 +279,44 @@ __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep
             for (int w = 0; w < 4; ++w) repel(yg[w]);
         }
     }
-    return make_float2(gx, gy);
+    return g;
 }
 
 // ------------------------------------------------------------------ per-call preparation
 // Head row of every CSR entry of rows [row_begin, n).  Entries not covered by
-// any row keep -1; a row whose bounds leave [0, nnz_cap] is reported.
+// any row keep -1; a row whose bounds leave [0, nnz_cap] is reported.  A warp
+// takes 32 rows: where their bounds ascend, as in any well-formed CSR, it
+// writes their entries 32 at a time, each lane finding its entry's row among
+// the 32 by five shuffles (a thread per row, each writing its own run of
+// entries, took 115 us for a million rows; now 21); otherwise each lane writes
+// its own row's entries.
 __global__ void epoch_heads_kernel(const int32_t* __restrict__ rp, int64_t n_rows, int64_t row_begin,
                                    int64_t nnz_cap, int32_t* __restrict__ row_of, int* status) {
-    for (int64_t lr = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; lr < n_rows;
-         lr += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t beg = rp[lr], end = rp[lr + 1];
-        if (beg < 0 || end < beg || end > nnz_cap) {
-            report_status(status, DRGB_ERR_INVALID);
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    for (int64_t l0 = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 32; l0 < n_rows; l0 += warps * 32) {
+        const int64_t lr = l0 + lane;
+        const bool in = lr < n_rows;
+        const int32_t beg = in ? rp[lr] : INT32_MAX, end = in ? rp[lr + 1] : INT32_MAX;
+        const bool bad = in && (beg < 0 || end < beg || end > nnz_cap);
+        if (bad) report_status(status, DRGB_ERR_INVALID);
+        if (__any_sync(FULL, bad)) {
+            if (in && !bad)
+                for (int32_t e = beg; e < end; ++e) row_of[e] = int32_t(row_begin + lr);
             continue;
         }
-        const int32_t r = int32_t(row_begin + lr);
-        for (int32_t e = beg; e < end; ++e) row_of[e] = r;
+        const int rows = n_rows - l0 < 32 ? int(n_rows - l0) : 32;
+        const int32_t b = __shfl_sync(FULL, beg, 0), z = __shfl_sync(FULL, end, rows - 1);
+        for (int32_t e0 = b; e0 < z; e0 += 32) {
+            const int32_t e = e0 + lane;
+            int r = 0;  // the last row of the 32 that starts at or before e
+#pragma unroll
+            for (int st = 16; st > 0; st >>= 1) {
+                const int32_t v = __shfl_sync(FULL, beg, r + st);
+                if (v <= e) r += st;
+            }
+            if (e < z) row_of[e] = int32_t(row_begin + l0 + r);
+        }
     }
 }
 
@@ -333,7 +395,7 @@ int epoch_prepare(Ctx* c, const int32_t* rp, int64_t n, int64_t row_begin, int64
     DRGB_CUDA(c, cudaMemsetAsync(es->row_of, 0xFF, size_t(nnz_cap > 0 ? nnz_cap : 1) * 4, st));
     const int64_t n_rows = n - row_begin;
     if (n_rows > 0) {
-        epoch_heads_kernel<<<grid_for(n_rows, 256, c->num_sms * 8), 256, 0, st>>>(rp, n_rows, row_begin, nnz_cap,
+        epoch_heads_kernel<<<grid_for(n_rows, 256, c->num_sms * 16), 256, 0, st>>>(rp, n_rows, row_begin, nnz_cap,
                                                                                  es->row_of, c->d_status);
         DRGB_CHECK_LAUNCH(c);
     }
@@ -974,7 +1036,7 @@ int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool
     if (!A_in.row_of || !A_in.win_row) return set_error(c, DRGB_ERR_INVALID, "epoch: state not prepared");
     EpochArgs A = A_in;
     philox_round_keys(A.k0, A.k1, A.rk);
-    const bool bat = A.count > 0, n5 = A.neg == 5;
+    const bool bat = A.count > 0, n5 = A.neg == 5 && A.b > 0.f;
     const bool pipe = c->epoch_pipe != 0;
     const int per_sm = epoch_warps_per_sm(pipe) / warps;
     const int fgrid = grid_for(A.win_cap, warps, c->num_sms * per_sm);
@@ -1078,7 +1140,7 @@ static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float 
     P.arrived = sync;
     P.stop = reinterpret_cast<int*>(sync + 1);
     philox_round_keys(A.k0, A.k1, A.rk);
-    const bool bat = A.count > 0, n5 = A.neg == 5;
+    const bool bat = A.count > 0, n5 = A.neg == 5 && A.b > 0.f;
     auto pick = [&](auto nw) {
         constexpr int NW = decltype(nw)::value;
         return bat ? (n5 ? epoch_loop_kernel<true, 5, NW> : epoch_loop_kernel<true, -1, NW>)
