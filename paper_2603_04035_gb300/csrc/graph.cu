@@ -5,16 +5,19 @@
 // in which atomics resolved.
 //
 // Passes (n rows, k neighbours, m_j = in-degree of j):
-//   1 rows      rho, sigma (64 bisection steps), w_{j|i}; out-list sorted by column
-//   2 indegree  histogram of tails
-//   3 scan      in_ptr
-//   4 scatter   in_src[in_ptr[j] + slot] = p   (p = i*k + s with idx[p] = j)
-//   5 sort      each in-list by p (rank sort, warp per row)
-//   6 merge     union of out-list and in-list by column -> tmp (cap k + m_i per row), w_max
-//   7 count     entries kept (T q >= 2^24)
-//   8 scan      row_ptr
-//   9 fill      col, w, q
-// Passes 6, 7 and 9 take a warp per row.
+//   1 rows      rho, sigma (64 bisection steps), w_{j|i}; out-list sorted by
+//               column; histogram of tails, whose counts give each entry a slot
+//   2 scan      in_ptr
+//   3 scatter   in_src[in_ptr[j] + slot] = p   (p = i*k + s with idx[p] = j)
+//   4 sort      in-lists longer than a warp, by p
+//   5 merge     union of out-list and in-list (sorted by p in the warp's
+//               registers) by column -> tmp (cap k + m_i per row); entries kept
+//               (T q >= 2^24)
+//   6 scan      row_ptr
+//   7 fill      col, w, q
+// Passes 5 and 7 take a warp per row.  The largest weight of a graph is 1: a
+// row's nearest neighbour has w = 1, and the union with 1 is 1; so q is
+// round(2^24 w) without a pass for the maximum.
 #include <mutex>
 
 #include "common.cuh"
@@ -26,162 +29,212 @@ static constexpr uint32_t Q_ONE = 1u << 24;
 
 // ---------------------------------------------------------------- pass 1
 // Rows are the n query points; neighbour indices lie in [0, db_n) and, when
-// self_check is set (a graph of X on itself), must differ from the row.
-__global__ void fuzzy_rows_kernel(const int32_t* __restrict__ idx, const float* __restrict__ dist,
-                                  int64_t n, int k, float target, float* __restrict__ w_dir,
-                                  int32_t* __restrict__ out_col, float* __restrict__ out_w,
-                                  float* __restrict__ rho_out, float* __restrict__ sigma_out,
-                                  int* __restrict__ status, int64_t db_n, int self_check) {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        float dr[DRGB_MAX_K];
-        int32_t jr[DRGB_MAX_K];
-        float mean = 0.f;
-        bool bad = false;
-        for (int s = 0; s < k; ++s) {
-            dr[s] = dist[i * k + s];
-            jr[s] = idx[i * k + s];
-            mean += dr[s];
-            bad |= !(dr[s] >= 0.f && dr[s] < INFINITY) || jr[s] < 0 || jr[s] >= db_n || (self_check && jr[s] == i);
+// in_cnt is given (a graph of X on itself), must differ from the row.
+//
+// A thread per row, its k <= KM values in registers: the bisection is k
+// exponentials and divides a step, in order.  Rows come and go through shared
+// memory, so that global accesses are whole lines.  (With the values in
+// indexable arrays, i.e. local memory: 136 us for 200,000 rows, 41 us for
+// 2,000.)
+static constexpr int FR_THREADS = 128;
+
+template <int KM>
+__global__ void __launch_bounds__(FR_THREADS)
+fuzzy_rows_kernel(const int32_t* __restrict__ idx, const float* __restrict__ dist, int64_t n, int k, float target,
+                  float* __restrict__ w_dir, int32_t* __restrict__ out_col, float* __restrict__ out_w,
+                  float* __restrict__ rho_out, float* __restrict__ sigma_out, int* __restrict__ status, int64_t db_n,
+                  int32_t* __restrict__ in_cnt, int32_t* __restrict__ slot) {
+    extern __shared__ int32_t s_rows[];  // four arrays of FR_THREADS rows of `pitch` words
+    const int pitch = k | 1;             // odd: the threads' rows start in distinct banks
+    const int words = FR_THREADS * pitch;
+    float* s_d = reinterpret_cast<float*>(s_rows);           // distances, then the weights in list order
+    int32_t* s_j = s_rows + words;                           // neighbours, then the sorted columns
+    float* s_w = reinterpret_cast<float*>(s_rows + 2 * words);  // their weights
+    int32_t* s_s = s_rows + 3 * words;                       // slots
+    const int tid = threadIdx.x;
+    for (int64_t i0 = int64_t(blockIdx.x) * FR_THREADS; i0 < n; i0 += int64_t(gridDim.x) * FR_THREADS) {
+        const int rows = n - i0 < FR_THREADS ? int(n - i0) : FR_THREADS;
+        for (int t = tid; t < rows * k; t += FR_THREADS) {
+            const int r = t / k, c = t - r * k;
+            s_d[r * pitch + c] = dist[i0 * k + t];
+            s_j[r * pitch + c] = idx[i0 * k + t];
         }
-        if (bad) report_status(status, DRGB_ERR_INVALID);
-        mean /= float(k);
-        const float rho = dr[0];
-        float lo = 0.f, hi = INFINITY, mid = 1.f;
-        for (int it = 0; it < 64; ++it) {
-            float psum = 0.f;
-            for (int s = 0; s < k; ++s) psum += expf(-fmaxf(0.f, dr[s] - rho) / mid);
-            if (psum > target) {
-                hi = mid;
-            } else {
-                lo = mid;
+        __syncthreads();
+        const int64_t i = i0 + tid;
+        if (tid < rows) {
+            float dr[KM];
+            int32_t jr[KM];
+            float mean = 0.f;
+            bool bad = false;
+#pragma unroll
+            for (int s = 0; s < KM; ++s) {
+                dr[s] = s < k ? s_d[tid * pitch + s] : 0.f;
+                jr[s] = s < k ? s_j[tid * pitch + s] : -1;
+                if (s < k) {
+                    mean += dr[s];
+                    bad |= !(dr[s] >= 0.f && dr[s] < INFINITY) || jr[s] < 0 || jr[s] >= db_n || (in_cnt && jr[s] == i);
+                }
             }
-            const float nxt = (hi == INFINITY) ? mid * 2.f : 0.5f * (lo + hi);
-            // a step that leaves mid unchanged repeats itself (same test, same
-            // bound): every later step would too, so the 64-step result is mid
-            if (nxt == mid) break;
-            mid = nxt;
-        }
-        const float sigma = fmaxf(mid, 1e-3f * mean);
-        if (rho_out) rho_out[i] = rho;
-        if (sigma_out) sigma_out[i] = sigma;
-        float wr[DRGB_MAX_K];
-        for (int s = 0; s < k; ++s) {
-            const float ex = dr[s] - rho;
-            wr[s] = ex > 0.f ? expf(-ex / sigma) : 1.f;
-            w_dir[i * k + s] = wr[s];
-        }
-        // out-list sorted by column (insertion sort; k <= DRGB_MAX_K)
-        for (int s = 1; s < k; ++s) {
-            int32_t jj = jr[s];
-            float ww = wr[s];
-            int t = s - 1;
-            while (t >= 0 && jr[t] > jj) {
-                jr[t + 1] = jr[t];
-                wr[t + 1] = wr[t];
-                --t;
+            if (bad) report_status(status, DRGB_ERR_INVALID);
+            mean /= float(k);
+            const float rho = dr[0];
+            // slots in the tails' in-lists (all requests in flight during the bisection)
+            int32_t sl[KM];
+            if (in_cnt) {
+#pragma unroll
+                for (int s = 0; s < KM; ++s)
+                    sl[s] = s < k && jr[s] >= 0 && jr[s] < db_n && jr[s] != i ? atomicAdd(&in_cnt[jr[s]], 1) : -1;
             }
-            jr[t + 1] = jj;
-            wr[t + 1] = ww;
+            float nx[KM];  // -max(0, d - rho)
+#pragma unroll
+            for (int s = 0; s < KM; ++s) nx[s] = -fmaxf(0.f, dr[s] - rho);
+            float lo = 0.f, hi = INFINITY, mid = 1.f;
+            for (int it = 0; it < 64; ++it) {
+                float psum = 0.f;
+#pragma unroll
+                for (int s = 0; s < KM; ++s)
+                    if (s < k) psum += expf(nx[s] / mid);
+                if (psum > target) {
+                    hi = mid;
+                } else {
+                    lo = mid;
+                }
+                const float nxt = (hi == INFINITY) ? mid * 2.f : 0.5f * (lo + hi);
+                // a step that leaves mid unchanged repeats itself (same test, same
+                // bound): every later step would too, so the 64-step result is mid
+                if (nxt == mid) break;
+                mid = nxt;
+            }
+            const float sigma = fmaxf(mid, 1e-3f * mean);
+            if (rho_out) rho_out[i] = rho;
+            if (sigma_out) sigma_out[i] = sigma;
+            bool dup = false;
+#pragma unroll
+            for (int s = 0; s < KM; ++s) {
+                if (s < k) {
+                    const float ex = dr[s] - rho;
+                    const float w = ex > 0.f ? expf(-ex / sigma) : 1.f;
+                    int rank = 0;  // place in the list sorted by column
+#pragma unroll
+                    for (int t = 0; t < KM; ++t) {
+                        if (t < k && t != s) {
+                            rank += jr[t] < jr[s] || (t < s && jr[t] == jr[s]);
+                            dup |= jr[t] == jr[s];
+                        }
+                    }
+                    s_d[tid * pitch + s] = w;
+                    s_j[tid * pitch + rank] = jr[s];
+                    s_w[tid * pitch + rank] = w;
+                    if (in_cnt) s_s[tid * pitch + s] = sl[s];
+                }
+            }
+            if (dup) report_status(status, DRGB_ERR_INVALID);  // a neighbour listed twice
         }
-        bool dup = false;
-        for (int s = 0; s < k; ++s) {
-            out_col[i * k + s] = jr[s];
-            out_w[i * k + s] = wr[s];
-            dup |= s > 0 && jr[s] == jr[s - 1];
+        __syncthreads();
+        for (int t = tid; t < rows * k; t += FR_THREADS) {
+            const int r = t / k, c = t - r * k;
+            w_dir[i0 * k + t] = s_d[r * pitch + c];
+            out_col[i0 * k + t] = s_j[r * pitch + c];
+            out_w[i0 * k + t] = s_w[r * pitch + c];
+            if (in_cnt) slot[i0 * k + t] = s_s[r * pitch + c];
         }
-        if (dup) report_status(status, DRGB_ERR_INVALID);  // a neighbour listed twice
+        __syncthreads();
     }
 }
 
-// ---------------------------------------------------------------- passes 2, 4
-__global__ void indegree_kernel(const int32_t* __restrict__ idx, int64_t n, int k,
-                                int32_t* __restrict__ in_cnt) {
-    const int64_t nk = n * k;
-    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < nk;
-         p += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t j = idx[p];
-        if (j >= 0 && j < n && j != p / k) atomicAdd(&in_cnt[j], 1);
-    }
+static int launch_fuzzy_rows(Ctx* c, const int32_t* idx, const float* dist, int64_t n, int k, int64_t db_n,
+                             float* w_dir, int32_t* out_col, float* out_w, float* rho, float* sigma, int32_t* in_cnt,
+                             int32_t* slot, cudaStream_t st) {
+    const float target = float(std::log2(double(k)));
+    const size_t smem = size_t(4) * FR_THREADS * (k | 1) * 4;
+    auto kernel = k <= 8 ? fuzzy_rows_kernel<8> : (k <= 16 ? fuzzy_rows_kernel<16> : fuzzy_rows_kernel<32>);
+    DRGB_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    kernel<<<grid_for(n, FR_THREADS, c->num_sms * 16), FR_THREADS, smem, st>>>(
+        idx, dist, n, k, target, w_dir, out_col, out_w, rho, sigma, c->d_status, db_n, in_cnt, slot);
+    DRGB_CHECK_LAUNCH(c);
+    return DRGB_OK;
 }
 
-__global__ void in_scatter_kernel(const int32_t* __restrict__ idx, int64_t n, int k,
-                                  const int32_t* __restrict__ in_ptr, int32_t* __restrict__ in_fill,
-                                  int32_t* __restrict__ in_src) {
-    const int64_t nk = n * k;
-    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < nk;
-         p += int64_t(gridDim.x) * blockDim.x) {
-        const int32_t j = idx[p];
-        if (j >= 0 && j < n && j != p / k) {
-            const int32_t slot = atomicAdd(&in_fill[j], 1);
-            in_src[in_ptr[j] + slot] = int32_t(p);
-        }
-    }
-}
-
-// ---------------------------------------------------------------- pass 5
-// Warp per row, ascending order of the row's (distinct) p values whatever
-// order the scatter produced.  A row of at most 32 elements (the common case:
-// the mean in-degree is k) is held one element per lane and every element
-// goes to its rank, counted through shuffles; rows of up to IS_WARP_MAX
-// elements are ranked by reading the row back for every element.  Longer
-// rows (hubs: at 70K the in-degree reaches 620) of up to IS_BIG_MAX elements
-// are listed in big_rows for in_sort_big_kernel; beyond that the warp ranks
-// them itself.
+// ---------------------------------------------------------------- pass 3
+// In-lists in the order of their slots (any order).  Lists longer than a warp
+// are noted for pass 4: those a warp ranks from the front of long_rows, those
+// a CTA sorts from its back (long_cnt counts both).
 static constexpr int IS_WARP_MAX = 128;
 static constexpr int IS_BIG_MAX = 8192;
-static constexpr int IS_BIG_THREADS = 256;
+static constexpr int IS_THREADS = 256;
 
-__global__ void in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ src,
-                               int32_t* __restrict__ dst, int64_t n, int32_t* __restrict__ big_rows,
-                               unsigned int* __restrict__ big_cnt) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t j = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n; j += warps) {
-        const int32_t b = in_ptr[j], m = in_ptr[j + 1] - b;
-        if (m <= 32) {
-            const int32_t x = lane < m ? src[b + lane] : INT32_MAX;
-            int32_t rank = 0;
-#pragma unroll
-            for (int t = 0; t < 32; ++t) {
-                const int32_t y = __shfl_sync(0xffffffffu, x, t);
-                rank += (t < m && y < x) ? 1 : 0;
-            }
-            if (lane < m) dst[b + rank] = x;
-            continue;
-        }
-        if (m > IS_WARP_MAX && m <= IS_BIG_MAX) {
-            if (lane == 0) big_rows[atomicAdd(big_cnt, 1u)] = int32_t(j);
-            continue;
-        }
-        for (int32_t a = lane; a < m; a += 32) {
-            const int32_t x = src[b + a];
-            int32_t rank = 0;
-            for (int32_t t = 0; t < m; ++t) rank += src[b + t] < x;
-            dst[b + rank] = x;
+__global__ void in_scatter_kernel(const int32_t* __restrict__ idx, int64_t n, int k,
+                                  const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ slot,
+                                  int32_t* __restrict__ in_src, int32_t* __restrict__ long_rows,
+                                  unsigned int* __restrict__ long_cnt) {
+    const int64_t nk = n * k;
+    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < nk;
+         p += int64_t(gridDim.x) * blockDim.x) {
+        const int32_t s = slot[p];
+        if (s >= 0) in_src[in_ptr[idx[p]] + s] = int32_t(p);
+        if (p < n) {
+            const int32_t m = in_ptr[p + 1] - in_ptr[p];
+            if (m > IS_WARP_MAX && m <= IS_BIG_MAX) long_rows[n - 1 - atomicAdd(&long_cnt[1], 1u)] = int32_t(p);
+            else if (m > 32) long_rows[atomicAdd(&long_cnt[0], 1u)] = int32_t(p);
         }
     }
 }
 
-// CTA per listed row: the row, padded with INT32_MAX to a power of two, is
-// sorted ascending by a bitonic network in shared memory.
-__global__ void __launch_bounds__(IS_BIG_THREADS)
-in_sort_big_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ src,
-                   int32_t* __restrict__ dst, const int32_t* __restrict__ big_rows,
-                   const unsigned int* __restrict__ big_cnt) {
+// ---------------------------------------------------------------- pass 4
+// Ascending order of the (distinct) p values of the in-lists longer than 32.
+// Up to IS_WARP_MAX: a warp ranks its elements against the whole list.  Longer
+// ones (hubs: at 70K the in-degree reaches 620), padded with INT32_MAX to a
+// power of two, are sorted by a CTA's bitonic network in shared memory; beyond
+// IS_BIG_MAX a warp ranks them from global memory.
+__global__ void __launch_bounds__(IS_THREADS)
+in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ src, int32_t* __restrict__ dst,
+               int64_t n, const int32_t* __restrict__ long_rows, const unsigned int* __restrict__ long_cnt) {
     extern __shared__ int32_t s_row[];  // [IS_BIG_MAX]
-    const unsigned cnt = *big_cnt;
-    for (unsigned r = blockIdx.x; r < cnt; r += gridDim.x) {
-        const int64_t j = big_rows[r];
-        const int32_t b = in_ptr[j], m = in_ptr[j + 1] - b;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned warps = gridDim.x * (IS_THREADS / 32), few = long_cnt[0], many = long_cnt[1];
+    for (unsigned r = blockIdx.x * (IS_THREADS / 32) + warp; r < few; r += warps) {
+        const int32_t j = long_rows[r], b = in_ptr[j], m = in_ptr[j + 1] - b;
+        if (m <= IS_WARP_MAX) {
+            int32_t* list = s_row + warp * IS_WARP_MAX;
+            int32_t x[IS_WARP_MAX / 32];
+            int32_t rank[IS_WARP_MAX / 32];
+#pragma unroll
+            for (int u = 0; u < IS_WARP_MAX / 32; ++u) {
+                const int a = lane + 32 * u;
+                x[u] = a < m ? src[b + a] : INT32_MAX;
+                list[a] = x[u];
+                rank[u] = 0;
+            }
+            __syncwarp();
+#pragma unroll 4
+            for (int t = 0; t < m; ++t) {
+                const int32_t y = list[t];
+#pragma unroll
+                for (int u = 0; u < IS_WARP_MAX / 32; ++u) rank[u] += y < x[u];
+            }
+#pragma unroll
+            for (int u = 0; u < IS_WARP_MAX / 32; ++u)
+                if (lane + 32 * u < m) dst[b + rank[u]] = x[u];
+            __syncwarp();
+        } else {
+            for (int32_t a = lane; a < m; a += 32) {
+                const int32_t x = src[b + a];
+                int32_t rank = 0;
+                for (int32_t t = 0; t < m; ++t) rank += src[b + t] < x;
+                dst[b + rank] = x;
+            }
+        }
+    }
+    for (unsigned r = blockIdx.x; r < many; r += gridDim.x) {
+        const int32_t j = long_rows[n - 1 - r], b = in_ptr[j], m = in_ptr[j + 1] - b;
         int P = 2 * IS_WARP_MAX;
         while (P < m) P <<= 1;
-        __syncthreads();  // the previous row's read-back is done
-        for (int a = threadIdx.x; a < P; a += IS_BIG_THREADS) s_row[a] = a < m ? src[b + a] : INT32_MAX;
+        __syncthreads();  // the previous lists are done with
+        for (int a = threadIdx.x; a < P; a += IS_THREADS) s_row[a] = a < m ? src[b + a] : INT32_MAX;
         __syncthreads();
         for (int kk = 2; kk <= P; kk <<= 1) {
             for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-                for (int a = threadIdx.x; a < P; a += IS_BIG_THREADS) {
+                for (int a = threadIdx.x; a < P; a += IS_THREADS) {
                     const int l = a ^ jj;
                     if (l > a) {
                         const int32_t x = s_row[a], y = s_row[l];
@@ -194,16 +247,32 @@ in_sort_big_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict
                 __syncthreads();
             }
         }
-        for (int a = threadIdx.x; a < m; a += IS_BIG_THREADS) dst[b + a] = s_row[a];
+        for (int a = threadIdx.x; a < m; a += IS_THREADS) dst[b + a] = s_row[a];
     }
 }
 
-// ---------------------------------------------------------------- pass 6
+// ---------------------------------------------------------------- pass 5
 __device__ __forceinline__ float fuzzy_union(float a, float b) {
     // a + b - ab, written symmetrically in (a, b) so that w_ij == w_ji exactly
     // and exactly 1 whenever either side is 1.
     const float hi = fmaxf(a, b), lo = fminf(a, b);
     return fmaf(lo, 1.0f - hi, hi);
+}
+
+__device__ __forceinline__ uint32_t schedule_word(float w) { return __float2uint_rn(float(Q_ONE) * w); }
+__device__ __forceinline__ bool word_fires(uint32_t q, int T) { return uint64_t(T) * q >= Q_ONE; }
+
+// First lane of a sorted list (one element a lane, INT32_MAX past its end)
+// whose element is >= x: 0 .. 32.
+__device__ __forceinline__ int warp_lower_bound(int32_t list, int32_t x) {
+    int r = 0;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1) {
+        const int32_t y = __shfl_sync(0xffffffffu, list, r + st - 1);
+        if (y < x) r += st;
+    }
+    const int32_t y = __shfl_sync(0xffffffffu, list, r);
+    return r + (y < x);
 }
 
 // Warp per row.  Out-list entry a (lane a < k; sorted by column, entries
@@ -212,173 +281,180 @@ __device__ __forceinline__ float fuzzy_union(float a, float b) {
 // for a column x that place is #(valid out columns < x) + #(in columns < x)
 // - #(columns < x present in both), and a column present in both is written
 // once, by its out entry, with the fuzzy union of the two weights.  Columns
-// are distinct within each list.
-__global__ void merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_w,
-                             const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ in_sorted,
-                             const float* __restrict__ w_dir, int64_t n, int k,
-                             int32_t* __restrict__ tcol, float* __restrict__ tw,
-                             int32_t* __restrict__ tcnt, unsigned int* __restrict__ wmax_bits) {
+// are distinct within each list.  The counts are binary searches among the
+// lanes (a walk over the other list by shuffles took 150 us for 200,000 rows,
+// and a sort of every in-list before it 57).
+// The next row's bounds and out-list are loaded while this one is merged.
+__global__ void __launch_bounds__(256)
+merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_w, const int32_t* __restrict__ in_ptr,
+             const int32_t* __restrict__ in_src, const int32_t* __restrict__ in_sorted,
+             const float* __restrict__ w_dir, int64_t n, int k, int T, int32_t* __restrict__ tcol,
+             float* __restrict__ tw, int32_t* __restrict__ tcnt, int32_t* __restrict__ keep_cnt) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    float local_max = 0.f;
-    for (int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const int32_t ib = in_ptr[i], m = in_ptr[i + 1] - ib;
-        const int64_t base = i * k + ib;
-        int32_t ca = INT32_MAX;  // this lane's out column (INT32_MAX: none or invalid)
-        float wa = 0.f;
-        if (lane < k) {
-            const int32_t c0 = out_col[i * k + lane];
-            if (c0 >= 0 && c0 < n && c0 != i) {
-                ca = c0;
-                wa = out_w[i * k + lane];
-            }
+    int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    int32_t ib_n = 0, ie_n = 0, oc_n = INT32_MAX;
+    float ow_n = 0.f;
+    auto prefetch = [&](int64_t r) {
+        if (r < n) {
+            ib_n = in_ptr[r];
+            ie_n = in_ptr[r + 1];
+            oc_n = lane < k ? out_col[r * k + lane] : INT32_MAX;
+            ow_n = lane < k ? out_w[r * k + lane] : 0.f;
         }
-        // out entries: in columns below ca, and ca's in weight if present
-        int32_t in_less = 0;
-        bool matched = false;
-        float w_in = 0.f;
-        for (int32_t t0 = 0; t0 < m; t0 += 32) {
-            int32_t cb = INT32_MAX;
-            float wb = 0.f;
-            if (t0 + lane < m) {
-                const int32_t p = in_sorted[ib + t0 + lane];
-                cb = p / k;
-                wb = w_dir[p];
-            }
-            const int cnt = m - t0 < 32 ? m - t0 : 32;
-            for (int u = 0; u < cnt; ++u) {
-                const int32_t cu = __shfl_sync(0xffffffffu, cb, u);
-                const float wu = __shfl_sync(0xffffffffu, wb, u);
-                in_less += cu < ca;
-                if (cu == ca) {
-                    matched = true;
-                    w_in = wu;
+    };
+    prefetch(i);
+    for (; i < n; i += warps) {
+        const int32_t ib = ib_n, m = ie_n - ib, c0 = oc_n;
+        const float wa = ow_n;
+        const int64_t base = i * k + ib;
+        // the first 32 in entries, sorted
+        int32_t p = lane < m ? (m <= 32 ? in_src[ib + lane] : in_sorted[ib + lane]) : INT32_MAX;
+        prefetch(i + warps);
+        if (m <= 32) {
+#pragma unroll
+            for (int kk = 2; kk <= 32; kk <<= 1) {
+#pragma unroll
+                for (int st = kk >> 1; st > 0; st >>= 1) {
+                    const int32_t o = __shfl_xor_sync(0xffffffffu, p, st);
+                    const bool keep_min = ((lane & kk) == 0) == ((lane & st) == 0);
+                    p = keep_min ? min(p, o) : max(p, o);
                 }
             }
         }
-        const bool va = ca != INT32_MAX;
+        const bool va = lane < k && c0 >= 0 && c0 < n && c0 != i;
         const unsigned vmask = __ballot_sync(0xffffffffu, va);
-        const unsigned mmask = __ballot_sync(0xffffffffu, va && matched);
+        int32_t in_less = 0, kept = 0;
+        float w_in = 0.f;
+        bool matched = false;
+        // out entries: in columns below c0, and c0's in weight if present
+        for (int32_t t0 = 0; t0 < m; t0 += 32) {
+            if (t0) p = t0 + lane < m ? in_sorted[ib + t0 + lane] : INT32_MAX;
+            const int32_t cb = p == INT32_MAX ? INT32_MAX : p / k;
+            const float wb = p == INT32_MAX ? 0.f : w_dir[p];
+            const int at = warp_lower_bound(cb, c0);
+            in_less += at;
+            const int32_t cm = __shfl_sync(0xffffffffu, cb, at & 31);
+            const float wm = __shfl_sync(0xffffffffu, wb, at & 31);
+            if (at < 32 && cm == c0 && va) {
+                matched = true;
+                w_in = wm;
+            }
+            if (m <= 32) {  // the common case: the in entries are at hand
+                const unsigned mmask = __ballot_sync(0xffffffffu, matched);
+                const int ao = warp_lower_bound(c0, cb);
+                const int32_t co = __shfl_sync(0xffffffffu, c0, ao & 31);
+                const unsigned below = ao >= 32 ? 0xffffffffu : (1u << ao) - 1u;
+                const bool mine = lane < m && !(ao < 32 && co == cb && (vmask >> ao & 1u));
+                if (mine) {
+                    const int32_t pos = lane + __popc(vmask & below) - __popc(mmask & below);
+                    tcol[base + pos] = cb;
+                    tw[base + pos] = wb;
+                }
+                kept += __popc(__ballot_sync(0xffffffffu, mine && word_fires(schedule_word(wb), T)));
+            }
+        }
+        const unsigned mmask = __ballot_sync(0xffffffffu, matched);
+        float wv = 0.f;
         if (va) {
             const int32_t pos = __popc(vmask & lt) + in_less - __popc(mmask & lt);
-            const float wv = matched ? fuzzy_union(wa, w_in) : wa;
-            tcol[base + pos] = ca;
+            wv = matched ? fuzzy_union(wa, w_in) : wa;
+            tcol[base + pos] = c0;
             tw[base + pos] = wv;
-            local_max = fmaxf(local_max, wv);
         }
-        // in entries without an out partner
-        for (int32_t t0 = 0; t0 < m; t0 += 32) {
-            const int32_t t = t0 + lane;
-            int32_t cb = INT32_MAX;
-            float wb = 0.f;
-            if (t < m) {
-                const int32_t p = in_sorted[ib + t];
-                cb = p / k;
-                wb = w_dir[p];
-            }
-            int32_t out_less = 0, both_less = 0;
-            bool partner = false;
-            for (int a = 0; a < k; ++a) {
-                const int32_t c_a = __shfl_sync(0xffffffffu, ca, a);
-                const bool lt_a = c_a < cb;
-                out_less += lt_a;
-                both_less += lt_a && ((mmask >> a) & 1u);
-                partner |= c_a == cb && c_a != INT32_MAX;
-            }
-            if (t < m && !partner) {
-                const int32_t pos = t + out_less - both_less;
-                tcol[base + pos] = cb;
-                tw[base + pos] = wb;
-                local_max = fmaxf(local_max, wb);
+        kept += __popc(__ballot_sync(0xffffffffu, va && word_fires(schedule_word(wv), T)));
+        if (m > 32) {  // in entries without an out partner
+            for (int32_t t0 = 0; t0 < m; t0 += 32) {
+                const int32_t t = t0 + lane;
+                const int32_t q = t < m ? in_sorted[ib + t] : INT32_MAX;
+                const int32_t cb = q == INT32_MAX ? INT32_MAX : q / k;
+                const float wb = q == INT32_MAX ? 0.f : w_dir[q];
+                const int ao = warp_lower_bound(c0, cb);
+                const int32_t co = __shfl_sync(0xffffffffu, c0, ao & 31);
+                const unsigned below = ao >= 32 ? 0xffffffffu : (1u << ao) - 1u;
+                const bool mine = t < m && !(ao < 32 && co == cb && (vmask >> ao & 1u));
+                if (mine) {
+                    const int32_t pos = t + __popc(vmask & below) - __popc(mmask & below);
+                    tcol[base + pos] = cb;
+                    tw[base + pos] = wb;
+                }
+                kept += __popc(__ballot_sync(0xffffffffu, mine && word_fires(schedule_word(wb), T)));
             }
         }
-        if (lane == 0) tcnt[i] = __popc(vmask) + m - __popc(mmask);
-    }
-    // non-negative floats order like their bit patterns
-    for (int o = 16; o > 0; o >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
-    if (lane == 0) atomicMax(wmax_bits, __float_as_uint(local_max));
-}
-
-__device__ __forceinline__ uint32_t schedule_word(float w, float w_max) {
-    return __float2uint_rn(float(Q_ONE) * (w / w_max));
-}
-
-// ---------------------------------------------------------------- passes 7, 9
-// Warp per row; the kept entries keep their order.
-__global__ void prune_count_kernel(const int32_t* __restrict__ in_ptr, const float* __restrict__ tw,
-                                   const int32_t* __restrict__ tcnt, int64_t n, int k, int T,
-                                   const unsigned int* __restrict__ wmax_bits,
-                                   int32_t* __restrict__ keep_cnt) {
-    const float w_max = __uint_as_float(*wmax_bits);
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const int64_t base = i * k + in_ptr[i];
-        const int32_t cnt = tcnt[i];
-        int32_t c = 0;
-        for (int32_t t0 = 0; t0 < cnt; t0 += 32) {
-            const int32_t t = t0 + lane;
-            const bool keep = t < cnt && uint64_t(T) * schedule_word(tw[base + t], w_max) >= Q_ONE;
-            c += __popc(__ballot_sync(0xffffffffu, keep));
+        if (lane == 0) {
+            tcnt[i] = __popc(vmask) + m - __popc(mmask);
+            keep_cnt[i] = kept;
         }
-        if (lane == 0) keep_cnt[i] = c;
     }
 }
 
-__global__ void fill_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ tcol,
-                            const float* __restrict__ tw, const int32_t* __restrict__ tcnt,
-                            int64_t n, int k, int T, const unsigned int* __restrict__ wmax_bits,
-                            const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col,
-                            float* __restrict__ w, uint32_t* __restrict__ q) {
-    const float w_max = __uint_as_float(*wmax_bits);
+// ---------------------------------------------------------------- pass 7
+// Warp per row; the kept entries keep their order.  A warp loads the bounds
+// and first 32 entries of FILL_ROWS rows before it writes any.
+static constexpr int FILL_ROWS = 4;
+
+__global__ void __launch_bounds__(256)
+fill_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ tcol, const float* __restrict__ tw,
+            const int32_t* __restrict__ tcnt, int64_t n, int k, int T, const int32_t* __restrict__ row_ptr,
+            int32_t* __restrict__ col, float* __restrict__ w, uint32_t* __restrict__ q) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const int64_t base = i * k + in_ptr[i];
-        const int32_t cnt = tcnt[i];
-        int64_t o = row_ptr[i];
-        for (int32_t t0 = 0; t0 < cnt; t0 += 32) {
-            const int32_t t = t0 + lane;
-            float wt = 0.f;
-            uint32_t qt = 0;
-            bool keep = false;
-            if (t < cnt) {
-                wt = tw[base + t];
-                qt = schedule_word(wt, w_max);
-                keep = uint64_t(T) * qt >= Q_ONE;
+    for (int64_t i0 = (int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * FILL_ROWS; i0 < n;
+         i0 += warps * FILL_ROWS) {
+        int64_t base[FILL_ROWS];
+        int32_t cnt[FILL_ROWS], o[FILL_ROWS], cv[FILL_ROWS];
+        float wv[FILL_ROWS];
+#pragma unroll
+        for (int u = 0; u < FILL_ROWS; ++u) {
+            const int64_t i = i0 + u;
+            base[u] = i < n ? i * k + in_ptr[i] : 0;
+            cnt[u] = i < n ? tcnt[i] : 0;
+            o[u] = i < n ? row_ptr[i] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < FILL_ROWS; ++u) {
+            wv[u] = lane < cnt[u] ? tw[base[u] + lane] : 0.f;
+            cv[u] = lane < cnt[u] ? tcol[base[u] + lane] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < FILL_ROWS; ++u) {
+            for (int32_t t0 = 0; t0 < cnt[u]; t0 += 32) {
+                const int32_t t = t0 + lane;
+                if (t0) {
+                    wv[u] = t < cnt[u] ? tw[base[u] + t] : 0.f;
+                    cv[u] = t < cnt[u] ? tcol[base[u] + t] : 0;
+                }
+                const uint32_t qt = schedule_word(wv[u]);
+                const bool keep = t < cnt[u] && word_fires(qt, T);
+                const unsigned km = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int64_t d = o[u] + __popc(km & lt);
+                    col[d] = cv[u];
+                    w[d] = wv[u];
+                    q[d] = qt;
+                }
+                o[u] += __popc(km);
             }
-            const unsigned km = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int64_t d = o + __popc(km & lt);
-                col[d] = tcol[base + t];
-                w[d] = wt;
-                q[d] = qt;
-            }
-            o += __popc(km);
         }
     }
 }
 
 int launch_directed_weights(Ctx* c, const int32_t* idx, const float* dist, int64_t n, int k, int64_t db_n,
                             float* w_dir, int32_t* out_col, float* out_w, cudaStream_t st) {
-    const float target = float(std::log2(double(k)));
-    fuzzy_rows_kernel<<<grid_for(n, 128, c->num_sms * 16), 128, 0, st>>>(idx, dist, n, k, target, w_dir, out_col,
-                                                                        out_w, nullptr, nullptr, c->d_status, db_n, 0);
-    DRGB_CHECK_LAUNCH(c);
-    return DRGB_OK;
+    return launch_fuzzy_rows(c, idx, dist, n, k, db_n, w_dir, out_col, out_w, nullptr, nullptr, nullptr, nullptr, st);
 }
 
 size_t fuzzy_scratch_bytes(int64_t n, int k) {
     const size_t nk = size_t(n) * k;
     size_t b = 0;
     b += Carve::round(nk * 4) * 3;          // w_dir, out_col, out_w
-    b += Carve::round((n + 1) * 4) * 4;     // in_cnt, in_ptr, in_fill, keep_cnt
+    b += Carve::round((n + 1) * 4) * 4;     // in_cnt, in_ptr, long_rows, keep_cnt
     b += Carve::round(nk * 4) * 2;          // in_src, in_sorted
     b += Carve::round(2 * nk * 4) * 2;      // tcol, tw
     b += Carve::round(n * 4);               // tcnt
-    b += Carve::round(256);                 // w_max
+    b += Carve::round(256);                 // long_cnt
     b += Carve::round(scan_scratch_elems(n) * 4);
     return b + 4096;
 }
@@ -393,53 +469,33 @@ int build_fuzzy_graph(Ctx* c, const int32_t* idx, const float* dist, int64_t n, 
     float* out_w = cv.take<float>(nk);
     int32_t* in_cnt = cv.take<int32_t>(n + 1);
     int32_t* in_ptr = cv.take<int32_t>(n + 1);
-    int32_t* in_fill = cv.take<int32_t>(n + 1);
+    int32_t* long_rows = cv.take<int32_t>(n + 1);
     int32_t* keep_cnt = cv.take<int32_t>(n + 1);
     int32_t* in_src = cv.take<int32_t>(nk);
     int32_t* in_sorted = cv.take<int32_t>(nk);
     int32_t* tcol = cv.take<int32_t>(2 * nk);
     float* tw = cv.take<float>(2 * nk);
     int32_t* tcnt = cv.take<int32_t>(n);
-    unsigned int* wmax = cv.take<unsigned int>(64);
+    unsigned int* long_cnt = cv.take<unsigned int>(64);
     int32_t* scan_tmp = cv.take<int32_t>(scan_scratch_elems(n));
+    int32_t* slot = tcol;  // free until the merge
 
     const int TB = 256;
     const int gmax = c->num_sms * 16;
-    const float target = float(std::log2(double(k)));
-    fuzzy_rows_kernel<<<grid_for(n, 128, gmax), 128, 0, st>>>(idx, dist, n, k, target, w_dir, out_col,
-                                                             out_w, rho, sigma, c->d_status, n, 1);
-    DRGB_CHECK_LAUNCH(c);
     DRGB_CUDA(c, cudaMemsetAsync(in_cnt, 0, (n + 1) * 4, st));
-    DRGB_CUDA(c, cudaMemsetAsync(in_fill, 0, (n + 1) * 4, st));
-    DRGB_CUDA(c, cudaMemsetAsync(wmax, 0, 4, st));
-    indegree_kernel<<<grid_for(int64_t(nk), TB, gmax), TB, 0, st>>>(idx, n, k, in_cnt);
+    DRGB_CUDA(c, cudaMemsetAsync(long_cnt, 0, 8, st));
+    int rc = launch_fuzzy_rows(c, idx, dist, n, k, n, w_dir, out_col, out_w, rho, sigma, in_cnt, slot, st);
+    if (rc || (rc = exclusive_scan(c, in_cnt, in_ptr, n, scan_tmp, st))) return rc;
+    in_scatter_kernel<<<grid_for(int64_t(nk), TB, gmax), TB, 0, st>>>(idx, n, k, in_ptr, slot, in_src, long_rows, long_cnt);
     DRGB_CHECK_LAUNCH(c);
-    int rc = exclusive_scan(c, in_cnt, in_ptr, n, scan_tmp, st);
-    if (rc) return rc;
-    in_scatter_kernel<<<grid_for(int64_t(nk), TB, gmax), TB, 0, st>>>(idx, n, k, in_ptr, in_fill, in_src);
+    in_sort_kernel<<<c->num_sms * 4, IS_THREADS, size_t(IS_BIG_MAX) * 4, st>>>(in_ptr, in_src, in_sorted, n, long_rows,
+                                                                               long_cnt);
     DRGB_CHECK_LAUNCH(c);
-    {
-        // rows longer than a warp ranks well go to a CTA each; keep_cnt is
-        // free until the prune pass and holds their list
-        int32_t* big_rows = keep_cnt;
-        unsigned int* big_cnt = wmax + 32;
-        DRGB_CUDA(c, cudaMemsetAsync(big_cnt, 0, 4, st));
-        in_sort_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(in_ptr, in_src, in_sorted, n, big_rows, big_cnt);
-        DRGB_CHECK_LAUNCH(c);
-        const size_t big_smem = size_t(IS_BIG_MAX) * 4;
-        in_sort_big_kernel<<<c->num_sms * 2, IS_BIG_THREADS, big_smem, st>>>(in_ptr, in_src, in_sorted, big_rows,
-                                                                              big_cnt);
-    }
+    merge_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(out_col, out_w, in_ptr, in_src, in_sorted, w_dir, n, k, T,
+                                                           tcol, tw, tcnt, keep_cnt);
     DRGB_CHECK_LAUNCH(c);
-    merge_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(out_col, out_w, in_ptr, in_sorted, w_dir, n, k,
-                                                           tcol, tw, tcnt, wmax);
-    DRGB_CHECK_LAUNCH(c);
-    prune_count_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(in_ptr, tw, tcnt, n, k, T, wmax, keep_cnt);
-    DRGB_CHECK_LAUNCH(c);
-    rc = exclusive_scan(c, keep_cnt, row_ptr, n, scan_tmp, st);
-    if (rc) return rc;
-    fill_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(in_ptr, tcol, tw, tcnt, n, k, T, wmax, row_ptr,
-                                                          col, w, q);
+    if ((rc = exclusive_scan(c, keep_cnt, row_ptr, n, scan_tmp, st))) return rc;
+    fill_kernel<<<grid_for(n, FILL_ROWS * TB / 32, gmax), TB, 0, st>>>(in_ptr, tcol, tw, tcnt, n, k, T, row_ptr, col, w, q);
     DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
