@@ -38,6 +38,18 @@ static constexpr uint32_t Q_ONE = 1u << 24;
 // 2,000.)
 static constexpr int FR_THREADS = 128;
 
+// x / m, correctly rounded, from y = 1 / m correctly rounded (Markstein's
+// theorem, IBM J. Res. Dev. 34, 1990: a quotient within one ulp, corrected by
+// its exact remainder times y, is the correctly rounded one; two corrections,
+// since x y itself may be off by more).  Straight-line code for quotients of
+// one divisor: the general divide's branch keeps a row's k divides from
+// overlapping (159 us for 200,000 rows, 46 us for 2,000).
+__device__ __forceinline__ float quotient(float x, float m, float y) {
+    float q = __fmul_rn(x, y);
+    q = fmaf(fmaf(-q, m, x), y, q);
+    return fmaf(fmaf(-q, m, x), y, q);
+}
+
 template <int KM>
 __global__ void __launch_bounds__(FR_THREADS)
 fuzzy_rows_kernel(const int32_t* __restrict__ idx, const float* __restrict__ dist, int64_t n, int k, float target,
@@ -88,12 +100,24 @@ fuzzy_rows_kernel(const int32_t* __restrict__ idx, const float* __restrict__ dis
             float nx[KM];  // -max(0, d - rho)
 #pragma unroll
             for (int s = 0; s < KM; ++s) nx[s] = -fmaxf(0.f, dr[s] - rho);
+            // whether the quotients nx / mid (mid within 2^+-64) and their
+            // remainders are all normal numbers
+            bool tame = true;
+#pragma unroll
+            for (int s = 0; s < KM; ++s)
+                if (s < k) tame = tame && (nx[s] == 0.f || (nx[s] < -8.67361738e-19f && nx[s] > -1.15292150e18f));
             float lo = 0.f, hi = INFINITY, mid = 1.f;
             for (int it = 0; it < 64; ++it) {
                 float psum = 0.f;
+                if (tame) {
+                    const float y = __frcp_rn(mid);
 #pragma unroll
-                for (int s = 0; s < KM; ++s)
-                    if (s < k) psum += expf(nx[s] / mid);
+                    for (int s = 0; s < KM; ++s)
+                        if (s < k) psum += expf(quotient(nx[s], mid, y));
+                } else {
+#pragma unroll 1
+                    for (int s = 0; s < k; ++s) psum += expf(-fmaxf(0.f, s_d[tid * pitch + s] - rho) / mid);
+                }
                 if (psum > target) {
                     hi = mid;
                 } else {
