@@ -34,6 +34,18 @@ static constexpr int SC_QPITCH = 66;    // float pairs per dimension of the quer
 static constexpr int SC_WARPS = SC_THREADS / 32;
 static constexpr int SC_ROWS = SC_Q / SC_WARPS;  // rows a warp selects
 
+// The cell order a SCAN_CELLS scan works on (see launch_knn_cells).
+struct CellScan {
+    const int32_t* rows;       // listed rows (point indices)
+    const int32_t* perm;       // point at a position
+    int K;
+    const int32_t* cell_beg;   // [K + 1] positions
+    const int32_t* chunk_beg;  // [K + 1] chunks
+    const int32_t* cell_cnt;   // [K] listed rows that reach the cell
+    const int32_t* cell_rows;  // [K][number of listed rows] which
+};
+static constexpr int64_t CELL_CHUNK = 1024;  // positions per chunk of a cell (at least)
+
 struct ScanArgs {
     const float* X;          // n x d database
     int64_t n;
@@ -51,6 +63,8 @@ struct ScanArgs {
     int32_t* idx;
     float* dist;
     bool partial;
+    // cells: see launch_knn_cells
+    CellScan cells;
     // ranks: targets and their squared distances (n_rows x k), counts added to
     const int32_t* tgt;
     const float* td;
@@ -74,11 +88,17 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return r;
 }
 
-// RANK = false: the k nearest of every query row in the chunk.  RANK = true:
-// for every target s of row r, the number of points of the chunk that precede
-// it in the FP32 (distance, index) order.
-template <bool RANK>
+// NEAREST: the k nearest of every query row in the chunk.  RANKS: for every
+// target s of row r, the number of points of the chunk that precede it in the
+// FP32 (distance, index) order.  CELLS: the k nearest among chunk blockIdx.y of
+// a cell for the listed rows that reach the cell; X is in cell order, and a
+// point's index is cells.perm of its position (ascending within a cell, so the
+// order by position is the order by index).
+enum { SCAN_NEAREST = 0, SCAN_RANKS = 1, SCAN_CELLS = 2 };
+
+template <int MODE>
 __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
+    constexpr bool RANK = MODE == SCAN_RANKS, CELLS = MODE == SCAN_CELLS;
     extern __shared__ __align__(16) unsigned char sc_raw[];
     const int d = A.d, k = A.k, kl = k <= 16 ? 16 : 32;
     const bool q_all = d <= 2 * SC_DC;  // the queries stay in shared memory
@@ -91,14 +111,37 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
     const int64_t r0 = int64_t(blockIdx.x) * SC_Q;
-    const int64_t p_begin = int64_t(blockIdx.y) * A.chunk;
-    const int64_t p_end = p_begin + A.chunk < A.n ? p_begin + A.chunk : A.n;
+    int64_t p_begin = int64_t(blockIdx.y) * A.chunk;
+    int64_t p_end = p_begin + A.chunk < A.n ? p_begin + A.chunk : A.n;
+    int64_t n_rows = A.n_rows;
+    const int32_t* list = A.list;
+    if constexpr (CELLS) {
+        const CellScan& S = A.cells;
+        if (int(blockIdx.y) >= S.chunk_beg[S.K]) return;
+        int C = 0;  // the cell holding this chunk: the last C with chunk_beg[C] <= blockIdx.y
+        for (int lo = 0, hi = S.K - 1; lo <= hi;) {
+            const int mid = (lo + hi) >> 1;
+            if (S.chunk_beg[mid] <= int(blockIdx.y)) {
+                C = mid;
+                lo = mid + 1;
+            } else {
+                hi = mid - 1;
+            }
+        }
+        n_rows = S.cell_cnt[C];
+        if (r0 >= n_rows) return;
+        list = S.cell_rows + int64_t(C) * A.n_rows;
+        p_begin = S.cell_beg[C] + (int64_t(blockIdx.y) - S.chunk_beg[C]) * A.chunk;
+        p_end = S.cell_beg[C + 1] - p_begin < A.chunk ? S.cell_beg[C + 1] : p_begin + A.chunk;
+    }
+    // where query q of this CTA goes in the outputs, and its row of Q
     auto place_of = [&](int q) -> int64_t {
-        const int64_t r = r0 + q < A.n_rows ? r0 + q : A.n_rows - 1;
-        return A.list ? int64_t(A.list[r]) : r;
+        const int64_t r = r0 + q < n_rows ? r0 + q : n_rows - 1;
+        return list ? int64_t(list[r]) : r;
     };
     auto query_of = [&](int q) -> int64_t {
         const int64_t p = place_of(q);
+        if constexpr (CELLS) return A.cells.rows[p];
         return A.rows ? A.rows[p] : p;
     };
     // dimensions [c0, c0 + cc) of the queries, negated and doubled
@@ -115,7 +158,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     for (int t = tid; t < SC_Q * kl; t += SC_THREADS) {
         const int q = t / kl, s = t - q * kl;
         if (RANK) {
-            const bool in = s < k && r0 + q < A.n_rows;
+            const bool in = s < k && r0 + q < n_rows;
             s_ld[t] = in ? A.td[(r0 + q) * k + s] : -1.f;
             s_li[t] = in ? A.tgt[(r0 + q) * k + s] : -1;
         } else {
@@ -126,7 +169,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
             // distance 0 (the test is strict)
             float T = INFINITY;
             if (A.ub) {
-                const float u = A.ub[place_of(q) * k + k - 1];
+                const float u = A.ub[(CELLS ? query_of(q) : place_of(q)) * k + k - 1];
                 T = fmaf(u * u, 1.0f + 1e-6f, 1.17549435e-38f);
                 if (!(T < INFINITY)) T = INFINITY;
             }
@@ -218,7 +261,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                 const int q = warp * SC_ROWS + rr;
                 const float4 v4 = *reinterpret_cast<const float4*>(s_d + q * SC_PITCH + 4 * lane);
                 float v[4] = {v4.x, v4.y, v4.z, v4.w};
-                const int64_t self = s_qi[q] - p0;
+                const int64_t self = CELLS ? -1 : s_qi[q] - p0;
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (4 * lane + j >= left || 4 * lane + j == self) v[j] = __int_as_float(0x7fc00000);  // compares false
@@ -251,7 +294,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                         if (lane == s) mine = c;
                     }
                     // the count of target s of row r0 + q
-                    if (lane < k && mine && r0 + q < A.n_rows) atomicAdd(&A.cnt[(r0 + q) * k + lane], mine);
+                    if (lane < k && mine && r0 + q < n_rows) atomicAdd(&A.cnt[(r0 + q) * k + lane], mine);
                 } else {
                     const float thr = ld[k - 1];
                     const float m = fminf(fminf(v[0], v[1]), fminf(v[2], v[3]));  // ignores the NaN marks
@@ -265,7 +308,11 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                             const int src = __ffs(todo) - 1;
                             todo &= todo - 1;
                             const float cd = __shfl_sync(0xffffffffu, v[j], src);
-                            const int32_t ci = int32_t(p0) + 4 * src + j;
+                            int32_t ci = int32_t(p0) + 4 * src + j;
+                            if constexpr (CELLS) {
+                                ci = A.cells.perm[ci];
+                                if (ci == s_qi[q]) continue;
+                            }
                             const bool less = D < cd || (D == cd && I < ci);
                             const int pos = __popc(__ballot_sync(0xffffffffu, less));
                             if (pos >= k) continue;  // overtaken by this tile's other points
@@ -297,8 +344,9 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
         for (int t = tid; t < SC_Q * k; t += SC_THREADS) {
             const int q = t / k, s = t - q * k;
             const int64_t r = r0 + q;
-            if (r >= A.n_rows) continue;
-            const int64_t o = A.partial ? int64_t(blockIdx.y) * A.n_rows + r : place_of(q);
+            if (r >= n_rows) continue;
+            const int64_t o = CELLS ? int64_t(blockIdx.y) * A.n_rows + place_of(q)
+                                    : (A.partial ? int64_t(blockIdx.y) * A.n_rows + r : place_of(q));
             const float D = s_ld[q * kl + s];
             const int32_t I = s_li[q * kl + s];
             A.idx[o * k + s] = I == INT32_MAX ? -1 : I;
@@ -422,13 +470,13 @@ size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
     return C > 1 ? 2 * (size_t(n_rows) * C * k * 4 + 512) : 0;
 }
 
-template <bool RANK>
+template <int MODE>
 static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
     A.chunk = ((A.n + C - 1) / C + SC_P - 1) / SC_P * SC_P;
     const size_t smem = scan_smem(A.d, A.k);
-    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<RANK>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     const dim3 grid(unsigned((A.n_rows + SC_Q - 1) / SC_Q), unsigned((A.n + A.chunk - 1) / A.chunk));
-    scan_kernel<RANK><<<grid, SC_THREADS, smem, st>>>(A);
+    scan_kernel<MODE><<<grid, SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
@@ -443,17 +491,118 @@ static int scan_nearest(Ctx* c, ScanArgs& A, int32_t* idx_out, float* dist_out, 
         A.idx = idx_out;
         A.dist = dist_out;
         A.partial = false;
-        return scan_launch<false>(c, A, 1, st);
+        return scan_launch<SCAN_NEAREST>(c, A, 1, st);
     }
     Carve cv(part);
     A.idx = cv.take<int32_t>(size_t(A.n_rows) * C * A.k);
     A.dist = cv.take<float>(size_t(A.n_rows) * C * A.k);
     A.partial = true;
-    int rc = scan_launch<false>(c, A, C, st);
+    int rc = scan_launch<SCAN_NEAREST>(c, A, C, st);
     if (rc) return rc;
     const int lists = int((A.n + A.chunk - 1) / A.chunk);
     return launch_merge_partials(c, A.idx, A.dist, A.n_rows, lists, A.k, A.list, idx_out,
                                  dist_out, st, none);
+}
+
+// chunk_beg[C] = sum over cells c < C of ceil(|c| / CH) (one warp, K <= 128);
+// the cells' row counts start at 0.
+__global__ void cell_chunks_kernel(const int32_t* __restrict__ cell_beg, int K, int32_t CH,
+                                   int32_t* __restrict__ chunk_beg, int32_t* __restrict__ cell_cnt) {
+    int32_t carry = 0;
+    for (int c0 = 0; c0 < K; c0 += 32) {
+        const int c = c0 + threadIdx.x;
+        const int32_t v = c < K ? (cell_beg[c + 1] - cell_beg[c] + CH - 1) / CH : 0;
+        int32_t incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (int(threadIdx.x) >= o) incl += y;
+        }
+        if (c < K) {
+            chunk_beg[c] = carry + incl - v;
+            cell_cnt[c] = 0;
+        }
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (threadIdx.x == 0) chunk_beg[K] = carry;
+}
+
+// The listed rows that can have one of their k nearest in cell C, for every C
+// (in any order).  For a point p of C, |x_q - p| >= |x_q - c_C| - |p - c_C|;
+// the FP32 values D~ of |x_q - c_C| and r~_C >= max |p - c_C| carry a relative
+// error below 1e-5 each (sums of at most 61 squares), and a point that can
+// enter the row's k nearest has FP32 distance <= u, exact distance <= u (1 +
+// 1.1e-5).  So C is left out when D~ - r~_C - 1e-5 (D~ + r~_C) > u (1 + 2e-5).
+// One warp per row, a cell per lane.
+__global__ void cell_reach_kernel(const float* __restrict__ X, int d, int k, const int32_t* __restrict__ rows,
+                                  int64_t cnt, int K, const float* __restrict__ cell_c,
+                                  const float* __restrict__ cell_r, const float* __restrict__ dist_in,
+                                  int32_t* __restrict__ cell_cnt, int32_t* __restrict__ cell_rows) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    for (int64_t r = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; r < cnt; r += warps) {
+        const int64_t q = rows[r];
+        const float u = dist_in[q * k + k - 1];
+        for (int C = lane; C < K; C += 32) {
+            float sq = 0.f;
+#pragma unroll 8
+            for (int c = 0; c < d; ++c) {
+                const float df = X[q * d + c] - cell_c[int64_t(C) * d + c];
+                sq = fmaf(df, df, sq);
+            }
+            const float Dc = sqrtf(sq), rc = cell_r[C];
+            if (Dc - rc - 1e-5f * (Dc + rc) > u * (1.0f + 2e-5f)) continue;  // false for u = INFINITY
+            cell_rows[int64_t(C) * cnt + atomicAdd(&cell_cnt[C], 1)] = int32_t(r);
+        }
+    }
+}
+
+int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, int k, const int32_t* rows,
+                     int64_t cnt, int K, const int32_t* perm, const int32_t* cell_beg, const float* cell_c,
+                     const float* cell_r, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
+                     size_t part_bytes, bool* done) {
+    *done = false;
+    // chunks of at least CELL_CHUNK positions, as many as the partial lists'
+    // scratch holds (at most n / CH + K chunks in all)
+    const size_t fixed = 3 * Carve::round(size_t(K + 1) * 4) + Carve::round(size_t(K) * cnt * 4) + 4096;
+    const size_t per_list = size_t(cnt) * k * 8;
+    if (K <= 1 || fixed >= part_bytes) return DRGB_OK;
+    const int64_t max_lists = int64_t((part_bytes - fixed) / per_list) - K;
+    if (max_lists <= 0) return DRGB_OK;
+    int64_t CH = CELL_CHUNK;
+    if (CH * max_lists < n) CH = (n + max_lists - 1) / max_lists;
+    CH = (CH + SC_P - 1) / SC_P * SC_P;
+    const int64_t nchunk = (n + CH - 1) / CH + K;
+    if (nchunk > 65535) return DRGB_OK;
+    Carve pc(part);
+    int32_t* chunk_beg = pc.take<int32_t>(K + 1);
+    int32_t* cell_cnt = pc.take<int32_t>(K);
+    int32_t* cell_rows = pc.take<int32_t>(size_t(K) * cnt);
+    ScanArgs A = {};
+    A.idx = pc.take<int32_t>(size_t(cnt) * nchunk * k);
+    A.dist = pc.take<float>(size_t(cnt) * nchunk * k);
+    cell_chunks_kernel<<<1, 32, 0, st>>>(cell_beg, K, int32_t(CH), chunk_beg, cell_cnt);
+    DRGB_CHECK_LAUNCH(c);
+    DRGB_CUDA(c, cudaMemsetAsync(A.idx, 0xFF, size_t(cnt) * nchunk * k * 4, st));  // lists that no CTA writes are empty
+    cell_reach_kernel<<<grid_for(cnt, 4, c->num_sms * 16), 128, 0, st>>>(X, d, k, rows, cnt, K, cell_c, cell_r, dist_out,
+                                                                       cell_cnt, cell_rows);
+    DRGB_CHECK_LAUNCH(c);
+    A.X = Xp;
+    A.Q = X;
+    A.n = n;
+    A.d = d;
+    A.k = k;
+    A.n_rows = cnt;
+    A.chunk = CH;
+    A.ub = dist_out;
+    A.partial = true;
+    A.cells = CellScan{rows, perm, K, cell_beg, chunk_beg, cell_cnt, cell_rows};
+    const size_t smem = scan_smem(d, k);
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<SCAN_CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    scan_kernel<SCAN_CELLS><<<dim3(unsigned((cnt + SC_Q - 1) / SC_Q), unsigned(nchunk)), SC_THREADS, smem, st>>>(A);
+    DRGB_CHECK_LAUNCH(c);
+    *done = true;
+    return launch_merge_partials(c, A.idx, A.dist, cnt, int(nchunk), k, rows, idx_out, dist_out, st);
 }
 
 int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, const int32_t* rows32, int64_t cnt,
@@ -573,7 +722,7 @@ int launch_rank(Ctx* c, const float* X, int64_t n, int d, int k, const int64_t* 
     A.tgt = tgt;
     A.td = td;
     A.cnt = cnt;
-    int rc = scan_launch<true>(c, A, scan_chunks(c, n_rows, n, k, 0, false), st);
+    int rc = scan_launch<SCAN_RANKS>(c, A, scan_chunks(c, n_rows, n, k, 0, false), st);
     if (rc) return rc;
     rank_excess_kernel<<<grid_for(n_rows, 128, c->num_sms * 8), 128, 0, st>>>(cnt, tgt, n_rows, k, excess_out);
     DRGB_CHECK_LAUNCH(c);

@@ -66,6 +66,19 @@ static constexpr size_t TC_SMEM =
     1024 + TC_A_BYTES + TC_STAGES * TC_B_BYTES + 256 + TC_QUEUE_BYTES + TC_THR_BYTES + TC_SCHED_BYTES;
 
 // ------------------------------------------------------------------ A1: staging
+// Bound on |s - s~| for K = 64 columns (FP32 accumulation and norms): a K = 16
+// step adds 16 exact products and the accumulator, each aligned with an error
+// below an FP32 unit (2^-23) of the largest magnitude, which is at most n_j + 2
+// |x_i| |x_j| <= 2 (n_i + n_max): 34 * 2^-23 (n_i + n_max) a step; the norms'
+// sums and split below 2^-17 of that, and in FP16 the split's last part may lie
+// below the smallest normal number (4 units of the scaled operands).  (2^-14 (n_i +
+// n_max), taken before, left 914 rows of 70,000 projected images uncertified.)
+template <bool F16>
+__device__ __forceinline__ float tc_eps(float ni, float n_max, float S) {
+    constexpr float rel = 4.0f * 34.0f * 1.1920929e-7f + 7.6293945e-6f;
+    return rel * (ni + n_max) + (F16 ? 4.0f * (S * S) : 0.f);
+}
+
 // Column statistics of X (d <= 64) for the operand staging.  Block b sums,
 // and takes the minimum and maximum of, every column over its range of rows
 // (a warp per row, lanes on dimensions (lane, lane + 32)) into partial[b]; the
@@ -663,7 +676,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             if (g_row >= 0) {
                 const float r_max = __uint_as_float(P.maxbits[1]), n_max = __uint_as_float(P.maxbits[0]);
                 const float ni = P.norm[g_row];
-                ua = ni + 6.103515625e-05f * (ni + n_max);
+                ua = ni + tc_eps<F16>(ni, n_max, operand_scale<F16>(P.maxbits));
                 uc = P.resid[g_row] + r_max;
             }
             s_ua[row] = ua;
@@ -868,205 +881,13 @@ tc_rerank_kernel(const float* __restrict__ Xp, const int32_t* __restrict__ perm,
             // never compared lie in skipped cells, beyond lbstop)
             const float s_thr = cand_s[p * TC_KP + TC_KP - 1] * (S * S);
             const float ni = norm[i];
-            const float eps = 6.103515625e-05f * (ni + n_max);  // 2^-14 (n_i + n_max)
+            const float eps = tc_eps<F16>(ni, n_max, S);
             const float lb2 = ni + s_thr - eps;
             const float lb = fminf(sqrtf(fmaxf(lb2, 0.f)) - resid[i] - r_max, lbstop[p]);
             const bool ok = n_valid >= k && lb > sqrtf(dk2) * (1.0f + 3.8e-6f);
             if (!ok) fail_rows[atomicAdd(fail_count, 1)] = int32_t(i);
         }
         __syncwarp();
-    }
-}
-
-// Exact re-scan of the uncertified rows over the cells they can reach.  The
-// cells are cut into chunks of at most CH positions (chunk_beg[C] = the first
-// chunk of cell C; chunks of one cell are consecutive), so that a large cell
-// does not become one long scan.  CTA (chunk y, listed row r) scans chunk y
-// of its cell C for row q = rows[r], unless the cell's sphere lies beyond the
-// row's re-ranked k-th distance u.
-// For a point p of C, |x_q - p| >= |x_q - c_C| - |p - c_C|; the FP32 values
-// D~ of |x_q - c_C| and r~_C >= max |p - c_C| carry a relative error below
-// 1e-5 each (sums of at most 61 squares), and a point that can enter the
-// row's k nearest has FP32 distance <= u, exact distance <= u (1 + 1.1e-5).
-// So C is skipped when D~ - r~_C - 1e-5 (D~ + r~_C) > u (1 + 2e-5).
-// The scan itself is the FP32 scan's arithmetic: squared distance
-// sum_c (x_qc - p_c)^2 over the dimensions in order, kept when below the
-// admission bound of the k-th distance, per thread sorted by distance, then
-// merged by (distance, index) within each warp and over the CTA's warps into
-// partial list (y, r), which launch_merge_partials combines over the chunks.
-// Within a cell, positions follow the point index (the cell sort is stable),
-// so every per-thread list is ordered by (distance, index).  The cell's
-// points are staged 128 at a time with asynchronous copies into two
-// alternating buffers, the next tile in flight while the current one is used.
-static constexpr int RS_THREADS = 128;
-static constexpr int RS_PITCH = 65;  // floats per staged point (d <= 61), odd: conflict-free
-static constexpr size_t RS_SMEM = size_t(2) * RS_THREADS * RS_PITCH * 4;
-static constexpr int64_t RS_CHUNK_MIN = 2048;  // positions per chunk of a cell (at least)
-
-// chunk_beg[C] = sum over cells c < C of ceil(|c| / CH) (one CTA, K <= 128).
-__global__ void tc_chunks_kernel(const int32_t* __restrict__ cell_beg, int K, int32_t CH,
-                                 int32_t* __restrict__ chunk_beg) {
-    if (threadIdx.x != 0) return;
-    int32_t acc = 0;
-    for (int c = 0; c < K; ++c) {
-        chunk_beg[c] = acc;
-        acc += (cell_beg[c + 1] - cell_beg[c] + CH - 1) / CH;
-    }
-    chunk_beg[K] = acc;
-}
-
-template <int KL>
-__global__ void __launch_bounds__(RS_THREADS)
-tc_rescan_kernel(const float* __restrict__ X, const float* __restrict__ Xp, const int32_t* __restrict__ perm,
-                 int d, int k, const int32_t* __restrict__ rows, int cnt, int K, int32_t CH,
-                 const int32_t* __restrict__ cell_beg, const int32_t* __restrict__ chunk_beg,
-                 const float* __restrict__ cell_c, const float* __restrict__ cell_r,
-                 const float* __restrict__ dist_in, int32_t* __restrict__ pidx, float* __restrict__ pd2) {
-    extern __shared__ __align__(16) float s_pts[];   // [2][RS_THREADS][RS_PITCH]
-    __shared__ float s_x[64];
-    __shared__ float s_part[RS_THREADS / 32];
-    __shared__ float s_wd[RS_THREADS / 32][32];
-    __shared__ int32_t s_wi[RS_THREADS / 32][32];
-    const int y = blockIdx.x, r = blockIdx.y, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const int32_t q = rows[r];
-    const int64_t out = (int64_t(y) * cnt + r) * k;
-    if (y >= chunk_beg[K]) {  // past the last chunk
-        if (t == 0) pidx[out] = -1;
-        return;
-    }
-    int C = 0;  // the cell holding chunk y: the last C with chunk_beg[C] <= y
-    for (int lo = 0, hi = K - 1; lo <= hi;) {
-        const int mid = (lo + hi) >> 1;
-        if (chunk_beg[mid] <= y) {
-            C = mid;
-            lo = mid + 1;
-        } else {
-            hi = mid - 1;
-        }
-    }
-    for (int c = t; c < 64; c += RS_THREADS) s_x[c] = c < d ? X[int64_t(q) * d + c] : 0.f;
-    __syncthreads();
-    float part = 0.f;
-    for (int c = t; c < d; c += RS_THREADS) {
-        const float df = s_x[c] - cell_c[int64_t(C) * d + c];
-        part = fmaf(df, df, part);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane == 0) s_part[w] = part;
-    __syncthreads();
-    const float Dc = sqrtf(s_part[0] + s_part[1] + s_part[2] + s_part[3]);
-    const float rc = cell_r[C];
-    const float u = dist_in[int64_t(q) * k + k - 1];
-    if (Dc - rc - 1e-5f * (Dc + rc) > u * (1.0f + 2e-5f)) {  // false for u = INFINITY
-        if (t == 0) pidx[out] = -1;
-        return;
-    }
-    // admission bound: as in the FP32 scan's re-scan (the smallest normal
-    // number keeps a k-th distance of 0 admitting distance 0)
-    float T = fmaf(u * u, 1.0f + 1e-6f, 1.17549435e-38f);
-    if (!(T < INFINITY)) T = INFINITY;
-    float D[KL];
-    int32_t I[KL];
-#pragma unroll
-    for (int s2 = 0; s2 < KL; ++s2) {
-        D[s2] = T;
-        I[s2] = -1;
-    }
-    const int32_t b = cell_beg[C] + (y - chunk_beg[C]) * CH;
-    const int32_t e = cell_beg[C + 1] - b < CH ? cell_beg[C + 1] : b + CH;
-    // warp w copies points w, w + 4, ... of a tile, lanes on dimensions
-    // (lane, lane + 32)
-    auto stage = [&](int32_t p0, float* buf) {
-        const int m = e - p0 < RS_THREADS ? e - p0 : RS_THREADS;
-        for (int row = w; row < m; row += RS_THREADS / 32) {
-            const float* src = Xp + int64_t(p0 + row) * d;
-            if (lane < d) cp_async4(buf + row * RS_PITCH + lane, src + lane);
-            if (lane + 32 < d) cp_async4(buf + row * RS_PITCH + lane + 32, src + lane + 32);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    if (b < e) stage(b, s_pts);
-    int buf = 0;
-    for (int32_t p0 = b; p0 < e; p0 += RS_THREADS, buf ^= 1) {
-        const bool more = p0 + RS_THREADS < e;
-        if (more) {
-            stage(p0 + RS_THREADS, s_pts + (buf ^ 1) * RS_THREADS * RS_PITCH);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();
-        const float* tile = s_pts + buf * RS_THREADS * RS_PITCH;
-        if (p0 + t < e) {
-            float a = 0.f;
-            for (int c = 0; c < d; ++c) {
-                const float df = s_x[c] - tile[t * RS_PITCH + c];
-                a = fmaf(df, df, a);
-            }
-            if (a < D[KL - 1]) {
-                const int32_t j = perm[p0 + t];
-                if (j != q) topk_insert<KL>(D, I, a, j);
-            }
-        }
-        __syncthreads();  // the buffer is refilled two tiles later
-    }
-    // the warp's k best by (distance, index): k rounds of a warp-wide minimum
-    // over the lanes' list heads, the owner popping its head
-    for (int s2 = 0; s2 < k; ++s2) {
-        float bd = I[0] >= 0 ? D[0] : INFINITY;
-        int32_t bi = I[0] >= 0 ? I[0] : INT32_MAX;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-            const int32_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (od < bd || (od == bd && oi < bi)) {
-                bd = od;
-                bi = oi;
-            }
-        }
-        if (lane == 0) {
-            s_wd[w][s2] = bd;
-            s_wi[w][s2] = bi == INT32_MAX ? -1 : bi;
-        }
-        if (I[0] >= 0 && I[0] == bi && D[0] == bd) {
-#pragma unroll
-            for (int s3 = 0; s3 < KL - 1; ++s3) {
-                D[s3] = D[s3 + 1];
-                I[s3] = I[s3 + 1];
-            }
-            D[KL - 1] = T;
-            I[KL - 1] = -1;
-        }
-    }
-    __syncthreads();
-    // the CTA's k best from the four sorted warp lists (lanes 0..3 hold heads)
-    if (w == 0) {
-        int ptr = 0;
-        for (int s2 = 0; s2 < k; ++s2) {
-            float hd = INFINITY;
-            int32_t hi = INT32_MAX;
-            if (lane < RS_THREADS / 32 && ptr < k && s_wi[lane][ptr] >= 0) {
-                hd = s_wd[lane][ptr];
-                hi = s_wi[lane][ptr];
-            }
-            float bd = hd;
-            int32_t bi = hi;
-#pragma unroll
-            for (int o = 2; o > 0; o >>= 1) {
-                const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-                const int32_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (od < bd || (od == bd && oi < bi)) {
-                    bd = od;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) {
-                pidx[out + s2] = bi == INT32_MAX ? -1 : bi;
-                pd2[out + s2] = bd;
-            }
-            if (lane < RS_THREADS / 32 && hi == bi && hd == bd && bi != INT32_MAX) ++ptr;
-        }
     }
 }
 
@@ -1209,29 +1030,12 @@ static int knn_tc_impl(Ctx* c, const float* X, int64_t n, int d, int k, int32_t*
     DRGB_CUDA(c, cudaMemcpyAsync(&cnt32, fail_count, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     DRGB_CUDA(c, cudaStreamSynchronize(st));
     const int64_t cnt = cnt32 < n ? cnt32 : n;
-    // chunks: at least RS_CHUNK_MIN positions, at most as many as the
-    // partial lists' scratch holds (at most n / CH + K chunks in all)
-    int64_t CH = RS_CHUNK_MIN;
-    const size_t per_list = size_t(cnt > 0 ? cnt : 1) * k * 8;
-    const int64_t max_lists = int64_t((TC_PART_BYTES - 4096) / per_list) - K;
-    if (max_lists > 0 && CH * max_lists < n) CH = (n + max_lists - 1) / max_lists;
-    const int64_t nchunk = (n + CH - 1) / CH + K;
-    if (cnt > 0 && K > 1 && max_lists > 0 && nchunk <= int64_t(INT32_MAX) && cnt <= 65535) {
-        Carve pc(part);
-        int32_t* pidx = pc.take<int32_t>(size_t(cnt) * nchunk * k);
-        float* pd2 = pc.take<float>(size_t(cnt) * nchunk * k);
-        int32_t* chunk_beg = pc.take<int32_t>(TC_CELLS + 1);
-        tc_chunks_kernel<<<1, 32, 0, st>>>(cell_beg, K, int32_t(CH), chunk_beg);
-        DRGB_CHECK_LAUNCH(c);
-        const dim3 grid(static_cast<unsigned>(nchunk), static_cast<unsigned>(cnt));
-        auto rs = k <= 16 ? tc_rescan_kernel<16> : tc_rescan_kernel<32>;
-        DRGB_CUDA(c, cudaFuncSetAttribute(rs, cudaFuncAttributeMaxDynamicSharedMemorySize, int(RS_SMEM)));
-        rs<<<grid, RS_THREADS, RS_SMEM, st>>>(X, Xp, perm, d, k, fail_rows, int(cnt), K, int32_t(CH), cell_beg,
-                                              chunk_beg, cell_c, cell_r, dist_out, pidx, pd2);
-        DRGB_CHECK_LAUNCH(c);
-        rc = launch_merge_partials(c, pidx, pd2, cnt, int(nchunk), k, fail_rows, idx_out, dist_out, st);
-    } else {
-        rc = launch_knn_exact_rows_n(c, X, n, d, k, fail_rows, cnt, idx_out, dist_out, st, part, TC_PART_BYTES);
+    if (cnt > 0) {
+        bool done = false;
+        rc = launch_knn_cells(c, X, Xp, n, d, k, fail_rows, cnt, K, perm, cell_beg, cell_c, cell_r, idx_out, dist_out, st,
+                              part, TC_PART_BYTES, &done);
+        if (rc == DRGB_OK && !done)
+            rc = launch_knn_exact_rows_n(c, X, n, d, k, fail_rows, cnt, idx_out, dist_out, st, part, TC_PART_BYTES);
     }
     if (rc) return rc;
     return stage_mark(c, 10, st);
