@@ -8,10 +8,10 @@
 //   1 rows      rho, sigma (64 bisection steps), w_{j|i}; out-list sorted by
 //               column; histogram of tails, whose counts give each entry a slot
 //   2 scan      in_ptr
-//   3 scatter   in_src[in_ptr[j] + slot] = p   (p = i*k + s with idx[p] = j)
-//   4 sort      in-lists longer than a warp, by p
-//   5 merge     union of out-list and in-list (sorted by p in the warp's
-//               registers) by column -> tmp (cap k + m_i per row); entries kept
+//   3 scatter   in_src[in_ptr[j] + slot] = (i, w_{j|i})   (idx[i*k + s] = j)
+//   4 sort      in-lists longer than a warp, by source
+//   5 merge     union of out-list and in-list (sorted in the warp's registers)
+//               by column -> tmp (cap k + m_i per row); entries kept
 //               (T q >= 2^24)
 //   6 scan      row_ptr
 //   7 fill      col, w, q
@@ -48,6 +48,12 @@ __device__ __forceinline__ float quotient(float x, float m, float y) {
     float q = __fmul_rn(x, y);
     q = fmaf(fmaf(-q, m, x), y, q);
     return fmaf(fmaf(-q, m, x), y, q);
+}
+
+__device__ __forceinline__ float hw_exp2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 template <int KM>
@@ -111,9 +117,20 @@ fuzzy_rows_kernel(const int32_t* __restrict__ idx, const float* __restrict__ dis
                 float psum = 0.f;
                 if (tame) {
                     const float y = __frcp_rn(mid);
+                    // A sum of hardware exponentials is within 1e-4 of the
+                    // precise one (each term within about 2^-20), so it decides
+                    // the step unless it is that close to the target: about the
+                    // first half of them.
+                    const float z = 1.44269504f * y;
 #pragma unroll
                     for (int s = 0; s < KM; ++s)
-                        if (s < k) psum += expf(quotient(nx[s], mid, y));
+                        if (s < k) psum += hw_exp2(nx[s] * z);
+                    if (fabsf(psum - target) <= 1e-4f) {
+                        psum = 0.f;
+#pragma unroll
+                        for (int s = 0; s < KM; ++s)
+                            if (s < k) psum += expf(quotient(nx[s], mid, y));
+                    }
                 } else {
 #pragma unroll 1
                     for (int s = 0; s < k; ++s) psum += expf(-fmaxf(0.f, s_d[tid * pitch + s] - rho) / mid);
@@ -189,13 +206,13 @@ static constexpr int IS_THREADS = 256;
 
 __global__ void in_scatter_kernel(const int32_t* __restrict__ idx, int64_t n, int k,
                                   const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ slot,
-                                  int32_t* __restrict__ in_src, int32_t* __restrict__ long_rows,
-                                  unsigned int* __restrict__ long_cnt) {
+                                  const float* __restrict__ w_dir, int2* __restrict__ in_src,
+                                  int32_t* __restrict__ long_rows, unsigned int* __restrict__ long_cnt) {
     const int64_t nk = n * k;
     for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < nk;
          p += int64_t(gridDim.x) * blockDim.x) {
         const int32_t s = slot[p];
-        if (s >= 0) in_src[in_ptr[idx[p]] + s] = int32_t(p);
+        if (s >= 0) in_src[in_ptr[idx[p]] + s] = make_int2(int32_t(p / k), __float_as_int(w_dir[p]));
         if (p < n) {
             const int32_t m = in_ptr[p + 1] - in_ptr[p];
             if (m > IS_WARP_MAX && m <= IS_BIG_MAX) long_rows[n - 1 - atomicAdd(&long_cnt[1], 1u)] = int32_t(p);
@@ -205,28 +222,28 @@ __global__ void in_scatter_kernel(const int32_t* __restrict__ idx, int64_t n, in
 }
 
 // ---------------------------------------------------------------- pass 4
-// Ascending order of the (distinct) p values of the in-lists longer than 32.
-// Up to IS_WARP_MAX: a warp ranks its elements against the whole list.  Longer
-// ones (hubs: at 70K the in-degree reaches 620), padded with INT32_MAX to a
-// power of two, are sorted by a CTA's bitonic network in shared memory; beyond
-// IS_BIG_MAX a warp ranks them from global memory.
+// Ascending order of the (distinct) sources of the in-lists longer than 32, in
+// place.  Up to IS_WARP_MAX: a warp ranks its elements against the whole list.
+// Longer ones (hubs: at 70K the in-degree reaches 620), padded with INT32_MAX to
+// a power of two, are sorted by a CTA's bitonic network in shared memory; beyond
+// IS_BIG_MAX a warp ranks them in global memory (through tmp, as large as src).
 __global__ void __launch_bounds__(IS_THREADS)
-in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ src, int32_t* __restrict__ dst,
-               int64_t n, const int32_t* __restrict__ long_rows, const unsigned int* __restrict__ long_cnt) {
-    extern __shared__ int32_t s_row[];  // [IS_BIG_MAX]
+in_sort_kernel(const int32_t* __restrict__ in_ptr, int2* __restrict__ src, int2* __restrict__ tmp, int64_t n,
+               const int32_t* __restrict__ long_rows, const unsigned int* __restrict__ long_cnt) {
+    extern __shared__ __align__(16) int2 s_row[];  // [IS_BIG_MAX]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned warps = gridDim.x * (IS_THREADS / 32), few = long_cnt[0], many = long_cnt[1];
     for (unsigned r = blockIdx.x * (IS_THREADS / 32) + warp; r < few; r += warps) {
         const int32_t j = long_rows[r], b = in_ptr[j], m = in_ptr[j + 1] - b;
         if (m <= IS_WARP_MAX) {
-            int32_t* list = s_row + warp * IS_WARP_MAX;
-            int32_t x[IS_WARP_MAX / 32];
+            int32_t* list = reinterpret_cast<int32_t*>(s_row) + warp * IS_WARP_MAX;
+            int2 x[IS_WARP_MAX / 32];
             int32_t rank[IS_WARP_MAX / 32];
 #pragma unroll
             for (int u = 0; u < IS_WARP_MAX / 32; ++u) {
                 const int a = lane + 32 * u;
-                x[u] = a < m ? src[b + a] : INT32_MAX;
-                list[a] = x[u];
+                x[u] = a < m ? src[b + a] : make_int2(INT32_MAX, 0);
+                list[a] = x[u].x;
                 rank[u] = 0;
             }
             __syncwarp();
@@ -234,19 +251,21 @@ in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ s
             for (int t = 0; t < m; ++t) {
                 const int32_t y = list[t];
 #pragma unroll
-                for (int u = 0; u < IS_WARP_MAX / 32; ++u) rank[u] += y < x[u];
+                for (int u = 0; u < IS_WARP_MAX / 32; ++u) rank[u] += y < x[u].x;
             }
 #pragma unroll
             for (int u = 0; u < IS_WARP_MAX / 32; ++u)
-                if (lane + 32 * u < m) dst[b + rank[u]] = x[u];
+                if (lane + 32 * u < m) src[b + rank[u]] = x[u];
             __syncwarp();
         } else {
             for (int32_t a = lane; a < m; a += 32) {
-                const int32_t x = src[b + a];
+                const int2 x = src[b + a];
                 int32_t rank = 0;
-                for (int32_t t = 0; t < m; ++t) rank += src[b + t] < x;
-                dst[b + rank] = x;
+                for (int32_t t = 0; t < m; ++t) rank += src[b + t].x < x.x;
+                tmp[b + rank] = x;
             }
+            __syncwarp();
+            for (int32_t a = lane; a < m; a += 32) src[b + a] = tmp[b + a];
         }
     }
     for (unsigned r = blockIdx.x; r < many; r += gridDim.x) {
@@ -254,15 +273,15 @@ in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ s
         int P = 2 * IS_WARP_MAX;
         while (P < m) P <<= 1;
         __syncthreads();  // the previous lists are done with
-        for (int a = threadIdx.x; a < P; a += IS_THREADS) s_row[a] = a < m ? src[b + a] : INT32_MAX;
+        for (int a = threadIdx.x; a < P; a += IS_THREADS) s_row[a] = a < m ? src[b + a] : make_int2(INT32_MAX, 0);
         __syncthreads();
         for (int kk = 2; kk <= P; kk <<= 1) {
             for (int jj = kk >> 1; jj > 0; jj >>= 1) {
                 for (int a = threadIdx.x; a < P; a += IS_THREADS) {
                     const int l = a ^ jj;
                     if (l > a) {
-                        const int32_t x = s_row[a], y = s_row[l];
-                        if ((x > y) == ((a & kk) == 0)) {
+                        const int2 x = s_row[a], y = s_row[l];
+                        if ((x.x > y.x) == ((a & kk) == 0)) {
                             s_row[a] = y;
                             s_row[l] = x;
                         }
@@ -271,7 +290,7 @@ in_sort_kernel(const int32_t* __restrict__ in_ptr, const int32_t* __restrict__ s
                 __syncthreads();
             }
         }
-        for (int a = threadIdx.x; a < m; a += IS_THREADS) dst[b + a] = s_row[a];
+        for (int a = threadIdx.x; a < m; a += IS_THREADS) src[b + a] = s_row[a];
     }
 }
 
@@ -311,8 +330,7 @@ __device__ __forceinline__ int warp_lower_bound(int32_t list, int32_t x) {
 // The next row's bounds and out-list are loaded while this one is merged.
 __global__ void __launch_bounds__(256)
 merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_w, const int32_t* __restrict__ in_ptr,
-             const int32_t* __restrict__ in_src, const int32_t* __restrict__ in_sorted,
-             const float* __restrict__ w_dir, int64_t n, int k, int T, int32_t* __restrict__ tcol,
+             const int2* __restrict__ in_src, int64_t n, int k, int T, int32_t* __restrict__ tcol,
              float* __restrict__ tw, int32_t* __restrict__ tcnt, int32_t* __restrict__ keep_cnt) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -334,16 +352,21 @@ merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_
         const float wa = ow_n;
         const int64_t base = i * k + ib;
         // the first 32 in entries, sorted
-        int32_t p = lane < m ? (m <= 32 ? in_src[ib + lane] : in_sorted[ib + lane]) : INT32_MAX;
+        int2 p = lane < m ? in_src[ib + lane] : make_int2(INT32_MAX, 0);
         prefetch(i + warps);
         if (m <= 32) {
 #pragma unroll
             for (int kk = 2; kk <= 32; kk <<= 1) {
+                if (kk > 16 && m <= 16) break;  // the first 16 lanes hold the list, ascending
 #pragma unroll
                 for (int st = kk >> 1; st > 0; st >>= 1) {
-                    const int32_t o = __shfl_xor_sync(0xffffffffu, p, st);
+                    const int32_t o = __shfl_xor_sync(0xffffffffu, p.x, st), ow = __shfl_xor_sync(0xffffffffu, p.y, st);
+                    // (the padding's keys are equal, and so are their weights)
                     const bool keep_min = ((lane & kk) == 0) == ((lane & st) == 0);
-                    p = keep_min ? min(p, o) : max(p, o);
+                    if (keep_min == (o < p.x)) {
+                        p.x = o;
+                        p.y = ow;
+                    }
                 }
             }
         }
@@ -354,9 +377,9 @@ merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_
         bool matched = false;
         // out entries: in columns below c0, and c0's in weight if present
         for (int32_t t0 = 0; t0 < m; t0 += 32) {
-            if (t0) p = t0 + lane < m ? in_sorted[ib + t0 + lane] : INT32_MAX;
-            const int32_t cb = p == INT32_MAX ? INT32_MAX : p / k;
-            const float wb = p == INT32_MAX ? 0.f : w_dir[p];
+            if (t0) p = t0 + lane < m ? in_src[ib + t0 + lane] : make_int2(INT32_MAX, 0);
+            const int32_t cb = p.x;
+            const float wb = __int_as_float(p.y);
             const int at = warp_lower_bound(cb, c0);
             in_less += at;
             const int32_t cm = __shfl_sync(0xffffffffu, cb, at & 31);
@@ -391,9 +414,9 @@ merge_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_
         if (m > 32) {  // in entries without an out partner
             for (int32_t t0 = 0; t0 < m; t0 += 32) {
                 const int32_t t = t0 + lane;
-                const int32_t q = t < m ? in_sorted[ib + t] : INT32_MAX;
-                const int32_t cb = q == INT32_MAX ? INT32_MAX : q / k;
-                const float wb = q == INT32_MAX ? 0.f : w_dir[q];
+                const int2 e = t < m ? in_src[ib + t] : make_int2(INT32_MAX, 0);
+                const int32_t cb = e.x;
+                const float wb = __int_as_float(e.y);
                 const int ao = warp_lower_bound(c0, cb);
                 const int32_t co = __shfl_sync(0xffffffffu, c0, ao & 31);
                 const unsigned below = ao >= 32 ? 0xffffffffu : (1u << ao) - 1u;
@@ -475,7 +498,7 @@ size_t fuzzy_scratch_bytes(int64_t n, int k) {
     size_t b = 0;
     b += Carve::round(nk * 4) * 3;          // w_dir, out_col, out_w
     b += Carve::round((n + 1) * 4) * 4;     // in_cnt, in_ptr, long_rows, keep_cnt
-    b += Carve::round(nk * 4) * 2;          // in_src, in_sorted
+    b += Carve::round(nk * 4) * 2;          // in_src (pairs)
     b += Carve::round(2 * nk * 4) * 2;      // tcol, tw
     b += Carve::round(n * 4);               // tcnt
     b += Carve::round(256);                 // long_cnt
@@ -495,14 +518,14 @@ int build_fuzzy_graph(Ctx* c, const int32_t* idx, const float* dist, int64_t n, 
     int32_t* in_ptr = cv.take<int32_t>(n + 1);
     int32_t* long_rows = cv.take<int32_t>(n + 1);
     int32_t* keep_cnt = cv.take<int32_t>(n + 1);
-    int32_t* in_src = cv.take<int32_t>(nk);
-    int32_t* in_sorted = cv.take<int32_t>(nk);
+    int2* in_src = cv.take<int2>(nk);
     int32_t* tcol = cv.take<int32_t>(2 * nk);
     float* tw = cv.take<float>(2 * nk);
     int32_t* tcnt = cv.take<int32_t>(n);
     unsigned int* long_cnt = cv.take<unsigned int>(64);
     int32_t* scan_tmp = cv.take<int32_t>(scan_scratch_elems(n));
-    int32_t* slot = tcol;  // free until the merge
+    int32_t* slot = tcol;  // free until the merge, as is the sort's
+    int2* sort_tmp = reinterpret_cast<int2*>(tw);
 
     const int TB = 256;
     const int gmax = c->num_sms * 16;
@@ -510,13 +533,15 @@ int build_fuzzy_graph(Ctx* c, const int32_t* idx, const float* dist, int64_t n, 
     DRGB_CUDA(c, cudaMemsetAsync(long_cnt, 0, 8, st));
     int rc = launch_fuzzy_rows(c, idx, dist, n, k, n, w_dir, out_col, out_w, rho, sigma, in_cnt, slot, st);
     if (rc || (rc = exclusive_scan(c, in_cnt, in_ptr, n, scan_tmp, st))) return rc;
-    in_scatter_kernel<<<grid_for(int64_t(nk), TB, gmax), TB, 0, st>>>(idx, n, k, in_ptr, slot, in_src, long_rows, long_cnt);
+    in_scatter_kernel<<<grid_for(int64_t(nk), TB, gmax), TB, 0, st>>>(idx, n, k, in_ptr, slot, w_dir, in_src, long_rows,
+                                                                       long_cnt);
     DRGB_CHECK_LAUNCH(c);
-    in_sort_kernel<<<c->num_sms * 4, IS_THREADS, size_t(IS_BIG_MAX) * 4, st>>>(in_ptr, in_src, in_sorted, n, long_rows,
+    DRGB_CUDA(c, cudaFuncSetAttribute(in_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, IS_BIG_MAX * 8));
+    in_sort_kernel<<<c->num_sms * 2, IS_THREADS, size_t(IS_BIG_MAX) * 8, st>>>(in_ptr, in_src, sort_tmp, n, long_rows,
                                                                                long_cnt);
     DRGB_CHECK_LAUNCH(c);
-    merge_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(out_col, out_w, in_ptr, in_src, in_sorted, w_dir, n, k, T,
-                                                           tcol, tw, tcnt, keep_cnt);
+    merge_kernel<<<grid_for(n, TB / 32, gmax), TB, 0, st>>>(out_col, out_w, in_ptr, in_src, n, k, T, tcol, tw,
+                                                           tcnt, keep_cnt);
     DRGB_CHECK_LAUNCH(c);
     if ((rc = exclusive_scan(c, keep_cnt, row_ptr, n, scan_tmp, st))) return rc;
     fill_kernel<<<grid_for(n, FILL_ROWS * TB / 32, gmax), TB, 0, st>>>(in_ptr, tcol, tw, tcnt, n, k, T, row_ptr, col, w, q);
