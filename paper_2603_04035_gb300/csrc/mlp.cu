@@ -750,6 +750,245 @@ __global__ void mlp_init_kernel(float* __restrict__ P, int d, uint32_t k0, uint3
     }
 }
 
+// ------------------------------------------------------------------ fused forward pass
+// Y = head(GELU(GELU(X W1^T + b1) W2^T + b2)) for whole 128-row tiles, one
+// persistent CTA per SM: both weight matrices stay in shared memory (160 KB),
+// X is cast into a swizzled operand tile, H1 goes through shared memory in two
+// halves of 128 columns, each multiplied into the second accumulator as soon as
+// it is written, and H2 never leaves the registers that form the head's sums.
+//
+// Bound: the two GELUs' erf (about 40 instructions an element on the FP32 pipe,
+// 18,000 cycles a tile against 3,200 of MMA), which the earlier form, two GEMMs
+// and a head over chunks of 65,536 rows, joined with three passes over the
+// activations.
+//
+// The sums are those of the training kernels: column pairs of the head in the
+// order of mlp_head_kernel (partial sums over columns u + 32 i, i ascending, for
+// u = 0..31, joined as its shuffles join lanes).
+static constexpr int FE_EPI_WARPS = 16;  // four per TMEM lane quarter
+static constexpr int FE_EPI = FE_EPI_WARPS * 32;
+static constexpr int FE_THREADS = FE_EPI + 32;  // the last warp loads the weights and issues the MMAs
+static constexpr int FE_W1 = MLP_H * MLP_IN * 2, FE_W2 = MLP_H * MLP_H * 2, FE_X = G_BM * MLP_IN * 2, FE_H = G_BM * 128 * 2;
+static constexpr size_t FE_SMEM = 1024 + FE_W1 + FE_W2 + FE_X + FE_H + 128 + (4 * MLP_H + 2) * 4;
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__global__ void __launch_bounds__(FE_THREADS, 1)
+mlp_embed_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
+                 const float* __restrict__ X, int64_t n, int d, const float* __restrict__ P,
+                 const float* __restrict__ W3f, float* __restrict__ Y, int* status) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint8_t* sW1 = base;
+    uint8_t* sW2 = sW1 + FE_W1;  // four K blocks of 64 columns x 256 rows
+    uint8_t* sX = sW2 + FE_W2;
+    uint8_t* sH = sX + FE_X;     // two K blocks of 64 columns x 128 rows; also the head's partial sums
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sH + FE_H);
+    uint64_t *w_full = bars, *x_full = bars + 1, *h_full = bars + 2, *d1_full = bars + 3, *h_free = bars + 4,
+             *d2_full = bars + 5, *mma_done = bars + 6;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 7);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    float* s_b1 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 128);
+    float* s_b2 = s_b1 + MLP_H;
+    float* s_w3 = s_b2 + MLP_H;  // [2][256], then the two biases
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t tiles = (n + G_BM - 1) / G_BM;
+    const int mine = int((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x);  // tiles blockIdx.x, + gridDim.x, ...
+
+    if (tid == 0) {
+        mbar_init(w_full, 1);
+        mbar_init(x_full, FE_EPI_WARPS);
+        mbar_init(h_full, FE_EPI_WARPS);
+        mbar_init(d1_full, 1);
+        mbar_init(h_free, 1);
+        mbar_init(d2_full, 1);
+        mbar_init(mma_done, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == FE_EPI_WARPS) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int t = tid; t < MLP_H; t += FE_THREADS) {
+        s_b1[t] = P[OFF_B1 + t];
+        s_b2[t] = P[OFF_B2 + t];
+        s_w3[t] = W3f[t];
+        s_w3[MLP_H + t] = W3f[MLP_H + t];
+        if (t < 2) s_w3[2 * MLP_H + t] = P[OFF_B3 + t];
+    }
+    for (int t = tid; t < FE_X / 16; t += FE_THREADS) reinterpret_cast<uint4*>(sX)[t] = make_uint4(0u, 0u, 0u, 0u);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == FE_EPI_WARPS) {
+        if (lane == 0) {
+            mbar_expect_tx(w_full, FE_W1 + FE_W2);
+            tma_load_2d(sW1, &tmW1, 0, 0, w_full);
+            for (int kb = 0; kb < 4; ++kb) tma_load_2d(sW2 + kb * (FE_W2 / 4), &tmW2, kb * 64, 0, w_full);
+            const uint32_t idesc = idesc_f16kind(G_BM, MLP_H, false);
+            const uint32_t D1 = tmem, D2 = tmem + MLP_H;
+            bool ok = mbar_wait(w_full, 0, abort_flag, status);
+            for (int t = 0; t < mine && ok; ++t) {
+                if (!mbar_wait(x_full, t & 1, abort_flag, status)) break;
+                tc_fence_after();
+                const uint64_t xd = sdesc_sw128(smem_u32(sX)), w1d = sdesc_sw128(smem_u32(sW1));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mma_f16kind(D1, xd + 2 * k, w1d + 2 * k, idesc, k > 0);
+                mma_commit(d1_full);
+                for (int half = 0; half < 2 && ok; ++half) {
+                    if (!(ok = mbar_wait(h_full, half, abort_flag, status))) break;
+                    tc_fence_after();
+                    for (int kb = 0; kb < 2; ++kb) {
+                        const uint64_t hd = sdesc_sw128(smem_u32(sH + kb * (FE_H / 2)));
+                        const uint64_t w2d = sdesc_sw128(smem_u32(sW2 + (2 * half + kb) * (FE_W2 / 4)));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            mma_f16kind(D2, hd + 2 * k, w2d + 2 * k, idesc, (half > 0 || kb > 0 || k > 0) ? 1u : 0u);
+                    }
+                    mma_commit(half == 0 ? h_free : d2_full);
+                }
+            }
+            // every MMA issued above has completed once this barrier fires
+            mma_commit(mma_done);
+            const unsigned long long t0 = global_timer();
+            while (!mbar_try(mma_done, 0) && global_timer() - t0 < 100000000ull) {
+            }
+        }
+    } else {
+        // A failed wait (reported in the status word) does not leave the loop:
+        // every later one then returns at once, and the warps still meet at
+        // their barriers.
+        const int quarter = warp & 3, g = warp >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t tq = tmem + (uint32_t(quarter * 32) << 16);
+        // this thread's elements of an X tile (128 d consecutive floats) and
+        // their places in the operand tile
+        constexpr int NX = G_BM * MLP_IN / FE_EPI;
+        uint32_t xo[NX];
+#pragma unroll
+        for (int u = 0; u < NX; ++u) {
+            const int e = tid + u * FE_EPI, r = e / d, c = e - r * d;
+            xo[u] = r < G_BM ? uint32_t(r * 128 + ((((c >> 3) ^ r) & 7) << 4) + (c & 7) * 2) : 0xffffffffu;
+        }
+        float xv[NX];
+        auto load_x = [&](int t) {
+            const int64_t e0 = (blockIdx.x + int64_t(t) * gridDim.x) * G_BM * d;
+#pragma unroll
+            for (int u = 0; u < NX; ++u) {
+                const int64_t e = e0 + tid + u * FE_EPI;
+                xv[u] = t < mine && xo[u] != 0xffffffffu && e < n * d ? X[e] : 0.f;
+            }
+        };
+        auto stage_x = [&]() {
+#pragma unroll
+            for (int u = 0; u < NX; ++u)
+                if (xo[u] != 0xffffffffu) *reinterpret_cast<bf16*>(sX + xo[u]) = __float2bfloat16_rn(xv[u]);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tc_fence_before();  // (the reads of the first accumulator)
+            __syncwarp();
+            if (lane == 0) mbar_arrive(x_full);
+        };
+        load_x(0);
+        if (mine > 0) stage_x();
+        load_x(1);
+        for (int t = 0; t < mine; ++t) {
+            mbar_wait(d1_full, t & 1, abort_flag, status);
+            tc_fence_after();
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                const int c0 = half * 128 + g * 32;
+                float v[32];
+                __syncwarp();
+                tmem_ld32(tq + uint32_t(c0), v);
+                uint32_t packed[16];
+#pragma unroll
+                for (int i = 0; i < 32; i += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(s_b1 + c0 + i);
+                    v[i] = gelu(v[i] + b4.x);
+                    v[i + 1] = gelu(v[i + 1] + b4.y);
+                    v[i + 2] = gelu(v[i + 2] + b4.z);
+                    v[i + 3] = gelu(v[i + 3] + b4.w);
+                    const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i], v[i + 1]), h1 = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
+                    packed[i / 2] = *reinterpret_cast<const uint32_t*>(&h0);
+                    packed[i / 2 + 1] = *reinterpret_cast<const uint32_t*>(&h1);
+                }
+                // the first half's products with H are done (the second's, of the
+                // tile before, were when its D2 was read)
+                if (half == 1) mbar_wait(h_free, t & 1, abort_flag, status);
+                uint8_t* hr = sH + (g >> 1) * (FE_H / 2) + row * 128;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<uint4*>(hr + ((((g & 1) * 4 + j) ^ (row & 7)) << 4)) =
+                        make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(h_full);
+            }
+            if (t + 1 < mine) stage_x();
+            load_x(t + 2);
+            mbar_wait(d2_full, t & 1, abort_flag, status);
+            tc_fence_after();
+            // residues u = 8 g .. 8 g + 7 of the columns modulo 32
+            float p0[8], p1[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) p0[u] = p1[u] = 0.f;
+#pragma unroll 1
+            for (int i = 0; i < 8; ++i) {
+                const int c0 = 32 * i + 8 * g;
+                float v[8];
+                __syncwarp();
+                tmem_ld8(tq + uint32_t(MLP_H + c0), v);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float h = __bfloat162float(__float2bfloat16_rn(gelu(v[u] + s_b2[c0 + u])));
+                    p0[u] = fmaf(h, s_w3[c0 + u], p0[u]);
+                    p1[u] = fmaf(h, s_w3[MLP_H + c0 + u], p1[u]);
+                }
+            }
+            tc_fence_before();
+            float* hs = reinterpret_cast<float*>(sH);  // [2][32][128]
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                hs[(8 * g + u) * 128 + row] = p0[u];
+                hs[(32 + 8 * g + u) * 128 + row] = p1[u];
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(FE_EPI) : "memory");
+            if (tid < 2 * G_BM) {
+                const int o = tid >> 7, r = tid & 127;
+                float q[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) q[u] = hs[(32 * o + u) * 128 + r] + hs[(32 * o + u + 16) * 128 + r];
+#pragma unroll
+                for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+                    for (int u = 0; u < w; ++u) q[u] += q[u + w];
+                const int64_t gr = (blockIdx.x + int64_t(t) * gridDim.x) * G_BM + r;
+                if (gr < n) Y[2 * gr + o] = q[0] + s_w3[2 * MLP_H + o];
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(FE_EPI) : "memory");
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == FE_EPI_WARPS) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
 // ------------------------------------------------------------------ host: one forward/backward
 // Opt the chunk kernels into their shared-memory sizes (before any capture).
 static int chunk_prepare(Ctx* c) {
@@ -1054,17 +1293,10 @@ int drgb_mlp_embed(drgb_ctx* c, const float* params, const float* X, int64_t n, 
     if (rc) return rc;
     if (!params || !X || !Y || n < 1) return set_error(c, DRGB_ERR_INVALID, "mlp_embed: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if ((rc = gemm_prepare(c))) return rc;
-    const int CH = 1 << 16;  // rows per chunk
-    const size_t bytes = Carve::round(size_t(CH) * MLP_IN * 2) + 2 * Carve::round(size_t(CH) * MLP_H * 2) +
-                         Carve::round(size_t(CH) * 2 * 4) + 2 * Carve::round(MLP_H * MLP_H * 2) +
-                         Carve::round(MLP_H * MLP_IN * 2) + Carve::round(2 * MLP_H * 4) + 8192;
+    const size_t bytes = 2 * Carve::round(MLP_H * MLP_H * 2) + Carve::round(MLP_H * MLP_IN * 2) +
+                         Carve::round(2 * MLP_H * 4) + 1024;
     if ((rc = ensure_scratch(c, bytes, st))) return rc;
     Carve cv(c->scratch);
-    bf16* Xb = cv.take<bf16>(size_t(CH) * MLP_IN);
-    bf16* H1 = cv.take<bf16>(size_t(CH) * MLP_H);
-    bf16* H2 = cv.take<bf16>(size_t(CH) * MLP_H);
-    float* z = cv.take<float>(size_t(CH) * 2);
     MlpWeights W;
     W.W2b = cv.take<bf16>(MLP_H * MLP_H);
     W.W2tb = cv.take<bf16>(MLP_H * MLP_H);
@@ -1072,24 +1304,13 @@ int drgb_mlp_embed(drgb_ctx* c, const float* params, const float* X, int64_t n, 
     W.W3f = cv.take<float>(2 * MLP_H);
     mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, W);
     DRGB_CHECK_LAUNCH(c);
-    for (int64_t r0 = 0; r0 < n; r0 += CH) {
-        const int mv = int(n - r0 < CH ? n - r0 : CH);
-        const int M = round_up(mv, 128);
-        mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, st>>>(X + r0 * d, d, nullptr, M, mv, Xb,
-                                                                            nullptr);
-        DRGB_CHECK_LAUNCH(c);
-        Gemm F1, F2;
-        if ((rc = gemm_setup(c, F1, Xb, W.W1b, M, MLP_H, MLP_IN, 128, EPI_GELU, 1))) return rc;
-        F1.g.bias = params + OFF_B1;
-        F1.g.out = H1;
-        if ((rc = gemm_setup(c, F2, H1, W.W2b, M, MLP_H, MLP_H, 128, EPI_GELU, 1))) return rc;
-        F2.g.bias = params + OFF_B2;
-        F2.g.out = H2;
-        if ((rc = gemm_launch(c, F1, st)) || (rc = gemm_launch(c, F2, st))) return rc;
-        mlp_head_kernel<<<grid_for(M / HEAD_ROWS, 8, c->num_sms * 8), 256, 0, st>>>(H2, W.W3f, params, M, z);
-        DRGB_CHECK_LAUNCH(c);
-        DRGB_CUDA(c, cudaMemcpyAsync(Y + 2 * r0, z, size_t(mv) * 8, cudaMemcpyDeviceToDevice, st));
-    }
+    CUtensorMap m1, m2;
+    if ((rc = make_map_k64(c, &m1, W.W1b, MLP_H, MLP_IN, MLP_H, false))) return rc;
+    if ((rc = make_map_k64(c, &m2, W.W2b, MLP_H, MLP_H, MLP_H, false))) return rc;
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(FE_SMEM)));
+    mlp_embed_kernel<<<grid_for((n + G_BM - 1) / G_BM, 1, c->num_sms), FE_THREADS, FE_SMEM, st>>>(m1, m2, X, n, d, params,
+                                                                                                W.W3f, Y, c->d_status);
+    DRGB_CHECK_LAUNCH(c);
     return DRGB_OK;
 }
 
