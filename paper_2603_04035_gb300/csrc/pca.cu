@@ -91,27 +91,33 @@ __global__ void pca_mean_kernel(const double* __restrict__ part, int chunks, int
 }
 
 // hi[j][i], lo[j][i] = the split of X[i][j] - mu[j] (zero outside n x D),
-// through 32 x 32 tiles in shared memory.
-__global__ void pca_stage_kernel(const float* __restrict__ X, const float* __restrict__ mu, int64_t n, int D,
+// through 64 x 32 tiles in shared memory, so that a warp stores 128 bytes of a
+// row (two points a lane).
+__global__ void __launch_bounds__(256) pca_stage_kernel(const float* __restrict__ X, const float* __restrict__ mu, int64_t n, int D,
                                  int64_t n_pad, int D_pad, __nv_bfloat16* __restrict__ hi,
                                  __nv_bfloat16* __restrict__ lo) {
-    __shared__ float tile[32][33];
-    const int64_t i0 = int64_t(blockIdx.x) * 32;
+    __shared__ float tile[64][33];
+    const int64_t i0 = int64_t(blockIdx.x) * 64;
     const int j0 = blockIdx.y * 32;
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int64_t i = i0 + r;
-        const int j = j0 + threadIdx.x;
-        tile[r][threadIdx.x] = (i < n && j < D) ? X[i * D + j] - mu[j] : 0.f;
+    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+    const int jx = j0 + tx;
+    const float m = jx < D ? mu[jx] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int64_t i = i0 + ty + 8 * u;
+        tile[ty + 8 * u][tx] = (i < n && jx < D) ? X[i * D + jx] - m : 0.f;
     }
     __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int j = j0 + r;
-        const int64_t i = i0 + threadIdx.x;
-        if (j < D_pad && i < n_pad) {
-            const float v = tile[threadIdx.x][r];
-            const __nv_bfloat16 h = __float2bfloat16_rn(v);
-            hi[int64_t(j) * n_pad + i] = h;
-            lo[int64_t(j) * n_pad + i] = __float2bfloat16_rn(v - __bfloat162float(h));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = ty + 8 * u, j = j0 + r;
+        const int64_t i = i0 + 2 * tx;
+        if (j < D_pad && i < n_pad) {  // n_pad is a multiple of 64
+            const float v0 = tile[2 * tx][r], v1 = tile[2 * tx + 1][r];
+            const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+            *reinterpret_cast<__nv_bfloat162*>(hi + int64_t(j) * n_pad + i) = h;
+            *reinterpret_cast<__nv_bfloat162*>(lo + int64_t(j) * n_pad + i) =
+                __floats2bfloat162_rn(v0 - __bfloat162float(h.x), v1 - __bfloat162float(h.y));
         }
     }
 }
@@ -154,11 +160,48 @@ __global__ void pca_cov_kernel(const double* __restrict__ T, const double* __res
 // Blocks are D x P row-major; columns < L are the locked vectors, columns
 // L..P-1 the active ones (m = P - L of them).
 
+// Whether this CTA is the last of `count` to arrive at `counter` (which it then
+// resets): what the others wrote before is visible to it.
+__device__ __forceinline__ bool last_to_arrive(unsigned int* counter, unsigned int count) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(counter, 1u) == count - 1;
+        if (s_last) *counter = 0;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+// sum of at(0 .. count - 1) in order, eight loads in flight.
+template <class T, class F>
+__device__ __forceinline__ T ordered_sum(int count, F&& at) {
+    T s = 0;
+    for (int z0 = 0; z0 < count; z0 += 8) {
+        T v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = z0 + u < count ? at(z0 + u) : T(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (z0 + u < count) s += v[u];
+    }
+    return s;
+}
+
+// Active columns: Y = alpha C X + beta X + gamma Z (locked columns: Y = X).
 // part[s][a][p] = sum over b in split s (PCA_KCHUNK rows) of C[a][b] X[b][p]:
 // a block takes PCA_CROWS rows of C and one split, both staged in shared
-// memory; a thread computes 4 adjacent columns of one row.
-__global__ void __launch_bounds__(256) pca_cmul_part_kernel(const float* __restrict__ C, int D,
-                                                            const float* __restrict__ X, float* __restrict__ part) {
+// memory; a thread computes 4 adjacent columns of one row.  The block that
+// finishes a row range last adds its splits, in order (instead of a launch of
+// its own, 5 us and a gap each).  (4 rows x 4 columns a thread, with a quarter of
+// the threads to load: 29 us a product against 19.)
+__global__ void __launch_bounds__(256) pca_cmul_kernel(const float* __restrict__ C, int D,
+                                                       const float* __restrict__ X, float* __restrict__ part,
+                                                       unsigned int* __restrict__ counters,
+                                                       const float* __restrict__ Z, float alpha, float beta,
+                                                       float gamma, int L, float* __restrict__ Y) {
     __shared__ __align__(16) float Xs[PCA_KCHUNK][PCA_P];
     __shared__ float Cs[PCA_CROWS][PCA_KCHUNK + 1];
     const int a0 = blockIdx.x * PCA_CROWS, b0 = blockIdx.y * PCA_KCHUNK;
@@ -202,22 +245,19 @@ __global__ void __launch_bounds__(256) pca_cmul_part_kernel(const float* __restr
     }
     if (a0 + r < D)
         *reinterpret_cast<float4*>(part + (int64_t(blockIdx.y) * D + a0 + r) * PCA_P + 4 * c4) = acc;
-}
-
-// Active columns: Y = alpha C X + beta X + gamma Z, C X the sum of the splits
-// in order; locked columns: Y = X.
-__global__ void pca_cmul_kernel(const float* __restrict__ part, int nsplit, int D, const float* __restrict__ X,
-                                const float* __restrict__ Z, float alpha, float beta, float gamma, int L,
-                                float* __restrict__ Y) {
+    if (!last_to_arrive(&counters[blockIdx.x], gridDim.y)) return;
     const int64_t total = int64_t(D) * PCA_P;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += int64_t(gridDim.x) * blockDim.x) {
-        const int p = int(t % PCA_P);
+    const int nsplit = gridDim.y;
+#pragma unroll
+    for (int u = 0; u < PCA_CROWS * PCA_P / 256; ++u) {
+        const int e = threadIdx.x + u * 256, a = a0 + e / PCA_P, p = e % PCA_P;
+        if (a >= D) continue;
+        const int64_t t = int64_t(a) * PCA_P + p;
         if (p < L) {
             Y[t] = X[t];
             continue;
         }
-        float s = 0.f;
-        for (int z = 0; z < nsplit; ++z) s += part[z * total + t];
+        const float s = ordered_sum<float>(nsplit, [&](int z) { return __ldcg(part + z * total + t); });
         float y = alpha * s + beta * X[t];
         if (Z) y = fmaf(gamma, Z[t], y);
         Y[t] = y;
@@ -228,9 +268,11 @@ __global__ void pca_cmul_kernel(const float* __restrict__ part, int nsplit, int 
 // q < m (chunks of PCA_GCHUNK rows, staged in shared memory).  The sum runs
 // in float-float arithmetic (Ogita, Rump & Oishi 2005, Dot2: the exact
 // product split by an FMA, the running sum by Knuth's TwoSum), about as
-// accurate as FP64 and all on the FP32 pipes, and is stored as FP64.
+// accurate as FP64 and all on the FP32 pipes, and is stored as FP64.  The last
+// chunk's block to finish adds the chunks in order into G.
 __global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                       int D, int L, double* __restrict__ Gp) {
+                                                       int D, int L, double* __restrict__ Gp,
+                                                       unsigned int* __restrict__ counters, double* __restrict__ G) {
     __shared__ float As[PCA_GCHUNK][PCA_P + 1];
     __shared__ float Bs[PCA_GCHUNK][PCA_P + 1];
     const int m = PCA_P - L;
@@ -263,29 +305,23 @@ __global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__
     }
     __syncthreads();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= PCA_P * m) return;
-    const int p = t / m, q = L + (t - p * m);
-    float hi = 0.f, lo = 0.f;
-    for (int a = 0; a < rows; ++a) {
-        const float x = As[a][p], y = Bs[a][q];
-        const float pr = __fmul_rn(x, y);
-        const float pe = fmaf(x, y, -pr);
-        const float s = __fadd_rn(hi, pr);
-        const float bb = __fsub_rn(s, hi);
-        const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(pr, bb));
-        hi = s;
-        lo = __fadd_rn(lo, __fadd_rn(se, pe));
+    if (t < PCA_P * m) {
+        const int p = t / m, q = L + (t - p * m);
+        float hi = 0.f, lo = 0.f;
+        for (int a = 0; a < rows; ++a) {
+            const float x = As[a][p], y = Bs[a][q];
+            const float pr = __fmul_rn(x, y);
+            const float pe = fmaf(x, y, -pr);
+            const float s = __fadd_rn(hi, pr);
+            const float bb = __fsub_rn(s, hi);
+            const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(pr, bb));
+            hi = s;
+            lo = __fadd_rn(lo, __fadd_rn(se, pe));
+        }
+        Gp[int64_t(blockIdx.y) * PCA_P * m + t] = double(hi) + double(lo);
     }
-    Gp[int64_t(blockIdx.y) * PCA_P * m + t] = double(hi) + double(lo);
-}
-
-// G[t] = sum_z Gp[z][t] (chunk order), t < P m.
-__global__ void pca_gsum_kernel(const double* __restrict__ Gp, int nch, int pm, double* __restrict__ G) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= pm) return;
-    double v = 0.0;
-    for (int z = 0; z < nch; ++z) v += Gp[int64_t(z) * pm + t];
-    G[t] = v;
+    if (!last_to_arrive(&counters[blockIdx.x], gridDim.y) || t >= PCA_P * m) return;
+    G[t] = ordered_sum<double>(gridDim.y, [&](int z) { return __ldcg(Gp + int64_t(z) * PCA_P * m + t); });
 }
 
 // rn[j] = sum_a (W[a][L + j] - theta_j Y[a][L + j])^2 (FP64), one warp per
@@ -297,6 +333,7 @@ __global__ void pca_resid_kernel(const float* __restrict__ Y, const float* __res
     const int k = L + j;
     const float th = theta[j];
     double s = 0.0;
+#pragma unroll 8
     for (int a = lane; a < D; a += 32) {
         const double r = double(W[int64_t(a) * PCA_P + k]) - double(th) * double(Y[int64_t(a) * PCA_P + k]);
         s = fma(r, r, s);
@@ -306,73 +343,105 @@ __global__ void pca_resid_kernel(const float* __restrict__ Y, const float* __res
     if (lane == 0) rn[j] = s;
 }
 
+// Tiles of 16 rows x 64 columns of the block: a thread takes 4 adjacent columns
+// of one row.  out[0..3] = sum_p Xs[r][p] Ms[p][4 c4 ..], p ascending.
+static constexpr int PCA_TROWS = 16;
+
+__device__ __forceinline__ float4 tile_product(const float (*Xs)[PCA_P + 1], const float (*Ms)[PCA_P], int r, int c4) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
+    for (int p = 0; p < PCA_P; ++p) {
+        const float x = Xs[r][p];
+        const float4 m = *reinterpret_cast<const float4*>(&Ms[p][4 * c4]);
+        s.x = fmaf(x, m.x, s.x);
+        s.y = fmaf(x, m.y, s.y);
+        s.z = fmaf(x, m.z, s.z);
+        s.w = fmaf(x, m.w, s.w);
+    }
+    return s;
+}
+
 // Locked columns: Y = X; active columns: Y[a][L + q] = sum_p X[a][p] M[p][q]
 // (M: P x m, device).
-__global__ void pca_apply_kernel(const float* __restrict__ X, int D, const float* __restrict__ M, int L,
-                                 float* __restrict__ Y) {
-    const int m = PCA_P - L;
-    const int64_t total = int64_t(D) * PCA_P;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += int64_t(gridDim.x) * blockDim.x) {
-        const int a = int(t / PCA_P), q = int(t - int64_t(a) * PCA_P);
-        if (q < L) {
-            Y[t] = X[t];
-            continue;
-        }
-        const float* Xa = X + int64_t(a) * PCA_P;
-        float s = 0.f;
-        for (int p = 0; p < PCA_P; ++p) s = fmaf(Xa[p], M[p * m + (q - L)], s);
-        Y[t] = s;
+__global__ void __launch_bounds__(256) pca_apply_kernel(const float* __restrict__ X, int D,
+                                                        const float* __restrict__ M, int L, float* __restrict__ Y) {
+    __shared__ __align__(16) float Ms[PCA_P][PCA_P];
+    __shared__ float Xs[PCA_TROWS][PCA_P + 1];
+    const int m = PCA_P - L, a0 = blockIdx.x * PCA_TROWS;
+#pragma unroll
+    for (int u = 0; u < PCA_P * PCA_P / 256; ++u) {
+        const int t = threadIdx.x + u * 256, p = t / PCA_P, q = t % PCA_P;
+        Ms[p][q] = q >= L ? M[p * m + (q - L)] : (p == q ? 1.f : 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < PCA_TROWS * PCA_P / 256; ++u) {
+        const int t = threadIdx.x + u * 256, r = t / PCA_P, p = t % PCA_P;
+        Xs[r][p] = a0 + r < D ? X[int64_t(a0 + r) * PCA_P + p] : 0.f;
+    }
+    __syncthreads();
+    const int r = threadIdx.x >> 4, c4 = threadIdx.x & 15;
+    if (a0 + r >= D) return;
+    const float4 s = tile_product(Xs, Ms, r, c4);
+    const float v[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int q = 4 * c4 + u;
+        Y[int64_t(a0 + r) * PCA_P + q] = q < L ? Xs[r][q] : v[u];
     }
 }
 
-// Mode 0 of the orthonormalisation step (the mode word is the factor
-// kernel's): Y = X T^-1 for the upper-triangular T = [I, W; 0, R]
-// (Y[:, :L] = X[:, :L], Y[:, L:] = (X[:, L:] - X[:, :L] W) R^-1), each thread
-// solving y T = x for one row by forward substitution.  Rows pass through
-// shared memory to keep global accesses coalesced.
-__global__ void __launch_bounds__(64) pca_tsolve_kernel(const float* __restrict__ X, int D,
-                                                        const float* __restrict__ T, const int* __restrict__ mode,
-                                                        float* __restrict__ Y) {
-    __shared__ float Ts[PCA_P][PCA_P];
-    __shared__ float rdiag[PCA_P];
-    __shared__ float Xs[64][PCA_P + 1];
-    const int a0 = blockIdx.x * 64;
-    const int rows = D - a0 < 64 ? D - a0 : 64;
-    if (*mode != 0) return;
-    for (int u = threadIdx.x; u < PCA_P * PCA_P; u += blockDim.x) Ts[u / PCA_P][u % PCA_P] = T[u];
-    for (int u = threadIdx.x; u < rows * PCA_P; u += blockDim.x) Xs[u / PCA_P][u % PCA_P] = X[int64_t(a0) * PCA_P + u];
-    __syncthreads();
-    if (threadIdx.x < PCA_P) rdiag[threadIdx.x] = 1.f / Ts[threadIdx.x][threadIdx.x];
-    __syncthreads();
-    if (int(threadIdx.x) < rows) {
-        float y[PCA_P];
+// The orthonormalisation step (the mode word is the factor kernel's).  Mode 0:
+// Y = X T^-1 for the upper-triangular T = [I, W; 0, R] (Y[:, :L] = X[:, :L], Y[:,
+// L:] = (X[:, L:] - X[:, :L] W) R^-1), a warp solving y T = x for one row: when y_j
+// is known, every lane subtracts y_j T[j][k] from its two columns k > j (a thread
+// per row, summing up to each column in turn, took 22 us).  Mode 1: Y = X T, T
+// general P x P.
+__global__ void __launch_bounds__(256) pca_ortho_kernel(const float* __restrict__ X, int D, const float* __restrict__ T,
+                                                        const int* __restrict__ mode, float* __restrict__ Y) {
+    __shared__ __align__(16) float Ts[PCA_P][PCA_P];
+    __shared__ float Xs[PCA_TROWS][PCA_P + 1];
+    const int a0 = blockIdx.x * PCA_TROWS, solve = *mode == 0;
 #pragma unroll
+    for (int u = 0; u < PCA_P * PCA_P / 256; ++u) {
+        const int t = threadIdx.x + u * 256;
+        Ts[t / PCA_P][t % PCA_P] = T[t];
+    }
+#pragma unroll
+    for (int u = 0; u < PCA_TROWS * PCA_P / 256; ++u) {
+        const int t = threadIdx.x + u * 256, r = t / PCA_P, p = t % PCA_P;
+        Xs[r][p] = a0 + r < D ? X[int64_t(a0 + r) * PCA_P + p] : 0.f;
+    }
+    __syncthreads();
+    if (solve) {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        const float d0 = 1.f / Ts[lane][lane], d1 = 1.f / Ts[lane + 32][lane + 32];
+        float v0[2], v1[2];  // two rows a warp
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            v0[h] = Xs[2 * w + h][lane];
+            v1[h] = Xs[2 * w + h][lane + 32];
+        }
+#pragma unroll 8
         for (int j = 0; j < PCA_P; ++j) {
-            float v = Xs[threadIdx.x][j];
+            const float t0 = Ts[j][lane], t1 = Ts[j][lane + 32];
 #pragma unroll
-            for (int i = 0; i < j; ++i) v = fmaf(-y[i], Ts[i][j], v);
-            y[j] = v * rdiag[j];
+            for (int h = 0; h < 2; ++h) {
+                const float y = j < 32 ? __shfl_sync(0xffffffffu, v0[h] * d0, j) : __shfl_sync(0xffffffffu, v1[h] * d1, j - 32);
+                if (lane > j) v0[h] = fmaf(-y, t0, v0[h]);
+                if (lane + 32 > j) v1[h] = fmaf(-y, t1, v1[h]);
+            }
         }
 #pragma unroll
-        for (int j = 0; j < PCA_P; ++j) Xs[threadIdx.x][j] = y[j];
-    }
-    __syncthreads();
-    for (int u = threadIdx.x; u < rows * PCA_P; u += blockDim.x) Y[int64_t(a0) * PCA_P + u] = Xs[u / PCA_P][u % PCA_P];
-}
-
-// Mode 1 of the orthonormalisation step: Y = X M, M general P x P, one
-// thread per output.
-__global__ void pca_mprod_kernel(const float* __restrict__ X, int D, const float* __restrict__ M,
-                                 const int* __restrict__ mode, float* __restrict__ Y) {
-    if (*mode != 1) return;
-    const int64_t total = int64_t(D) * PCA_P;
-    for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += int64_t(gridDim.x) * blockDim.x) {
-        const int a = int(t / PCA_P), q = int(t % PCA_P);
-        const float* Xa = X + int64_t(a) * PCA_P;
-        float s = 0.f;
-#pragma unroll 16
-        for (int p = 0; p < PCA_P; ++p) s = fmaf(Xa[p], M[p * PCA_P + q], s);
-        Y[t] = s;
+        for (int h = 0; h < 2; ++h) {
+            const int a = a0 + 2 * w + h;
+            if (a < D) {
+                Y[int64_t(a) * PCA_P + lane] = v0[h] * d0;
+                Y[int64_t(a) * PCA_P + lane + 32] = v1[h] * d1;
+            }
+        }
+    } else {
+        const int r = threadIdx.x >> 4, c4 = threadIdx.x & 15;
+        if (a0 + r < D) *reinterpret_cast<float4*>(Y + int64_t(a0 + r) * PCA_P + 4 * c4) = tile_product(Xs, Ts, r, c4);
     }
 }
 
@@ -412,54 +481,93 @@ __global__ void pca_start_kernel(int D, float* __restrict__ X) {
     }
 }
 
-// Z[i][k] = sum_j (X[i][j] - mu[j]) V[j][k] for k < dim: 64 x 64 output
-// tiles, 16 x 16 threads with 4 x 4 outputs each, D in steps of 32.
-__global__ void __launch_bounds__(256) pca_project_kernel(const float* __restrict__ X, const float* __restrict__ mu,
+// Z[i][k] = sum_j (X[i][j] - mu[j]) V[j][k] for k < dim, j ascending: 128 x 64
+// output tiles by 128 threads, a thread taking 8 rows (as packed pairs) x 8
+// columns, D in steps of 16; the next step's loads are in flight during this
+// one's products.  Bound: FP32 issue and shared-memory reads, about equal with
+// 8 x 8 outputs a thread (70,000 x 784: 325 us with 4 x 4).
+static constexpr int PJ_ROWS = 128, PJ_STEP = 16, PJ_PITCH = 132;
+
+__global__ void __launch_bounds__(128) pca_project_kernel(const float* __restrict__ X, const float* __restrict__ mu,
                                                           const float* __restrict__ V, int64_t n, int D, int dim,
                                                           float* __restrict__ Z) {
-    __shared__ float As[64][33];
-    __shared__ float Bs[32][65];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int64_t i0 = int64_t(blockIdx.x) * 64;
-    float acc[4][4] = {};
-    for (int j0 = 0; j0 < D; j0 += 32) {
-        for (int t = threadIdx.x; t < 64 * 32; t += 256) {
-            const int r = t / 32, cc = t % 32;
-            const int64_t i = i0 + r;
-            const int j = j0 + cc;
-            As[r][cc] = (i < n && j < D) ? X[i * D + j] - mu[j] : 0.f;
-        }
-        for (int t = threadIdx.x; t < 32 * 64; t += 256) {
-            const int r = t / 64, cc = t % 64;
-            const int j = j0 + r;
-            Bs[r][cc] = (j < D && cc < dim) ? V[int64_t(j) * PCA_P + cc] : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
-            float a[4], b[4];
+    __shared__ __align__(16) float As[2][PJ_STEP][PJ_PITCH];  // [j][row]
+    __shared__ __align__(16) float Bs[2][PJ_STEP][PCA_P];     // [j][column]
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int64_t i0 = int64_t(blockIdx.x) * PJ_ROWS;
+    const int jl = tid & 7, rl = tid >> 3;  // a warp reads 8 features of 4 rows
+    // raw loads: the mean is subtracted when they are stored, a step later, so
+    // that nothing waits for them before this step's products
+    float av[16], bv[8], mv[2];
+    auto load = [&](int j0) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = As[ty * 4 + u][kk];
-                b[u] = Bs[kk][tx * 4 + u];
+        for (int v = 0; v < 2; ++v) mv[v] = j0 + jl + 8 * v < D ? mu[j0 + jl + 8 * v] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int64_t i = i0 + rl + 16 * u;
+                const int j = j0 + jl + 8 * v;
+                av[2 * u + v] = (i < n && j < D) ? X[i * D + j] : mv[v];
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+        for (int u = 0; u < 8; ++u) {
+            const int t = tid + 128 * u, j = j0 + (t >> 6), cc = t & 63;
+            bv[u] = (j < D && cc < dim) ? V[int64_t(j) * PCA_P + cc] : 0.f;
         }
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) As[buf][jl + 8 * v][rl + 16 * u] = av[2 * u + v] - mv[v];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int t = tid + 128 * u;
+            Bs[buf][t >> 6][t & 63] = bv[u];
+        }
+    };
+    uint64_t acc[4][8];  // [row pair][column]: rows 4 ty + {0, 2}, 64 + 4 ty + {0, 2}
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) acc[u][v] = 0ull;
+    load(0);
+    store(0);
+    int buf = 0;
+    for (int j0 = 0; j0 < D; j0 += PJ_STEP, buf ^= 1) {
         __syncthreads();
-    }
+        const bool more = j0 + PJ_STEP < D;
+        if (more) load(j0 + PJ_STEP);
+#pragma unroll 4
+        for (int kk = 0; kk < PJ_STEP; ++kk) {
+            const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][4 * ty]);
+            const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&As[buf][kk][64 + 4 * ty]);
+            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][32 + 4 * tx]);
+            const uint64_t a[4] = {a0.x, a0.y, a1.x, a1.y};
+            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int64_t i = i0 + ty * 4 + u;
-        if (i >= n) continue;
+            for (int v = 0; v < 8; ++v) {
+                uint64_t bb;
+                asm("mov.b64 %0, {%1, %1};" : "=l"(bb) : "f"(b[v]));
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int k = tx * 4 + v;
-            if (k < dim) Z[i * dim + k] = acc[u][v];
+                for (int u = 0; u < 4; ++u) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[u][v]) : "l"(a[u]), "l"(bb));
+            }
         }
+        if (more) store(buf ^ 1);  // (last read before the barrier of the previous step)
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            float2 z;
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(z.x), "=f"(z.y) : "l"(acc[u][v]));
+            const int64_t i = i0 + 4 * ty + 2 * (u & 1) + 64 * (u >> 1);
+            const int k = 4 * tx + (v & 3) + 32 * (v >> 2);
+            if (k < dim && i < n) Z[i * dim + k] = z.x;
+            if (k < dim && i + 1 < n) Z[(i + 1) * dim + k] = z.y;
+        }
 }
 
 // V_out[k][j] = V[j][k] (components as rows).
@@ -480,7 +588,7 @@ static constexpr int PCA_JAC_SWEEPS = 6;
 // Pass 0, and any pass after a shifted one: S = sym(G[L:]) - W^T W (the Gram
 // of the active columns after projection off the locked ones; W is tiny, so
 // W^T W is taken in FP32), S (+ shift) = R^T R in FP64, and T = [I, W; 0, R]
-// (P x P, FP32) with mode 0 for pca_tsolve_kernel, which forms X T^-1 =
+// (P x P, FP32) with mode 0 for pca_ortho_kernel, which forms X T^-1 =
 // [X_L, (X_a - X_L W) R^-1] (Cholesky QR).  Pass 0 also requires min R_jj >
 // 1e-5 max R_jj; where the plain factor fails that or breaks down, it is
 // retaken of S + 1e-10 tr(S) I (shifted Cholesky QR, Fukaya et al. 2020),
@@ -536,26 +644,38 @@ __global__ void __launch_bounds__(PCA_CHOL_THREADS) pca_chol_kernel(const double
         }
         if (tid == 0) s_fail = 0;
         __syncthreads();
-        for (int j = 0; j < m; ++j) {
-            if (tid == 0) {  // one FP64 square root and reciprocal per column
-                double d = R[j * m + j];
-                if (!(d > 0.0)) {
-                    s_fail = 1;
-                    d = 1.0;
-                }
-                const double rjj = sqrt(d);
-                R[j * m + j] = rjj;
-                s_rinv = 1.0 / rjj;
+        // one FP64 square root and reciprocal per column, by warp 0 beside the
+        // other warps' update of the previous column (they take longer than
+        // the update: 94 us a factor when they followed it)
+        auto pivot = [&](int j) {
+            double d = R[j * m + j];
+            if (!(d > 0.0)) {
+                s_fail = 1;
+                d = 1.0;
             }
-            __syncthreads();
+            const double rjj = sqrt(d);
+            R[j * m + j] = rjj;
+            s_rinv = 1.0 / rjj;
+        };
+        if (tid == 0) pivot(0);
+        __syncthreads();
+        for (int j = 0; j < m; ++j) {
             const double rinv = s_rinv;
             for (int i = j + 1 + tid; i < m; i += nt) R[j * m + i] *= rinv;
             __syncthreads();
-            {
-                const int k = j + 1 + (tid & (PCA_P - 1));  // a column per lane group, rows by stride
+            if (tid < 32) {
+                if (tid == 0 && j + 1 < m) {
+                    const double r1 = R[j * m + j + 1];
+                    R[(j + 1) * m + j + 1] -= r1 * r1;
+                    pivot(j + 1);
+                }
+            } else if (tid < 32 + 7 * PCA_P) {
+                const int u = tid - 32;
+                const int k = j + 1 + (u & (PCA_P - 1));  // a column per lane group, rows by stride
                 if (k < m) {
                     const double rjk = R[j * m + k];
-                    for (int i = j + 1 + (tid >> 6); i <= k; i += nt >> 6) R[i * m + k] -= R[j * m + i] * rjk;
+                    for (int i = j + 1 + (u >> 6); i <= k; i += 7)
+                        if (k != j + 1) R[i * m + k] -= R[j * m + i] * rjk;
                 }
             }
             __syncthreads();
@@ -789,7 +909,7 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
     const int S = pca_splits(n_pad);
     const int64_t dpp = int64_t(D_pad) * D_pad;
     Carve cv(scratch);
-    double* part = cv.take<double>(size_t(PCA_MEAN_CHUNKS) * D);
+    double* part = cv.take<double>(size_t(PCA_MEAN_CHUNKS) * D);  // later the products' arrival counters
     float* mu = cv.take<float>(D);
     __nv_bfloat16* hi = cv.take<__nv_bfloat16>(size_t(D_pad) * n_pad);
     __nv_bfloat16* lo = cv.take<__nv_bfloat16>(size_t(D_pad) * n_pad);
@@ -818,7 +938,7 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
     DRGB_CHECK_LAUNCH(c);
     pca_mean_kernel<<<D, 256, 0, st>>>(part, chunks, n, D, mu);
     DRGB_CHECK_LAUNCH(c);
-    pca_stage_kernel<<<dim3(unsigned(n_pad / 32), unsigned(D_pad / 32)), dim3(32, 8), 0, st>>>(X, mu, n, D, n_pad,
+    pca_stage_kernel<<<dim3(unsigned(n_pad / 64), unsigned(D_pad / 32)), dim3(32, 8), 0, st>>>(X, mu, n, D, n_pad,
                                                                                            D_pad, hi, lo);
     DRGB_CHECK_LAUNCH(c);
     // covariance: hi hi^T and hi lo^T, accumulation chains of at most
@@ -852,26 +972,26 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
     } else {
         DRGB_CUDA(c, cudaFuncSetAttribute(pca_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           int(PCA_CHOL_SMEM)));
-        const int gblk = grid_for(int64_t(D) * P, 256, c->num_sms * 4);
+        const int tblk = (D + PCA_TROWS - 1) / PCA_TROWS;
+        unsigned int* counters = reinterpret_cast<unsigned int*>(part);  // one per row range of C X, then of the Gram
+        const int crows = (D + PCA_CROWS - 1) / PCA_CROWS;
+        DRGB_CUDA(c, cudaMemsetAsync(counters, 0, (size_t(crows) + P * P / 256 + 1) * sizeof(unsigned int), st));
         int L = 0;  // locked (converged and deflated) leading pairs
         const int nks = (D + PCA_KCHUNK - 1) / PCA_KCHUNK;
         auto cmul = [&](const float* A, const float* Zz, double al, double be, double ga, float* B) -> int {
-            pca_cmul_part_kernel<<<dim3((D + PCA_CROWS - 1) / PCA_CROWS, nks), 256, 0, st>>>(C, D, A, cpart);
-            DRGB_CHECK_LAUNCH(c);
-            pca_cmul_kernel<<<gblk, 256, 0, st>>>(cpart, nks, D, A, Zz, float(al), float(be), float(ga), L, B);
+            pca_cmul_kernel<<<dim3(crows, nks), 256, 0, st>>>(C, D, A, cpart, counters, Zz, float(al), float(be), float(ga),
+                                                             L, B);
             DRGB_CHECK_LAUNCH(c);
             return DRGB_OK;
         };
         auto gram = [&](const float* A, const float* B) -> int {
             const int m = P - L;
-            pca_gram_kernel<<<dim3((P * m + 255) / 256, nch), 256, 0, st>>>(A, B, D, L, Gd);
-            DRGB_CHECK_LAUNCH(c);
-            pca_gsum_kernel<<<(P * m + 255) / 256, 256, 0, st>>>(Gd, nch, P * m, Gsum);
+            pca_gram_kernel<<<dim3((P * m + 255) / 256, nch), 256, 0, st>>>(A, B, D, L, Gd, counters + crows, Gsum);
             DRGB_CHECK_LAUNCH(c);
             return DRGB_OK;
         };
         auto apply = [&](const float* A, float* B) -> int {
-            pca_apply_kernel<<<gblk, 256, 0, st>>>(A, D, Md, L, B);
+            pca_apply_kernel<<<tblk, 256, 0, st>>>(A, D, Md, L, B);
             DRGB_CHECK_LAUNCH(c);
             return DRGB_OK;
         };
@@ -883,9 +1003,7 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
                 if (r) return r;
                 pca_chol_kernel<<<1, PCA_CHOL_THREADS, PCA_CHOL_SMEM, st>>>(Gsum, L, pass, dflags, Md);
                 DRGB_CHECK_LAUNCH(c);
-                pca_tsolve_kernel<<<(D + 63) / 64, 64, 0, st>>>(A, D, Md, dflags + PCA_MODE, tmp);
-                DRGB_CHECK_LAUNCH(c);
-                pca_mprod_kernel<<<gblk, 256, 0, st>>>(A, D, Md, dflags + PCA_MODE, tmp);
+                pca_ortho_kernel<<<tblk, 256, 0, st>>>(A, D, Md, dflags + PCA_MODE, tmp);
                 DRGB_CHECK_LAUNCH(c);
                 std::swap(A, tmp);
             }
@@ -987,7 +1105,7 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
     }
     pca_sign_kernel<<<(dim * 32 + 255) / 256, 256, 0, st>>>(V, D, P, dim);
     DRGB_CHECK_LAUNCH(c);
-    pca_project_kernel<<<unsigned((n + 63) / 64), 256, 0, st>>>(X, mu, V, n, D, dim, Z);
+    pca_project_kernel<<<unsigned((n + PJ_ROWS - 1) / PJ_ROWS), 128, 0, st>>>(X, mu, V, n, D, dim, Z);
     DRGB_CHECK_LAUNCH(c);
     if (comps) {
         pca_components_kernel<<<grid_for(int64_t(D) * dim, 256, c->num_sms * 4), 256, 0, st>>>(V, D, dim, comps);
