@@ -71,10 +71,10 @@ struct ScanArgs {
     int32_t* cnt;
 };
 
-static size_t scan_smem(int d, int k) {
+static size_t scan_smem(int d, int k, bool ranks) {
     const int qd = d <= 2 * SC_DC ? d : 2 * SC_DC, kl = k <= 16 ? 16 : 32;
     return size_t(2) * SC_DC * SC_PITCH * 4 + size_t(qd) * SC_QPITCH * 8 + size_t(SC_Q) * SC_PITCH * 4 +
-           size_t(SC_Q) * kl * 8 + (SC_Q * 4);
+           size_t(SC_Q) * kl * 8 + (SC_Q * 4) + (ranks ? size_t(SC_Q) * kl * 4 : 0);
 }
 
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
@@ -86,6 +86,22 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     uint64_t r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+static constexpr int SC_RANK_FEW = 24;  // points near enough to matter up to which they are walked one by one
+static constexpr int SC_BULK = 6;  // candidates of 32 from which sorting them beats inserting them one by one
+
+// One step of a sorting network over the lanes: keep the smaller (keep_min) or
+// the larger, by (distance, index), of this lane's pair and lane ^ st's.
+__device__ __forceinline__ void cmp_swap(float& d, int32_t& i, int st, bool keep_min) {
+    const float od = __shfl_xor_sync(0xffffffffu, d, st);
+    const int32_t oi = __shfl_xor_sync(0xffffffffu, i, st);
+    const bool less = od < d || (od == d && oi < i);
+    const bool same = od == d && oi == i;
+    if (!same && less == keep_min) {
+        d = od;
+        i = oi;
+    }
 }
 
 // NEAREST: the k nearest of every query row in the chunk.  RANKS: for every
@@ -108,6 +124,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     float* s_ld = s_d + SC_Q * SC_PITCH;                                      // [SC_Q][kl] list (or target) distances
     int32_t* s_li = reinterpret_cast<int32_t*>(s_ld + SC_Q * kl);             // [SC_Q][kl] their indices
     int32_t* s_qi = s_li + SC_Q * kl;                                         // [SC_Q] point excluded (-1: none)
+    int32_t* s_cnt = s_qi + SC_Q;                                             // RANKS: [SC_Q][kl] counts
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
     const int64_t r0 = int64_t(blockIdx.x) * SC_Q;
@@ -159,6 +176,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
         const int q = t / kl, s = t - q * kl;
         if (RANK) {
             const bool in = s < k && r0 + q < n_rows;
+            s_cnt[t] = 0;
             s_ld[t] = in ? A.td[(r0 + q) * k + s] : -1.f;
             s_li[t] = in ? A.tgt[(r0 + q) * k + s] : -1;
         } else {
@@ -276,25 +294,46 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                     if (!__any_sync(0xffffffffu, v[0] <= tmax || v[1] <= tmax || v[2] <= tmax || v[3] <= tmax)) continue;
                     const int32_t jl = lane < k ? li[lane] : -1;
                     int32_t mine = 0;
-                    for (int s = 0; s < k; ++s) {
-                        const float t = __shfl_sync(0xffffffffu, tl, s);
-                        const int32_t tj = __shfl_sync(0xffffffffu, jl, s);
-                        int c = 0;
-                        if (tj < p0) {  // every point of the tile comes after the target's index
+                    unsigned near[4];
+                    int few = 0;
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) c += v[j] < t;
-                        } else if (tj >= p0 + SC_P) {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) c += v[j] <= t;
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) c += v[j] < t || (v[j] == t && gp + j < tj);
-                        }
-                        c = __reduce_add_sync(0xffffffffu, c);
-                        if (lane == s) mine = c;
+                    for (int j = 0; j < 4; ++j) {
+                        near[j] = __ballot_sync(0xffffffffu, v[j] <= tmax);
+                        few += __popc(near[j]);
                     }
-                    // the count of target s of row r0 + q
-                    if (lane < k && mine && r0 + q < n_rows) atomicAdd(&A.cnt[(r0 + q) * k + lane], mine);
+                    if (few <= SC_RANK_FEW) {
+                        // lane s compares the few points that can precede any
+                        // target with target s
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            unsigned todo = near[j];
+                            while (todo) {
+                                const int src = __ffs(todo) - 1;
+                                todo &= todo - 1;
+                                const float cd = __shfl_sync(0xffffffffu, v[j], src);
+                                mine += cd < tl || (cd == tl && int32_t(p0) + 4 * src + j < jl);
+                            }
+                        }
+                    } else {
+                        for (int s = 0; s < k; ++s) {
+                            const float t = __shfl_sync(0xffffffffu, tl, s);
+                            const int32_t tj = __shfl_sync(0xffffffffu, jl, s);
+                            int c = 0;
+                            if (tj < p0) {  // every point of the tile comes after the target's index
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) c += v[j] < t;
+                            } else if (tj >= p0 + SC_P) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) c += v[j] <= t;
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) c += v[j] < t || (v[j] == t && gp + j < tj);
+                            }
+                            c = __reduce_add_sync(0xffffffffu, c);
+                            if (lane == s) mine = c;
+                        }
+                    }
+                    if (lane < k) s_cnt[q * kl + lane] += mine;  // (the warp's own rows)
                 } else {
                     const float thr = ld[k - 1];
                     const float m = fminf(fminf(v[0], v[1]), fminf(v[2], v[3]));  // ignores the NaN marks
@@ -304,6 +343,34 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         unsigned todo = __ballot_sync(0xffffffffu, v[j] < thr);
+                        if (__popc(todo) > SC_BULK) {
+                            // many at once (a list that is still filling): sort
+                            // the 32 and keep the 32 smallest of them and the list
+                            const bool in = v[j] < thr;
+                            float cd = in ? v[j] : INFINITY;
+                            int32_t ci = in ? int32_t(p0) + 4 * lane + j : INT32_MAX;
+                            if constexpr (CELLS) {
+                                if (in) ci = A.cells.perm[ci];
+                                if (ci == s_qi[q]) {
+                                    cd = INFINITY;
+                                    ci = INT32_MAX;
+                                }
+                            }
+#pragma unroll
+                            for (int kk = 2; kk <= 32; kk <<= 1) {
+#pragma unroll
+                                for (int st = kk >> 1; st > 0; st >>= 1) cmp_swap(cd, ci, st, ((lane & kk) == 0) == ((lane & st) == 0));
+                            }
+                            const float od = __shfl_sync(0xffffffffu, cd, 31 - lane);
+                            const int32_t oi = __shfl_sync(0xffffffffu, ci, 31 - lane);
+                            if (od < D || (od == D && oi < I)) {
+                                D = od;
+                                I = oi;
+                            }
+#pragma unroll
+                            for (int st = 16; st > 0; st >>= 1) cmp_swap(D, I, st, (lane & st) == 0);
+                            todo = 0;
+                        }
                         while (todo) {
                             const int src = __ffs(todo) - 1;
                             todo &= todo - 1;
@@ -339,7 +406,14 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
         }
         __syncthreads();  // the buffer and the tile may be overwritten
     }
-    if constexpr (!RANK) {
+    if constexpr (RANK) {
+        __syncthreads();
+        for (int t = tid; t < SC_Q * k; t += SC_THREADS) {
+            const int q = t / k, s = t - q * k;
+            const int32_t c = s_cnt[q * kl + s];
+            if (r0 + q < n_rows && c) atomicAdd(&A.cnt[(r0 + q) * k + s], c);
+        }
+    } else {
         __syncthreads();
         for (int t = tid; t < SC_Q * k; t += SC_THREADS) {
             const int q = t / k, s = t - q * k;
@@ -473,7 +547,7 @@ size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
 template <int MODE>
 static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
     A.chunk = ((A.n + C - 1) / C + SC_P - 1) / SC_P * SC_P;
-    const size_t smem = scan_smem(A.d, A.k);
+    const size_t smem = scan_smem(A.d, A.k, MODE == SCAN_RANKS);
     DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     const dim3 grid(unsigned((A.n_rows + SC_Q - 1) / SC_Q), unsigned((A.n + A.chunk - 1) / A.chunk));
     scan_kernel<MODE><<<grid, SC_THREADS, smem, st>>>(A);
@@ -597,7 +671,7 @@ int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, 
     A.ub = dist_out;
     A.partial = true;
     A.cells = CellScan{rows, perm, K, cell_beg, chunk_beg, cell_cnt, cell_rows};
-    const size_t smem = scan_smem(d, k);
+    const size_t smem = scan_smem(d, k, false);
     DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<SCAN_CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     scan_kernel<SCAN_CELLS><<<dim3(unsigned((cnt + SC_Q - 1) / SC_Q), unsigned(nchunk)), SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
