@@ -202,6 +202,7 @@ int drgb_fit_transform_batched(drgb_ctx* c, const float* X_cat, const int64_t* o
             drgb_tuning_cache_lookup(c->tuning_cache.c_str(), key.c_str(), &cached_w, &cached_p) == DRGB_OK) {
             c->epoch_warps = cached_w;
             c->epoch_pipe = cached_p;
+            c->epoch_pipe_set = true;
         } else {
             float us = 0.f;
             EpochScratch es;

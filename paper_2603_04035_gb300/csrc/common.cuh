@@ -31,6 +31,7 @@ struct Ctx {
     int64_t launches = 0;         // kernels launched (host-side count)
     int epoch_warps = 8;          // warps per CTA of the epoch force kernel (tuning)
     int epoch_pipe = 1;           // epoch force kernel form: 1 pipelined, 0 flat (tuning)
+    bool epoch_pipe_set = false;  // the form was chosen (set or tuned), not the default
     std::string device_name;      // for tuning-cache keys
     std::string tuning_cache;     // JSON file of tuned settings ("" = none)
     bool profiling = false;       // record stage events in fit_transform

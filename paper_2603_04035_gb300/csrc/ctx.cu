@@ -348,6 +348,7 @@ int drgb_set_tuning(drgb_ctx* c, int32_t param, int32_t value) {
             if (value != 0 && value != 1)
                 return set_error(c, DRGB_ERR_INVALID, "epoch kernel form must be 0 (flat) or 1 (pipelined)");
             c->epoch_pipe = value;
+            c->epoch_pipe_set = true;
             return DRGB_OK;
         default:
             return set_error(c, DRGB_ERR_INVALID, "unknown tuning parameter %d", param);

@@ -1027,6 +1027,8 @@ __global__ void __launch_bounds__(LOOP_WARPS * 32, loop_ctas_per_sm(LOOP_WARPS))
     }
 }
 
+static constexpr int64_t EPOCH_FLAT_ROWS = 200000;
+
 bool epoch_warps_supported(int warps) { return warps == 4 || warps == 8; }
 
 int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool after_epoch) {
@@ -1037,7 +1039,12 @@ int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool
     EpochArgs A = A_in;
     philox_round_keys(A.k0, A.k1, A.rk);
     const bool bat = A.count > 0, n5 = A.neg == 5 && A.b > 0.f;
-    const bool pipe = c->epoch_pipe != 0;
+    // Untuned, a large single instance takes the flat form: its gathers miss L1,
+    // and 40 warps an SM hide that better than 24 with two groups each (us an
+    // epoch, pipelined / flat: 70,000 rows 19.5 / 26.6, 130,000 35.7 / 36.6,
+    // 250,000 65.4 / 60.8, a million 208.5 / 197.3, two million 396 / 380; batches of
+    // small instances 48.0 / 49.8).
+    const bool pipe = c->epoch_pipe != 0 && (c->epoch_pipe_set || bat || A.n < EPOCH_FLAT_ROWS);
     const int per_sm = epoch_warps_per_sm(pipe) / warps;
     const int fgrid = grid_for(A.win_cap, warps, c->num_sms * per_sm);
     auto go = [&](auto kernel) -> int {
@@ -1260,6 +1267,8 @@ int autotune_epoch(Ctx* c, const float2* Y, float2* Ya, float2* Yb, const int32_
     DRGB_CUDA(c, cudaEventCreate(&e0));
     DRGB_CUDA(c, cudaEventCreate(&e1));
     const int saved_pipe = c->epoch_pipe;
+    const bool saved_set = c->epoch_pipe_set;
+    c->epoch_pipe_set = true;
     int best_w = c->epoch_warps, best_p = c->epoch_pipe, rc = DRGB_OK;
     float best = 1e30f;
     const int t0 = T / 4 < T - trials ? T / 4 : (T - trials > 0 ? T - trials : 0);
@@ -1299,7 +1308,9 @@ int autotune_epoch(Ctx* c, const float2* Y, float2* Ya, float2* Yb, const int32_
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->epoch_pipe = saved_pipe;
+    c->epoch_pipe_set = saved_set;
     if (rc) return rc;
+    c->epoch_pipe_set = true;
     c->epoch_warps = best_w;
     c->epoch_pipe = best_p;
     if (best_us) *best_us = best;
