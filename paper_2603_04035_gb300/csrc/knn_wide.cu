@@ -40,7 +40,7 @@ static constexpr size_t WD_SMEM =
     1024 + size_t(WD_STAGES) * WD_STAGE + 256 + TC_QUEUE_BYTES + size_t(2) * WD_BM * TC_NQ * 4;
 static constexpr int WD_MAX_D = 1021;     // K <= 1024: the norms' split stays in FP16's range
 static constexpr int WD_MAX_SPLITS = 64;
-static constexpr int WD_STAT_BLOCKS = 256;  // row ranges of the database's column statistics
+static constexpr int WD_STAT_BLOCKS = 256;  // row ranges of the database's column statistics (at most)
 static constexpr int WD_STAT_QBLOCKS = 64;  // and of the queries'
 
 // ------------------------------------------------------------------ staging
@@ -48,11 +48,11 @@ static constexpr int WD_STAT_QBLOCKS = 64;  // and of the queries'
 // covers a range of rows, a thread per column.
 __global__ void __launch_bounds__(256) wide_stats_kernel(const float* __restrict__ X, int64_t n,
                                                          const float* __restrict__ Q, int64_t nq, int d,
-                                                         float* __restrict__ partial) {
-    const bool db = blockIdx.x < WD_STAT_BLOCKS;
+                                                         unsigned db_blocks, float* __restrict__ partial) {
+    const bool db = blockIdx.x < db_blocks;
     const float* M = db ? X : Q;
-    const int64_t rows = db ? n : nq, nb = db ? WD_STAT_BLOCKS : gridDim.x - WD_STAT_BLOCKS;
-    const int64_t b = db ? blockIdx.x : blockIdx.x - WD_STAT_BLOCKS;
+    const int64_t rows = db ? n : nq, nb = db ? db_blocks : gridDim.x - db_blocks;
+    const int64_t b = db ? blockIdx.x : blockIdx.x - db_blocks;
     const int64_t per = (rows + nb - 1) / nb, r0 = b * per, r1 = r0 + per < rows ? r0 + per : rows;
     for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < d; c += gridDim.y * blockDim.x) {
         float s = 0.f, lo = INFINITY, hi = -INFINITY;
@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(256) wide_stats_kernel(const float* __restrict
 // Column means and the largest |x - mean| (maxbits[2]); 32 columns a block,
 // eight threads a column.  Rounding is monotone, so fl(max - m) and fl(m - min)
 // bound every |fl(x - m)| of the column.
-__global__ void __launch_bounds__(256) wide_mean_kernel(const float* __restrict__ partial, int blocks, int64_t n,
-                                                        int d, float* __restrict__ mean,
+__global__ void __launch_bounds__(256) wide_mean_kernel(const float* __restrict__ partial, int blocks, int db_blocks,
+                                                        int64_t n, int d, float* __restrict__ mean,
                                                         unsigned int* __restrict__ maxbits) {
     __shared__ double s_s[8][32];
     __shared__ float s_lo[8][32], s_hi[8][32];
@@ -82,12 +82,22 @@ __global__ void __launch_bounds__(256) wide_mean_kernel(const float* __restrict_
     double s = 0.0;
     float lo = INFINITY, hi = -INFINITY;
     if (c < d)
-#pragma unroll 4
-        for (int b = g; b < blocks; b += 8) {
-            const float* p = partial + int64_t(b) * 3 * d + c;
-            if (b < WD_STAT_BLOCKS) s += double(p[0]);
-            lo = fminf(lo, p[d]);
-            hi = fmaxf(hi, p[2 * d]);
+        for (int b0 = g; b0 < blocks; b0 += 64) {  // eight blocks' loads in flight
+            float vs[8], vl[8], vh[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int b = b0 + 8 * u;
+                const float* p = partial + int64_t(b < blocks ? b : g) * 3 * d + c;
+                vs[u] = b < db_blocks ? p[0] : 0.f;
+                vl[u] = p[d];
+                vh[u] = p[2 * d];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                s += double(vs[u]);
+                lo = fminf(lo, vl[u]);
+                hi = fmaxf(hi, vh[u]);
+            }
         }
     s_s[g][threadIdx.x] = s;
     s_lo[g][threadIdx.x] = lo;
@@ -482,7 +492,9 @@ struct WideShape {
 // Splits of the database: those that leave the fewest idle CTAs in the last
 // wave, at most so many that a split has 4 tiles (its lists start empty, and
 // filling them is the dearest part).
-static WideShape wide_shape(const Ctx* c, int64_t nq, int64_t n, int d) {
+// `shared`: other searches run beside this one, so splits, each of which fills
+// lists of its own, are made only until the search has an eighth of the SMs.
+static WideShape wide_shape(const Ctx* c, int64_t nq, int64_t n, int d, bool shared = false) {
     WideShape w;
     w.K = (d + 3 + 63) / 64 * 64;
     w.kch = w.K / 64;
@@ -495,7 +507,8 @@ static WideShape wide_shape(const Ctx* c, int64_t nq, int64_t n, int d) {
     for (int s = 1; s <= WD_MAX_SPLITS && (s == 1 || w.n_tiles / s >= 4); ++s) {
         const int per = (w.n_tiles + s - 1) / s;
         const int64_t waves = (blocks * s + c->num_sms - 1) / c->num_sms;
-        const double cost = double(waves) * (per + 6.0);  // a CTA's start costs about 6 tiles
+        // a CTA's start costs about 6 tiles
+        const double cost = shared ? (blocks * s * 8 < c->num_sms ? 1e9 - s : double(s)) : double(waves) * (per + 6.0);
         if (cost < best * 0.98) {
             best = cost;
             pick = s;
@@ -529,7 +542,7 @@ bool knn_wide_preferred(int64_t nq, int64_t n, int d, int k) {
 int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n, int d,
              int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* scratch, int32_t* defer_rows,
              int32_t* defer_count) {
-    const WideShape w = wide_shape(c, nq, n, d);
+    const WideShape w = wide_shape(c, nq, n, d, defer_rows != nullptr);
     Carve cv(scratch);
     float* partial = cv.take<float>(size_t(WD_STAT_BLOCKS + WD_STAT_QBLOCKS) * 3 * d);
     float* mean = cv.take<float>(d);
@@ -549,10 +562,11 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     if ((rc = stage_mark(c, 8, st))) return rc;
     DRGB_CUDA(c, cudaMemsetAsync(maxbits, 0, 64, st));
     DRGB_CUDA(c, cudaMemsetAsync(fail_count, 0, 64, st));
-    const int blocks = WD_STAT_BLOCKS + (separate ? WD_STAT_QBLOCKS : 0);
-    wide_stats_kernel<<<dim3(blocks, (d + 255) / 256), 256, 0, st>>>(X, n, Q, nq, d, partial);
+    const int db_blocks = grid_for(n, 32, WD_STAT_BLOCKS);
+    const int blocks = db_blocks + (separate ? grid_for(nq, 32, WD_STAT_QBLOCKS) : 0);
+    wide_stats_kernel<<<dim3(blocks, (d + 255) / 256), 256, 0, st>>>(X, n, Q, nq, d, db_blocks, partial);
     DRGB_CHECK_LAUNCH(c);
-    wide_mean_kernel<<<(d + 31) / 32, dim3(32, 8), 0, st>>>(partial, blocks, n, d, mean, maxbits);
+    wide_mean_kernel<<<(d + 31) / 32, dim3(32, 8), 0, st>>>(partial, blocks, db_blocks, n, d, mean, maxbits);
     DRGB_CHECK_LAUNCH(c);
     wide_stage_kernel<false><<<grid_for(w.n_pad, 8, c->num_sms * 8), 256, 0, st>>>(X, nullptr, n, w.n_pad, d, w.K, mean,
                                                                                   maxbits, XB, nullptr, nullptr);
