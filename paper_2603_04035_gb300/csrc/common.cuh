@@ -167,6 +167,12 @@ __device__ __forceinline__ int64_t mulshift_index(uint32_t u, int64_t n) {
 }
 
 // ------------------------------------------------------------------ launch helpers
+// Programmatic dependent launch: wait until the grids that this one depends on
+// have completed and their writes are visible; let the next grid be scheduled.
+// Without a programmatic dependency both are no-ops.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 inline int grid_for(int64_t work, int per_block, int max_blocks) {
     int64_t g = (work + per_block - 1) / per_block;
     if (g < 1) g = 1;

@@ -421,9 +421,7 @@ int epoch_prepare(Ctx* c, const int32_t* rp, int64_t n, int64_t row_begin, int64
 // may start while that one finishes.  Everything before grid_dep_wait() reads
 // only the CSR and the prepared tables (which no epoch writes); Y is read and
 // written only after it, when the previous epoch's grid has completed and its
-// writes are visible.  Without a programmatic dependency both are no-ops.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// writes are visible.
 
 // CSR chunks (of 32 entries) a warp loads at once before testing them.  The
 // window's CSR words are streamed in bursts so that several loads are in

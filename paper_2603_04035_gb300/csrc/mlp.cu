@@ -16,6 +16,7 @@
 // rows per edge, M = B R rows):
 //   sample     edges proportional to w (integer rejection on q) + negatives
 //   gather     X rows -> Xb (M x 64) and Xb^T (64 x M), BF16
+//              (both for the next step, beside this step's backward pass)
 //   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16, H1 also
 //              transposed) ; GELU'(pre_l) (FP32, blocked)
 //   head       z = H2 W3^T + b3 ; loss and dL/dz per edge
@@ -31,6 +32,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <vector>
 
 #include "common.cuh"
@@ -96,6 +98,16 @@ struct GemmSmem {
 };
 static constexpr int G_PITCH = 36;  // floats per row of a warp's 32 x 32 transposing tile (16-byte rows)
 
+// The kernels of a training step are launched with programmatic dependencies:
+// each is scheduled while the one before drains and then waits here, before its
+// first access to memory that another writes.  Only then may the next one
+// start, so at most two kernels of the chain are resident.  (A step of 4096
+// edges: 144 to 136 us.)
+__device__ __forceinline__ void step_dep() {
+    grid_dep_wait();
+    grid_dep_launch();
+}
+
 template <int BN, int EPI>
 __global__ void __launch_bounds__(G_THREADS, 2)
 mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs G) {
@@ -134,12 +146,13 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (EPI == EPI_GELU && threadIdx.x >= 64 && threadIdx.x < 64 + BN) s_bias[threadIdx.x - 64] = G.bias[n0 + threadIdx.x - 64];
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    step_dep();
+    if (EPI == EPI_GELU && threadIdx.x >= 64 && threadIdx.x < 64 + BN) s_bias[threadIdx.x - 64] = G.bias[n0 + threadIdx.x - 64];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -330,18 +343,34 @@ static int gemm_prepare(Ctx* c) {
     return DRGB_OK;
 }
 
-template <int BN, int EPI>
-static int gemm_launch_t(Ctx* c, const Gemm& G, cudaStream_t st) {
-    mlp_gemm_kernel<BN, EPI><<<G.grid, G_THREADS, GemmSmem<BN>::TOTAL, st>>>(G.a, G.b, G.g);
-    DRGB_CHECK_LAUNCH(c);
+// Launch with (dep) or without a programmatic dependency on the kernel before.
+template <class... P, class... A>
+static int launch_step(Ctx* c, void (*kernel)(P...), dim3 grid, int block, size_t smem, bool dep, cudaStream_t st,
+                       const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dep ? 1 : 0;
+    DRGB_CUDA(c, cudaLaunchKernelEx(&cfg, kernel, P(args)...));
     return DRGB_OK;
 }
 
-static int gemm_launch(Ctx* c, const Gemm& G, cudaStream_t st) {
-    if (G.bn == 128 && G.epi == EPI_GELU) return gemm_launch_t<128, EPI_GELU>(c, G, st);
-    if (G.bn == 128 && G.epi == EPI_GELU_GRAD) return gemm_launch_t<128, EPI_GELU_GRAD>(c, G, st);
-    if (G.bn == 128 && G.epi == EPI_F32) return gemm_launch_t<128, EPI_F32>(c, G, st);
-    if (G.bn == 64 && G.epi == EPI_F32) return gemm_launch_t<64, EPI_F32>(c, G, st);
+template <int BN, int EPI>
+static int gemm_launch_t(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
+    return launch_step(c, mlp_gemm_kernel<BN, EPI>, G.grid, G_THREADS, GemmSmem<BN>::TOTAL, dep, st, G.a, G.b, G.g);
+}
+
+static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
+    if (G.bn == 128 && G.epi == EPI_GELU) return gemm_launch_t<128, EPI_GELU>(c, G, dep, st);
+    if (G.bn == 128 && G.epi == EPI_GELU_GRAD) return gemm_launch_t<128, EPI_GELU_GRAD>(c, G, dep, st);
+    if (G.bn == 128 && G.epi == EPI_F32) return gemm_launch_t<128, EPI_F32>(c, G, dep, st);
+    if (G.bn == 64 && G.epi == EPI_F32) return gemm_launch_t<64, EPI_F32>(c, G, dep, st);
     return set_error(c, DRGB_ERR_INVALID, "mlp gemm: unsupported tile");
 }
 
@@ -356,7 +385,7 @@ int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, in
     G.g.out_f32 = partials;
     if ((rc = bn == 128 ? gemm_attr<128, EPI_F32>(c) : gemm_attr<64, EPI_F32>(c))) return rc;
     if (splits_used) *splits_used = int(G.grid.z);
-    return gemm_launch(c, G, st);
+    return gemm_launch(c, G, false, st);
 }
 
 // ------------------------------------------------------------------ SIMT kernels
@@ -388,12 +417,13 @@ __global__ void mlp_cast_kernel(const float* __restrict__ P, MlpWeights W) {
 
 // Edge sampling proportional to w: try uniform entries e, accept when the
 // next 24 random bits fall below q_e = round(2^24 w_e); 64 tries at most.
+// Draws the batch of step *step_dev + 1.
 __global__ void mlp_sample_kernel(const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                                   const uint32_t* __restrict__ q, int64_t n, int64_t nnz, int B, int neg,
                                   const uint32_t* __restrict__ step_dev, uint32_t k0, uint32_t k1,
                                   const int32_t* __restrict__ row_of, int32_t* __restrict__ rows) {
     const int R = 2 + neg;
-    const uint32_t step = *step_dev;
+    const uint32_t step = *step_dev + 1;
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < B; s += gridDim.x * blockDim.x) {
         uint32_t e = 0;
         for (uint32_t r = 0; r < 64; ++r) {
@@ -431,11 +461,15 @@ __global__ void mlp_heads_kernel(const int32_t* __restrict__ rp, int64_t n, int6
     }
 }
 
-// Gather BF16 rows (zero-padded to 64 columns) and their transpose.
+// Gather BF16 rows (zero-padded to 64 columns) and their transpose; with
+// `kept` the row numbers are copied there.
 __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int32_t* __restrict__ rows, int M,
-                                  int M_valid, bf16* __restrict__ Xb, bf16* __restrict__ Xbt) {
+                                  int M_valid, bf16* __restrict__ Xb, bf16* __restrict__ Xbt,
+                                  int32_t* __restrict__ kept) {
     __shared__ bf16 tile[32][33];
     const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+    if (kept && c0 == 0 && threadIdx.y == 0 && r0 + int(threadIdx.x) < M_valid)
+        kept[r0 + threadIdx.x] = rows[r0 + threadIdx.x];
     for (int ty = threadIdx.y; ty < 32; ty += blockDim.y) {
         const int r = r0 + ty, cc = c0 + threadIdx.x;
         float v = 0.f;
@@ -453,11 +487,15 @@ __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int3
 }
 
 // z = H2 W3^T + b3: one warp per row, lanes on columns lane + 32 i; four rows'
-// loads are in flight together.
+// loads are in flight together.  Advances the step counter, which is at the
+// step before until here.
 static constexpr int HEAD_ROWS = 4;
 
 __global__ void __launch_bounds__(256) mlp_head_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
-                                                       const float* __restrict__ P, int M, float* __restrict__ z) {
+                                                       const float* __restrict__ P, int M, float* __restrict__ z,
+                                                       uint32_t* __restrict__ step_dev) {
+    step_dep();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;
     const int lane = threadIdx.x & 31;
     float w0[MLP_H / 32], w1[MLP_H / 32];
 #pragma unroll
@@ -501,6 +539,7 @@ __global__ void __launch_bounds__(256) mlp_head_kernel(const bf16* __restrict__ 
 // gradient where clamped); loss and dL/dz are divided by the batch size.
 __global__ void mlp_loss_kernel(const float* __restrict__ z, const int32_t* __restrict__ rows, int B, int neg,
                                 float a, float b, float* __restrict__ dz, float* __restrict__ loss_part) {
+    step_dep();
     const int R = 2 + neg;
     const float lo = 1e-4f, hi = 1.0f - 1e-4f, invB = 1.0f / float(B);
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < B; s += gridDim.x * blockDim.x) {
@@ -564,6 +603,7 @@ mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, c
     float2* s_z = reinterpret_cast<float2*>(s_h + MLP_CHUNK * 32);  // [MLP_CHUNK]: dz
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
     const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
+    step_dep();
     for (int t = tid; t < rows * 4; t += MC_THREADS) {
         const int r = t >> 2, i = t & 3;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s_h + r * 32 + 8 * i)),
@@ -630,6 +670,7 @@ mlp_colsum_kernel(const float* __restrict__ A, int M, float* __restrict__ part) 
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
     const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
+    step_dep();
     for (int r = tid; r < rows; r += MC_THREADS) {
         const float* p = A + blocked_at(r0 + r, c0, MLP_H);
 #pragma unroll
@@ -667,12 +708,12 @@ struct GradParts {
 template <class F>
 __device__ __forceinline__ float sum_splits(int count, F&& at) {
     float s = 0.f;
-    for (int z0 = 0; z0 < count; z0 += 8) {  // eight loads in flight, added in order
-        float v[8];
+    for (int z0 = 0; z0 < count; z0 += 32) {  // 32 loads in flight, added in order
+        float v[32];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = z0 + u < count ? at(z0 + u) : 0.f;
+        for (int u = 0; u < 32; ++u) v[u] = z0 + u < count ? at(z0 + u) : 0.f;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < 32; ++u)
             if (z0 + u < count) s += v[u];
     }
     return s;
@@ -708,8 +749,9 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(GradParts g, AdamArgs A
         else if (p < OFF_B2) s = sum_splits(g.s2, [&](int z) { return g.dW2[int64_t(z) * MLP_H * MLP_H + (p - OFF_W2)]; });
         else if (p < OFF_W3) s = sum_splits(g.n2, [&](int z) { return g.db2[int64_t(z) * MLP_H + (p - OFF_B2)]; });
         else s = sum_splits(g.n3, [&](int z) { return g.w3[int64_t(z) * (2 * MLP_H + 2) + (p - OFF_W3)]; });
-        grad[p] = s;
-        if (ADAM) {
+        if (!ADAM) {
+            grad[p] = s;
+        } else {
             const float mm = A.b1 * A.m[p] + (1.0f - A.b1) * s;
             const float vv = A.b2 * A.v[p] + (1.0f - A.b2) * s * s;
             A.m[p] = mm;
@@ -720,10 +762,11 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(GradParts g, AdamArgs A
             mlp_cast_one(w, p, A.W);
         }
     }
-    if (blockIdx.x == 0 && loss_out) {
+    if (blockIdx.x == gridDim.x - 1 && loss_out) {  // (a block without parameters)
         __shared__ float red[256];
         float s = 0.f;
-        for (int t = threadIdx.x; t < g.B; t += blockDim.x) s += g.loss[t];
+#pragma unroll 16
+        for (int t = threadIdx.x; t < g.B; t += 256) s += g.loss[t];
         red[threadIdx.x] = s;
         __syncthreads();
         for (int o = blockDim.x / 2; o > 0; o >>= 1) {
@@ -733,8 +776,6 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(GradParts g, AdamArgs A
         if (threadIdx.x == 0) loss_out[step] = red[0];
     }
 }
-
-__global__ void mlp_step_advance_kernel(uint32_t* step_dev) { *step_dev += 1; }
 
 // Initial weights: U(-1/sqrt(fan_in), 1/sqrt(fan_in)) from Philox, biases 0,
 // columns of W1 beyond d exactly 0.
@@ -1065,12 +1106,32 @@ static MlpBuffers mlp_carve(void* base, int M) {
     return b;
 }
 
-// A second branch of the step: with a stream, work forks off `st` and joins
-// it again through the events; without one it runs in line.
+// Further branches of a training step: dW2 beside dH1 and what follows from
+// it, and the next step's batch.  The batch does not depend on the weights: its
+// rows are drawn beside the backward pass, into the space of z (read last by
+// the losses), and gathered beside the update, when dW1 has read this step's
+// Xb.  In line the two took 27 us of a step (dependent loads from memory, under
+// one warp an SM): a step of 4096 edges went from 160 to 144 us, one of 512
+// from 74 to 58.
+// Without the streams everything runs in line and no batch is prepared.
 struct MlpFork {
-    cudaStream_t side = nullptr;
-    cudaEvent_t forked = nullptr, joined = nullptr;
+    cudaStream_t side = nullptr, ahead = nullptr;
+    cudaEvent_t ev[5] = {};
+    std::function<int(cudaStream_t)> draw, gather;
 };
+
+// `to` continues after what `from` holds so far.
+static int mlp_order(Ctx* c, cudaEvent_t ev, cudaStream_t from, cudaStream_t to) {
+    DRGB_CUDA(c, cudaEventRecord(ev, from));
+    DRGB_CUDA(c, cudaStreamWaitEvent(to, ev, 0));
+    return DRGB_OK;
+}
+
+// Padding rows carry no gradient (their part of dz is written by nothing else).
+static int mlp_zero_padding(Ctx* c, const MlpBuffers& b, int rows, cudaStream_t st) {
+    if (b.M > rows) DRGB_CUDA(c, cudaMemsetAsync(b.dz + 2 * int64_t(rows), 0, size_t(b.M - rows) * 2 * 4, st));
+    return DRGB_OK;
+}
 
 // Forward + backward of the batch whose rows are already gathered (Xb, Xbt)
 // with B edges of R rows; leaves the gradient in b.grad and the loss in
@@ -1089,40 +1150,36 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     F2.g.bias = P + OFF_B2;
     F2.g.dgelu = b.dg2;
     F2.g.out = b.H2b;
-    if ((rc = gemm_launch(c, F1, st))) return rc;
-    if ((rc = gemm_launch(c, F2, st))) return rc;
-    mlp_head_kernel<<<grid_for(M / HEAD_ROWS, 8, c->num_sms * 8), 256, 0, st>>>(b.H2b, b.W.W3f, P, M, b.z);
-    DRGB_CHECK_LAUNCH(c);
-    if (M > B * (2 + neg))  // padding rows carry no gradient
-        DRGB_CUDA(c, cudaMemsetAsync(b.dz + 2 * int64_t(B) * (2 + neg), 0,
-                                     (size_t(M) - size_t(B) * (2 + neg)) * 2 * 4, st));
-    mlp_loss_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, st>>>(b.z, b.rows, B, neg, a, bb, b.dz, b.loss_part);
-    DRGB_CHECK_LAUNCH(c);
+    if ((rc = gemm_launch(c, F1, false, st)) || (rc = gemm_launch(c, F2, true, st)) ||
+        (rc = launch_step(c, mlp_head_kernel, dim3(grid_for(M / HEAD_ROWS, 8, c->num_sms * 8)), 256, 0, true, st, b.H2b,
+                          b.W.W3f, P, M, b.z, b.step)) ||
+        (rc = launch_step(c, mlp_loss_kernel, dim3(grid_for(B, 32, c->num_sms * 8)), 32, 0, true, st, b.z, b.rows, B, neg,
+                          a, bb, b.dz, b.loss_part)))
+        return rc;
+    if (fork.ahead && ((rc = mlp_order(c, fork.ev[0], st, fork.ahead)) || (rc = fork.draw(fork.ahead)))) return rc;
     const dim3 cgrid(b.n_chunks, MLP_H / 32);
-    mlp_l3back_kernel<<<cgrid, MC_THREADS, L3_SMEM, st>>>(b.dz, b.W.W3f, b.dg2, b.H2b, M, b.D2b, b.D2bt, b.pb2, b.pw3);
-    DRGB_CHECK_LAUNCH(c);
-    // dW2 = dpre2^T H1 (K = M, split), beside dH1 and what follows from it
-    if (fork.side) {
-        DRGB_CUDA(c, cudaEventRecord(fork.forked, st));
-        DRGB_CUDA(c, cudaStreamWaitEvent(fork.side, fork.forked, 0));
-    }
+    if ((rc = launch_step(c, mlp_l3back_kernel, cgrid, MC_THREADS, L3_SMEM, true, st, b.dz, b.W.W3f, b.dg2, b.H2b, M,
+                          b.D2b, b.D2bt, b.pb2, b.pw3)))
+        return rc;
+    // dW2 = dpre2^T H1 (K = M, split)
+    if (fork.side && (rc = mlp_order(c, fork.ev[1], st, fork.side))) return rc;
     if ((rc = gemm_setup(c, DW2, b.D2bt, b.H1bt, MLP_H, MLP_H, M, 128, EPI_F32, MLP_SPLITS))) return rc;
     DW2.g.out_f32 = b.pW2;
-    if ((rc = gemm_launch(c, DW2, fork.side ? fork.side : st))) return rc;
-    if (fork.side) DRGB_CUDA(c, cudaEventRecord(fork.joined, fork.side));
+    if ((rc = gemm_launch(c, DW2, false, fork.side ? fork.side : st))) return rc;
     // dpre1 = (dpre2 W2) . GELU'(pre1): A = dpre2 [M x 256(out)], B = W2^T [256(in) x 256(out)]
     if ((rc = gemm_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H, MLP_H, 128, EPI_GELU_GRAD, 1))) return rc;
     DH1.g.dgelu = b.dg1;
     DH1.g.out_t = b.D1bt;
     DH1.g.out_f32 = b.D1f;
-    if ((rc = gemm_launch(c, DH1, st))) return rc;
-    mlp_colsum_kernel<<<cgrid, MC_THREADS, CS_SMEM, st>>>(b.D1f, M, b.pb1);
-    DRGB_CHECK_LAUNCH(c);
+    if ((rc = gemm_launch(c, DH1, fork.side != nullptr, st)) ||
+        (rc = launch_step(c, mlp_colsum_kernel, cgrid, MC_THREADS, CS_SMEM, true, st, b.D1f, M, b.pb1)))
+        return rc;
     // dW1 = dpre1^T Xb: A = dpre1^T [256 x M], B = Xb^T [64 x M]
     if ((rc = gemm_setup(c, DW1, b.D1bt, b.Xbt, MLP_H, MLP_IN, M, 64, EPI_F32, MLP_SPLITS))) return rc;
     DW1.g.out_f32 = b.pW1;
-    if ((rc = gemm_launch(c, DW1, st))) return rc;
-    if (fork.side) DRGB_CUDA(c, cudaStreamWaitEvent(st, fork.joined, 0));
+    if ((rc = gemm_launch(c, DW1, true, st))) return rc;
+    if (fork.ahead && ((rc = mlp_order(c, fork.ev[2], st, fork.ahead)) || (rc = fork.gather(fork.ahead)))) return rc;
+    if (fork.side && (rc = mlp_order(c, fork.ev[3], fork.side, st))) return rc;
     GradParts gp;
     gp.dW1 = b.pW1;
     gp.s1 = int(DW1.grid.z);
@@ -1136,10 +1193,11 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     gp.n3 = b.n_chunks;
     gp.loss = b.loss_part;
     gp.B = B;
-    const int ugrid = grid_for(MLP_P, 256, c->num_sms * 4);
+    const int ugrid = int((MLP_P + 255) / 256) + 1;  // the last block adds the losses
     if (adam) mlp_update_kernel<true><<<ugrid, 256, 0, st>>>(gp, *adam, b.grad, loss_out, b.step);
     else mlp_update_kernel<false><<<ugrid, 256, 0, st>>>(gp, AdamArgs{}, b.grad, loss_out, b.step);
     DRGB_CHECK_LAUNCH(c);
+    if (fork.ahead && (rc = mlp_order(c, fork.ev[4], fork.ahead, st))) return rc;
     return DRGB_OK;
 }
 
@@ -1183,10 +1241,11 @@ int drgb_mlp_grad(drgb_ctx* c, const float* params, const float* X, int64_t n, i
     MlpBuffers bu = mlp_carve(c->scratch, M);
     DRGB_CUDA(c, cudaMemsetAsync(bu.rows, 0, size_t(M) * 4, st));
     DRGB_CUDA(c, cudaMemcpyAsync(bu.rows, rows, size_t(Mv) * 4, cudaMemcpyDeviceToDevice, st));
-    DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0, 64, st));
+    DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0xFF, 64, st));  // (the step before the first)
+    if ((rc = mlp_zero_padding(c, bu, Mv, st))) return rc;
     mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, bu.W);
     DRGB_CHECK_LAUNCH(c);
-    mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, st>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt);
+    mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, st>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt, nullptr);
     DRGB_CHECK_LAUNCH(c);
     if ((rc = mlp_fwd_bwd(c, bu, params, n_edges, neg, a, b, loss_out, nullptr, MlpFork{}, st))) return rc;
     DRGB_CUDA(c, cudaMemcpyAsync(grad_out, bu.grad, MLP_P * 4, cudaMemcpyDeviceToDevice, st));
@@ -1213,7 +1272,8 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
     MlpBuffers bu = mlp_carve(c->scratch, M);
     int32_t* row_of = bytes > least ? reinterpret_cast<int32_t*>(static_cast<char*>(c->scratch) + Carve::round(least)) : nullptr;
     DRGB_CUDA(c, cudaMemsetAsync(bu.rows, 0, size_t(M) * 4, st));
-    DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0, 64, st));
+    DRGB_CUDA(c, cudaMemsetAsync(bu.step, 0xFF, 64, st));  // (the step before the first)
+    if ((rc = mlp_zero_padding(c, bu, Mv, st))) return rc;
     if (row_of) {
         DRGB_CUDA(c, cudaMemsetAsync(row_of, 0xFF, size_t(nnz) * 4, st));
         mlp_heads_kernel<<<grid_for(n, 256, c->num_sms * 8), 256, 0, st>>>(row_ptr, n, nnz, row_of);
@@ -1223,40 +1283,47 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
     DRGB_CHECK_LAUNCH(c);
     const uint32_t k0 = uint32_t(mp->seed), k1 = uint32_t(mp->seed >> 32);
 
+    MlpFork fork;
+    int32_t* const next_rows = reinterpret_cast<int32_t*>(bu.z);
+    fork.draw = [&](cudaStream_t s) -> int {
+        mlp_sample_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, s>>>(row_ptr, col, q, n, nnz, B, neg, bu.step, k0,
+                                                                        k1, row_of, next_rows);
+        DRGB_CHECK_LAUNCH(c);
+        return DRGB_OK;
+    };
+    fork.gather = [&](cudaStream_t s) -> int {
+        mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, s>>>(X, d, next_rows, M, Mv, bu.Xb, bu.Xbt, bu.rows);
+        DRGB_CHECK_LAUNCH(c);
+        return DRGB_OK;
+    };
+    if (mp->steps > 0 && ((rc = fork.draw(st)) || (rc = fork.gather(st)))) return rc;
+
     // capture one step, replay it mp->steps times (the step counter lives on
     // the device, so every replay draws a fresh batch)
     cudaStream_t cap = nullptr;
-    MlpFork fork;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     auto release = [&]() {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
-        if (fork.forked) cudaEventDestroy(fork.forked);
-        if (fork.joined) cudaEventDestroy(fork.joined);
+        for (cudaEvent_t ev : fork.ev)
+            if (ev) cudaEventDestroy(ev);
         if (fork.side) cudaStreamDestroy(fork.side);
+        if (fork.ahead) cudaStreamDestroy(fork.ahead);
         if (cap) cudaStreamDestroy(cap);
     };
     cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&fork.side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork.forked, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork.joined, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&fork.ahead, cudaStreamNonBlocking);
+    for (cudaEvent_t& ev : fork.ev)
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) {
         release();
         return set_error(c, DRGB_ERR_CUDA, "mlp_train: begin capture: %s", cudaGetErrorString(e));
     }
     const AdamArgs adam{params, adam_m, adam_v, mp->lr, mp->beta1, mp->beta2, mp->eps, bu.W};
-    do {
-        mlp_sample_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, cap>>>(row_ptr, col, q, n, nnz, B, neg, bu.step,
-                                                                          k0, k1, row_of, bu.rows);
-        if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
-        mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, cap>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt);
-        if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
-        if ((rc = mlp_fwd_bwd(c, bu, params, B, neg, a, b, losses, &adam, fork, cap))) break;
-        mlp_step_advance_kernel<<<1, 1, 0, cap>>>(bu.step);
-        if ((rc = [&]() { DRGB_CHECK_LAUNCH(c); return DRGB_OK; }())) break;
-    } while (0);
+    rc = mlp_fwd_bwd(c, bu, params, B, neg, a, b, losses, &adam, fork, cap);
     e = cudaStreamEndCapture(cap, &graph);
     if (rc == DRGB_OK && e != cudaSuccess) rc = set_error(c, DRGB_ERR_CUDA, "mlp_train: end capture: %s", cudaGetErrorString(e));
     if (rc == DRGB_OK && (e = cudaGraphInstantiate(&exec, graph, 0)) != cudaSuccess)
@@ -1280,7 +1347,8 @@ int drgb_mlp_sample(drgb_ctx* c, const int32_t* row_ptr, const int32_t* col, con
     int rc = ensure_scratch(c, 256, st);
     if (rc) return rc;
     uint32_t* step_dev = static_cast<uint32_t*>(c->scratch);
-    DRGB_CUDA(c, cudaMemcpyAsync(step_dev, &step, 4, cudaMemcpyHostToDevice, st));
+    const uint32_t before = step - 1;
+    DRGB_CUDA(c, cudaMemcpyAsync(step_dev, &before, 4, cudaMemcpyHostToDevice, st));
     mlp_sample_kernel<<<grid_for(n_edges, 128, c->num_sms * 8), 128, 0, st>>>(row_ptr, col, q, n, nnz, n_edges, neg,
                                                                              step_dev, uint32_t(seed),
                                                                              uint32_t(seed >> 32), nullptr, rows);
