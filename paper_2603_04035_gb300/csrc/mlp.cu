@@ -5,20 +5,22 @@
 // fuzzy graph, then used to embed new points.
 //
 // Every dense product runs on the tcgen05 tensor cores through one kernel,
-// mlp_gemm_kernel: C[M x N] = A[M x K] * B[N x K]^T with both operands K-major
-// BF16 (TMA, 128-byte swizzle), FP32 accumulation in TMEM, and a fused
-// epilogue: bias + GELU (forward), GELU derivative (backward) or plain FP32
-// (weight gradients, split over K).  Activations are also written transposed,
-// so the weight-gradient products are K-major as well.  The 256 -> 2 layer,
-// the loss, the reductions and Adam are small SIMT kernels.
+// mlp_gemm_kernel: C[M x N] = A[M x K] * B[N x K]^T with BF16 operands (TMA,
+// 128-byte swizzle), FP32 accumulation in TMEM, and a fused epilogue: bias +
+// GELU (forward), GELU derivative (backward) or plain FP32 (weight gradients,
+// split over K).  The weight gradients sum over the batch's rows: they take the
+// activations as they lie, MN-major (with transposed copies for K-major
+// operands, written by two GEMM epilogues, the layer 3 kernel and the gather, a
+// step of 4096 edges took 136 us against 125).  The 256 -> 2 layer, the loss,
+// the reductions and Adam are small SIMT kernels.
 //
 // One training step (batch of B edges, each with `neg` negatives, R = 2 + neg
 // rows per edge, M = B R rows):
 //   sample     edges proportional to w (integer rejection on q) + negatives
-//   gather     X rows -> Xb (M x 64) and Xb^T (64 x M), BF16
+//   gather     X rows -> Xb (M x 64), BF16
 //              (both for the next step, beside this step's backward pass)
-//   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16, H1 also
-//              transposed) ; GELU'(pre_l) (FP32, blocked)
+//   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16) ;
+//              GELU'(pre_l) (FP32, blocked)
 //   head       z = H2 W3^T + b3 ; loss and dL/dz per edge
 //   L3 back    dpre2 = (dz W3) . GELU'(pre2) ; dW3, db3, db2 partial sums
 //   dW2        dpre2^T H1     (split-K, FP32 partials; beside dH1 and dW1)
@@ -84,7 +86,6 @@ struct GemmArgs {
     const float* bias;    // EPI_GELU: [N]
     float* dgelu;         // GELU'(pre), blocked: EPI_GELU out (nullable), EPI_GELU_GRAD in
     bf16* out;            // [M][N] (nullable)
-    bf16* out_t;          // [N][M] transposed (nullable)
     float* out_f32;       // EPI_F32: [splits][M][N]; EPI_GELU_GRAD: blocked FP32 copy (nullable)
     int* status;
 };
@@ -108,11 +109,14 @@ __device__ __forceinline__ void step_dep() {
     grid_dep_launch();
 }
 
-template <int BN, int EPI>
+// With KROWS the operands are stored K rows x M (N) columns, as activations of a
+// batch are for a product over its rows, and staged as boxes of 64 x 64.
+template <int BN, int EPI, bool KROWS>
 __global__ void __launch_bounds__(G_THREADS, 2)
 mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs G) {
     using SM = GemmSmem<BN>;
     constexpr int STAGES = SM::STAGES;
+    constexpr int BOX = 64 * 64 * 2;
     static_assert(STAGES * (SM::A_BYTES + SM::B_BYTES) >= G_EPI_WARPS * 32 * G_PITCH * 4, "epilogue tiles fit the ring");
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned (swizzled operand tiles); an offset from the shared
@@ -165,8 +169,17 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int s = kb % STAGES;
                 if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) & 1) ^ 1, abort_flag, G.status)) break;
                 mbar_expect_tx(&full[s], SM::A_BYTES + SM::B_BYTES);
-                tma_load_2d(sA + s * SM::A_BYTES, &tmA, (kb0 + kb) * 64, m0, &full[s]);
-                tma_load_2d(sB + s * SM::B_BYTES, &tmB, (kb0 + kb) * 64, n0, &full[s]);
+                if (KROWS) {
+#pragma unroll
+                    for (int j = 0; j < G_BM / 64; ++j)
+                        tma_load_2d(sA + s * SM::A_BYTES + j * BOX, &tmA, m0 + 64 * j, (kb0 + kb) * 64, &full[s]);
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j)
+                        tma_load_2d(sB + s * SM::B_BYTES + j * BOX, &tmB, n0 + 64 * j, (kb0 + kb) * 64, &full[s]);
+                } else {
+                    tma_load_2d(sA + s * SM::A_BYTES, &tmA, (kb0 + kb) * 64, m0, &full[s]);
+                    tma_load_2d(sB + s * SM::B_BYTES, &tmB, (kb0 + kb) * 64, n0, &full[s]);
+                }
             }
             if (kb < nkb) {  // aborted: let issued loads land before exit
                 for (int u = (kb > STAGES ? kb - STAGES : 0); u < kb; ++u) {
@@ -178,15 +191,18 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16kind(G_BM, BN, false);
+            const uint32_t idesc = idesc_f16kind(G_BM, BN, false) | (KROWS ? IDESC_MN_MAJOR : 0u);
+            constexpr int KSTEP = KROWS ? 2048 / 16 : 32 / 16;  // 16 of K, in descriptor units
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
                 if (!mbar_wait(&full[s], (kb / STAGES) & 1, abort_flag, G.status)) break;
                 tc_fence_after();
-                const uint64_t ad = sdesc_sw128(smem_u32(sA + s * SM::A_BYTES));
-                const uint64_t bd = sdesc_sw128(smem_u32(sB + s * SM::B_BYTES));
+                const uint32_t pa = smem_u32(sA + s * SM::A_BYTES), pb = smem_u32(sB + s * SM::B_BYTES);
+                const uint64_t ad = KROWS ? sdesc_sw128_mn(pa, BOX) : sdesc_sw128(pa);
+                const uint64_t bd = KROWS ? sdesc_sw128_mn(pb, BOX) : sdesc_sw128(pb);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) mma_f16kind(tmem, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                for (int k = 0; k < 4; ++k)
+                    mma_f16kind(tmem, ad + KSTEP * k, bd + KSTEP * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
                 mma_commit(&empty[s]);
             }
             mma_commit(acc_full);
@@ -282,10 +298,6 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                 *reinterpret_cast<const uint4*>(wt + r * 20 + 4 * i);
                         }
                     }
-                    if (G.out_t) {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) G.out_t[int64_t(gc0 + i) * G.M + gr] = __float2bfloat16_rn(v[i]);
-                    }
                 }
             }
         }
@@ -304,16 +316,21 @@ struct Gemm {
     dim3 grid;
     int bn;
     int epi;
+    bool krows;
 };
 
-// C[M x N] = A[M x K] B[N x K]^T with A, B row-major BF16 (K contiguous).
+// C[M x N] = A[M x K] B[N x K]^T with A, B row-major BF16 (K contiguous), or
+// with `krows` A[K x M]^T B[K x N].
 static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int N, int K, int bn, int epi,
-                      int splits) {
+                      int splits, bool krows = false) {
     if (M % G_BM || N % bn || K % 64 || splits < 1)
         return set_error(c, DRGB_ERR_INVALID, "mlp gemm: bad shape %d x %d x %d", M, N, K);
-    int rc = make_map_k64(c, &G.a, A, M, K, G_BM, false);
-    if (rc) return rc;
-    if ((rc = make_map_k64(c, &G.b, B, N, K, bn, false))) return rc;
+    int rc;
+    if (krows) {
+        if ((rc = make_map_k64(c, &G.a, A, K, M, 64, false)) || (rc = make_map_k64(c, &G.b, B, K, N, 64, false))) return rc;
+    } else {
+        if ((rc = make_map_k64(c, &G.a, A, M, K, G_BM, false)) || (rc = make_map_k64(c, &G.b, B, N, K, bn, false))) return rc;
+    }
     std::memset(&G.g, 0, sizeof(G.g));
     G.g.M = M;
     G.g.N = N;
@@ -324,12 +341,13 @@ static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int 
     G.grid = dim3(M / G_BM, N / bn, (kbs + G.g.kb_per_split - 1) / G.g.kb_per_split);
     G.bn = bn;
     G.epi = epi;
+    G.krows = krows;
     return DRGB_OK;
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool KROWS>
 static int gemm_attr(Ctx* c) {
-    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_gemm_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_gemm_kernel<BN, EPI, KROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       int(GemmSmem<BN>::TOTAL)));
     return DRGB_OK;
 }
@@ -337,8 +355,8 @@ static int gemm_attr(Ctx* c) {
 // Opt the GEMM instantiations into their shared-memory size (before any capture).
 static int gemm_prepare(Ctx* c) {
     int rc;
-    if ((rc = gemm_attr<128, EPI_GELU>(c)) || (rc = gemm_attr<128, EPI_GELU_GRAD>(c)) ||
-        (rc = gemm_attr<128, EPI_F32>(c)) || (rc = gemm_attr<64, EPI_F32>(c)))
+    if ((rc = gemm_attr<128, EPI_GELU, false>(c)) || (rc = gemm_attr<128, EPI_GELU_GRAD, false>(c)) ||
+        (rc = gemm_attr<128, EPI_F32, true>(c)) || (rc = gemm_attr<64, EPI_F32, true>(c)))
         return rc;
     return DRGB_OK;
 }
@@ -361,16 +379,18 @@ static int launch_step(Ctx* c, void (*kernel)(P...), dim3 grid, int block, size_
     return DRGB_OK;
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool KROWS>
 static int gemm_launch_t(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
-    return launch_step(c, mlp_gemm_kernel<BN, EPI>, G.grid, G_THREADS, GemmSmem<BN>::TOTAL, dep, st, G.a, G.b, G.g);
+    return launch_step(c, mlp_gemm_kernel<BN, EPI, KROWS>, G.grid, G_THREADS, GemmSmem<BN>::TOTAL, dep, st, G.a, G.b, G.g);
 }
 
 static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
-    if (G.bn == 128 && G.epi == EPI_GELU) return gemm_launch_t<128, EPI_GELU>(c, G, dep, st);
-    if (G.bn == 128 && G.epi == EPI_GELU_GRAD) return gemm_launch_t<128, EPI_GELU_GRAD>(c, G, dep, st);
-    if (G.bn == 128 && G.epi == EPI_F32) return gemm_launch_t<128, EPI_F32>(c, G, dep, st);
-    if (G.bn == 64 && G.epi == EPI_F32) return gemm_launch_t<64, EPI_F32>(c, G, dep, st);
+    if (G.bn == 128 && G.epi == EPI_GELU && !G.krows) return gemm_launch_t<128, EPI_GELU, false>(c, G, dep, st);
+    if (G.bn == 128 && G.epi == EPI_GELU_GRAD && !G.krows) return gemm_launch_t<128, EPI_GELU_GRAD, false>(c, G, dep, st);
+    if (G.bn == 128 && G.epi == EPI_F32)
+        return G.krows ? gemm_launch_t<128, EPI_F32, true>(c, G, dep, st) : gemm_launch_t<128, EPI_F32, false>(c, G, dep, st);
+    if (G.bn == 64 && G.epi == EPI_F32)
+        return G.krows ? gemm_launch_t<64, EPI_F32, true>(c, G, dep, st) : gemm_launch_t<64, EPI_F32, false>(c, G, dep, st);
     return set_error(c, DRGB_ERR_INVALID, "mlp gemm: unsupported tile");
 }
 
@@ -383,7 +403,7 @@ int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, in
     int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, EPI_F32, splits);
     if (rc) return rc;
     G.g.out_f32 = partials;
-    if ((rc = bn == 128 ? gemm_attr<128, EPI_F32>(c) : gemm_attr<64, EPI_F32>(c))) return rc;
+    if ((rc = bn == 128 ? gemm_attr<128, EPI_F32, false>(c) : gemm_attr<64, EPI_F32, false>(c))) return rc;
     if (splits_used) *splits_used = int(G.grid.z);
     return gemm_launch(c, G, false, st);
 }
@@ -461,29 +481,23 @@ __global__ void mlp_heads_kernel(const int32_t* __restrict__ rp, int64_t n, int6
     }
 }
 
-// Gather BF16 rows (zero-padded to 64 columns) and their transpose; with
-// `kept` the row numbers are copied there.
+// Gather BF16 rows (zero-padded to 64 columns), a warp per row; with `kept` the
+// row numbers are copied there.
 __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int32_t* __restrict__ rows, int M,
-                                  int M_valid, bf16* __restrict__ Xb, bf16* __restrict__ Xbt,
-                                  int32_t* __restrict__ kept) {
-    __shared__ bf16 tile[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    if (kept && c0 == 0 && threadIdx.y == 0 && r0 + int(threadIdx.x) < M_valid)
-        kept[r0 + threadIdx.x] = rows[r0 + threadIdx.x];
-    for (int ty = threadIdx.y; ty < 32; ty += blockDim.y) {
-        const int r = r0 + ty, cc = c0 + threadIdx.x;
-        float v = 0.f;
-        if (r < M_valid && cc < d) v = X[int64_t(rows ? rows[r] : r) * d + cc];
-        const bf16 b = __float2bfloat16_rn(v);
-        if (r < M) Xb[int64_t(r) * MLP_IN + cc] = b;
-        tile[ty][threadIdx.x] = b;
-    }
-    __syncthreads();
-    if (Xbt)
-        for (int ty = threadIdx.y; ty < 32; ty += blockDim.y) {
-            const int cc = c0 + ty, r = r0 + threadIdx.x;
-            if (r < M) Xbt[int64_t(cc) * M + r] = tile[threadIdx.x][ty];
+                                  int M_valid, bf16* __restrict__ Xb, int32_t* __restrict__ kept) {
+    const int lane = threadIdx.x & 31;
+    for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < M; r += (gridDim.x * blockDim.x) >> 5) {
+        float v[2] = {0.f, 0.f};
+        if (r < M_valid) {
+            const int32_t src = rows[r];
+            if (kept && lane == 0) kept[r] = src;
+            const float* x = X + int64_t(src) * d + 2 * lane;
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (2 * lane + j < d) v[j] = x[j];
         }
+        reinterpret_cast<__nv_bfloat162*>(Xb)[int64_t(r) * (MLP_IN / 2) + lane] = __floats2bfloat162_rn(v[0], v[1]);
+    }
 }
 
 // z = H2 W3^T + b3: one warp per row, lanes on columns lane + 32 i; four rows'
@@ -590,13 +604,13 @@ static constexpr int MLP_CHUNK = 512;
 static constexpr int MC_THREADS = 256;
 static constexpr int MC_PITCH = MLP_CHUNK * 4 + 4;  // floats per float4 column: lanes of a row hit distinct banks
 
-// dpre2 = (dz W3) . GELU'(pre2) (BF16 row-major and transposed) and, over the
+// dpre2 = (dz W3) . GELU'(pre2) (BF16) and, over the
 // chunk, db2 = sum dpre2, dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
 static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 64 + MLP_CHUNK * 8;
 
 __global__ void __launch_bounds__(MC_THREADS, 2)
 mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2,
-                  const bf16* __restrict__ H2, int M, bf16* __restrict__ D, bf16* __restrict__ Dt,
+                  const bf16* __restrict__ H2, int M, bf16* __restrict__ D,
                   float* __restrict__ pb2, float* __restrict__ pw3) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]: dpre2, float4 columns
     bf16* s_h = reinterpret_cast<bf16*>(s_v + 8 * MC_PITCH);       // [MLP_CHUNK][32]: H2
@@ -626,7 +640,6 @@ mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, c
                 const int cc = c0 + 4 * i + j;
                 const float g = dz2.x * W3f[cc] + dz2.y * W3f[MLP_H + cc];
                 v[j] = g * v[j];
-                Dt[int64_t(cc) * M + r0 + r] = __float2bfloat16_rn(v[j]);
             }
             *reinterpret_cast<float4*>(s_v + i * MC_PITCH + 4 * r) = make_float4(v[0], v[1], v[2], v[3]);
             const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
@@ -1041,7 +1054,7 @@ static int chunk_prepare(Ctx* c) {
 struct MlpBuffers {
     int M;                       // rows of the batch (padded to 128)
     int32_t* rows;
-    bf16 *Xb, *Xbt, *H1b, *H1bt, *H2b, *D2b, *D2bt, *D1b, *D1bt;
+    bf16 *Xb, *H1b, *H2b, *D2b, *D1b;
     float *dg1, *dg2, *z, *dz, *D1f, *loss_part;
     float *pW2, *pW1, *pb1, *pb2, *pw3;
     float* grad;
@@ -1055,8 +1068,8 @@ static size_t mlp_batch_bytes(int M) {
     const size_t m = size_t(M);
     const int nch = int((m + MLP_CHUNK - 1) / MLP_CHUNK);
     size_t b = Carve::round(m * 4);                                   // rows
-    b += 2 * Carve::round(m * MLP_IN * 2);                            // Xb, Xbt
-    b += 7 * Carve::round(m * MLP_H * 2);                             // H1b, H1bt, H2b, D2b, D2bt, D1b, D1bt
+    b += Carve::round(m * MLP_IN * 2);                                // Xb
+    b += 4 * Carve::round(m * MLP_H * 2);                             // H1b, H2b, D2b, D1b
     b += 3 * Carve::round(m * MLP_H * 4);                             // dg1, dg2, D1f
     b += 2 * Carve::round(m * 2 * 4) + Carve::round(m * 4);           // z, dz, loss_part
     b += Carve::round(size_t(MLP_SPLITS) * MLP_H * MLP_H * 4);        // pW2
@@ -1078,14 +1091,10 @@ static MlpBuffers mlp_carve(void* base, int M) {
     b.s_split = MLP_SPLITS;
     b.rows = cv.take<int32_t>(m);
     b.Xb = cv.take<bf16>(m * MLP_IN);
-    b.Xbt = cv.take<bf16>(m * MLP_IN);
     b.H1b = cv.take<bf16>(m * MLP_H);
-    b.H1bt = cv.take<bf16>(m * MLP_H);
     b.H2b = cv.take<bf16>(m * MLP_H);
     b.D2b = cv.take<bf16>(m * MLP_H);
-    b.D2bt = cv.take<bf16>(m * MLP_H);
     b.D1b = cv.take<bf16>(m * MLP_H);
-    b.D1bt = cv.take<bf16>(m * MLP_H);
     b.dg1 = cv.take<float>(m * MLP_H);
     b.dg2 = cv.take<float>(m * MLP_H);
     b.D1f = cv.take<float>(m * MLP_H);
@@ -1133,7 +1142,7 @@ static int mlp_zero_padding(Ctx* c, const MlpBuffers& b, int rows, cudaStream_t 
     return DRGB_OK;
 }
 
-// Forward + backward of the batch whose rows are already gathered (Xb, Xbt)
+// Forward + backward of the batch whose rows are already gathered (Xb)
 // with B edges of R rows; leaves the gradient in b.grad and the loss in
 // loss_out[*step] (if given), and with `adam` updates the weights.
 static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, float a, float bb,
@@ -1145,7 +1154,6 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     F1.g.bias = P + OFF_B1;
     F1.g.dgelu = b.dg1;
     F1.g.out = b.H1b;
-    F1.g.out_t = b.H1bt;
     if ((rc = gemm_setup(c, F2, b.H1b, b.W.W2b, M, MLP_H, MLP_H, 128, EPI_GELU, 1))) return rc;
     F2.g.bias = P + OFF_B2;
     F2.g.dgelu = b.dg2;
@@ -1159,23 +1167,23 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     if (fork.ahead && ((rc = mlp_order(c, fork.ev[0], st, fork.ahead)) || (rc = fork.draw(fork.ahead)))) return rc;
     const dim3 cgrid(b.n_chunks, MLP_H / 32);
     if ((rc = launch_step(c, mlp_l3back_kernel, cgrid, MC_THREADS, L3_SMEM, true, st, b.dz, b.W.W3f, b.dg2, b.H2b, M,
-                          b.D2b, b.D2bt, b.pb2, b.pw3)))
+                          b.D2b, b.pb2, b.pw3)))
         return rc;
     // dW2 = dpre2^T H1 (K = M, split)
     if (fork.side && (rc = mlp_order(c, fork.ev[1], st, fork.side))) return rc;
-    if ((rc = gemm_setup(c, DW2, b.D2bt, b.H1bt, MLP_H, MLP_H, M, 128, EPI_F32, MLP_SPLITS))) return rc;
+    if ((rc = gemm_setup(c, DW2, b.D2b, b.H1b, MLP_H, MLP_H, M, 128, EPI_F32, MLP_SPLITS, true))) return rc;
     DW2.g.out_f32 = b.pW2;
     if ((rc = gemm_launch(c, DW2, false, fork.side ? fork.side : st))) return rc;
     // dpre1 = (dpre2 W2) . GELU'(pre1): A = dpre2 [M x 256(out)], B = W2^T [256(in) x 256(out)]
     if ((rc = gemm_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H, MLP_H, 128, EPI_GELU_GRAD, 1))) return rc;
     DH1.g.dgelu = b.dg1;
-    DH1.g.out_t = b.D1bt;
+    DH1.g.out = b.D1b;
     DH1.g.out_f32 = b.D1f;
     if ((rc = gemm_launch(c, DH1, fork.side != nullptr, st)) ||
         (rc = launch_step(c, mlp_colsum_kernel, cgrid, MC_THREADS, CS_SMEM, true, st, b.D1f, M, b.pb1)))
         return rc;
-    // dW1 = dpre1^T Xb: A = dpre1^T [256 x M], B = Xb^T [64 x M]
-    if ((rc = gemm_setup(c, DW1, b.D1bt, b.Xbt, MLP_H, MLP_IN, M, 64, EPI_F32, MLP_SPLITS))) return rc;
+    // dW1 = dpre1^T Xb
+    if ((rc = gemm_setup(c, DW1, b.D1b, b.Xb, MLP_H, MLP_IN, M, 64, EPI_F32, MLP_SPLITS, true))) return rc;
     DW1.g.out_f32 = b.pW1;
     if ((rc = gemm_launch(c, DW1, true, st))) return rc;
     if (fork.ahead && ((rc = mlp_order(c, fork.ev[2], st, fork.ahead)) || (rc = fork.gather(fork.ahead)))) return rc;
@@ -1245,7 +1253,7 @@ int drgb_mlp_grad(drgb_ctx* c, const float* params, const float* X, int64_t n, i
     if ((rc = mlp_zero_padding(c, bu, Mv, st))) return rc;
     mlp_cast_kernel<<<grid_for(MLP_P, 256, c->num_sms * 4), 256, 0, st>>>(params, bu.W);
     DRGB_CHECK_LAUNCH(c);
-    mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, st>>>(X, d, bu.rows, M, Mv, bu.Xb, bu.Xbt, nullptr);
+    mlp_gather_kernel<<<grid_for(M, 8, c->num_sms * 8), 256, 0, st>>>(X, d, bu.rows, M, Mv, bu.Xb, nullptr);
     DRGB_CHECK_LAUNCH(c);
     if ((rc = mlp_fwd_bwd(c, bu, params, n_edges, neg, a, b, loss_out, nullptr, MlpFork{}, st))) return rc;
     DRGB_CUDA(c, cudaMemcpyAsync(grad_out, bu.grad, MLP_P * 4, cudaMemcpyDeviceToDevice, st));
@@ -1292,7 +1300,7 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
         return DRGB_OK;
     };
     fork.gather = [&](cudaStream_t s) -> int {
-        mlp_gather_kernel<<<dim3(M / 32, MLP_IN / 32), dim3(32, 8), 0, s>>>(X, d, next_rows, M, Mv, bu.Xb, bu.Xbt, bu.rows);
+        mlp_gather_kernel<<<grid_for(M, 8, c->num_sms * 8), 256, 0, s>>>(X, d, next_rows, M, Mv, bu.Xb, bu.rows);
         DRGB_CHECK_LAUNCH(c);
         return DRGB_OK;
     };

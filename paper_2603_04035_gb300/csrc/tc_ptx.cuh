@@ -88,6 +88,18 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr) {
     d |= uint64_t(2) << 61;                       // 128-byte swizzle
     return d;
 }
+// The same for an operand stored K rows x MN columns (MN-major): its tile is
+// boxes of 64 MN columns (128 bytes) x 64 K rows, `box` bytes apart.
+__device__ __forceinline__ uint64_t sdesc_sw128_mn(uint32_t addr, uint32_t box) {
+    uint64_t d = 0;
+    d |= uint64_t((addr & 0x3FFFFu) >> 4);
+    d |= uint64_t(box >> 4) << 16;                 // leading byte offset: next 64 columns
+    d |= uint64_t(1024 >> 4) << 32;                // stride byte offset: next 8 K rows
+    d |= uint64_t(1) << 46;
+    d |= uint64_t(2) << 61;
+    return d;
+}
+static constexpr uint32_t IDESC_MN_MAJOR = (1u << 15) | (1u << 16);  // A and B MN-major
 // Instruction descriptor (kind::f16): D = F32, A = B = BF16 (format 1) or
 // FP16 (format 0), both K-major, M x N.
 __host__ __device__ constexpr uint32_t idesc_f16kind(int M, int N, bool f16) {
