@@ -4,11 +4,10 @@
 // trained with Adam on the UMAP cross-entropy over edges of the method's own
 // fuzzy graph, then used to embed new points.
 //
-// Every dense product runs on the tcgen05 tensor cores through one kernel,
-// mlp_gemm_kernel: C[M x N] = A[M x K] * B[N x K]^T with BF16 operands (TMA,
-// 128-byte swizzle), FP32 accumulation in TMEM, and a fused epilogue: bias +
-// GELU (forward), GELU derivative (backward) or plain FP32 (weight gradients,
-// split over K).  The weight gradients sum over the batch's rows: they take the
+// Every dense product runs on the tcgen05 tensor cores with BF16 operands (TMA,
+// 128-byte swizzle) and FP32 accumulation in TMEM: mlp_layer_kernel with a fused
+// epilogue (bias + GELU forward, the GELU derivative backward), mlp_gemm_kernel
+// for the weight gradients (plain FP32, split over K).  The weight gradients sum over the batch's rows: they take the
 // activations as they lie, MN-major (with transposed copies for K-major
 // operands, written by two GEMM epilogues, the layer 3 kernel and the gather, a
 // step of 4096 edges took 136 us against 125).  The 256 -> 2 layer, the loss,
@@ -21,9 +20,10 @@
 //              (both for the next step, beside this step's backward pass)
 //   F1, F2     pre_l = H_{l-1} W_l^T + b_l ; H_l = GELU(pre_l)  (BF16) ;
 //              GELU'(pre_l) (FP32, blocked)
-//   head       z = H2 W3^T + b3 ; loss and dL/dz per edge
-//   L3 back    dpre2 = (dz W3) . GELU'(pre2) ; dW3, db3, db2 partial sums
-//   dW2        dpre2^T H1     (split-K, FP32 partials; beside dH1 and dW1)
+//   head       z = H2 W3^T + b3, loss and dL/dz per edge
+//   L3 back    dpre2 = (dz W3) . GELU'(pre2) ; db2 partial sums
+//   dW3, dW2   dW3, db3 partial sums ; dpre2^T H1 (split-K, FP32 partials), on a
+//              branch of their own
 //   dH1        dpre1 = (dpre2 W2) . GELU'(pre1)
 //   dW1        dpre1^T Xb     (split-K) ; db1 partial sums
 //   update     gradient (fixed summation order), Adam, BF16 copies
@@ -64,14 +64,10 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // ------------------------------------------------------------------ tensor-core GEMM
-// 128 x 128 (or 64) tiles, two CTAs per SM: the epilogue (bias, GELU and its
-// derivative: about 60 instructions an element) is the larger part, and 16
-// epilogue warps an SM hide its latency (4 warps on one CTA per SM, with
-// 128 x 256 tiles: 41-52 us for 28,672 rows; now 12-17).
 static constexpr int G_BM = 128;
+// 128 x 128 (or 64) tiles of C, split over K, two CTAs per SM.
 static constexpr int G_EPI_WARPS = 8;  // two per TMEM lane quarter, one per column half
 static constexpr int G_THREADS = 64 + G_EPI_WARPS * 32;  // warp 0 TMA, warp 1 MMA
-enum { EPI_GELU = 0, EPI_GELU_GRAD = 1, EPI_F32 = 2 };
 
 // Blocked FP32 layout of an M x N matrix that only epilogues (and kernels of
 // the same tiling) exchange: 128 x 32 blocks, within a block float4 columns of
@@ -83,10 +79,7 @@ __host__ __device__ __forceinline__ int64_t blocked_at(int64_t row, int col, int
 struct GemmArgs {
     int M, N, K;          // M, N multiples of 128 / BN; K multiple of 64
     int kb_per_split;     // 64-wide K blocks per split (grid z)
-    const float* bias;    // EPI_GELU: [N]
-    float* dgelu;         // GELU'(pre), blocked: EPI_GELU out (nullable), EPI_GELU_GRAD in
-    bf16* out;            // [M][N] (nullable)
-    float* out_f32;       // EPI_F32: [splits][M][N]; EPI_GELU_GRAD: blocked FP32 copy (nullable)
+    float* out_f32;       // [splits][M][N]
     int* status;
 };
 
@@ -95,7 +88,7 @@ struct GemmSmem {
     static constexpr int STAGES = BN == 128 ? 3 : 4;
     static constexpr int A_BYTES = G_BM * 64 * 2;
     static constexpr int B_BYTES = BN * 64 * 2;
-    static constexpr size_t TOTAL = 1024 + size_t(STAGES) * (A_BYTES + B_BYTES) + 256 + BN * 4;
+    static constexpr size_t TOTAL = 1024 + size_t(STAGES) * (A_BYTES + B_BYTES) + 256;
 };
 static constexpr int G_PITCH = 36;  // floats per row of a warp's 32 x 32 transposing tile (16-byte rows)
 
@@ -111,7 +104,7 @@ __device__ __forceinline__ void step_dep() {
 
 // With KROWS the operands are stored K rows x M (N) columns, as activations of a
 // batch are for a product over its rows, and staged as boxes of 64 x 64.
-template <int BN, int EPI, bool KROWS>
+template <int BN, bool KROWS>
 __global__ void __launch_bounds__(G_THREADS, 2)
 mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs G) {
     using SM = GemmSmem<BN>;
@@ -131,7 +124,6 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     uint64_t* mma_done = acc_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    float* s_bias = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 256);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * G_BM, n0 = blockIdx.y * BN;
@@ -156,7 +148,6 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     step_dep();
-    if (EPI == EPI_GELU && threadIdx.x >= 64 && threadIdx.x < 64 + BN) s_bias[threadIdx.x - 64] = G.bias[n0 + threadIdx.x - 64];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -213,8 +204,6 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else {
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        const int row = quarter * 32 + lane;
-        const int64_t gr = m0 + row;
         // once the accumulator is complete the operand ring is free: each warp
         // transposes its 32 x 32 pieces through its own part of it
         float* tile = reinterpret_cast<float*>(base) + (warp - 2) * 32 * G_PITCH;
@@ -227,77 +216,16 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 __syncwarp();
                 tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(c * 32), v);
                 const int gc0 = n0 + c * 32;
-                if (EPI == EPI_F32) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 4)
-                        *reinterpret_cast<float4*>(tile + lane * G_PITCH + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                    __syncwarp();
-                    float* o = G.out_f32 + (int64_t(blockIdx.z) * G.M + m0 + quarter * 32) * G.N + gc0;
+                for (int i = 0; i < 32; i += 4)
+                    *reinterpret_cast<float4*>(tile + lane * G_PITCH + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                __syncwarp();
+                float* o = G.out_f32 + (int64_t(blockIdx.z) * G.M + m0 + quarter * 32) * G.N + gc0;
 #pragma unroll
-                    for (int it = 0; it < 8; ++it) {  // four rows of 128 bytes an instruction
-                        const int r = it * 4 + (lane >> 3), i = 4 * (lane & 7);
-                        *reinterpret_cast<float4*>(o + int64_t(r) * G.N + i) =
-                            *reinterpret_cast<const float4*>(tile + r * G_PITCH + i);
-                    }
-                } else {
-                    float* bl = nullptr;  // this lane's float4 column of the blocked matrices
-                    const int64_t bo = blocked_at(gr, gc0, G.N);
-                    if (EPI == EPI_GELU) {
-                        if (G.dgelu) bl = G.dgelu + bo;
-#pragma unroll
-                        for (int i = 0; i < 32; i += 4) {
-                            const float4 b4 = *reinterpret_cast<const float4*>(s_bias + c * 32 + i);
-                            v[i] += b4.x;
-                            v[i + 1] += b4.y;
-                            v[i + 2] += b4.z;
-                            v[i + 3] += b4.w;
-                            if (bl)
-                                *reinterpret_cast<float4*>(bl + i * 128) = make_float4(
-                                    gelu_grad(v[i]), gelu_grad(v[i + 1]), gelu_grad(v[i + 2]), gelu_grad(v[i + 3]));
-                            v[i] = gelu(v[i]);
-                            v[i + 1] = gelu(v[i + 1]);
-                            v[i + 2] = gelu(v[i + 2]);
-                            v[i + 3] = gelu(v[i + 3]);
-                        }
-                    } else {  // EPI_GELU_GRAD
-                        const float* p = G.dgelu + bo;
-#pragma unroll
-                        for (int i = 0; i < 32; i += 4) {
-                            const float4 x = *reinterpret_cast<const float4*>(p + i * 128);
-                            v[i] *= x.x;
-                            v[i + 1] *= x.y;
-                            v[i + 2] *= x.z;
-                            v[i + 3] *= x.w;
-                        }
-                        if (G.out_f32) {
-                            bl = G.out_f32 + bo;
-#pragma unroll
-                            for (int i = 0; i < 32; i += 4)
-                                *reinterpret_cast<float4*>(bl + i * 128) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                        }
-                    }
-                    if (G.out) {
-                        uint32_t* wt = reinterpret_cast<uint32_t*>(tile);  // rows of 20 words: 16-byte reads and writes
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            uint32_t packed[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[8 * i + 2 * j], v[8 * i + 2 * j + 1]);
-                                packed[j] = *reinterpret_cast<const uint32_t*>(&h2);
-                            }
-                            *reinterpret_cast<uint4*>(wt + lane * 20 + 4 * i) =
-                                make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                        }
-                        __syncwarp();
-                        bf16* o = G.out + (int64_t(m0) + quarter * 32) * G.N + gc0;
-#pragma unroll
-                        for (int it = 0; it < 4; ++it) {  // eight rows of 64 bytes an instruction
-                            const int r = it * 8 + (lane >> 2), i = lane & 3;
-                            *reinterpret_cast<uint4*>(o + int64_t(r) * G.N + 8 * i) =
-                                *reinterpret_cast<const uint4*>(wt + r * 20 + 4 * i);
-                        }
-                    }
+                for (int it = 0; it < 8; ++it) {  // four rows of 128 bytes an instruction
+                    const int r = it * 4 + (lane >> 3), i = 4 * (lane & 7);
+                    *reinterpret_cast<float4*>(o + int64_t(r) * G.N + i) =
+                        *reinterpret_cast<const float4*>(tile + r * G_PITCH + i);
                 }
             }
         }
@@ -315,14 +243,13 @@ struct Gemm {
     GemmArgs g;
     dim3 grid;
     int bn;
-    int epi;
     bool krows;
 };
 
 // C[M x N] = A[M x K] B[N x K]^T with A, B row-major BF16 (K contiguous), or
 // with `krows` A[K x M]^T B[K x N].
-static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int N, int K, int bn, int epi,
-                      int splits, bool krows = false) {
+static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int N, int K, int bn,
+                      int splits, bool krows) {
     if (M % G_BM || N % bn || K % 64 || splits < 1)
         return set_error(c, DRGB_ERR_INVALID, "mlp gemm: bad shape %d x %d x %d", M, N, K);
     int rc;
@@ -340,24 +267,14 @@ static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int 
     G.g.status = c->d_status;
     G.grid = dim3(M / G_BM, N / bn, (kbs + G.g.kb_per_split - 1) / G.g.kb_per_split);
     G.bn = bn;
-    G.epi = epi;
     G.krows = krows;
     return DRGB_OK;
 }
 
-template <int BN, int EPI, bool KROWS>
+template <int BN, bool KROWS>
 static int gemm_attr(Ctx* c) {
-    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_gemm_kernel<BN, EPI, KROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_gemm_kernel<BN, KROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       int(GemmSmem<BN>::TOTAL)));
-    return DRGB_OK;
-}
-
-// Opt the GEMM instantiations into their shared-memory size (before any capture).
-static int gemm_prepare(Ctx* c) {
-    int rc;
-    if ((rc = gemm_attr<128, EPI_GELU, false>(c)) || (rc = gemm_attr<128, EPI_GELU_GRAD, false>(c)) ||
-        (rc = gemm_attr<128, EPI_F32, true>(c)) || (rc = gemm_attr<64, EPI_F32, true>(c)))
-        return rc;
     return DRGB_OK;
 }
 
@@ -379,18 +296,10 @@ static int launch_step(Ctx* c, void (*kernel)(P...), dim3 grid, int block, size_
     return DRGB_OK;
 }
 
-template <int BN, int EPI, bool KROWS>
-static int gemm_launch_t(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
-    return launch_step(c, mlp_gemm_kernel<BN, EPI, KROWS>, G.grid, G_THREADS, GemmSmem<BN>::TOTAL, dep, st, G.a, G.b, G.g);
-}
-
 static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
-    if (G.bn == 128 && G.epi == EPI_GELU && !G.krows) return gemm_launch_t<128, EPI_GELU, false>(c, G, dep, st);
-    if (G.bn == 128 && G.epi == EPI_GELU_GRAD && !G.krows) return gemm_launch_t<128, EPI_GELU_GRAD, false>(c, G, dep, st);
-    if (G.bn == 128 && G.epi == EPI_F32)
-        return G.krows ? gemm_launch_t<128, EPI_F32, true>(c, G, dep, st) : gemm_launch_t<128, EPI_F32, false>(c, G, dep, st);
-    if (G.bn == 64 && G.epi == EPI_F32)
-        return G.krows ? gemm_launch_t<64, EPI_F32, true>(c, G, dep, st) : gemm_launch_t<64, EPI_F32, false>(c, G, dep, st);
+    auto go = [&](auto kernel, size_t smem) { return launch_step(c, kernel, G.grid, G_THREADS, smem, dep, st, G.a, G.b, G.g); };
+    if (G.bn == 128) return go(G.krows ? mlp_gemm_kernel<128, true> : mlp_gemm_kernel<128, false>, GemmSmem<128>::TOTAL);
+    if (G.bn == 64) return go(G.krows ? mlp_gemm_kernel<64, true> : mlp_gemm_kernel<64, false>, GemmSmem<64>::TOTAL);
     return set_error(c, DRGB_ERR_INVALID, "mlp gemm: unsupported tile");
 }
 
@@ -400,12 +309,254 @@ int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, in
                    int* splits_used, cudaStream_t st) {
     Gemm G;
     const int bn = (N % 128 == 0) ? 128 : 64;
-    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, EPI_F32, splits);
+    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, splits, false);
     if (rc) return rc;
     G.g.out_f32 = partials;
-    if ((rc = bn == 128 ? gemm_attr<128, EPI_F32, false>(c) : gemm_attr<64, EPI_F32, false>(c))) return rc;
+    if ((rc = bn == 128 ? gemm_attr<128, false>(c) : gemm_attr<64, false>(c))) return rc;
     if (splits_used) *splits_used = int(G.grid.z);
     return gemm_launch(c, G, false, st);
+}
+
+// ------------------------------------------------------------------ layers of a batch
+// One layer of the training step over M rows, N = MLP_H: forward
+// (pre = A B^T + bias; out = GELU(pre), dgelu = GELU'(pre)) or backward
+// (d = (A B^T) . dgelu; out, out_f32 = d).  128 x 64 tiles in persistent CTAs, two
+// per SM: the producer and MMA warps run up to two tiles ahead (the accumulator
+// has two buffers) of eight epilogue warps, each on 32 x 32 of a tile.
+//
+// Bound: the epilogue (forward about 60 instructions an element for GELU and
+// its derivative; backward the latency of its reads), so the split evens that
+// out: 28,672 rows are 896 tiles on 304 CTAs, 2.95 rounds of them.  As 448 CTAs of
+// 128 x 128 (1.47 rounds, each load, MMA and epilogue in turn) F1 took 27.1, F2
+// 28.5 and dH1 21.3 us; a step went from 125 to 109 us.
+static constexpr int LY_BN = 64, LY_STAGES = 3;
+static constexpr int LY_A = G_BM * 64 * 2, LY_B = LY_BN * 64 * 2;
+static constexpr int LY_TILE = 32 * G_PITCH * 4;  // a warp's transposing tile
+static constexpr size_t LY_SMEM = 1024 + size_t(LY_STAGES) * (LY_A + LY_B) + G_EPI_WARPS * LY_TILE + MLP_H * 4 + 128;
+
+struct LayerArgs {
+    int M, K;             // multiples of 128 and 64
+    const float* bias;    // forward: [MLP_H]
+    float* dgelu;         // blocked: forward out, backward in
+    bf16* out;            // [M][MLP_H]
+    float* out_f32;       // backward: blocked
+    int* status;
+};
+
+template <bool BACK>
+__global__ void __launch_bounds__(G_THREADS, 2)
+mlp_layer_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, LayerArgs G) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint8_t* sA = base;
+    uint8_t* sB = base + LY_STAGES * LY_A;
+    uint8_t* s_tile = sB + LY_STAGES * LY_B;
+    float* s_bias = reinterpret_cast<float*>(s_tile + G_EPI_WARPS * LY_TILE);
+    uint64_t* full = reinterpret_cast<uint64_t*>(s_bias + MLP_H);
+    uint64_t* empty = full + LY_STAGES;
+    uint64_t* acc_full = empty + LY_STAGES;  // [2]
+    uint64_t* acc_free = acc_full + 2;       // [2]
+    uint64_t* mma_done = acc_free + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    constexpr int NT = MLP_H / LY_BN;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tiles = G.M / G_BM * NT, nkb = G.K / 64;
+    const int mine = (tiles - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x);  // tiles blockIdx.x, + gridDim.x, ...
+
+    if (tid == 0) {
+        for (int s = 0; s < LY_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int u = 0; u < 2; ++u) {
+            mbar_init(&acc_full[u], 1);
+            mbar_init(&acc_free[u], G_EPI_WARPS);
+        }
+        mbar_init(mma_done, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(2 * LY_BN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    step_dep();
+    if (!BACK)
+        for (int t = tid; t < MLP_H; t += G_THREADS) s_bias[t] = G.bias[t];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            for (int i = 0; i < mine && ok; ++i) {
+                const int t = int(blockIdx.x) + i * int(gridDim.x), m0 = t / NT * G_BM, n0 = t % NT * LY_BN;
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const int s = it % LY_STAGES;
+                    if (it >= LY_STAGES && !(ok = mbar_wait(&empty[s], ((it / LY_STAGES) & 1) ^ 1, abort_flag, G.status))) break;
+                    mbar_expect_tx(&full[s], LY_A + LY_B);
+                    tma_load_2d(sA + s * LY_A, &tmA, kb * 64, m0, &full[s]);
+                    tma_load_2d(sB + s * LY_B, &tmB, kb * 64, n0, &full[s]);
+                }
+            }
+            if (!ok) {  // aborted: let issued loads land before exit
+                for (int u = (it > LY_STAGES ? it - LY_STAGES : 0); u < it; ++u) {
+                    const unsigned long long t0 = global_timer();
+                    while (!mbar_try(&full[u % LY_STAGES], (u / LY_STAGES) & 1) && global_timer() - t0 < 100000000ull) {
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = idesc_f16kind(G_BM, LY_BN, false);
+            int it = 0;
+            bool ok = true;
+            for (int i = 0; i < mine && ok; ++i) {
+                const int u = i & 1;
+                if (i >= 2 && !(ok = mbar_wait(&acc_free[u], ((i >> 1) & 1) ^ 1, abort_flag, G.status))) break;
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const int s = it % LY_STAGES;
+                    if (!(ok = mbar_wait(&full[s], (it / LY_STAGES) & 1, abort_flag, G.status))) break;
+                    tc_fence_after();
+                    const uint64_t ad = sdesc_sw128(smem_u32(sA + s * LY_A)), bd = sdesc_sw128(smem_u32(sB + s * LY_B));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        mma_f16kind(tmem + u * LY_BN, ad + 2 * k, bd + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                    mma_commit(&empty[s]);
+                }
+                if (ok) mma_commit(&acc_full[u]);
+            }
+            mma_commit(mma_done);  // every MMA issued above has completed once this fires
+            const unsigned long long t0 = global_timer();
+            while (!mbar_try(mma_done, 0) && global_timer() - t0 < 100000000ull) {
+            }
+        }
+    } else {
+        const int quarter = warp & 3, half = (warp - 2) >> 2;
+        float* tile = reinterpret_cast<float*>(s_tile + (warp - 2) * LY_TILE);
+        auto at = [&](int i, int& m0, int& c0) {
+            const int t = int(blockIdx.x) + i * int(gridDim.x);
+            m0 = t / NT * G_BM + quarter * 32;
+            c0 = t % NT * LY_BN + half * 32;
+        };
+        float x[32];  // backward: GELU' of the tile to come
+        auto load_x = [&](int i) {
+            if (!BACK || i >= mine) return;
+            int m0, c0;
+            at(i, m0, c0);
+            const float* p = G.dgelu + blocked_at(m0 + lane, c0, MLP_H);
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 f = *reinterpret_cast<const float4*>(p + j * 128);
+                x[j] = f.x;
+                x[j + 1] = f.y;
+                x[j + 2] = f.z;
+                x[j + 3] = f.w;
+            }
+        };
+        load_x(0);
+        for (int i = 0; i < mine; ++i) {
+            const int u = i & 1;
+            int m0, c0;
+            at(i, m0, c0);
+            if (!mbar_wait(&acc_full[u], (i >> 1) & 1, abort_flag, G.status)) break;
+            tc_fence_after();
+            float v[32];
+            __syncwarp();
+            tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(u * LY_BN + half * 32), v);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_free[u]);
+            const int64_t bo = blocked_at(m0 + lane, c0, MLP_H);  // this lane's float4 column of the blocked matrices
+            if (!BACK) {
+                float* bl = G.dgelu + bo;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(s_bias + c0 + j);
+                    v[j] += b4.x;
+                    v[j + 1] += b4.y;
+                    v[j + 2] += b4.z;
+                    v[j + 3] += b4.w;
+                    *reinterpret_cast<float4*>(bl + j * 128) =
+                        make_float4(gelu_grad(v[j]), gelu_grad(v[j + 1]), gelu_grad(v[j + 2]), gelu_grad(v[j + 3]));
+                    v[j] = gelu(v[j]);
+                    v[j + 1] = gelu(v[j + 1]);
+                    v[j + 2] = gelu(v[j + 2]);
+                    v[j + 3] = gelu(v[j + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] *= x[j];
+                load_x(i + 1);
+                float* bl = G.out_f32 + bo;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4)
+                    *reinterpret_cast<float4*>(bl + j * 128) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+            uint32_t* wt = reinterpret_cast<uint32_t*>(tile);  // rows of 20 words: 16-byte reads and writes
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                uint32_t packed[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[8 * j + 2 * k], v[8 * j + 2 * k + 1]);
+                    packed[k] = *reinterpret_cast<const uint32_t*>(&h2);
+                }
+                *reinterpret_cast<uint4*>(wt + lane * 20 + 4 * j) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+            }
+            __syncwarp();
+            bf16* o = G.out + int64_t(m0) * MLP_H + c0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {  // eight rows of 64 bytes an instruction
+                const int r = j * 8 + (lane >> 2), k = lane & 3;
+                *reinterpret_cast<uint4*>(o + int64_t(r) * MLP_H + 8 * k) = *reinterpret_cast<const uint4*>(wt + r * 20 + 4 * k);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * LY_BN) : "memory");
+    }
+}
+
+struct Layer {
+    CUtensorMap a, b;
+    LayerArgs g;
+};
+
+static int layer_setup(Ctx* c, Layer& L, const bf16* A, const bf16* B, int M, int K) {
+    int rc;
+    if ((rc = make_map_k64(c, &L.a, A, M, K, G_BM, false)) || (rc = make_map_k64(c, &L.b, B, MLP_H, K, LY_BN, false))) return rc;
+    std::memset(&L.g, 0, sizeof(L.g));
+    L.g.M = M;
+    L.g.K = K;
+    L.g.status = c->d_status;
+    return DRGB_OK;
+}
+
+template <bool BACK>
+static int layer_launch(Ctx* c, const Layer& L, bool dep, cudaStream_t st) {
+    const dim3 grid(grid_for(int64_t(L.g.M / G_BM) * (MLP_H / LY_BN), 1, 2 * c->num_sms));
+    return launch_step(c, mlp_layer_kernel<BACK>, grid, G_THREADS, LY_SMEM, dep, st, L.a, L.b, L.g);
+}
+
+// Opt the training kernels into their shared-memory sizes (before any capture).
+static int gemm_prepare(Ctx* c) {
+    int rc;
+    if ((rc = gemm_attr<128, true>(c)) || (rc = gemm_attr<64, true>(c))) return rc;
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_layer_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LY_SMEM)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(mlp_layer_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(LY_SMEM)));
+    return DRGB_OK;
 }
 
 // ------------------------------------------------------------------ SIMT kernels
@@ -500,17 +651,25 @@ __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int3
     }
 }
 
-// z = H2 W3^T + b3: one warp per row, lanes on columns lane + 32 i; four rows'
-// loads are in flight together.  Advances the step counter, which is at the
-// step before until here.
+// z = H2 W3^T + b3 of an edge's rows (head, tail, negatives) and its UMAP
+// cross-entropy, with Phi = 1 / (1 + a d^b) clamped to [1e-4, 1 - 1e-4] (zero
+// gradient where clamped); loss and dL/dz are divided by the batch size.
+// Advances the step counter, which is at the step before until here.
+//
+// One warp per edge: the rows' products with lanes on columns lane + 32 i, four
+// rows' loads in flight together, then one lane per row for the loss (powf and
+// logf of all rows at once), whose terms are added in row order.  Latency-bound:
+// as two kernels, with a thread per edge for the losses, 8 + 7 us.  (This and
+// the split of the layer 3 backward below took a step of 4096 edges from 109 to
+// 101 us.)
 static constexpr int HEAD_ROWS = 4;
 
-__global__ void __launch_bounds__(256) mlp_head_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
-                                                       const float* __restrict__ P, int M, float* __restrict__ z,
-                                                       uint32_t* __restrict__ step_dev) {
-    step_dep();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;
+__global__ void __launch_bounds__(256) mlp_head_loss_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
+                                                            const float* __restrict__ P, const int32_t* __restrict__ rows,
+                                                            int B, int neg, float a, float b, float* __restrict__ dz,
+                                                            float* __restrict__ loss_part, uint32_t* __restrict__ step_dev) {
     const int lane = threadIdx.x & 31;
+    // (the weights are older than the kernel before)
     float w0[MLP_H / 32], w1[MLP_H / 32];
 #pragma unroll
     for (int i = 0; i < MLP_H / 32; ++i) {
@@ -518,80 +677,72 @@ __global__ void __launch_bounds__(256) mlp_head_kernel(const bf16* __restrict__ 
         w1[i] = W3f[MLP_H + lane + 32 * i];
     }
     const float b0 = P[OFF_B3], b1 = P[OFF_B3 + 1];
-    const int64_t warps = (int64_t(gridDim.x) * blockDim.x) >> 5;
-    // M is a multiple of 128, so groups of HEAD_ROWS rows are whole
-    for (int64_t r0 = ((int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * HEAD_ROWS; r0 < M; r0 += warps * HEAD_ROWS) {
-        bf16 h[HEAD_ROWS][MLP_H / 32];
-#pragma unroll
-        for (int u = 0; u < HEAD_ROWS; ++u)
-#pragma unroll
-            for (int i = 0; i < MLP_H / 32; ++i) h[u][i] = H2[(r0 + u) * MLP_H + lane + 32 * i];
-#pragma unroll
-        for (int u = 0; u < HEAD_ROWS; ++u) {
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-            for (int i = 0; i < MLP_H / 32; ++i) {
-                const float x = __bfloat162float(h[u][i]);
-                s0 = fmaf(x, w0[i], s0);
-                s1 = fmaf(x, w1[i], s1);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            }
-            if (lane == 0) {
-                z[2 * (r0 + u)] = s0 + b0;
-                z[2 * (r0 + u) + 1] = s1 + b1;
-            }
-        }
-    }
-}
-
-// UMAP cross-entropy of each edge (head, tail, negatives) on the embedded
-// rows, with Phi = 1 / (1 + a d^b) clamped to [1e-4, 1 - 1e-4] (zero
-// gradient where clamped); loss and dL/dz are divided by the batch size.
-__global__ void mlp_loss_kernel(const float* __restrict__ z, const int32_t* __restrict__ rows, int B, int neg,
-                                float a, float b, float* __restrict__ dz, float* __restrict__ loss_part) {
     step_dep();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *step_dev += 1;
     const int R = 2 + neg;
     const float lo = 1e-4f, hi = 1.0f - 1e-4f, invB = 1.0f / float(B);
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < B; s += gridDim.x * blockDim.x) {
+    const int warps = int((gridDim.x * blockDim.x) >> 5);
+    for (int s = int((blockIdx.x * blockDim.x + threadIdx.x) >> 5); s < B; s += warps) {
         const int64_t r0 = int64_t(s) * R;
-        const float zi0 = z[2 * r0], zi1 = z[2 * r0 + 1];
-        float gi0 = 0.f, gi1 = 0.f, L = 0.f;
-        for (int t = 1; t < R; ++t) {
-            const int64_t r = r0 + t;
-            float g0 = 0.f, g1 = 0.f;
-            if (t >= 2 && rows[r] == rows[r0]) {  // a negative that is the head itself
-                dz[2 * r] = 0.f;
-                dz[2 * r + 1] = 0.f;
-                continue;
+        const int32_t row = lane < R ? rows[r0 + lane] : 0;
+        float z0 = 0.f, z1 = 0.f;  // of row r0 + lane
+        for (int q = 0; q < R; q += HEAD_ROWS) {
+            bf16 h[HEAD_ROWS][MLP_H / 32];
+#pragma unroll
+            for (int u = 0; u < HEAD_ROWS; ++u) {
+                const int64_t r = r0 + (q + u < R ? q + u : R - 1);
+#pragma unroll
+                for (int i = 0; i < MLP_H / 32; ++i) h[u][i] = H2[r * MLP_H + lane + 32 * i];
             }
-            const float d0 = zi0 - z[2 * r], d1 = zi1 - z[2 * r + 1];
+#pragma unroll
+            for (int u = 0; u < HEAD_ROWS; ++u) {
+                float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                for (int i = 0; i < MLP_H / 32; ++i) {
+                    const float x = __bfloat162float(h[u][i]);
+                    s0 = fmaf(x, w0[i], s0);
+                    s1 = fmaf(x, w1[i], s1);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                }
+                if (lane == q + u) {
+                    z0 = s0 + b0;
+                    z1 = s1 + b1;
+                }
+            }
+        }
+        const float d0 = __shfl_sync(0xffffffffu, z0, 0) - z0, d1 = __shfl_sync(0xffffffffu, z1, 0) - z1;
+        const int32_t head = __shfl_sync(0xffffffffu, row, 0);
+        float g0 = 0.f, g1 = 0.f, l = 0.f;
+        if (lane >= 1 && lane < R && !(lane >= 2 && row == head)) {  // (a negative that is the head itself adds nothing)
             const float d = d0 * d0 + d1 * d1;
             const float adb = d > 0.f ? a * powf(d, b) : 0.f;
             const float phi = 1.0f / (1.0f + adb);
             const bool inside = phi > lo && phi < hi;
             const float pc = fminf(fmaxf(phi, lo), hi);
             float dLdd = 0.f;
-            if (t == 1) {
-                L += -logf(pc);
+            if (lane == 1) {
+                l = -logf(pc);
                 if (inside) dLdd = b * adb / (d * (1.0f + adb));  // a b d^(b-1) / (1 + a d^b)
             } else {
-                L += -logf(1.0f - pc);
+                l = -logf(1.0f - pc);
                 if (inside) dLdd = -b / (d * (1.0f + adb));
             }
             g0 = dLdd * 2.0f * d0 * invB;
             g1 = dLdd * 2.0f * d1 * invB;
-            gi0 += g0;
-            gi1 += g1;
-            dz[2 * r] = -g0;
-            dz[2 * r + 1] = -g1;
         }
-        dz[2 * r0] = gi0;
-        dz[2 * r0 + 1] = gi1;
-        loss_part[s] = L * invB;
+        float gi0 = 0.f, gi1 = 0.f, L = 0.f;
+        for (int t = 1; t < R; ++t) {
+            gi0 += __shfl_sync(0xffffffffu, g0, t);
+            gi1 += __shfl_sync(0xffffffffu, g1, t);
+            L += __shfl_sync(0xffffffffu, l, t);
+        }
+        if (lane < R)
+            *reinterpret_cast<float2*>(dz + 2 * (r0 + lane)) = lane == 0 ? make_float2(gi0, gi1) : make_float2(-g0, -g1);
+        if (lane == 0) loss_part[s] = L * invB;
     }
 }
 
@@ -604,69 +755,89 @@ static constexpr int MLP_CHUNK = 512;
 static constexpr int MC_THREADS = 256;
 static constexpr int MC_PITCH = MLP_CHUNK * 4 + 4;  // floats per float4 column: lanes of a row hit distinct banks
 
-// dpre2 = (dz W3) . GELU'(pre2) (BF16) and, over the
-// chunk, db2 = sum dpre2, dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
-static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 64 + MLP_CHUNK * 8;
+// dpre2 = (dz W3) . GELU'(pre2) (BF16) and, over the chunk, db2 = sum dpre2.
+// Loads 64 KB a CTA, a warp per float4 column; one warp then adds while the
+// others write dpre2 from shared memory.  (With dW3's sums and H2's tile in the
+// same CTA, two CTAs an SM and 1.47 rounds of them, 26 us; mlp_w3grad_kernel now
+// runs beside it.)
+static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 8;
 
-__global__ void __launch_bounds__(MC_THREADS, 2)
-mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2,
-                  const bf16* __restrict__ H2, int M, bf16* __restrict__ D,
-                  float* __restrict__ pb2, float* __restrict__ pw3) {
+__global__ void __launch_bounds__(MC_THREADS, 3)
+mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2, int M,
+                  bf16* __restrict__ D, float* __restrict__ pb2) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]: dpre2, float4 columns
-    bf16* s_h = reinterpret_cast<bf16*>(s_v + 8 * MC_PITCH);       // [MLP_CHUNK][32]: H2
-    float2* s_z = reinterpret_cast<float2*>(s_h + MLP_CHUNK * 32);  // [MLP_CHUNK]: dz
-    const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
-    const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
-    step_dep();
-    for (int t = tid; t < rows * 4; t += MC_THREADS) {
-        const int r = t >> 2, i = t & 3;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s_h + r * 32 + 8 * i)),
-                     "l"(H2 + int64_t(r0 + r) * MLP_H + c0 + 8 * i) : "memory");
+    float2* s_z = reinterpret_cast<float2*>(s_v + 8 * MC_PITCH);  // [MLP_CHUNK]: dz
+    const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;  // a multiple of 128
+    float wx[4], wy[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {  // (the weights are older than the kernel before)
+        wx[j] = W3f[c0 + 4 * warp + j];
+        wy[j] = W3f[MLP_H + c0 + 4 * warp + j];
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int r = tid; r < rows; r += MC_THREADS) {
-        const float2 dz2 = *reinterpret_cast<const float2*>(dz + 2 * int64_t(r0 + r));
-        s_z[r] = dz2;
-        const float* p = dgelu2 + blocked_at(r0 + r, c0, MLP_H);
-        float4 x[8];
+    step_dep();
+    for (int r = tid; r < rows; r += MC_THREADS) s_z[r] = *reinterpret_cast<const float2*>(dz + 2 * int64_t(r0 + r));
+    __syncthreads();
+    for (int q = 0; q < rows; q += 128) {
+        const float* p = dgelu2 + blocked_at(r0 + q + lane, c0 + 4 * warp, MLP_H);
+        float4 x[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float4*>(p + i * 512);
-        uint32_t packed[16];
+        for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const float4*>(p + u * 128);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float v[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+        for (int u = 0; u < 4; ++u) {
+            const int r = q + 32 * u + lane;
+            const float2 dz2 = s_z[r];
+            float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int cc = c0 + 4 * i + j;
-                const float g = dz2.x * W3f[cc] + dz2.y * W3f[MLP_H + cc];
+                const float g = dz2.x * wx[j] + dz2.y * wy[j];
                 v[j] = g * v[j];
             }
-            *reinterpret_cast<float4*>(s_v + i * MC_PITCH + 4 * r) = make_float4(v[0], v[1], v[2], v[3]);
-            const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-            packed[2 * i] = *reinterpret_cast<const uint32_t*>(&a);
-            packed[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&b);
+            *reinterpret_cast<float4*>(s_v + warp * MC_PITCH + 4 * r) = make_float4(v[0], v[1], v[2], v[3]);
         }
-        uint4* o = reinterpret_cast<uint4*>(D + int64_t(r0 + r) * MLP_H + c0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) o[i] = make_uint4(packed[4 * i], packed[4 * i + 1], packed[4 * i + 2], packed[4 * i + 3]);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31;
     if (warp == 0) {
         const float* col = s_v + (lane >> 2) * MC_PITCH + (lane & 3);
         float s = 0.f;
 #pragma unroll 16
         for (int r = 0; r < rows; ++r) s += col[4 * r];
         pb2[int64_t(blockIdx.x) * MLP_H + c0 + lane] = s;
-    } else if (warp <= 2) {
-        const int o = warp - 1;
-        const float* zo = reinterpret_cast<const float*>(s_z) + o;
+    } else {
+        for (int t = tid - 32; t < rows * 4; t += MC_THREADS - 32) {  // 16 bytes a lane, four lanes a row
+            const int r = t >> 2, i = t & 3;
+            const float4 f = *reinterpret_cast<const float4*>(s_v + 2 * i * MC_PITCH + 4 * r);
+            const float4 g = *reinterpret_cast<const float4*>(s_v + (2 * i + 1) * MC_PITCH + 4 * r);
+            const __nv_bfloat162 h[4] = {__floats2bfloat162_rn(f.x, f.y), __floats2bfloat162_rn(f.z, f.w),
+                                         __floats2bfloat162_rn(g.x, g.y), __floats2bfloat162_rn(g.z, g.w)};
+            *reinterpret_cast<uint4*>(D + int64_t(r0 + r) * MLP_H + c0 + 8 * i) = *reinterpret_cast<const uint4*>(h);
+        }
+    }
+}
+
+// Over the chunk: dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
+__global__ void __launch_bounds__(MC_THREADS)
+mlp_w3grad_kernel(const float* __restrict__ dz, const bf16* __restrict__ H2, int M, float* __restrict__ pw3) {
+    __shared__ __align__(16) bf16 s_h[MLP_CHUNK * 32];  // H2
+    __shared__ float2 s_z[MLP_CHUNK];                   // dz
+    const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
+    for (int t = tid; t < rows * 4; t += MC_THREADS) {
+        const int r = t >> 2, i = t & 3;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s_h + r * 32 + 8 * i)),
+                     "l"(H2 + int64_t(r0 + r) * MLP_H + c0 + 8 * i) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int r = tid; r < rows; r += MC_THREADS) s_z[r] = *reinterpret_cast<const float2*>(dz + 2 * int64_t(r0 + r));
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (warp < 2) {
+        const float* zo = reinterpret_cast<const float*>(s_z) + warp;
         float s = 0.f;
 #pragma unroll 16
         for (int r = 0; r < rows; ++r) s += zo[2 * r] * __bfloat162float(s_h[r * 32 + lane]);
-        pw3[int64_t(blockIdx.x) * (2 * MLP_H + 2) + o * MLP_H + c0 + lane] = s;
-    } else if (warp == 3 && c0 == 0 && lane < 2) {
+        pw3[int64_t(blockIdx.x) * (2 * MLP_H + 2) + warp * MLP_H + c0 + lane] = s;
+    } else if (warp == 2 && c0 == 0 && lane < 2) {
         const float* zo = reinterpret_cast<const float*>(s_z) + lane;
         float s = 0.f;
 #pragma unroll 16
@@ -817,7 +988,7 @@ __global__ void mlp_init_kernel(float* __restrict__ P, int d, uint32_t k0, uint3
 // activations.
 //
 // The sums are those of the training kernels: column pairs of the head in the
-// order of mlp_head_kernel (partial sums over columns u + 32 i, i ascending, for
+// order of mlp_head_loss_kernel (partial sums over columns u + 32 i, i ascending, for
 // u = 0..31, joined as its shuffles join lanes).
 static constexpr int FE_EPI_WARPS = 16;  // four per TMEM lane quarter
 static constexpr int FE_EPI = FE_EPI_WARPS * 32;
@@ -1055,7 +1226,8 @@ struct MlpBuffers {
     int M;                       // rows of the batch (padded to 128)
     int32_t* rows;
     bf16 *Xb, *H1b, *H2b, *D2b, *D1b;
-    float *dg1, *dg2, *z, *dz, *D1f, *loss_part;
+    int32_t* next_rows;
+    float *dg1, *dg2, *dz, *D1f, *loss_part;
     float *pW2, *pW1, *pb1, *pb2, *pw3;
     float* grad;
     MlpWeights W;
@@ -1071,7 +1243,7 @@ static size_t mlp_batch_bytes(int M) {
     b += Carve::round(m * MLP_IN * 2);                                // Xb
     b += 4 * Carve::round(m * MLP_H * 2);                             // H1b, H2b, D2b, D1b
     b += 3 * Carve::round(m * MLP_H * 4);                             // dg1, dg2, D1f
-    b += 2 * Carve::round(m * 2 * 4) + Carve::round(m * 4);           // z, dz, loss_part
+    b += Carve::round(m * 2 * 4) + 2 * Carve::round(m * 4);           // dz, next_rows, loss_part
     b += Carve::round(size_t(MLP_SPLITS) * MLP_H * MLP_H * 4);        // pW2
     b += Carve::round(size_t(MLP_SPLITS) * MLP_H * MLP_IN * 4);       // pW1
     b += 2 * Carve::round(size_t(nch) * MLP_H * 4);                   // pb1, pb2
@@ -1098,7 +1270,7 @@ static MlpBuffers mlp_carve(void* base, int M) {
     b.dg1 = cv.take<float>(m * MLP_H);
     b.dg2 = cv.take<float>(m * MLP_H);
     b.D1f = cv.take<float>(m * MLP_H);
-    b.z = cv.take<float>(m * 2);
+    b.next_rows = cv.take<int32_t>(m);
     b.dz = cv.take<float>(m * 2);
     b.loss_part = cv.take<float>(m);
     b.pW2 = cv.take<float>(size_t(MLP_SPLITS) * MLP_H * MLP_H);
@@ -1117,15 +1289,14 @@ static MlpBuffers mlp_carve(void* base, int M) {
 
 // Further branches of a training step: dW2 beside dH1 and what follows from
 // it, and the next step's batch.  The batch does not depend on the weights: its
-// rows are drawn beside the backward pass, into the space of z (read last by
-// the losses), and gathered beside the update, when dW1 has read this step's
-// Xb.  In line the two took 27 us of a step (dependent loads from memory, under
+// rows are drawn beside the backward pass and gathered beside the update, when
+// dW1 has read this step's Xb.  In line the two took 27 us of a step (dependent loads from memory, under
 // one warp an SM): a step of 4096 edges went from 160 to 144 us, one of 512
 // from 74 to 58.
 // Without the streams everything runs in line and no batch is prepared.
 struct MlpFork {
     cudaStream_t side = nullptr, ahead = nullptr;
-    cudaEvent_t ev[5] = {};
+    cudaEvent_t ev[6] = {};
     std::function<int(cudaStream_t)> draw, gather;
 };
 
@@ -1149,41 +1320,43 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
                        float* loss_out, const AdamArgs* adam, const MlpFork& fork, cudaStream_t st) {
     const int M = b.M;
     int rc;
-    Gemm F1, F2, DW2, DH1, DW1;
-    if ((rc = gemm_setup(c, F1, b.Xb, b.W.W1b, M, MLP_H, MLP_IN, 128, EPI_GELU, 1))) return rc;
+    Layer F1, F2, DH1;
+    Gemm DW2, DW1;
+    if ((rc = layer_setup(c, F1, b.Xb, b.W.W1b, M, MLP_IN))) return rc;
     F1.g.bias = P + OFF_B1;
     F1.g.dgelu = b.dg1;
     F1.g.out = b.H1b;
-    if ((rc = gemm_setup(c, F2, b.H1b, b.W.W2b, M, MLP_H, MLP_H, 128, EPI_GELU, 1))) return rc;
+    if ((rc = layer_setup(c, F2, b.H1b, b.W.W2b, M, MLP_H))) return rc;
     F2.g.bias = P + OFF_B2;
     F2.g.dgelu = b.dg2;
     F2.g.out = b.H2b;
-    if ((rc = gemm_launch(c, F1, false, st)) || (rc = gemm_launch(c, F2, true, st)) ||
-        (rc = launch_step(c, mlp_head_kernel, dim3(grid_for(M / HEAD_ROWS, 8, c->num_sms * 8)), 256, 0, true, st, b.H2b,
-                          b.W.W3f, P, M, b.z, b.step)) ||
-        (rc = launch_step(c, mlp_loss_kernel, dim3(grid_for(B, 32, c->num_sms * 8)), 32, 0, true, st, b.z, b.rows, B, neg,
-                          a, bb, b.dz, b.loss_part)))
+    if ((rc = layer_launch<false>(c, F1, false, st)) || (rc = layer_launch<false>(c, F2, true, st)) ||
+        (rc = launch_step(c, mlp_head_loss_kernel, dim3(grid_for(B, 8, c->num_sms * 8)), 256, 0, true, st, b.H2b, b.W.W3f,
+                          P, b.rows, B, neg, a, bb, b.dz, b.loss_part, b.step)))
         return rc;
     if (fork.ahead && ((rc = mlp_order(c, fork.ev[0], st, fork.ahead)) || (rc = fork.draw(fork.ahead)))) return rc;
+    // dW3, then dW2 = dpre2^T H1 (K = M, split), on their branch
     const dim3 cgrid(b.n_chunks, MLP_H / 32);
-    if ((rc = launch_step(c, mlp_l3back_kernel, cgrid, MC_THREADS, L3_SMEM, true, st, b.dz, b.W.W3f, b.dg2, b.H2b, M,
-                          b.D2b, b.pb2, b.pw3)))
+    const cudaStream_t side = fork.side ? fork.side : st;
+    if (fork.side && (rc = mlp_order(c, fork.ev[1], st, side))) return rc;
+    if ((rc = launch_step(c, mlp_l3back_kernel, cgrid, MC_THREADS, L3_SMEM, fork.side != nullptr, st, b.dz, b.W.W3f, b.dg2,
+                          M, b.D2b, b.pb2)) ||
+        (rc = launch_step(c, mlp_w3grad_kernel, cgrid, MC_THREADS, 0, false, side, b.dz, b.H2b, M, b.pw3)))
         return rc;
-    // dW2 = dpre2^T H1 (K = M, split)
-    if (fork.side && (rc = mlp_order(c, fork.ev[1], st, fork.side))) return rc;
-    if ((rc = gemm_setup(c, DW2, b.D2b, b.H1b, MLP_H, MLP_H, M, 128, EPI_F32, MLP_SPLITS, true))) return rc;
+    if (fork.side && (rc = mlp_order(c, fork.ev[5], st, side))) return rc;
+    if ((rc = gemm_setup(c, DW2, b.D2b, b.H1b, MLP_H, MLP_H, M, 128, MLP_SPLITS, true))) return rc;
     DW2.g.out_f32 = b.pW2;
-    if ((rc = gemm_launch(c, DW2, false, fork.side ? fork.side : st))) return rc;
+    if ((rc = gemm_launch(c, DW2, false, side))) return rc;
     // dpre1 = (dpre2 W2) . GELU'(pre1): A = dpre2 [M x 256(out)], B = W2^T [256(in) x 256(out)]
-    if ((rc = gemm_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H, MLP_H, 128, EPI_GELU_GRAD, 1))) return rc;
+    if ((rc = layer_setup(c, DH1, b.D2b, b.W.W2tb, M, MLP_H))) return rc;
     DH1.g.dgelu = b.dg1;
     DH1.g.out = b.D1b;
     DH1.g.out_f32 = b.D1f;
-    if ((rc = gemm_launch(c, DH1, fork.side != nullptr, st)) ||
+    if ((rc = layer_launch<true>(c, DH1, fork.side != nullptr, st)) ||
         (rc = launch_step(c, mlp_colsum_kernel, cgrid, MC_THREADS, CS_SMEM, true, st, b.D1f, M, b.pb1)))
         return rc;
     // dW1 = dpre1^T Xb
-    if ((rc = gemm_setup(c, DW1, b.D1b, b.Xb, MLP_H, MLP_IN, M, 64, EPI_F32, MLP_SPLITS, true))) return rc;
+    if ((rc = gemm_setup(c, DW1, b.D1b, b.Xb, MLP_H, MLP_IN, M, 64, MLP_SPLITS, true))) return rc;
     DW1.g.out_f32 = b.pW1;
     if ((rc = gemm_launch(c, DW1, true, st))) return rc;
     if (fork.ahead && ((rc = mlp_order(c, fork.ev[2], st, fork.ahead)) || (rc = fork.gather(fork.ahead)))) return rc;
@@ -1292,7 +1465,7 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
     const uint32_t k0 = uint32_t(mp->seed), k1 = uint32_t(mp->seed >> 32);
 
     MlpFork fork;
-    int32_t* const next_rows = reinterpret_cast<int32_t*>(bu.z);
+    int32_t* const next_rows = bu.next_rows;
     fork.draw = [&](cudaStream_t s) -> int {
         mlp_sample_kernel<<<grid_for(B, 32, c->num_sms * 8), 32, 0, s>>>(row_ptr, col, q, n, nnz, B, neg, bu.step, k0,
                                                                         k1, row_of, next_rows);
