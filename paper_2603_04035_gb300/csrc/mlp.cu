@@ -1296,7 +1296,7 @@ static MlpBuffers mlp_carve(void* base, int M) {
 // Without the streams everything runs in line and no batch is prepared.
 struct MlpFork {
     cudaStream_t side = nullptr, ahead = nullptr;
-    cudaEvent_t ev[6] = {};
+    cudaEvent_t ev[7] = {};
     std::function<int(cudaStream_t)> draw, gather;
 };
 
@@ -1335,7 +1335,7 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
                           P, b.rows, B, neg, a, bb, b.dz, b.loss_part, b.step)))
         return rc;
     if (fork.ahead && ((rc = mlp_order(c, fork.ev[0], st, fork.ahead)) || (rc = fork.draw(fork.ahead)))) return rc;
-    // dW3, then dW2 = dpre2^T H1 (K = M, split), on their branch
+    // dW3, dW2 = dpre2^T H1 (K = M, split) and later db1 on a branch of their own
     const dim3 cgrid(b.n_chunks, MLP_H / 32);
     const cudaStream_t side = fork.side ? fork.side : st;
     if (fork.side && (rc = mlp_order(c, fork.ev[1], st, side))) return rc;
@@ -1352,14 +1352,15 @@ static int mlp_fwd_bwd(Ctx* c, MlpBuffers& b, const float* P, int B, int neg, fl
     DH1.g.dgelu = b.dg1;
     DH1.g.out = b.D1b;
     DH1.g.out_f32 = b.D1f;
-    if ((rc = layer_launch<true>(c, DH1, fork.side != nullptr, st)) ||
-        (rc = launch_step(c, mlp_colsum_kernel, cgrid, MC_THREADS, CS_SMEM, true, st, b.D1f, M, b.pb1)))
-        return rc;
+    if ((rc = layer_launch<true>(c, DH1, fork.side != nullptr, st))) return rc;
+    if (fork.side && (rc = mlp_order(c, fork.ev[2], st, side))) return rc;
     // dW1 = dpre1^T Xb
     if ((rc = gemm_setup(c, DW1, b.D1b, b.Xb, MLP_H, MLP_IN, M, 64, MLP_SPLITS, true))) return rc;
     DW1.g.out_f32 = b.pW1;
-    if ((rc = gemm_launch(c, DW1, true, st))) return rc;
-    if (fork.ahead && ((rc = mlp_order(c, fork.ev[2], st, fork.ahead)) || (rc = fork.gather(fork.ahead)))) return rc;
+    if ((rc = gemm_launch(c, DW1, fork.side != nullptr, st)) ||
+        (rc = launch_step(c, mlp_colsum_kernel, cgrid, MC_THREADS, CS_SMEM, false, side, b.D1f, M, b.pb1)))
+        return rc;
+    if (fork.ahead && ((rc = mlp_order(c, fork.ev[6], st, fork.ahead)) || (rc = fork.gather(fork.ahead)))) return rc;
     if (fork.side && (rc = mlp_order(c, fork.ev[3], fork.side, st))) return rc;
     GradParts gp;
     gp.dW1 = b.pW1;
