@@ -680,7 +680,16 @@ __global__ void __launch_bounds__(NW * 32, epoch_warps_per_sm(PIPE) / NW)
         return;
     }
     const CsrGlobal csr{A.q, A.col, A.row_of};
-    for (int32_t W = int32_t(blockIdx.x) * NW + w; W < n_win; W += int32_t(gridDim.x) * NW)
+    // Single instances in the pipelined form deal the windows out over all CTAs (to
+    // every CTA's first warp first), so that fewer windows than warps load every
+    // SM alike (us an epoch, CTAs of consecutive windows / dealt out: 50,000 rows
+    // 18.8 / 15.9, 60,000 19.3 / 17.5, 130,000 35.5 / 34.4).  Batches keep an
+    // instance's windows together, whose positions stay in L1 (48 us, dealt out
+    // 56), and so does the flat form for large instances (a million rows 193, dealt
+    // out 198).
+    constexpr bool DEAL = PIPE && !BATCHED;
+    const int32_t grid = int32_t(gridDim.x), blk = int32_t(blockIdx.x);
+    for (int32_t W = DEAL ? blk + w * grid : blk * NW + w; W < n_win; W += grid * NW)
         epoch_window<BATCHED, NEG, PIPE, EPOCH_BURST>(A, S, csr, W, lane, s_ej[w], s_hd[w], &s_carry[w], &s_chead[w],
                                                       two_ab, two_b);
 }
@@ -1044,7 +1053,7 @@ int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool
     // small instances 48.0 / 49.8).
     const bool pipe = c->epoch_pipe != 0 && (c->epoch_pipe_set || bat || A.n < EPOCH_FLAT_ROWS);
     const int per_sm = epoch_warps_per_sm(pipe) / warps;
-    const int fgrid = grid_for(A.win_cap, warps, c->num_sms * per_sm);
+    const int fgrid = grid_for(A.win_cap, pipe && !bat ? 1 : warps, c->num_sms * per_sm);
     auto go = [&](auto kernel) -> int {
         // Ask for no more shared memory than the resident CTAs hold (their
         // queues plus the 1 KB the hardware reserves per CTA); the rest of the
@@ -1128,8 +1137,9 @@ static void fill_args(EpochArgs& A, const int32_t* rp, const int32_t* col, const
 // Windows (by capacity) up to which an epoch loop runs as one cooperative launch
 // (epoch_loop_kernel): microseconds an epoch against the chained launches, 15
 // neighbours: 2,000 rows 3.2 / 9.2, 8,000 5.1 / 13.4, 12,000 6.3 / 15.0, 20,000
-// 11.3 / 15.9, 30,000 12.0 / 17.0, 45,000 16.7 / 18.8, 70,000 24.1 / 20.2.
-static constexpr int64_t LOOP_MAX_WINDOWS_PER_SM = 18;
+// 10.9 / 11.5, 30,000 11.8 / 14.2, 35,000 14.5 / 14.5, 40,000 15.1 / 14.7, 50,000
+// 19.0 / 15.9 (35,000 rows are 11.5 windows an SM).
+static constexpr int64_t LOOP_MAX_WINDOWS_PER_SM = 11;
 static constexpr int LOOP_MAX_EPOCHS = 1000000;  // the barrier counts epochs x CTAs in 32 bits
 
 static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float lr0, int t_begin, int t_end, int T,
