@@ -18,8 +18,9 @@
 // 128 queries on 152 SMs leave a quarter of two waves idle, and a batch of
 // 1,000 queries has 8 blocks.  The splits' lists are merged by the re-rank.
 //
-// Bound: the selection (about 250 list insertions a query and split, whose
-// branches a warp of 32 rows takes on most chunks) up to K of about 256, the
+// Bound: the selection (about 250 list insertions a query for the first split
+// and 30 for a later one, whose branches a warp of 32 rows takes on most chunks) up
+// to K of about 256, the
 // tensor pipe and the L2 reads of both operands (48 KB per 128 x 256 x 64
 // step) above.
 #include <cuda.h>
@@ -124,7 +125,8 @@ __global__ void __launch_bounds__(256) wide_stage_kernel(const float* __restrict
                                                          int64_t n, int64_t n_pad, int d, int K,
                                                          const float* __restrict__ mean,
                                                          unsigned int* __restrict__ maxbits, op16* __restrict__ out,
-                                                         float* __restrict__ norm, float* __restrict__ resid) {
+                                                         float* __restrict__ norm, float* __restrict__ resid,
+                                                         int32_t* __restrict__ bound) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
     const float S = operand_scale<true>(maxbits), inv_S = 1.0f / S;
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(256) wide_stage_kernel(const float* __restrict
             if (QUERY) {
                 norm[i] = sq * S * S;
                 resid[i] = delta;
+                bound[i] = 0x7F800000;  // +inf (an ordered_key)
             } else {
                 nmax = fmaxf(nmax, sq * S * S);
                 rmax = fmaxf(rmax, delta);
@@ -187,12 +190,16 @@ __global__ void __launch_bounds__(256) wide_stage_kernel(const float* __restrict
 }
 
 // ------------------------------------------------------------------ GEMM + select
+// A float as an integer of the same order (its own inverse on the bits).
+__device__ __forceinline__ int32_t ordered_key(int32_t bits) { return bits ^ ((bits >> 31) & 0x7FFFFFFF); }
+
 struct WideParams {
     int64_t nq;
     int n_tiles, kch, tiles_per_split;
     int32_t* cand_idx;   // [split][n queries padded][TC_KP]
     float* cand_s;
     int64_t nq_pad;
+    int32_t* bound;      // [n queries]: the splits' common bound, an ordered_key (null: one split)
     int* status;
     unsigned long long* tiles_done;  // += tiles this CTA multiplies (null: not counted)
 };
@@ -314,10 +321,26 @@ knn_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         for (int j = 0; j < TC_NQ; ++j) q_mine[j] = INFINITY;
         asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI_WARPS * 32) : "memory");
         int qn = 0;
-        auto row_bound = [&]() { return list_bound(L, q_other); };
-        auto flush = [&]() { list_merge(L, I, qn, q, qb, q_mine); };
+        // A split's lists start empty, and a list of 32 from N columns in random
+        // order takes about 32 (1 + ln(N / 32)) insertions.  Its bound on the row's
+        // 32nd-best value holds for the other splits too, so each merge
+        // publishes it and every tile starts from the smallest published: a later
+        // split inserts little (the kernel at 30,000 x 200, 3 splits: 690 to 526 us).
+        // A value between the row's 32nd best and a stale bound is queued in vain.
+        int32_t* const bound = P.bound && q0 + row < P.nq ? P.bound + q0 + row : nullptr;
+        float known = INFINITY;
+        auto row_bound = [&]() { return fminf(list_bound(L, q_other), known); };
+        auto flush = [&]() {
+            list_merge(L, I, qn, q, qb, q_mine);
+            const float b = list_bound(L, q_other);
+            if (bound && b < known) {
+                known = b;
+                atomicMin(bound, ordered_key(__float_as_int(b)));
+            }
+        };
         for (int t = 0; t < nt; ++t) {
             const int buf = t & 1, use = t >> 1;
+            if (bound) known = fminf(known, __int_as_float(ordered_key(*static_cast<volatile int32_t*>(bound))));
             if (!mbar_wait(&acc_full[buf], use & 1, abort_flag, P.status)) break;
             tc_fence_after();
             const uint32_t tbase = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * WD_BN + half * 128);
@@ -365,9 +388,14 @@ knn_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 // candidate over the dimensions in order, 32 dimensions at a time staged by
 // asynchronous copies into two alternating buffers, and a bitonic network
 // orders the candidates by (distance, index).
+//
+// V floats a copy and a read, 4 or 2 where d and the matrices' alignment allow
+// it: with one, the load/store pipe bounds it (30,000 x 200: 167 us; with four
+// 115, 6.7 TB/s of the candidates' rows from L2).  The pitch keeps the lanes' reads of 32 rows on distinct banks.
 static constexpr int WR_WARPS = 4;
-static constexpr int WR_PITCH = 33;
+constexpr int wr_pitch(int v) { return v == 4 ? 36 : 32 + v; }
 
+template <int V>
 __global__ void __launch_bounds__(WR_WARPS * 32)
 wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const float* __restrict__ Q, bool separate,
                    const int64_t* __restrict__ rows, int64_t nq, int64_t nq_pad, int splits,
@@ -375,8 +403,9 @@ wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const f
                    const float* __restrict__ norm, const float* __restrict__ resid,
                    const unsigned int* __restrict__ maxbits, float eps_rel, int32_t* __restrict__ idx_out,
                    float* __restrict__ dist_out, int32_t* __restrict__ fail_rows, int32_t* __restrict__ fail_count) {
-    __shared__ float s_rows[WR_WARPS][2][32 * WR_PITCH];
-    __shared__ float s_q[WR_WARPS][2][32];
+    constexpr int PITCH = wr_pitch(V), PER = 32 / V;  // copies a row of 32 dimensions
+    __shared__ __align__(16) float s_rows[WR_WARPS][2][32 * PITCH];
+    __shared__ __align__(16) float s_q[WR_WARPS][2][32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float n_max = __uint_as_float(maxbits[0]), r_max = __uint_as_float(maxbits[1]);
     const float S = operand_scale<true>(maxbits);
@@ -409,16 +438,18 @@ wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const f
         const float* xq = Q + qi * d;
         const int cv = valid ? ci : -1;
         auto stage = [&](int c0, int buf) {
-            const int c = c0 + lane;
-            if (c < d)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(&s_q[w][buf][lane])),
-                             "l"(xq + c) : "memory");
+            const int c = c0 + V * (lane % PER);
+            if (lane < PER && c < d)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(&s_q[w][buf][V * lane])),
+                             "l"(xq + c), "n"(4 * V) : "memory");
 #pragma unroll 8
-            for (int t = 0; t < 32; ++t) {
+            for (int t0 = 0; t0 < 32; t0 += V) {
+                const int t = t0 + lane / PER;
                 const int ct = __shfl_sync(0xffffffffu, cv, t);
                 if (ct >= 0 && c < d)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(
-                                     &s_rows[w][buf][t * WR_PITCH + lane])), "l"(X + int64_t(ct) * d + c) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(
+                                     &s_rows[w][buf][t * PITCH + V * (lane % PER)])), "l"(X + int64_t(ct) * d + c),
+                                 "n"(4 * V) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
@@ -434,11 +465,16 @@ wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const f
             __syncwarp();
             if (valid) {
                 const int cc = d - c0 < 32 ? d - c0 : 32;
-                const float* row = &s_rows[w][buf][lane * WR_PITCH];
+                const float* row = &s_rows[w][buf][lane * PITCH];
 #pragma unroll 8
-                for (int c = 0; c < cc; ++c) {
-                    const float df = s_q[w][buf][c] - row[c];
-                    a = fmaf(df, df, a);
+                for (int c = 0; c < cc; c += V) {
+                    struct alignas(4 * V) Vec { float v[V]; };
+                    const Vec x = *reinterpret_cast<const Vec*>(&s_q[w][buf][c]), y = *reinterpret_cast<const Vec*>(row + c);
+#pragma unroll
+                    for (int u = 0; u < V; ++u) {
+                        const float df = x.v[u] - y.v[u];
+                        a = fmaf(df, df, a);
+                    }
                 }
             }
             __syncwarp();  // the buffer is refilled two steps later
@@ -569,10 +605,10 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     wide_mean_kernel<<<(d + 31) / 32, dim3(32, 8), 0, st>>>(partial, blocks, db_blocks, n, d, mean, maxbits);
     DRGB_CHECK_LAUNCH(c);
     wide_stage_kernel<false><<<grid_for(w.n_pad, 8, c->num_sms * 8), 256, 0, st>>>(X, nullptr, n, w.n_pad, d, w.K, mean,
-                                                                                  maxbits, XB, nullptr, nullptr);
+                                                                                  maxbits, XB, nullptr, nullptr, nullptr);
     DRGB_CHECK_LAUNCH(c);
     wide_stage_kernel<true><<<grid_for(w.nq_pad, 8, c->num_sms * 8), 256, 0, st>>>(Q, rows, nq, w.nq_pad, d, w.K, mean,
-                                                                                  maxbits, XA, norm, resid);
+                                                                                  maxbits, XA, norm, resid, fail_rows);
     DRGB_CHECK_LAUNCH(c);
     CUtensorMap mA, mB;
     if ((rc = make_map_k64(c, &mA, XA, w.nq_pad, w.K, WD_BM, true))) return rc;
@@ -586,6 +622,7 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     P.cand_idx = cand_idx;
     P.cand_s = cand_s;
     P.nq_pad = w.nq_pad;
+    P.bound = w.splits > 1 ? fail_rows : nullptr;  // (nothing has failed yet)
     P.status = c->d_status;
     P.tiles_done = nullptr;
     if (graph) {
@@ -602,7 +639,9 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     // largest magnitude, which is at most n_j + 2 |x_i| |x_j| <= 2 (n_i + n_max):
     // 34 * 2^-23 (n_i + n_max) a step, plus the FP32 norms' own error
     const float eps_rel = float(w.K / 16) * 34.0f * 1.1920929e-7f + 7.6293945e-6f;
-    wide_rerank_kernel<<<grid_for(nq, WR_WARPS, c->num_sms * 6), WR_WARPS * 32, 0, st>>>(
+    auto whole = [&](int v) { return d % v == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Q)) & (4 * v - 1)) == 0; };
+    auto rerank = whole(4) ? wide_rerank_kernel<4> : whole(2) ? wide_rerank_kernel<2> : wide_rerank_kernel<1>;
+    rerank<<<grid_for(nq, WR_WARPS, c->num_sms * 6), WR_WARPS * 32, 0, st>>>(
         X, n, d, k, Q, separate, rows, nq, w.nq_pad, w.splits, cand_idx, cand_s, norm, resid, maxbits, eps_rel,
         idx_out, dist_out, defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count);
     DRGB_CHECK_LAUNCH(c);
