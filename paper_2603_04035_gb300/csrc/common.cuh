@@ -173,6 +173,34 @@ __device__ __forceinline__ int64_t mulshift_index(uint32_t u, int64_t n) {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A chain of short kernels launched with launch_dep: each is scheduled while the
+// one before drains and waits in dep_enter, before its first access to memory
+// that an earlier one writes.  Only then may the next one start, so at most two
+// kernels of the chain are resident, and whatever came before the previous one is
+// complete when a kernel starts.
+__device__ __forceinline__ void dep_enter() {
+    grid_dep_wait();
+    grid_dep_launch();
+}
+
+// Launch with (dep) or without a programmatic dependency on the kernel before.
+template <class... P, class... A>
+int launch_dep(Ctx* c, void (*kernel)(P...), dim3 grid, int block, size_t smem, bool dep, cudaStream_t st,
+               const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dep ? 1 : 0;
+    DRGB_CUDA(c, cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+    return DRGB_OK;
+}
+
 inline int grid_for(int64_t work, int per_block, int max_blocks) {
     int64_t g = (work + per_block - 1) / per_block;
     if (g < 1) g = 1;

@@ -204,6 +204,7 @@ __global__ void __launch_bounds__(256) pca_cmul_kernel(const float* __restrict__
                                                        float gamma, int L, float* __restrict__ Y) {
     __shared__ __align__(16) float Xs[PCA_KCHUNK][PCA_P];
     __shared__ float Cs[PCA_CROWS][PCA_KCHUNK + 1];
+    dep_enter();
     const int a0 = blockIdx.x * PCA_CROWS, b0 = blockIdx.y * PCA_KCHUNK;
     const int kb = D - b0 < PCA_KCHUNK ? D - b0 : PCA_KCHUNK;
     // all of a thread's loads are issued before any is stored, so the block
@@ -275,6 +276,7 @@ __global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__
                                                        unsigned int* __restrict__ counters, double* __restrict__ G) {
     __shared__ float As[PCA_GCHUNK][PCA_P + 1];
     __shared__ float Bs[PCA_GCHUNK][PCA_P + 1];
+    dep_enter();
     const int m = PCA_P - L;
     const int a0 = blockIdx.y * PCA_GCHUNK;
     const int rows = D - a0 < PCA_GCHUNK ? D - a0 : PCA_GCHUNK;
@@ -328,6 +330,7 @@ __global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__
 // active column.
 __global__ void pca_resid_kernel(const float* __restrict__ Y, const float* __restrict__ W,
                                  const float* __restrict__ theta, int D, int L, double* __restrict__ rn) {
+    dep_enter();
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (j >= PCA_P - L) return;
     const int k = L + j;
@@ -367,6 +370,7 @@ __global__ void __launch_bounds__(256) pca_apply_kernel(const float* __restrict_
                                                         const float* __restrict__ M, int L, float* __restrict__ Y) {
     __shared__ __align__(16) float Ms[PCA_P][PCA_P];
     __shared__ float Xs[PCA_TROWS][PCA_P + 1];
+    dep_enter();
     const int m = PCA_P - L, a0 = blockIdx.x * PCA_TROWS;
 #pragma unroll
     for (int u = 0; u < PCA_P * PCA_P / 256; ++u) {
@@ -400,6 +404,7 @@ __global__ void __launch_bounds__(256) pca_ortho_kernel(const float* __restrict_
                                                         const int* __restrict__ mode, float* __restrict__ Y) {
     __shared__ __align__(16) float Ts[PCA_P][PCA_P];
     __shared__ float Xs[PCA_TROWS][PCA_P + 1];
+    dep_enter();
     const int a0 = blockIdx.x * PCA_TROWS, solve = *mode == 0;
 #pragma unroll
     for (int u = 0; u < PCA_P * PCA_P / 256; ++u) {
@@ -603,6 +608,7 @@ static constexpr size_t PCA_CHOL_SMEM = size_t(2) * PCA_P * PCA_P * sizeof(doubl
 __global__ void __launch_bounds__(PCA_CHOL_THREADS) pca_chol_kernel(const double* __restrict__ G, int L, int pass,
                                                                    int* __restrict__ flags, float* __restrict__ T) {
     extern __shared__ double csm[];
+    dep_enter();
     const int m = PCA_P - L;
     const int tid = threadIdx.x, nt = blockDim.x;
     if (pass > 0 && flags[0] == 0) {  // Newton-Schulz step
@@ -739,6 +745,7 @@ __global__ void __launch_bounds__(PCA_JAC_THREADS) pca_jacobi_kernel(const doubl
     __shared__ float s_thr;
     __shared__ int s_rot;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    dep_enter();
     for (int t = tid; t < m * m; t += blockDim.x) {
         const int i = t / m, j = t - i * m;
         double a = 0.0, b = 0.0;
@@ -979,21 +986,16 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
         int L = 0;  // locked (converged and deflated) leading pairs
         const int nks = (D + PCA_KCHUNK - 1) / PCA_KCHUNK;
         auto cmul = [&](const float* A, const float* Zz, double al, double be, double ga, float* B) -> int {
-            pca_cmul_kernel<<<dim3(crows, nks), 256, 0, st>>>(C, D, A, cpart, counters, Zz, float(al), float(be), float(ga),
-                                                             L, B);
-            DRGB_CHECK_LAUNCH(c);
-            return DRGB_OK;
+            return launch_dep(c, pca_cmul_kernel, dim3(crows, nks), 256, 0, true, st, C, D, A, cpart, counters, Zz,
+                              float(al), float(be), float(ga), L, B);
         };
         auto gram = [&](const float* A, const float* B) -> int {
             const int m = P - L;
-            pca_gram_kernel<<<dim3((P * m + 255) / 256, nch), 256, 0, st>>>(A, B, D, L, Gd, counters + crows, Gsum);
-            DRGB_CHECK_LAUNCH(c);
-            return DRGB_OK;
+            return launch_dep(c, pca_gram_kernel, dim3((P * m + 255) / 256, nch), 256, 0, true, st, A, B, D, L, Gd,
+                              counters + crows, Gsum);
         };
         auto apply = [&](const float* A, float* B) -> int {
-            pca_apply_kernel<<<tblk, 256, 0, st>>>(A, D, Md, L, B);
-            DRGB_CHECK_LAUNCH(c);
-            return DRGB_OK;
+            return launch_dep(c, pca_apply_kernel, dim3(tblk), 256, 0, true, st, A, D, Md, L, B);
         };
         // orthonormalise the active columns against the locked ones and among
         // themselves: Cholesky QR twice, three times after a shifted factor
@@ -1001,10 +1003,10 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
             for (int pass = 0; pass < 3; ++pass) {
                 int r = gram(A, A);
                 if (r) return r;
-                pca_chol_kernel<<<1, PCA_CHOL_THREADS, PCA_CHOL_SMEM, st>>>(Gsum, L, pass, dflags, Md);
-                DRGB_CHECK_LAUNCH(c);
-                pca_ortho_kernel<<<tblk, 256, 0, st>>>(A, D, Md, dflags + PCA_MODE, tmp);
-                DRGB_CHECK_LAUNCH(c);
+                if ((r = launch_dep(c, pca_chol_kernel, dim3(1), PCA_CHOL_THREADS, PCA_CHOL_SMEM, true, st, Gsum, L, pass,
+                                    dflags, Md)) ||
+                    (r = launch_dep(c, pca_ortho_kernel, dim3(tblk), 256, 0, true, st, A, D, Md, dflags + PCA_MODE, tmp)))
+                    return r;
                 std::swap(A, tmp);
             }
             return DRGB_OK;
@@ -1017,11 +1019,12 @@ int pca_run(Ctx* c, const float* X, int64_t n, int D, int dim, float* Z, float* 
             const int m = P - L;
             int r = cmul(Xb, nullptr, 1.0, 0.0, 0.0, Zb);
             if (r || (r = gram(Xb, Zb))) return r;
-            pca_jacobi_kernel<<<1, PCA_JAC_THREADS, 0, st>>>(Gsum, 1, 0, m, L, m, Md, m, L, 1, thf, rr_out);
-            DRGB_CHECK_LAUNCH(c);
-            if ((r = apply(Xb, Yb)) || (r = apply(Zb, Wb))) return r;
-            pca_resid_kernel<<<(m * 32 + 255) / 256, 256, 0, st>>>(Yb, Wb, thf, D, L, rr_out + P);
-            DRGB_CHECK_LAUNCH(c);
+            if ((r = launch_dep(c, pca_jacobi_kernel, dim3(1), PCA_JAC_THREADS, 0, true, st, Gsum, 1, 0, m, L, m, Md, m, L, 1,
+                                thf, rr_out)) ||
+                (r = apply(Xb, Yb)) || (r = apply(Zb, Wb)) ||
+                (r = launch_dep(c, pca_resid_kernel, dim3((m * 32 + 255) / 256), 256, 0, true, st, Yb, Wb, thf, D, L,
+                                rr_out + P)))
+                return r;
             DRGB_CUDA(c, cudaMemcpyAsync(hr.data(), rr_out, size_t(2) * P * 8, cudaMemcpyDeviceToHost, st));
             DRGB_CUDA(c, cudaMemcpyAsync(hflags, dflags, sizeof(hflags), cudaMemcpyDeviceToHost, st));
             DRGB_CUDA(c, cudaStreamSynchronize(st));
