@@ -63,6 +63,7 @@ struct ScanArgs {
     int32_t* idx;
     float* dist;
     bool partial;
+    int32_t* bound;          // partial: [n_rows], the chunks' common bound as float bits (nullable)
     // cells: see launch_knn_cells
     CellScan cells;
     // ranks: targets and their squared distances (n_rows x k), counts added to
@@ -88,6 +89,7 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return r;
 }
 
+static constexpr int32_t SC_UNBOUND = 0x7F7F7F7F;  // no bound published yet (every byte the same)
 static constexpr int SC_RANK_FEW = 24;  // points near enough to matter up to which they are walked one by one
 static constexpr int SC_BULK = 6;  // candidates of 32 from which sorting them beats inserting them one by one
 
@@ -244,6 +246,15 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
+        // The chunks' lists all start empty; a chunk's k-th distance bounds the
+        // row's, so each chunk publishes its own and a tile admits nothing beyond the
+        // smallest (points at the same distance are admitted: the index decides).
+        // Read here, a lane per row of the warp, before the tile's distances.
+        float known = INFINITY;
+        if (MODE == SCAN_NEAREST && A.bound && ch == nch - 1 && lane < SC_ROWS && r0 + warp * SC_ROWS + lane < n_rows) {
+            const int32_t b = *static_cast<volatile int32_t*>(A.bound + r0 + warp * SC_ROWS + lane);
+            if (b != SC_UNBOUND) known = __int_as_float(b);
+        }
         const int c0 = ch * SC_DC;
         const int cc = d - c0 < SC_DC ? d - c0 : SC_DC;
         const float* xs = s_x + (st & 1) * SC_DC * SC_PITCH + 4 * tx;
@@ -335,7 +346,10 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                     }
                     if (lane < k) s_cnt[q * kl + lane] += mine;  // (the warp's own rows)
                 } else {
-                    const float thr = ld[k - 1];
+                    const float shared_k = MODE == SCAN_NEAREST ? __shfl_sync(0xffffffffu, known, rr) : INFINITY;
+                    // (just above it, and no subnormal)
+                    const float thr = shared_k < INFINITY
+                        ? fminf(ld[k - 1], fmaxf(__int_as_float(__float_as_int(shared_k) + 1), 1.17549435e-38f)) : ld[k - 1];
                     const float m = fminf(fminf(v[0], v[1]), fminf(v[2], v[3]));  // ignores the NaN marks
                     if (!__any_sync(0xffffffffu, m < thr)) continue;
                     float D = lane < kl ? ld[lane] : INFINITY;
@@ -399,6 +413,8 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
                         ld[lane] = D;
                         li[lane] = I;
                     }
+                    if (MODE == SCAN_NEAREST && A.bound && lane == k - 1 && D < shared_k && r0 + q < n_rows)
+                        atomicMin(A.bound + r0 + q, __float_as_int(D));
                     __syncwarp();
                 }
             }
@@ -541,7 +557,7 @@ static int scan_chunks(const Ctx* c, int64_t n_rows, int64_t n, int k, size_t pa
 
 size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
     const int C = scan_chunks(c, n_rows, n, k, ~size_t(0) >> 1, true);
-    return C > 1 ? 2 * (size_t(n_rows) * C * k * 4 + 512) : 0;
+    return C > 1 ? 2 * (size_t(n_rows) * C * k * 4 + 512) + size_t(n_rows) * 4 + 512 : 0;
 }
 
 template <int MODE>
@@ -571,6 +587,10 @@ static int scan_nearest(Ctx* c, ScanArgs& A, int32_t* idx_out, float* dist_out, 
     A.idx = cv.take<int32_t>(size_t(A.n_rows) * C * A.k);
     A.dist = cv.take<float>(size_t(A.n_rows) * C * A.k);
     A.partial = true;
+    // with room beside the lists the chunks share their bounds
+    const size_t lists_end = size_t(reinterpret_cast<char*>(cv.take<char>(0)) - static_cast<char*>(part));
+    A.bound = lists_end + size_t(A.n_rows) * 4 <= part_bytes ? cv.take<int32_t>(A.n_rows) : nullptr;
+    if (A.bound) DRGB_CUDA(c, cudaMemsetAsync(A.bound, SC_UNBOUND & 0xFF, size_t(A.n_rows) * 4, st));
     int rc = scan_launch<SCAN_NEAREST>(c, A, C, st);
     if (rc) return rc;
     const int lists = int((A.n + A.chunk - 1) / A.chunk);
