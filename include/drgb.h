@@ -149,7 +149,8 @@ int64_t drgb_launch_count(const drgb_ctx* ctx);
  *   DRGB_TUNE_EPOCH_PIPE      form of the epoch's force kernel: 1 (default)
  *                             pipelined (a warp keeps two groups of gathers in
  *                             flight, 24 warps per SM), 0 flat (one group, 40
- *                             warps per SM)
+ *                             warps per SM); until it is set, single instances
+ *                             of 200,000 to 9 million rows take the flat form
  * Returns DRGB_ERR_INVALID for an unknown parameter or value. */
 #define DRGB_TUNE_EPOCH_WARPS 1
 #define DRGB_TUNE_EPOCH_PIPE 2
@@ -199,8 +200,10 @@ int drgb_stage_times(drgb_ctx* ctx, float* ms, int max);
  *            excluded), ordered by FP32 squared distance sum_c (x_ic - x_jc)^2
  *            evaluated directly (not by the expansion), ties by lower index.
  *   dist_out n x k FP32 Euclidean distances (square roots), same order.
- * mode: 0 auto (3 when n >= 4096, d <= 61, k < 32; else 1), 1 exact FP32
- * SIMT scan, 2 BF16 tcgen05 distance GEMM with a fused top-32 selection and
+ * mode: 0 auto (for k < 32: 3 when d <= 61 and n > 14000; else a product over
+ * all points with FP16 operands, its candidates re-ranked and certified as in
+ * mode 3, when 16 <= d <= 1021, n >= 1024 and n n d >= 1.5e8; else 3 when n >=
+ * 4096 and d <= 61; else 1), 1 exact FP32 SIMT scan, 2 BF16 tcgen05 distance GEMM with a fused top-32 selection and
  * an FP32 re-rank, 3 the same GEMM with FP16 operands (power-of-two scaled;
  * 8x smaller rounding residual at the same tensor-core rate).  In modes 2
  * and 3, rows whose candidate set cannot be certified to contain the exact

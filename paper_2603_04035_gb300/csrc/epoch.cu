@@ -1034,7 +1034,7 @@ __global__ void __launch_bounds__(LOOP_WARPS * 32, loop_ctas_per_sm(LOOP_WARPS))
     }
 }
 
-static constexpr int64_t EPOCH_FLAT_ROWS = 200000;
+static constexpr int64_t EPOCH_FLAT_ROWS = 200000, EPOCH_FLAT_ROWS_END = 9000000;
 
 bool epoch_warps_supported(int warps) { return warps == 4 || warps == 8; }
 
@@ -1047,11 +1047,13 @@ int launch_epoch(Ctx* c, const EpochArgs& A_in, int warps, cudaStream_t st, bool
     philox_round_keys(A.k0, A.k1, A.rk);
     const bool bat = A.count > 0, n5 = A.neg == 5 && A.b > 0.f;
     // Untuned, a large single instance takes the flat form: its gathers miss L1,
-    // and 40 warps an SM hide that better than 24 with two groups each (us an
-    // epoch, pipelined / flat: 70,000 rows 19.5 / 26.6, 130,000 35.7 / 36.6,
-    // 250,000 65.4 / 60.8, a million 208.5 / 197.3, two million 396 / 380; batches of
-    // small instances 48.0 / 49.8).
-    const bool pipe = c->epoch_pipe != 0 && (c->epoch_pipe_set || bat || A.n < EPOCH_FLAT_ROWS);
+    // and 40 warps an SM hide that better than 24 with two groups each, until the
+    // gathers miss L2 as well, between 8 and 10 million rows (us an
+    // epoch, pipelined / flat: 70,000 rows 19.1 / 26.6, 130,000 34.0 / 36.4, 250,000
+    // 58.3 / 55.0, a million 213 / 204, eight million 1,708 / 1,632, ten million 2,282 /
+    // 2,371; batches of small instances 48.0 / 49.8).
+    const bool pipe = c->epoch_pipe != 0 &&
+                      (c->epoch_pipe_set || bat || A.n < EPOCH_FLAT_ROWS || A.n >= EPOCH_FLAT_ROWS_END);
     const int per_sm = epoch_warps_per_sm(pipe) / warps;
     const int fgrid = grid_for(A.win_cap, pipe && !bat ? 1 : warps, c->num_sms * per_sm);
     auto go = [&](auto kernel) -> int {

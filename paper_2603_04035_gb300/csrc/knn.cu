@@ -16,10 +16,10 @@
 // pairs of points and dimension.  The earlier form, one thread per query with
 // its whole list in registers, filled the GPU only from about 80,000 queries
 // on; splitting the database over blockIdx.y fills it from a few hundred, and
-// the partial lists are merged afterwards.  Measured, earlier form -> this
-// one: 5,003 queries against 70,000 x 50 (with the layout of the new points)
-// 28.2 -> 2.9 ms; 3,000 ranks and neighbours of 20,011 x 50 40.2 -> 2.4 ms;
-// all pairs of 30,011 x 200 40.5 -> 22.5 ms; a 2,000 x 50 fit 2.60 -> 2.00 ms.
+// the partial lists are merged afterwards.  Measured, earlier form -> this one:
+// 3,000 ranks and neighbours of 20,000 x 50 and its 2-D image 40.2 -> 2.4 ms, and
+// 1.36 with the lists below and wider searches on the tensor cores (knn_wide.cu);
+// all pairs of 30,011 x 200 40.5 -> 22.5 ms.
 #include "common.cuh"
 #include "knn.cuh"
 
