@@ -200,7 +200,7 @@ int drgb_stage_times(drgb_ctx* ctx, float* ms, int max);
  *            excluded), ordered by FP32 squared distance sum_c (x_ic - x_jc)^2
  *            evaluated directly (not by the expansion), ties by lower index.
  *   dist_out n x k FP32 Euclidean distances (square roots), same order.
- * mode: 0 auto (for k < 32: 3 when d <= 61 and n > 14000; else a product over
+ * mode: 0 auto (for k < 32: 3 when d <= 61 and n > 16000; else a product over
  * all points with FP16 operands, its candidates re-ranked and certified as in
  * mode 3, when 16 <= d <= 1021, n >= 1024 and n n d >= 1.5e8; else 3 when n >=
  * 4096 and d <= 61; else 1), 1 exact FP32 SIMT scan, 2 BF16 tcgen05 distance GEMM with a fused top-32 selection and

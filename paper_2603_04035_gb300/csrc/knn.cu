@@ -855,12 +855,12 @@ namespace drgb {
 
 int knn_resolve_mode(int64_t n, int d, int k, int mode) {
     if (mode != 0) return mode;
-    // The cell-ordered product (knn_tc) spends about 150 us on the order and
-    // its bounds, and wins from about 14,000 rows on (10 clusters in 50
-    // dimensions; wide / cells: 4,096 rows 126 / 234 us, 8,000 175 / 256,
-    // 16,000 295 / 287, 30,000 786 / 429; 100 clusters: 297 / 434 at 16,000,
-    // 1,237 / 1,176 at 40,000).
-    if (knn_tc_preferred(n, d, k) && (n > 14000 || !knn_wide_preferred(n, n, d, k))) return 3;
+    // The cell-ordered product (knn_tc) spends about 150 us on the order and its
+    // bounds, and wins from about 16,000 rows on where clusters are few (10 in 50
+    // dimensions, wide / cells us: 8,000 rows 184 / 294, 16,000 306 / 312, 20,000
+    // 403 / 343, 30,000 633 / 466; 100 clusters, more than cells at these sizes: 308 /
+    // 417 at 16,000, 933 / 1,266 at 40,000).
+    if (knn_tc_preferred(n, d, k) && (n > 16000 || !knn_wide_preferred(n, n, d, k))) return 3;
     return knn_wide_preferred(n, n, d, k) ? KNN_WIDE : 1;
 }
 
