@@ -666,12 +666,12 @@ def roofline(args, n, d, nnz, updates, stage_acc, steps, peaks, peak_src, T, til
     mhz = float(peaks.get("sm_max_mhz", 2070.0))
     peak = SM_COUNT * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12
     achieved = flops / (knn_ms / 1e3) / 1e12
-    return {"kernel": "knn_exact_kernel", "bound": "alu", "achieved": achieved, "peak": peak,
+    return {"kernel": "scan_kernel", "bound": "alu", "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak,
             "peak_source": f"FP32 FMA: {SM_COUNT} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x "
                            f"{mhz:.0f} MHz ({peak_src} clock)",
             "flops_per_launch": flops, "launch_ms": knn_ms,
-            "traffic": kernel_traffic("knn_exact_kernel", "paper_2603_04035_gb300/csrc/knn.cu", args.workload)}
+            "traffic": kernel_traffic("scan_kernel", "paper_2603_04035_gb300/csrc/knn.cu", args.workload)}
 
 
 # ---------------------------------------------------------------- batched form

@@ -1,6 +1,7 @@
 // Initialisation and the synchronous SGD epoch (the method's per-epoch step:
 // attraction along active CSR entries, repulsion from Philox negatives, clip
-// to +-4, Y' = Y + lr g), plus the epoch loop replayed as a CUDA graph.
+// to +-4, Y' = Y + lr g), plus the epoch loop: one cooperative launch for small
+// graphs, else a CUDA graph of one launch per epoch.
 //
 // Layout: Y is n x 2 FP32 read as float2 (one 8-byte gather per point); the
 // CSR is head-sorted (row_ptr int32, col int32, q uint32 schedule words).

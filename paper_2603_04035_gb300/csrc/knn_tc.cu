@@ -17,7 +17,7 @@
 // GEMM + select (A2): one CTA owns 128 query rows (TMEM lanes) and streams the
 // database tiles of 256 rows that its cell schedule admits (points are staged
 // in the spatial cell order of knn_order.cu; see knn_tc_kernel for the cell
-// bounds).  Warp 0 issues TMA loads into a 4-stage ring,
+// bounds).  Warp 0 issues TMA loads into a 3-stage ring,
 // warp 1 issues 4 MMAs (M128 N256 K16) per tile into one of two TMEM
 // accumulators, and 8 epilogue warps (two per TMEM lane quarter, one per
 // column half) read the accumulator with tcgen05.ld, reject a 32-column chunk
