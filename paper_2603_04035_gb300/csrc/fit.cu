@@ -1,8 +1,9 @@
 // fit_transform(X) -> Y: the whole hot path on one stream (Section 2.1, the
 // public API; Section 3, the timed fit_transform).  [PCA to pca_dim ->] k-NN
-// graph -> fuzzy graph -> a, b -> initialisation -> T epochs (one captured
-// graph), all enqueued before the single synchronisation at the end (the
-// optional PCA synchronises on its own first).
+// graph -> fuzzy graph -> a, b -> initialisation -> T epochs (one cooperative
+// launch, or one captured graph), all enqueued before the synchronisation at the
+// end; a tensor-core k-NN reads its count of uncertified rows before that, and the
+// optional PCA synchronises on its own first.
 #include "common.cuh"
 #include "epoch.cuh"
 #include "graph.cuh"
