@@ -128,16 +128,19 @@ int drgb_wait_selftest(drgb_ctx* ctx, int64_t limit_us, int32_t arrive, void* st
 int drgb_gather_probe(drgb_ctx* ctx, const float* Y, int64_t n, int32_t rounds, uint32_t seed,
                       double* gathers_per_s, void* stream);
 
-/* Bytes of scratch the context currently holds (for memory accounting). */
+/* Bytes of scratch the context currently holds, in all its buffers (for memory
+ * accounting). */
 int64_t drgb_ctx_scratch_bytes(const drgb_ctx* ctx);
 
 /* Cap on the context's scratch memory (no counterpart in the paper, whose
  * runs fail with out-of-memory when a problem does not fit, Section 3.3):
  * bytes > 0 makes every later call that would need more scratch than `bytes`
  * fail with DRGB_ERR_WORKSPACE before anything is enqueued (the message
- * gives both sizes), and frees the current scratch now if it is larger
- * (waiting for the device); 0 (the default) removes the cap.  A refused call
- * leaves the context usable.  Errors: DRGB_ERR_INVALID (NULL, bytes < 0). */
+ * gives both sizes), and frees what the context now holds above it (waiting
+ * for the device); 0 (the default) removes the cap.  All buffers together stay
+ * within the cap; a buffer that only makes a search faster is not allocated, or
+ * is given back, where another call needs the room.  A refused call leaves the
+ * context usable.  Errors: DRGB_ERR_INVALID (NULL, bytes < 0). */
 int drgb_set_scratch_limit(drgb_ctx* ctx, int64_t bytes);
 
 /* Number of kernels this context has launched (graph replays count every

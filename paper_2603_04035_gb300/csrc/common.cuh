@@ -75,6 +75,13 @@ int set_error(Ctx* c, int code, const char* fmt, ...);
         DRGB_CUDA(ctx, cudaGetLastError());  \
     } while (0)
 
+// Device memory the context holds that counts against its limit: the scratch and
+// the k-NN buffer.  The k-NN buffer is what a call can do without: it is given
+// back (waiting for its users) where the limit or the device leaves the scratch
+// no room beside it.
+size_t held_bytes(const Ctx* c);
+int release_knn_buf(Ctx* c);
+
 // Ensure the context holds at least `bytes` of scratch.  Growing synchronises
 // `stream` first, so that work still using the old buffer has finished.
 int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream);

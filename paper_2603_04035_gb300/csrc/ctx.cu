@@ -22,11 +22,25 @@ int set_error(Ctx* c, int code, const char* fmt, ...) {
     return code;
 }
 
+size_t held_bytes(const Ctx* c) { return c->scratch_bytes + c->knn_buf_bytes; }
+
+int release_knn_buf(Ctx* c) {
+    if (!c->knn_buf) return DRGB_OK;
+    DRGB_CUDA(c, cudaFree(c->knn_buf));  // waits for work that may still use it
+    c->knn_buf = nullptr;
+    c->knn_buf_bytes = 0;
+    return DRGB_OK;
+}
+
 int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
     if (bytes <= c->scratch_bytes) return DRGB_OK;
     if (c->scratch_limit && bytes > c->scratch_limit)
         return set_error(c, DRGB_ERR_WORKSPACE, "scratch of %zu bytes needed, above the context's limit of %zu bytes",
                          bytes, c->scratch_limit);
+    if (c->scratch_limit && bytes + c->knn_buf_bytes > c->scratch_limit) {
+        int rc = release_knn_buf(c);
+        if (rc) return rc;
+    }
     if (c->scratch) {
         DRGB_CUDA(c, cudaStreamSynchronize(stream));
         DRGB_CUDA(c, cudaFree(c->scratch));
@@ -34,10 +48,17 @@ int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
         c->scratch_bytes = 0;
     }
     size_t want = bytes + bytes / 8;  // headroom against frequent regrowth
-    if (c->scratch_limit && want > c->scratch_limit) want = c->scratch_limit;
+    if (c->scratch_limit && want > c->scratch_limit - c->knn_buf_bytes) want = c->scratch_limit - c->knn_buf_bytes;
     cudaError_t e = cudaMalloc(&c->scratch, want);
+    if (e != cudaSuccess && c->knn_buf) {
+        cudaGetLastError();
+        int rc = release_knn_buf(c);
+        if (rc) return rc;
+        e = cudaMalloc(&c->scratch, want);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
+        c->scratch = nullptr;
         return set_error(c, DRGB_ERR_CUDA, "scratch allocation of %zu bytes failed: %s", want,
                          cudaGetErrorString(e));
     }
@@ -320,13 +341,17 @@ int drgb_ctx_destroy(drgb_ctx* c) {
 
 const char* drgb_last_error(const drgb_ctx* c) { return c ? c->err.c_str() : "null context"; }
 
-int64_t drgb_ctx_scratch_bytes(const drgb_ctx* c) { return c ? int64_t(c->scratch_bytes) : 0; }
+int64_t drgb_ctx_scratch_bytes(const drgb_ctx* c) { return c ? int64_t(held_bytes(c)) : 0; }
 
 int drgb_set_scratch_limit(drgb_ctx* c, int64_t bytes) {
     if (!c) return DRGB_ERR_INVALID;
     if (bytes < 0) return set_error(c, DRGB_ERR_INVALID, "scratch limit must be >= 0");
     c->scratch_limit = size_t(bytes);
-    if (bytes && c->scratch && c->scratch_bytes > size_t(bytes)) {  // honour the cap now
+    if (bytes && held_bytes(c) > size_t(bytes)) {  // honour the cap now
+        int rc = release_knn_buf(c);
+        if (rc) return rc;
+    }
+    if (bytes && c->scratch && c->scratch_bytes > size_t(bytes)) {
         DRGB_CUDA(c, cudaFree(c->scratch));  // waits for work that may still use it
         c->scratch = nullptr;
         c->scratch_bytes = 0;

@@ -906,17 +906,18 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     // buffer, and the wide form reads a count back); so does one that the
     // scratch limit or the device leaves no room for.
     size_t want = stream_captures(st) ? 0 : knn_scratch_bytes(c, n, d, k, m, nullptr);
-    if (want && c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) want = 0;
     if (want > c->knn_buf_bytes) {
-        if (c->knn_buf) DRGB_CUDA(c, cudaFree(c->knn_buf));  // waits for its users
-        c->knn_buf = nullptr;
-        c->knn_buf_bytes = 0;
-        if (cudaMalloc(&c->knn_buf, want) == cudaSuccess) {
-            c->knn_buf_bytes = want;
-        } else {
-            cudaGetLastError();
-            c->knn_buf = nullptr;
+        if (c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) {
             want = 0;
+        } else {
+            if ((rc = release_knn_buf(c))) return rc;
+            if (cudaMalloc(&c->knn_buf, want) == cudaSuccess) {
+                c->knn_buf_bytes = want;
+            } else {
+                cudaGetLastError();
+                c->knn_buf = nullptr;
+                want = 0;
+            }
         }
     }
     if (!want) return knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);

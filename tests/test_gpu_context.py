@@ -1,0 +1,92 @@
+"""What a context promises around the kernels: its memory cap covers every
+buffer it keeps (gpu)."""
+import ctypes as C
+
+import pytest
+
+from gpu_util import drgb_module
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture
+def drgb():
+    """The module with a context of its own."""
+    m = drgb_module()
+    m.context()
+    lib = m._lib.load()
+    own = C.c_void_p()
+    assert lib.drgb_ctx_create(0, C.byref(own)) == 0
+    saved, m._contexts[0] = m._contexts[0], own.value
+    yield m
+    m._contexts[0] = saved
+    lib.drgb_ctx_destroy(own)
+
+
+def _points(n, d, seed=0):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    c = 5.0 * torch.randn((20, d), generator=g, device="cuda")
+    return c[torch.randint(0, 20, (n,), generator=g, device="cuda")] + torch.randn((n, d), generator=g, device="cuda")
+
+
+def _render(drgb, side):
+    """A call whose scratch is 16 bytes a pixel."""
+    import torch
+    Y, rgb = torch.rand(10, 2, device="cuda"), torch.rand(10, 3, device="cuda")
+    return drgb.render(Y, rgb, width=side, height=side, radius=2.0)
+
+
+# ------------------------------------------------------------------ memory
+@pytest.mark.parametrize("mode", [0, 1])
+def test_held_memory_is_reported_and_capped(drgb, mode):
+    import torch
+    lib, ctx = drgb._lib.load(), drgb.context()
+    X = _points(20000, 150)
+    want = drgb.knn_graph(X, 15, mode=mode)  # (outputs and modules are loaded once)
+    torch.cuda.synchronize()
+    own = C.c_void_p()
+    assert lib.drgb_ctx_create(0, C.byref(own)) == 0
+    saved, drgb._contexts[0] = drgb._contexts[0], own.value
+    try:
+        torch.cuda.synchronize()
+        free0 = torch.cuda.mem_get_info()[0]
+        got = drgb.knn_graph(X, 15, mode=mode)
+        torch.cuda.synchronize()
+        lost = free0 - torch.cuda.mem_get_info()[0]
+        assert lib.drgb_ctx_scratch_bytes(own) >= lost - 4 * MB
+        assert lib.drgb_set_scratch_limit(own, 1 * MB) == 0
+        assert lib.drgb_ctx_scratch_bytes(own) <= 1 * MB
+        assert free0 - torch.cuda.mem_get_info()[0] <= 4 * MB
+        again = drgb.knn_graph(X, 15, mode=mode)  # without room for lists: the same result
+        torch.cuda.synchronize()
+        assert lib.drgb_ctx_scratch_bytes(own) <= 1 * MB
+    finally:
+        drgb._contexts[0] = saved
+        lib.drgb_ctx_destroy(own)
+    for r in (got, again):
+        assert torch.equal(r[0], want[0]) and torch.equal(r[1], want[1])
+
+
+def test_buffers_of_two_kinds_share_one_cap(drgb):
+    import torch
+    lib, ctx = drgb._lib.load(), drgb.context()
+    held = lambda: lib.drgb_ctx_scratch_bytes(ctx)
+    cap = 200 * MB
+    X = _points(5000, 150)
+    want = drgb.knn_graph(X, 15)
+    _render(drgb, 3400)  # 176 MB beside the search's buffer
+    torch.cuda.synchronize()
+    assert held() > cap
+    assert lib.drgb_set_scratch_limit(ctx, cap) == 0
+    assert held() <= cap
+    for _ in range(2):  # each needs less than the cap by itself
+        _render(drgb, 3400)
+        assert held() <= cap
+        got = drgb.knn_graph(X, 15)
+        torch.cuda.synchronize()
+        assert held() <= cap
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert lib.drgb_set_scratch_limit(ctx, 0) == 0
