@@ -205,6 +205,7 @@ int launch_dep(Ctx* c, void (*kernel)(P...), dim3 grid, int block, size_t smem, 
     cfg.attrs = attr;
     cfg.numAttrs = dep ? 1 : 0;
     DRGB_CUDA(c, cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+    ++c->launches;
     return DRGB_OK;
 }
 

@@ -1480,7 +1480,10 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
         return set_error(c, DRGB_ERR_CUDA, "mlp_train: begin capture: %s", cudaGetErrorString(e));
     }
     const AdamArgs adam{params, adam_m, adam_v, mp->lr, mp->beta1, mp->beta2, mp->eps, bu.W};
+    const int64_t before = c->launches;
     rc = mlp_fwd_bwd(c, bu, params, B, neg, a, b, losses, &adam, fork, cap);
+    const int64_t step_launches = c->launches - before;
+    c->launches = before;  // counted as they are replayed
     e = cudaStreamEndCapture(cap, &graph);
     if (rc == DRGB_OK && e != cudaSuccess) rc = set_error(c, DRGB_ERR_CUDA, "mlp_train: end capture: %s", cudaGetErrorString(e));
     if (rc == DRGB_OK && (e = cudaGraphInstantiate(&exec, graph, 0)) != cudaSuccess)
@@ -1488,6 +1491,7 @@ int drgb_mlp_train(drgb_ctx* c, const float* X, int64_t n, int32_t d, const int3
     for (int s = 0; rc == DRGB_OK && s < mp->steps; ++s) {
         e = cudaGraphLaunch(exec, st);
         if (e != cudaSuccess) rc = set_error(c, DRGB_ERR_CUDA, "mlp_train: launch: %s", cudaGetErrorString(e));
+        else c->launches += step_launches;
     }
     release();
     if (rc) return rc;

@@ -1,5 +1,5 @@
 """What a context promises around the kernels: its memory cap covers every
-buffer it keeps (gpu)."""
+buffer it keeps, every kernel is counted (gpu)."""
 import ctypes as C
 
 import pytest
@@ -90,3 +90,32 @@ def test_buffers_of_two_kinds_share_one_cap(drgb):
         assert held() <= cap
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     assert lib.drgb_set_scratch_limit(ctx, 0) == 0
+
+
+# ------------------------------------------------------------------ counters
+def _counted(drgb, f):
+    before = drgb.launch_count()
+    f()
+    return drgb.launch_count() - before
+
+
+def test_every_kernel_is_counted(drgb):
+    import torch
+    X = _points(3000, 50)
+    P = drgb.mlp_init(50, seed=1)
+    rows = torch.randint(0, 3000, (64 * 7,), dtype=torch.int32, device="cuda")
+    # weights, gather, two layers, head, layer 3 backward, three weight
+    # gradients, dH1, column sums, gradient
+    assert _counted(drgb, lambda: drgb.mlp_grad(P, X, rows, 64, 5, 1.577, 0.895)) == 12
+    g = drgb.fuzzy_weights(*drgb.knn_graph(X, 15), 200)
+
+    def train(steps):
+        Q = P.clone()
+        drgb.mlp_train(X, g, 1.577, 0.895, Q, torch.zeros_like(Q), torch.zeros_like(Q), steps, batch_edges=64)
+    few, more = (_counted(drgb, lambda s=s: train(s)) for s in (3, 8))
+    # a step: a gradient's ten without weights and gather, the next batch's two
+    assert more - few == 5 * 12
+    assert few == 3 * 12 + 4  # and before the first: heads, weights, batch
+    # at least the start's three orthonormalisations of three kernels and one
+    # Rayleigh-Ritz step of six beside means, covariance and projection
+    assert _counted(drgb, lambda: drgb.pca(_points(2000, 100), 5)) >= 9 + 6 + 8
