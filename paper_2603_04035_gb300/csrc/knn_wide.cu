@@ -593,9 +593,10 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     int32_t* fail_rows = cv.take<int32_t>(nq);
     void* part = cv.take<char>(WD_PART_BYTES);
 
-    const bool graph = !separate && !rows;  // a graph of X on itself: the context's k-NN counters report it
+    const bool graph = !separate && !rows;  // a graph of X on itself: the context's k-NN counters and times report it
+    auto mark = [&](int idx) { return graph ? stage_mark(c, idx, st) : DRGB_OK; };
     int rc;
-    if ((rc = stage_mark(c, 8, st))) return rc;
+    if ((rc = mark(8))) return rc;
     DRGB_CUDA(c, cudaMemsetAsync(maxbits, 0, 64, st));
     DRGB_CUDA(c, cudaMemsetAsync(fail_count, 0, 64, st));
     const int db_blocks = grid_for(n, 32, WD_STAT_BLOCKS);
@@ -630,10 +631,10 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
         c->knn_tiles_total = (w.nq_pad / WD_BM) * w.n_tiles;
         DRGB_CUDA(c, cudaMemsetAsync(c->d_counter + 4, 0, 8, st));
     }
-    if ((rc = stage_mark(c, 6, st))) return rc;
+    if ((rc = mark(6))) return rc;
     knn_wide_kernel<<<dim3(unsigned(w.nq_pad / WD_BM), w.splits), WD_THREADS, WD_SMEM, st>>>(mA, mB, P);
     DRGB_CHECK_LAUNCH(c);
-    if ((rc = stage_mark(c, 7, st))) return rc;
+    if ((rc = mark(7))) return rc;
     // |s - s~| for K columns: a K = 16 step adds 16 exact products and the
     // accumulator, each aligned with an error below an FP32 unit (2^-23) of the
     // largest magnitude, which is at most n_j + 2 |x_i| |x_j| <= 2 (n_i + n_max):
@@ -645,7 +646,7 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
         X, n, d, k, Q, separate, rows, nq, w.nq_pad, w.splits, cand_idx, cand_s, norm, resid, maxbits, eps_rel,
         idx_out, dist_out, defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count);
     DRGB_CHECK_LAUNCH(c);
-    if ((rc = stage_mark(c, 9, st))) return rc;
+    if ((rc = mark(9))) return rc;
     if (defer_rows) return DRGB_OK;  // the caller re-scans them
     if (graph) DRGB_CUDA(c, cudaMemcpyAsync(c->d_counter, fail_count, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     int32_t cnt = 0;
@@ -654,7 +655,7 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     if (cnt > 0 && (rc = launch_knn_exact_listed(c, Q, separate, rows, X, n, d, k, fail_rows, cnt, idx_out, dist_out,
                                                  st, part, WD_PART_BYTES)))
         return rc;
-    return stage_mark(c, 10, st);
+    return mark(10);
 }
 
 }  // namespace drgb

@@ -1,5 +1,6 @@
 """What a context promises around the kernels: its memory cap covers every
-buffer it keeps, every kernel is counted (gpu)."""
+buffer it keeps, every kernel is counted, and the stage times of a fit stay the
+fit's (gpu)."""
 import ctypes as C
 
 import pytest
@@ -119,3 +120,21 @@ def test_every_kernel_is_counted(drgb):
     # at least the start's three orthonormalisations of three kernels and one
     # Rayleigh-Ritz step of six beside means, covariance and projection
     assert _counted(drgb, lambda: drgb.pca(_points(2000, 100), 5)) >= 9 + 6 + 8
+
+
+def test_stage_times_stay_the_fits(drgb):
+    import torch
+    X = _points(5000, 50)
+    drgb.set_profiling(True)
+    try:
+        Y = drgb.fit_transform(X, n_epochs=20)
+        t = drgb.stage_times()
+        drgb.transform(X, Y, _points(4000, 50, 1), n_epochs=9)
+        drgb.eval_recall(X, Y, 15, 1000)
+        drgb.eval_recall_heldout(X, Y, X[:4000].contiguous(), Y[:4000].contiguous(), 15)
+        drgb.knn_graph(_points(3000, 50, 2), 15)
+        drgb.knn_graph(_points(3000, 200, 2), 15)
+        torch.cuda.synchronize()
+        assert drgb.stage_times() == t
+    finally:
+        drgb.set_profiling(False)
