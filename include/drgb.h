@@ -206,22 +206,24 @@ int drgb_stage_times(drgb_ctx* ctx, float* ms, int max);
  * mode: 0 auto (for k < 32: 3 when d <= 61 and n > 16000; else a product over
  * all points with FP16 operands, its candidates re-ranked and certified as in
  * mode 3, when 16 <= d <= 1021, n >= 1024 and n n d >= 1.5e8; else 3 when n >=
- * 4096 and d <= 61; else 1), 1 exact FP32 SIMT scan, 2 BF16 tcgen05 distance GEMM with a fused top-32 selection and
- * an FP32 re-rank, 3 the same GEMM with FP16 operands (power-of-two scaled;
- * 8x smaller rounding residual at the same tensor-core rate).  In modes 2
- * and 3, rows whose candidate set cannot be certified to contain the exact
- * FP32 k nearest are recomputed by the exact scan (over the spatial cells
- * each such row can reach), so every mode returns the same exact result;
- * these modes synchronise `stream` once, to read the number of such rows
- * (drgb_knn_uncertified reports it).
+ * 4096 and d <= 61; else 1), 1 exact FP32 SIMT scan, 2 BF16 tcgen05 distance
+ * GEMM with a fused top-32 selection and an FP32 re-rank, 3 the same GEMM with
+ * FP16 operands (power-of-two scaled; 8x smaller rounding residual at the same
+ * tensor-core rate).  Rows whose candidate set cannot be certified to contain the
+ * exact FP32 k nearest are recomputed by the exact scan (in modes 2 and 3 over
+ * the spatial cells each such row can reach), so every mode returns the same
+ * exact result; drgb_knn_uncertified reports their number.
+ * Modes 2 and 3, and auto mode where it takes mode 3 (or falls back on it for
+ * want of memory), synchronise `stream` once; other calls are asynchronous but
+ * where the context's memory has to grow.
  * Errors: DRGB_ERR_INVALID if n < k + 1, k < 1, k > DRGB_MAX_K, d < 1,
  * a pointer is NULL or X is not 4-byte aligned. */
 int drgb_knn_graph(drgb_ctx* ctx, const float* X, int64_t n, int32_t d, int32_t k,
                    int32_t mode, int32_t* idx_out, float* dist_out, void* stream);
 
 /* Number of rows whose 16-bit candidate set was not certified during the last
- * tensor-core (mode 2 or 3) drgb_knn_graph call on `ctx` (synchronous: waits
- * for that call). */
+ * tensor-core drgb_knn_graph call (mode 2 or 3, or auto mode unless it scans) on
+ * `ctx` (synchronous: waits for that call). */
 int drgb_knn_uncertified(drgb_ctx* ctx, int64_t* count, void* stream);
 
 /* Work of the last tensor-core drgb_knn_graph call on `ctx`: the number of

@@ -2,7 +2,7 @@
 // public API; Section 3, the timed fit_transform).  [PCA to pca_dim ->] k-NN
 // graph -> fuzzy graph -> a, b -> initialisation -> T epochs (one cooperative
 // launch, or one captured graph), all enqueued before the synchronisation at the
-// end; a tensor-core k-NN reads its count of uncertified rows before that, and the
+// end; the cell-ordered k-NN reads its count of uncertified rows before that, and the
 // optional PCA synchronises on its own first.
 #include "common.cuh"
 #include "epoch.cuh"

@@ -64,6 +64,11 @@ struct ScanArgs {
     float* dist;
     bool partial;
     int32_t* bound;          // partial: [n_rows], the chunks' common bound as float bits (nullable)
+    // listed: see scan_listed_kernel
+    const int32_t* count;
+    char* part;
+    size_t part_bytes;
+    int64_t slots;
     // cells: see launch_knn_cells
     CellScan cells;
     // ranks: targets and their squared distances (n_rows x k), counts added to
@@ -89,7 +94,7 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return r;
 }
 
-static constexpr int32_t SC_UNBOUND = 0x7F7F7F7F;  // no bound published yet (every byte the same)
+static constexpr int32_t SC_UNBOUND = KNN_UNBOUND;
 static constexpr int SC_RANK_FEW = 24;  // points near enough to matter up to which they are walked one by one
 static constexpr int SC_BULK = 6;  // candidates of 32 from which sorting them beats inserting them one by one
 
@@ -115,7 +120,7 @@ __device__ __forceinline__ void cmp_swap(float& d, int32_t& i, int st, bool keep
 enum { SCAN_NEAREST = 0, SCAN_RANKS = 1, SCAN_CELLS = 2 };
 
 template <int MODE>
-__global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
+__device__ __forceinline__ void scan_block(const ScanArgs& A, const unsigned bx, const unsigned by) {
     constexpr bool RANK = MODE == SCAN_RANKS, CELLS = MODE == SCAN_CELLS;
     extern __shared__ __align__(16) unsigned char sc_raw[];
     const int d = A.d, k = A.k, kl = k <= 16 ? 16 : 32;
@@ -129,18 +134,18 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     int32_t* s_cnt = s_qi + SC_Q;                                             // RANKS: [SC_Q][kl] counts
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
-    const int64_t r0 = int64_t(blockIdx.x) * SC_Q;
-    int64_t p_begin = int64_t(blockIdx.y) * A.chunk;
+    const int64_t r0 = int64_t(bx) * SC_Q;
+    int64_t p_begin = int64_t(by) * A.chunk;
     int64_t p_end = p_begin + A.chunk < A.n ? p_begin + A.chunk : A.n;
     int64_t n_rows = A.n_rows;
     const int32_t* list = A.list;
     if constexpr (CELLS) {
         const CellScan& S = A.cells;
-        if (int(blockIdx.y) >= S.chunk_beg[S.K]) return;
-        int C = 0;  // the cell holding this chunk: the last C with chunk_beg[C] <= blockIdx.y
+        if (int(by) >= S.chunk_beg[S.K]) return;
+        int C = 0;  // the cell holding this chunk: the last C with chunk_beg[C] <= by
         for (int lo = 0, hi = S.K - 1; lo <= hi;) {
             const int mid = (lo + hi) >> 1;
-            if (S.chunk_beg[mid] <= int(blockIdx.y)) {
+            if (S.chunk_beg[mid] <= int(by)) {
                 C = mid;
                 lo = mid + 1;
             } else {
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
         n_rows = S.cell_cnt[C];
         if (r0 >= n_rows) return;
         list = S.cell_rows + int64_t(C) * A.n_rows;
-        p_begin = S.cell_beg[C] + (int64_t(blockIdx.y) - S.chunk_beg[C]) * A.chunk;
+        p_begin = S.cell_beg[C] + (int64_t(by) - S.chunk_beg[C]) * A.chunk;
         p_end = S.cell_beg[C + 1] - p_begin < A.chunk ? S.cell_beg[C + 1] : p_begin + A.chunk;
     }
     // where query q of this CTA goes in the outputs, and its row of Q
@@ -435,13 +440,76 @@ __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
             const int q = t / k, s = t - q * k;
             const int64_t r = r0 + q;
             if (r >= n_rows) continue;
-            const int64_t o = CELLS ? int64_t(blockIdx.y) * A.n_rows + place_of(q)
-                                    : (A.partial ? int64_t(blockIdx.y) * A.n_rows + r : place_of(q));
+            const int64_t o = CELLS ? int64_t(by) * A.n_rows + place_of(q)
+                                    : (A.partial ? int64_t(by) * A.n_rows + r : place_of(q));
             const float D = s_ld[q * kl + s];
             const int32_t I = s_li[q * kl + s];
             A.idx[o * k + s] = I == INT32_MAX ? -1 : I;
             A.dist[o * k + s] = A.partial ? D : sqrtf(D);
         }
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
+    scan_block<MODE>(A, blockIdx.x, blockIdx.y);
+}
+
+// Database chunks of a scan: enough (row block, chunk) CTAs for one to four
+// whole waves of `slots` CTAs, whichever leaves the fewest idle, chunks of at
+// least two tiles, the partial lists within part_bytes.
+__host__ __device__ inline int scan_split(int64_t slots, int64_t n_rows, int64_t n, int k, size_t part_bytes, bool lists) {
+    const int64_t blocks = (n_rows + SC_Q - 1) / SC_Q;
+    int64_t best = 1;
+    double best_use = 0.0;
+    for (int w = 1; w <= 4; ++w) {
+        const int64_t C = slots * w / blocks;
+        const double use = double(blocks * C) / double(slots * w);
+        if (C >= 1 && use > best_use + 0.02) {
+            best = C;
+            best_use = use;
+        }
+    }
+    const int64_t most = n / (2 * SC_P);
+    if (best > most) best = most;
+    if (best > 128) best = 128;
+    if (lists) {
+        const int64_t fit = part_bytes > 1024 ? int64_t((part_bytes / 2 - 512) / (size_t(n_rows) * k * 4)) : 0;
+        if (best > fit) best = fit;
+    }
+    return best > 1 ? int(best) : 1;
+}
+
+// Points of a chunk when the database is cut into C.
+__host__ __device__ inline int64_t scan_chunk(int64_t n, int C) { return ((n + C - 1) / C + SC_P - 1) / SC_P * SC_P; }
+
+// A scan of *A.count listed rows, a number that only the device knows: every CTA
+// and the merge after it derive the split from it.  Unsplit, the lists are the
+// outputs.
+__device__ __forceinline__ int listed_split(ScanArgs& A, int32_t count) {
+    A.n_rows = count;
+    const int C = scan_split(A.slots, count, A.n, A.k, A.part_bytes, true);
+    A.chunk = scan_chunk(A.n, C);
+    A.partial = C > 1;
+    if (!A.partial) {
+        A.bound = nullptr;
+        return 1;
+    }
+    A.idx = reinterpret_cast<int32_t*>(A.part);
+    A.dist = reinterpret_cast<float*>(A.part + ((size_t(count) * C * A.k * 4 + 255) & ~size_t(255)));
+    return int((A.n + A.chunk - 1) / A.chunk);
+}
+
+// CTAs take the (row block, chunk) pairs in turn; none are left where nothing is listed.
+__global__ void __launch_bounds__(SC_THREADS, 2) scan_listed_kernel(const ScanArgs A0) {
+    const int32_t count = *A0.count;
+    if (count <= 0) return;
+    ScanArgs A = A0;
+    const int lists = listed_split(A, count);
+    const int64_t blocks = (count + SC_Q - 1) / SC_Q;
+    for (int64_t t = blockIdx.x; t < blocks * lists; t += gridDim.x) {
+        scan_block<SCAN_NEAREST>(A, unsigned(t % blocks), unsigned(t / blocks));
+        __syncthreads();  // the lists in shared memory have been written out
     }
 }
 
@@ -456,9 +524,9 @@ __device__ __forceinline__ bool lex_less(float a, int32_t i, float b, int32_t j)
 }
 
 template <int K>
-__global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const float* __restrict__ pd2,
-                                      int64_t cnt, int C, int k, const int32_t* __restrict__ rows32,
-                                      int32_t none, int32_t* __restrict__ idx_out, float* __restrict__ dist_out) {
+__device__ __forceinline__ void merge_lists(const int32_t* __restrict__ pidx, const float* __restrict__ pd2,
+                                            int64_t cnt, int C, int k, const int32_t* __restrict__ rows32,
+                                            int32_t none, int32_t* __restrict__ idx_out, float* __restrict__ dist_out) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
     for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); r < cnt; r += warps) {
@@ -530,29 +598,26 @@ __global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const fl
     }
 }
 
-// Database chunks of a scan: enough (row block, chunk) CTAs for one to four
-// whole waves of two CTAs per SM, whichever leaves the fewest idle, chunks of
-// at least two tiles, the partial lists within part_bytes.
+template <int K>
+__global__ void merge_partials_kernel(const int32_t* __restrict__ pidx, const float* __restrict__ pd2,
+                                      int64_t cnt, int C, int k, const int32_t* __restrict__ rows32,
+                                      int32_t none, int32_t* __restrict__ idx_out, float* __restrict__ dist_out) {
+    merge_lists<K>(pidx, pd2, cnt, C, k, rows32, none, idx_out, dist_out);
+}
+
+// The partial lists of scan_listed_kernel with the same arguments (idx and dist: the outputs).
+template <int K>
+__global__ void merge_listed_kernel(const ScanArgs A0, int32_t none) {
+    const int32_t count = *A0.count;
+    if (count <= 0) return;
+    ScanArgs A = A0;
+    const int lists = listed_split(A, count);
+    if (A.partial) merge_lists<K>(A.idx, A.dist, count, lists, A.k, A.list, none, A0.idx, A0.dist);
+}
+
+// Two CTAs an SM.
 static int scan_chunks(const Ctx* c, int64_t n_rows, int64_t n, int k, size_t part_bytes, bool lists) {
-    const int64_t blocks = (n_rows + SC_Q - 1) / SC_Q, slots = 2 * int64_t(c->num_sms);
-    int64_t best = 1;
-    double best_use = 0.0;
-    for (int w = 1; w <= 4; ++w) {
-        const int64_t C = slots * w / blocks;
-        const double use = double(blocks * C) / double(slots * w);
-        if (C >= 1 && use > best_use + 0.02) {
-            best = C;
-            best_use = use;
-        }
-    }
-    const int64_t most = n / (2 * SC_P);
-    if (best > most) best = most;
-    if (best > 128) best = 128;
-    if (lists) {
-        const int64_t fit = part_bytes > 1024 ? int64_t((part_bytes / 2 - 512) / (size_t(n_rows) * k * 4)) : 0;
-        if (best > fit) best = fit;
-    }
-    return best > 1 ? int(best) : 1;
+    return scan_split(2 * int64_t(c->num_sms), n_rows, n, k, part_bytes, lists);
 }
 
 size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
@@ -562,7 +627,7 @@ size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
 
 template <int MODE>
 static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
-    A.chunk = ((A.n + C - 1) / C + SC_P - 1) / SC_P * SC_P;
+    A.chunk = scan_chunk(A.n, C);
     const size_t smem = scan_smem(A.d, A.k, MODE == SCAN_RANKS);
     DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     const dim3 grid(unsigned((A.n_rows + SC_Q - 1) / SC_Q), unsigned((A.n + A.chunk - 1) / A.chunk));
@@ -714,8 +779,8 @@ int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, con
 }
 
 int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t* rows, const float* X, int64_t n,
-                            int d, int k, const int32_t* list, int64_t cnt, int32_t* idx_out, float* dist_out,
-                            cudaStream_t st, void* part, size_t part_bytes) {
+                            int d, int k, const int32_t* list, const int32_t* count, int32_t* bound, int32_t* idx_out,
+                            float* dist_out, cudaStream_t st, void* part, size_t part_bytes) {
     ScanArgs A = {};
     A.X = X;
     A.Q = Q;
@@ -725,9 +790,23 @@ int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t
     A.k = k;
     A.list = list;
     A.rows = rows;
-    A.n_rows = cnt;
+    A.count = count;
     A.ub = dist_out;
-    return scan_nearest(c, A, idx_out, dist_out, part, part_bytes, -1, st);
+    A.idx = idx_out;
+    A.dist = dist_out;
+    A.bound = bound;
+    A.part = static_cast<char*>(part);
+    A.part_bytes = part_bytes;
+    A.slots = 2 * int64_t(c->num_sms);
+    const size_t smem = scan_smem(d, k, false);
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_listed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    scan_listed_kernel<<<int(A.slots), SC_THREADS, smem, st>>>(A);
+    DRGB_CHECK_LAUNCH(c);
+    const int mb = c->num_sms * 4;
+    if (k <= 16) merge_listed_kernel<16><<<mb, 128, 0, st>>>(A, -1);
+    else merge_listed_kernel<32><<<mb, 128, 0, st>>>(A, -1);
+    DRGB_CHECK_LAUNCH(c);
+    return DRGB_OK;
 }
 
 int launch_merge_partials(Ctx* c, const int32_t* pidx, const float* pd2, int64_t cnt, int C, int k,
@@ -894,18 +973,23 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     if (mode < 0 || mode > 3) return set_error(c, DRGB_ERR_INVALID, "knn_graph: bad mode %d", mode);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int m = knn_resolve_mode(n, d, k, mode);
-    if (m == 2 || m == 3 || (m == KNN_WIDE && knn_tc_preferred(n, d, k))) {
-        size_t least = 0, bytes = knn_scratch_bytes(c, n, d, k, m, &least);
-        if ((rc = ensure_scratch_within(c, &bytes, least, st))) return rc;
-        return knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->scratch, c->scratch_bytes);
-    }
+    auto by_cells = [&](int how) -> int {
+        size_t least = 0, bytes = knn_scratch_bytes(c, n, d, k, how, &least);
+        int r = ensure_scratch_within(c, &bytes, least, st);
+        return r ? r : knn_run(c, X, n, d, k, how, idx_out, dist_out, st, c->scratch, c->scratch_bytes);
+    };
+    if (m == 2 || m == 3) return by_cells(m);
+    // Sizes that the cell-ordered form takes as well fall back on it, and are refused
+    // where it is (its scratch above the limit, a captured stream).
+    const bool cells = m == KNN_WIDE && knn_tc_preferred(n, d, k);
+    const bool captured = stream_captures(st);
+    if (cells && (captured || (c->scratch_limit && knn_tc_scratch_bytes(n, d) > c->scratch_limit))) return by_cells(3);
     // The other forms can do without scratch, and what they want is a buffer
     // of its own, so that one enqueued on one stream may overlap other calls'
     // use of the context's scratch on another; they take turns at it through
     // an event.  A captured call scans unsplit (its graph may outlive the
-    // buffer, and the wide form reads a count back); so does one that the
-    // scratch limit or the device leaves no room for.
-    size_t want = stream_captures(st) ? 0 : knn_scratch_bytes(c, n, d, k, m, nullptr);
+    // buffer); so does one that the scratch limit or the device leaves no room for.
+    size_t want = captured ? 0 : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
     if (want > c->knn_buf_bytes) {
         if (c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) {
             want = 0;
@@ -920,7 +1004,7 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
             }
         }
     }
-    if (!want) return knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
+    if (!want) return cells ? by_cells(3) : knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
     if (!c->knn_ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&c->knn_ev, cudaEventDisableTiming));
     DRGB_CUDA(c, cudaStreamWaitEvent(st, c->knn_ev, 0));
     const bool profiling = c->profiling;

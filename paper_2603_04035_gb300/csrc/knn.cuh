@@ -49,10 +49,12 @@ int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, 
                      int64_t cnt, int K, const int32_t* perm, const int32_t* cell_beg, const float* cell_c,
                      const float* cell_r, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
                      size_t part_bytes, bool* done);
-// The same for the queries list[0 .. cnt) of a query set (as for knn_wide).
+// The same for the queries list[0 .. *count) of a query set (as for knn_wide),
+// a count that stays on the device; bound[0 .. *count): KNN_UNBOUND.
+static constexpr int32_t KNN_UNBOUND = 0x7F7F7F7F;  // no bound published yet (every byte the same)
 int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t* rows, const float* X, int64_t n,
-                            int d, int k, const int32_t* list, int64_t cnt, int32_t* idx_out, float* dist_out,
-                            cudaStream_t st, void* part, size_t part_bytes);
+                            int d, int k, const int32_t* list, const int32_t* count, int32_t* bound, int32_t* idx_out,
+                            float* dist_out, cudaStream_t st, void* part, size_t part_bytes);
 // Merge C partial k-lists per listed row: list l of row r at
 // (l * cnt + r) * k in pidx/pd2 (squared distances, ascending by (distance,
 // index), ended early by index -1); the k best by (distance, index) go to
@@ -80,8 +82,8 @@ int knn_tc(Ctx* c, const float* X, int64_t n, int d, int k, bool f16, int32_t* i
 size_t knn_rescan_part_bytes();
 
 // The same for larger problems on the tensor cores (knn_wide.cu).
-// Synchronises `st` once (the count of uncertified queries) unless it is
-// deferred to the caller (as for knn_tc).  `scratch` holds knn_wide_scratch_bytes.
+// Uncertified queries are re-scanned without their number being read back, unless
+// that is deferred to the caller (as for knn_tc).  `scratch` holds knn_wide_scratch_bytes.
 bool knn_wide_preferred(int64_t nq, int64_t n, int d, int k);
 size_t knn_wide_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d);
 int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n, int d,

@@ -402,7 +402,8 @@ wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const f
                    const int32_t* __restrict__ cand_idx, const float* __restrict__ cand_s,
                    const float* __restrict__ norm, const float* __restrict__ resid,
                    const unsigned int* __restrict__ maxbits, float eps_rel, int32_t* __restrict__ idx_out,
-                   float* __restrict__ dist_out, int32_t* __restrict__ fail_rows, int32_t* __restrict__ fail_count) {
+                   float* __restrict__ dist_out, int32_t* __restrict__ fail_rows, int32_t* __restrict__ fail_count,
+                   int32_t* __restrict__ fail_bound) {
     constexpr int PITCH = wr_pitch(V), PER = 32 / V;  // copies a row of 32 dimensions
     __shared__ __align__(16) float s_rows[WR_WARPS][2][32 * PITCH];
     __shared__ __align__(16) float s_q[WR_WARPS][2][32];
@@ -514,7 +515,11 @@ wide_rerank_kernel(const float* __restrict__ X, int64_t n, int d, int k, const f
             const float lb2 = ni + s32 * (S * S) - eps_rel * (ni + n_max) - 4.0f * (S * S);
             const float lb = sqrtf(fmaxf(lb2, 0.f)) - resid[p] - r_max;
             const bool ok = n_valid >= k && lb > sqrtf(dk2) * (1.0f + float(d + 8) * 5.9604645e-8f);
-            if (!ok) fail_rows[atomicAdd(fail_count, 1)] = int32_t(p);
+            if (!ok) {
+                const int32_t slot = atomicAdd(fail_count, 1);
+                fail_rows[slot] = int32_t(p);
+                if (fail_bound) fail_bound[slot] = KNN_UNBOUND;
+            }
         }
     }
 }
@@ -562,7 +567,7 @@ size_t knn_wide_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d) {
     return Carve::round(size_t(WD_STAT_BLOCKS + WD_STAT_QBLOCKS) * 3 * d * 4) + Carve::round(size_t(d) * 4) +
            Carve::round(size_t(w.nq_pad) * w.K * 2) + Carve::round(size_t(w.n_pad) * w.K * 2) +
            2 * Carve::round(size_t(w.nq_pad) * 4) + 2 * Carve::round(64) +
-           2 * Carve::round(size_t(w.splits) * w.nq_pad * TC_KP * 4) + Carve::round(size_t(nq) * 4) + WD_PART_BYTES +
+           2 * Carve::round(size_t(w.splits) * w.nq_pad * TC_KP * 4) + 2 * Carve::round(size_t(nq) * 4) + WD_PART_BYTES +
            8192;
 }
 
@@ -591,6 +596,7 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     int32_t* cand_idx = cv.take<int32_t>(size_t(w.splits) * w.nq_pad * TC_KP);
     float* cand_s = cv.take<float>(size_t(w.splits) * w.nq_pad * TC_KP);
     int32_t* fail_rows = cv.take<int32_t>(nq);
+    int32_t* fail_bound = cv.take<int32_t>(nq);
     void* part = cv.take<char>(WD_PART_BYTES);
 
     const bool graph = !separate && !rows;  // a graph of X on itself: the context's k-NN counters and times report it
@@ -644,16 +650,16 @@ int knn_wide(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* r
     auto rerank = whole(4) ? wide_rerank_kernel<4> : whole(2) ? wide_rerank_kernel<2> : wide_rerank_kernel<1>;
     rerank<<<grid_for(nq, WR_WARPS, c->num_sms * 6), WR_WARPS * 32, 0, st>>>(
         X, n, d, k, Q, separate, rows, nq, w.nq_pad, w.splits, cand_idx, cand_s, norm, resid, maxbits, eps_rel,
-        idx_out, dist_out, defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count);
+        idx_out, dist_out, defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count,
+        defer_rows ? nullptr : fail_bound);
     DRGB_CHECK_LAUNCH(c);
     if ((rc = mark(9))) return rc;
     if (defer_rows) return DRGB_OK;  // the caller re-scans them
     if (graph) DRGB_CUDA(c, cudaMemcpyAsync(c->d_counter, fail_count, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-    int32_t cnt = 0;
-    DRGB_CUDA(c, cudaMemcpyAsync(&cnt, fail_count, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    DRGB_CUDA(c, cudaStreamSynchronize(st));
-    if (cnt > 0 && (rc = launch_knn_exact_listed(c, Q, separate, rows, X, n, d, k, fail_rows, cnt, idx_out, dist_out,
-                                                 st, part, WD_PART_BYTES)))
+    // The number of uncertified queries stays on the device: read back, it would
+    // hold the host, and whatever else it has to enqueue, until the search is done.
+    if ((rc = launch_knn_exact_listed(c, Q, separate, rows, X, n, d, k, fail_rows, fail_count, fail_bound, idx_out,
+                                      dist_out, st, part, WD_PART_BYTES)))
         return rc;
     return mark(10);
 }

@@ -1,6 +1,6 @@
 """What a context promises around the kernels: its memory cap covers every
-buffer it keeps, every kernel is counted, and the stage times of a fit stay the
-fit's (gpu)."""
+buffer it keeps, searches that were enqueued return before they run, every
+kernel is counted, and the stage times of a fit stay the fit's (gpu)."""
 import ctypes as C
 
 import pytest
@@ -91,6 +91,35 @@ def test_buffers_of_two_kinds_share_one_cap(drgb):
         assert held() <= cap
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     assert lib.drgb_set_scratch_limit(ctx, 0) == 0
+
+
+# ------------------------------------------------------------------ streams
+# sizes at which auto mode takes the product over all points, below and above
+# the cell-ordered form's width, and the scan
+SEARCHES = [(2000, 50, 0), (9000, 50, 0), (3000, 200, 0), (2000, 50, 1), (3000, 200, 1), (900, 20, 0)]
+
+
+def _busy(stream):
+    """About half a second of a one-thread kernel on `stream`; an event after it."""
+    import torch
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(1_000_000_000)
+        ev = torch.cuda.Event()
+        ev.record(stream)
+    return ev
+
+
+@pytest.mark.parametrize("n,d,mode", SEARCHES)
+def test_search_returns_before_it_runs(drgb, n, d, mode):
+    import torch
+    X = _points(n, d)
+    want = drgb.knn_graph(X, 15, mode=mode)
+    torch.cuda.synchronize()
+    busy = _busy(torch.cuda.current_stream())
+    got = drgb.knn_graph(X, 15, mode=mode)
+    assert not busy.query()  # enqueued behind it
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
 
 
 # ------------------------------------------------------------------ counters
