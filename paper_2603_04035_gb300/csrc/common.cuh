@@ -14,6 +14,16 @@
 namespace drgb {
 
 // ------------------------------------------------------------------ context
+// A buffer of one k-NN search at a time: searches on different streams take
+// different ones, while there are any, and need not wait for each other.
+struct KnnBuf {
+    void* p = nullptr;
+    size_t bytes = 0;
+    cudaStream_t last = nullptr;  // stream of its last use,
+    cudaEvent_t ev = nullptr;     // and what marks the end of it (null: not used yet)
+};
+static constexpr int KNN_BUFS = 8;
+
 struct Ctx {
     int device = 0;
     int num_sms = 0;
@@ -22,9 +32,7 @@ struct Ctx {
     void* scratch = nullptr;      // grown on demand, 256-byte aligned carve-outs
     size_t scratch_bytes = 0;
     size_t scratch_limit = 0;     // largest scratch the context may allocate (0 = no limit)
-    void* knn_buf = nullptr;      // buffer of drgb_knn_graph's scans and wide products (see there)
-    size_t knn_buf_bytes = 0;
-    cudaEvent_t knn_ev = nullptr;  // its last use
+    KnnBuf knn_bufs[KNN_BUFS];    // of drgb_knn_graph's scans and wide products
     int* d_status = nullptr;      // device status word (0 = ok, else DRGB_ERR_*)
     unsigned long long* d_counter = nullptr;  // [0] uncertified rows, [4] k-NN tile products computed
     int64_t knn_tiles_total = 0;              // tile products of a full scan (last tensor-core k-NN)
@@ -76,11 +84,17 @@ int set_error(Ctx* c, int code, const char* fmt, ...);
     } while (0)
 
 // Device memory the context holds that counts against its limit: the scratch and
-// the k-NN buffer.  The k-NN buffer is what a call can do without: it is given
-// back (waiting for its users) where the limit or the device leaves the scratch
-// no room beside it.
+// the k-NN buffers.  The k-NN buffers are what calls can do without: they are given
+// back (waiting for their users) where the limit or the device leaves the scratch
+// no room beside them.
+size_t knn_buf_bytes(const Ctx* c);
 size_t held_bytes(const Ctx* c);
-int release_knn_buf(Ctx* c);
+int release_knn_bufs(Ctx* c);
+
+// A k-NN buffer of at least `bytes` for work on `st`, which now waits for the
+// buffer's last user; null where the limit or the device leaves none.  The caller
+// records its end (KnnBuf::ev) on `st` when it has enqueued its work.
+int take_knn_buf(Ctx* c, size_t bytes, cudaStream_t st, KnnBuf** out);
 
 // Ensure the context holds at least `bytes` of scratch.  Growing synchronises
 // `stream` first, so that work still using the old buffer has finished.

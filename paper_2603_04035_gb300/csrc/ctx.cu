@@ -22,13 +22,83 @@ int set_error(Ctx* c, int code, const char* fmt, ...) {
     return code;
 }
 
-size_t held_bytes(const Ctx* c) { return c->scratch_bytes + c->knn_buf_bytes; }
+size_t knn_buf_bytes(const Ctx* c) {
+    size_t b = 0;
+    for (const KnnBuf& k : c->knn_bufs) b += k.bytes;
+    return b;
+}
 
-int release_knn_buf(Ctx* c) {
-    if (!c->knn_buf) return DRGB_OK;
-    DRGB_CUDA(c, cudaFree(c->knn_buf));  // waits for work that may still use it
-    c->knn_buf = nullptr;
-    c->knn_buf_bytes = 0;
+size_t held_bytes(const Ctx* c) { return c->scratch_bytes + knn_buf_bytes(c); }
+
+static int release_knn_buf(Ctx* c, KnnBuf& b) {
+    if (!b.p) return DRGB_OK;
+    DRGB_CUDA(c, cudaFree(b.p));  // waits for work that may still use it
+    b.p = nullptr;
+    b.bytes = 0;
+    return DRGB_OK;
+}
+
+int release_knn_bufs(Ctx* c) {
+    for (KnnBuf& b : c->knn_bufs) {
+        int rc = release_knn_buf(c, b);
+        if (rc) return rc;
+    }
+    return DRGB_OK;
+}
+
+// While a stream is captured in the global mode, a thread may allocate or ask for
+// an event only after saying that it touches no captured work.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+int take_knn_buf(Ctx* c, size_t bytes, cudaStream_t st, KnnBuf** out) {
+    *out = nullptr;
+    RelaxedCapture relaxed;
+    bool busy[KNN_BUFS];  // in use on another stream
+    for (int i = 0; i < KNN_BUFS; ++i) {
+        const KnnBuf& b = c->knn_bufs[i];
+        busy[i] = b.p && b.ev && b.last != st && cudaEventQuery(b.ev) != cudaSuccess;
+        if (busy[i]) cudaGetLastError();  // (not ready)
+    }
+    auto pick = [&](auto&& better) {  // the best buffer that is free
+        int at = -1;
+        for (int i = 0; i < KNN_BUFS; ++i)
+            if (!busy[i] && (at < 0 || better(c->knn_bufs[i], c->knn_bufs[at]))) at = i;
+        return at;
+    };
+    // the smallest that fits; else the largest grows, or a new one is made
+    int at = pick([&](const KnnBuf& x, const KnnBuf& y) {
+        const bool fx = x.bytes >= bytes, fy = y.bytes >= bytes;
+        return fx != fy ? fx : (fx ? x.bytes < y.bytes : x.bytes > y.bytes);
+    });
+    if (at >= 0 && c->knn_bufs[at].bytes < bytes) {
+        KnnBuf& b = c->knn_bufs[at];
+        int rc = release_knn_buf(c, b);
+        if (rc) return rc;
+        auto room = [&]() { return !c->scratch_limit || held_bytes(c) + bytes <= c->scratch_limit; };
+        for (int i = 0; i < KNN_BUFS && !room(); ++i)
+            if (!busy[i] && (rc = release_knn_buf(c, c->knn_bufs[i]))) return rc;
+        if (room()) {
+            if (cudaMalloc(&b.p, bytes) == cudaSuccess) {
+                b.bytes = bytes;
+            } else {
+                cudaGetLastError();
+                b.p = nullptr;
+            }
+        }
+        if (!b.p) at = -1;
+    }
+    for (int i = 0; i < KNN_BUFS && at < 0; ++i)  // else one in use, after its user
+        if (busy[i] && c->knn_bufs[i].bytes >= bytes) at = i;
+    if (at < 0) return DRGB_OK;
+    KnnBuf& b = c->knn_bufs[at];
+    if (!b.ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&b.ev, cudaEventDisableTiming));
+    else DRGB_CUDA(c, cudaStreamWaitEvent(st, b.ev, 0));
+    b.last = st;
+    *out = &b;
     return DRGB_OK;
 }
 
@@ -37,8 +107,8 @@ int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
     if (c->scratch_limit && bytes > c->scratch_limit)
         return set_error(c, DRGB_ERR_WORKSPACE, "scratch of %zu bytes needed, above the context's limit of %zu bytes",
                          bytes, c->scratch_limit);
-    if (c->scratch_limit && bytes + c->knn_buf_bytes > c->scratch_limit) {
-        int rc = release_knn_buf(c);
+    if (c->scratch_limit && bytes + knn_buf_bytes(c) > c->scratch_limit) {
+        int rc = release_knn_bufs(c);
         if (rc) return rc;
     }
     if (c->scratch) {
@@ -48,11 +118,11 @@ int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
         c->scratch_bytes = 0;
     }
     size_t want = bytes + bytes / 8;  // headroom against frequent regrowth
-    if (c->scratch_limit && want > c->scratch_limit - c->knn_buf_bytes) want = c->scratch_limit - c->knn_buf_bytes;
+    if (c->scratch_limit && want > c->scratch_limit - knn_buf_bytes(c)) want = c->scratch_limit - knn_buf_bytes(c);
     cudaError_t e = cudaMalloc(&c->scratch, want);
-    if (e != cudaSuccess && c->knn_buf) {
+    if (e != cudaSuccess && knn_buf_bytes(c)) {
         cudaGetLastError();
-        int rc = release_knn_buf(c);
+        int rc = release_knn_bufs(c);
         if (rc) return rc;
         e = cudaMalloc(&c->scratch, want);
     }
@@ -329,8 +399,10 @@ int drgb_ctx_destroy(drgb_ctx* c) {
     cudaDeviceSynchronize();
     if (c->epoch_exec) cudaGraphExecDestroy(c->epoch_exec);
     if (c->scratch) cudaFree(c->scratch);
-    if (c->knn_buf) cudaFree(c->knn_buf);
-    if (c->knn_ev) cudaEventDestroy(c->knn_ev);
+    for (auto& b : c->knn_bufs) {
+        if (b.p) cudaFree(b.p);
+        if (b.ev) cudaEventDestroy(b.ev);
+    }
     if (c->d_status) cudaFree(c->d_status);
     for (auto& e : c->stage_ev)
         if (e) cudaEventDestroy(e);
@@ -348,7 +420,7 @@ int drgb_set_scratch_limit(drgb_ctx* c, int64_t bytes) {
     if (bytes < 0) return set_error(c, DRGB_ERR_INVALID, "scratch limit must be >= 0");
     c->scratch_limit = size_t(bytes);
     if (bytes && held_bytes(c) > size_t(bytes)) {  // honour the cap now
-        int rc = release_knn_buf(c);
+        int rc = release_knn_bufs(c);
         if (rc) return rc;
     }
     if (bytes && c->scratch && c->scratch_bytes > size_t(bytes)) {

@@ -984,33 +984,19 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     const bool cells = m == KNN_WIDE && knn_tc_preferred(n, d, k);
     const bool captured = stream_captures(st);
     if (cells && (captured || (c->scratch_limit && knn_tc_scratch_bytes(n, d) > c->scratch_limit))) return by_cells(3);
-    // The other forms can do without scratch, and what they want is a buffer
-    // of its own, so that one enqueued on one stream may overlap other calls'
-    // use of the context's scratch on another; they take turns at it through
-    // an event.  A captured call scans unsplit (its graph may outlive the
-    // buffer); so does one that the scratch limit or the device leaves no room for.
-    size_t want = captured ? 0 : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
-    if (want > c->knn_buf_bytes) {
-        if (c->scratch_limit && c->scratch_bytes + want > c->scratch_limit) {
-            want = 0;
-        } else {
-            if ((rc = release_knn_buf(c))) return rc;
-            if (cudaMalloc(&c->knn_buf, want) == cudaSuccess) {
-                c->knn_buf_bytes = want;
-            } else {
-                cudaGetLastError();
-                c->knn_buf = nullptr;
-                want = 0;
-            }
-        }
-    }
-    if (!want) return cells ? by_cells(3) : knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
-    if (!c->knn_ev) DRGB_CUDA(c, cudaEventCreateWithFlags(&c->knn_ev, cudaEventDisableTiming));
-    DRGB_CUDA(c, cudaStreamWaitEvent(st, c->knn_ev, 0));
+    // The other forms can do without scratch, and what they want is a buffer of
+    // their own, so that one enqueued on one stream may overlap other calls' use of
+    // the context's scratch, and other searches, on another.  A captured call
+    // scans unsplit (its graph may outlive the buffer); so does one that the scratch
+    // limit or the device leaves no room for.
+    const size_t want = captured ? 0 : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
+    KnnBuf* buf = nullptr;
+    if (want && (rc = take_knn_buf(c, want, st, &buf))) return rc;
+    if (!buf) return cells ? by_cells(3) : knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);
     const bool profiling = c->profiling;
     c->profiling = false;  // the stage times are a fit's
-    rc = knn_run(c, X, n, d, k, m, idx_out, dist_out, st, c->knn_buf, want);
+    rc = knn_run(c, X, n, d, k, m, idx_out, dist_out, st, buf->p, want);
     c->profiling = profiling;
-    DRGB_CUDA(c, cudaEventRecord(c->knn_ev, st));
+    DRGB_CUDA(c, cudaEventRecord(buf->ev, st));
     return rc;
 }

@@ -1,6 +1,7 @@
 """What a context promises around the kernels: its memory cap covers every
-buffer it keeps, searches that were enqueued return before they run, every
-kernel is counted, and the stage times of a fit stay the fit's (gpu)."""
+buffer it keeps, searches that were enqueued return before they run and do not
+wait for other streams', every kernel is counted, and the stage times of a fit
+stay the fit's (gpu)."""
 import ctypes as C
 
 import pytest
@@ -120,6 +121,68 @@ def test_search_returns_before_it_runs(drgb, n, d, mode):
     assert not busy.query()  # enqueued behind it
     torch.cuda.synchronize()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("n,d,mode", SEARCHES)
+def test_searches_on_two_streams_do_not_wait_for_each_other(drgb, n, d, mode):
+    import torch
+    X = _points(n, d)
+    want = drgb.knn_graph(X, 15, mode=mode)
+    torch.cuda.synchronize()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(2):  # (the second time nothing grows)
+        busy = _busy(s1)
+        with torch.cuda.stream(s1):
+            a = drgb.knn_graph(X, 15, mode=mode)
+        with torch.cuda.stream(s2):
+            b = drgb.knn_graph(X, 15, mode=mode)
+        s2.synchronize()
+        assert not busy.query()
+        torch.cuda.synchronize()
+        for r in (a, b):
+            assert torch.equal(r[0], want[0]) and torch.equal(r[1], want[1])
+
+
+def test_searches_on_many_streams_with_growth(drgb):
+    # more streams than the context keeps buffers, sizes that grow in between
+    import torch
+    sets = [_points(n, d, n) for n, d in ((1500, 70), (3000, 200), (6000, 90), (2000, 50))]
+    want = [drgb.knn_graph(X, 15, mode=1) for X in sets]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(12)]
+    outs = []
+    for i in range(48):
+        with torch.cuda.stream(streams[i % 12]):
+            outs.append((i % 4, drgb.knn_graph(sets[i % 4], 15)))
+    torch.cuda.synchronize()
+    for k, r in outs:
+        assert torch.equal(r[0], want[k][0]) and torch.equal(r[1], want[k][1])
+
+
+def test_search_beside_a_capture_on_another_stream(drgb):
+    # a stream being captured in the global mode forbids what may synchronise the
+    # device; a search enqueued on another stream meanwhile still runs
+    import torch
+    lib, ctx = drgb._lib.load(), drgb.context()
+    X = _points(2000, 50)
+    want = drgb.knn_graph(X, 15)
+    X2 = _points(2600, 50)
+    want2 = drgb.knn_graph(X2, 15, mode=1)
+    idx, dist = torch.empty_like(want2[0]), torch.empty_like(want2[1])
+    lib.drgb_set_scratch_limit(ctx, 1)  # (the buffer has to be allocated again)
+    lib.drgb_set_scratch_limit(ctx, 0)
+    other = torch.cuda.Stream()
+    z = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        z.add_(1.0)
+        rc = lib.drgb_knn_graph(ctx, C.c_void_p(X2.data_ptr()), 2600, 50, 15, 0, C.c_void_p(idx.data_ptr()),
+                                C.c_void_p(dist.data_ptr()), C.c_void_p(other.cuda_stream))
+    g.replay()
+    torch.cuda.synchronize()
+    assert rc == 0 and float(z[0]) == 1.0
+    assert torch.equal(idx, want2[0]) and torch.equal(dist, want2[1])
 
 
 # ------------------------------------------------------------------ counters
