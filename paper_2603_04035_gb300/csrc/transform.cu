@@ -14,9 +14,11 @@
 namespace drgb {
 
 // Schedule words of the new rows (w_max = 1: every row's nearest neighbour has
-// membership 1) and the start positions.
+// membership 1) and the start positions.  A row with non-finite or overflowing
+// distances has no neighbours (-1; the weights' kernel reports it): it starts
+// from those it has.
 __global__ void transform_setup_kernel(const int32_t* __restrict__ out_col, const float* __restrict__ out_w,
-                                       int64_t n_new, int k, const float2* __restrict__ Y_train,
+                                       int64_t n_new, int k, const float2* __restrict__ Y_train, int64_t n_train,
                                        uint32_t* __restrict__ q, float2* __restrict__ Y_new_a,
                                        float2* __restrict__ Y_new_b) {
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_new;
@@ -24,10 +26,13 @@ __global__ void transform_setup_kernel(const int32_t* __restrict__ out_col, cons
         float sx = 0.f, sy = 0.f, sw = 0.f;
         for (int s = 0; s < k; ++s) {
             const float w = out_w[i * k + s];
-            const float2 y = Y_train[out_col[i * k + s]];
-            sx = fmaf(w, y.x, sx);
-            sy = fmaf(w, y.y, sy);
-            sw += w;
+            const int32_t j = out_col[i * k + s];
+            if (j >= 0 && j < n_train) {
+                const float2 y = Y_train[j];
+                sx = fmaf(w, y.x, sx);
+                sy = fmaf(w, y.y, sy);
+                sw += w;
+            }
             q[i * k + s] = __float2uint_rn(16777216.0f * w);
         }
         const float2 y0 = make_float2(sx / sw, sy / sw);
@@ -89,7 +94,7 @@ extern "C" int drgb_transform(drgb_ctx* c, const float* X_train, const float* Y_
     DRGB_CUDA(c, cudaMemcpyAsync(Ya, Y_train, size_t(n_train) * 8, cudaMemcpyDeviceToDevice, st));
     DRGB_CUDA(c, cudaMemcpyAsync(Yb, Y_train, size_t(n_train) * 8, cudaMemcpyDeviceToDevice, st));
     transform_setup_kernel<<<grid_for(n_new, 256, c->num_sms * 8), 256, 0, st>>>(
-        out_col, out_w, n_new, k, reinterpret_cast<const float2*>(Y_train), q, Ya + n_train, Yb + n_train);
+        out_col, out_w, n_new, k, reinterpret_cast<const float2*>(Y_train), n_train, q, Ya + n_train, Yb + n_train);
     DRGB_CHECK_LAUNCH(c);
     arange_kernel<<<grid_for(n_new + 1, 256, c->num_sms * 8), 256, 0, st>>>(rp, n_new, k);
     DRGB_CHECK_LAUNCH(c);
