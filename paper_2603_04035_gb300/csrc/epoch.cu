@@ -1145,8 +1145,11 @@ static void fill_args(EpochArgs& A, const int32_t* rp, const int32_t* col, const
 static constexpr int64_t LOOP_MAX_WINDOWS_PER_SM = 11;
 static constexpr int LOOP_MAX_EPOCHS = 1000000;  // the barrier counts epochs x CTAs in 32 bits
 
+// *done is false, and no epoch has run, where the device, or the part of it that
+// the stream may use, does not hold the grid at once: the caller chains launches.
 static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float lr0, int t_begin, int t_end, int T,
-                          unsigned int* sync, cudaStream_t st) {
+                          unsigned int* sync, cudaStream_t st, bool* done) {
+    *done = false;
     DRGB_CUDA(c, cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned int), st));
     LoopArgs P;
     P.buf[0] = Y;
@@ -1176,8 +1179,8 @@ static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float 
     const size_t need = size_t(per_sm) * (fa.sharedSizeBytes + 1024);
     const int pct = int((need * 100 + c->smem_per_sm - 1) / (c->smem_per_sm ? c->smem_per_sm : 1));
     DRGB_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct < 100 ? pct : 100));
-    const int64_t ctas = grid_for(A.win_cap, 1, c->num_sms * (per_sm > 0 ? per_sm : 1));
-    if (A.win_cap > ctas * LOOP_WINDOWS) return set_error(c, DRGB_ERR_CUDA, "epoch loop: too few CTAs fit the device");
+    const int64_t ctas = per_sm > 0 ? grid_for(A.win_cap, 1, c->num_sms * per_sm) : 0;
+    if (A.win_cap > ctas * LOOP_WINDOWS) return DRGB_OK;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(ctas));
     cfg.blockDim = dim3(nw * 32);
@@ -1187,8 +1190,14 @@ static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    DRGB_CUDA(c, cudaLaunchKernelEx(&cfg, kernel, static_cast<const EpochArgs&>(A), static_cast<const LoopArgs&>(P)));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<const EpochArgs&>(A), static_cast<const LoopArgs&>(P));
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return DRGB_OK;
+    }
+    DRGB_CUDA(c, e);
     DRGB_CHECK_LAUNCH(c);
+    *done = true;
     if ((t_end - t_begin) & 1)
         DRGB_CUDA(c, cudaMemcpyAsync(Y, Y_tmp, size_t(A.n) * sizeof(float2), cudaMemcpyDeviceToDevice, st));
     return DRGB_OK;
@@ -1213,7 +1222,9 @@ int run_epochs(Ctx* c, float2* Y, float2* Y_tmp, const int32_t* rp, const int32_
         es.win_cap <= LOOP_MAX_WINDOWS_PER_SM * c->num_sms) {
         EpochArgs A;
         fill_args(A, rp, col, q, n, a, b, neg, seed, c->d_status, es, count, inst_off, inst_seed, row_begin, neg_n);
-        return run_epoch_loop(c, Y, Y_tmp, A, lr0, t_begin, t_end, T, es.sync, st);
+        bool done = false;
+        rc = run_epoch_loop(c, Y, Y_tmp, A, lr0, t_begin, t_end, T, es.sync, st, &done);
+        if (rc || done) return rc;
     }
     cudaStream_t cap;
     DRGB_CUDA(c, cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
