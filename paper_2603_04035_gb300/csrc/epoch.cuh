@@ -9,8 +9,8 @@ namespace drgb {
 static constexpr int EPOCH_WIN = 512;
 
 struct EpochArgs {
-    const float2* __restrict__ Y_in;
-    float2* __restrict__ Y_out;
+    const float2* Y_in;  // (written by the launch before, which may still run: nothing is promised of it)
+    float2* Y_out;
     const int32_t* __restrict__ row_ptr;
     const int32_t* __restrict__ col;
     const uint32_t* __restrict__ q;

@@ -636,8 +636,8 @@ __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int3
 // 101 us.)
 static constexpr int HEAD_ROWS = 4;
 
-__global__ void __launch_bounds__(256) mlp_head_loss_kernel(const bf16* __restrict__ H2, const float* __restrict__ W3f,
-                                                            const float* __restrict__ P, const int32_t* __restrict__ rows,
+__global__ void __launch_bounds__(256) mlp_head_loss_kernel(const bf16* H2, const float* W3f,
+                                                            const float* P, const int32_t* rows,
                                                             int B, int neg, float a, float b, float* __restrict__ dz,
                                                             float* __restrict__ loss_part, uint32_t* __restrict__ step_dev) {
     const int lane = threadIdx.x & 31;
@@ -735,7 +735,7 @@ static constexpr int MC_PITCH = MLP_CHUNK * 4 + 4;  // floats per float4 column:
 static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 8;
 
 __global__ void __launch_bounds__(MC_THREADS, 3)
-mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2, int M,
+mlp_l3back_kernel(const float* dz, const float* W3f, const float* dgelu2, int M,
                   bf16* __restrict__ D, float* __restrict__ pb2) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]: dpre2, float4 columns
     float2* s_z = reinterpret_cast<float2*>(s_v + 8 * MC_PITCH);  // [MLP_CHUNK]: dz
@@ -789,7 +789,7 @@ mlp_l3back_kernel(const float* __restrict__ dz, const float* __restrict__ W3f, c
 
 // Over the chunk: dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
 __global__ void __launch_bounds__(MC_THREADS)
-mlp_w3grad_kernel(const float* __restrict__ dz, const bf16* __restrict__ H2, int M, float* __restrict__ pw3) {
+mlp_w3grad_kernel(const float* dz, const bf16* H2, int M, float* __restrict__ pw3) {
     __shared__ __align__(16) bf16 s_h[MLP_CHUNK * 32];  // H2
     __shared__ float2 s_z[MLP_CHUNK];                   // dz
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -822,7 +822,7 @@ mlp_w3grad_kernel(const float* __restrict__ dz, const bf16* __restrict__ H2, int
 static constexpr size_t CS_SMEM = size_t(8) * MC_PITCH * 4;
 
 __global__ void __launch_bounds__(MC_THREADS, 3)
-mlp_colsum_kernel(const float* __restrict__ A, int M, float* __restrict__ part) {
+mlp_colsum_kernel(const float* A, int M, float* __restrict__ part) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
     const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;

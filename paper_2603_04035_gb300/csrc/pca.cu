@@ -202,8 +202,8 @@ __device__ __forceinline__ T ordered_sum(int count, F&& at) {
 static constexpr int PCA_CSPLITS = 8;
 static constexpr int PCA_CTHREADS = 64 * PCA_CSPLITS;
 
-__global__ void __launch_bounds__(PCA_CTHREADS) pca_cmul_kernel(const float* __restrict__ C, int D,
-                                                                const float* __restrict__ X, const float* __restrict__ Z,
+__global__ void __launch_bounds__(PCA_CTHREADS) pca_cmul_kernel(const float* C, int D,
+                                                                const float* X, const float* Z,
                                                                 float alpha, float beta, float gamma, int L,
                                                                 float* __restrict__ Y) {
     __shared__ __align__(16) float Cs[PCA_CSPLITS * PCA_KCHUNK][PCA_CROWS];
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(PCA_CTHREADS) pca_cmul_kernel(const float* __r
 // product split by an FMA, the running sum by Knuth's TwoSum), about as
 // accurate as FP64 and all on the FP32 pipes, and is stored as FP64.  The last
 // chunk's block to finish adds the chunks in order into G.
-__global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__ A, const float* __restrict__ B,
+__global__ void __launch_bounds__(256) pca_gram_kernel(const float* A, const float* B,
                                                        int D, int L, double* __restrict__ Gp,
                                                        unsigned int* __restrict__ counters, double* __restrict__ G) {
     __shared__ float As[PCA_GCHUNK][PCA_P + 1];
@@ -346,8 +346,8 @@ __global__ void __launch_bounds__(256) pca_gram_kernel(const float* __restrict__
 
 // rn[j] = sum_a (W[a][L + j] - theta_j Y[a][L + j])^2 (FP64), one warp per
 // active column.
-__global__ void pca_resid_kernel(const float* __restrict__ Y, const float* __restrict__ W,
-                                 const float* __restrict__ theta, int D, int L, double* __restrict__ rn) {
+__global__ void pca_resid_kernel(const float* Y, const float* W,
+                                 const float* theta, int D, int L, double* __restrict__ rn) {
     dep_enter();
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (j >= PCA_P - L) return;
@@ -384,8 +384,8 @@ __device__ __forceinline__ float4 tile_product(const float (*Xs)[PCA_P + 1], con
 
 // Locked columns: Y = X; active columns: Y[a][L + q] = sum_p X[a][p] M[p][q]
 // (M: P x m, device).
-__global__ void __launch_bounds__(256) pca_apply_kernel(const float* __restrict__ X, int D,
-                                                        const float* __restrict__ M, int L, float* __restrict__ Y) {
+__global__ void __launch_bounds__(256) pca_apply_kernel(const float* X, int D,
+                                                        const float* M, int L, float* __restrict__ Y) {
     __shared__ __align__(16) float Ms[PCA_P][PCA_P];
     __shared__ float Xs[PCA_TROWS][PCA_P + 1];
     dep_enter();
@@ -418,8 +418,8 @@ __global__ void __launch_bounds__(256) pca_apply_kernel(const float* __restrict_
 // is known, every lane subtracts y_j T[j][k] from its two columns k > j (a thread
 // per row, summing up to each column in turn, took 22 us).  Mode 1: Y = X T, T
 // general P x P.
-__global__ void __launch_bounds__(256) pca_ortho_kernel(const float* __restrict__ X, int D, const float* __restrict__ T,
-                                                        const int* __restrict__ mode, float* __restrict__ Y) {
+__global__ void __launch_bounds__(256) pca_ortho_kernel(const float* X, int D, const float* T,
+                                                        const int* mode, float* __restrict__ Y) {
     __shared__ __align__(16) float Ts[PCA_P][PCA_P];
     __shared__ float Xs[PCA_TROWS][PCA_P + 1];
     dep_enter();
@@ -623,7 +623,7 @@ static constexpr int PCA_JAC_SWEEPS = 6;
 // orthonormality.
 static constexpr int PCA_MODE = 2;  // index of the mode word in the flags
 static constexpr size_t PCA_CHOL_SMEM = size_t(2) * PCA_P * PCA_P * sizeof(double) + size_t(PCA_P) * PCA_P * 4;
-__global__ void __launch_bounds__(PCA_CHOL_THREADS) pca_chol_kernel(const double* __restrict__ G, int L, int pass,
+__global__ void __launch_bounds__(PCA_CHOL_THREADS) pca_chol_kernel(const double* G, int L, int pass,
                                                                    int* __restrict__ flags, float* __restrict__ T) {
     extern __shared__ double csm[];
     dep_enter();
@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(PCA_CHOL_THREADS) pca_chol_kernel(const double
 // leaves its vectors' residuals larger, which the locking test sees).  Output, by decreasing eigenvalue: th_f, th_d,
 // and eigenvector k as column k of Vout rows row_out..row_out+m-1 (leading
 // dimension ldv); rows < row_out are zeroed when zero_lead.
-__global__ void __launch_bounds__(PCA_JAC_THREADS) pca_jacobi_kernel(const double* __restrict__ Gp, int nparts,
+__global__ void __launch_bounds__(PCA_JAC_THREADS) pca_jacobi_kernel(const double* Gp, int nparts,
                                                                     int64_t part_stride, int ld, int row0, int m,
                                                                     float* __restrict__ Vout, int ldv, int row_out,
                                                                     int zero_lead, float* __restrict__ th_f,
