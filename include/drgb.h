@@ -116,6 +116,16 @@ int drgb_sync(drgb_ctx* ctx, void* stream);
  * out of range. */
 int drgb_wait_selftest(drgb_ctx* ctx, int64_t limit_us, int32_t arrive, void* stream);
 
+/* Self-test of the tensor cores' sums (no counterpart in the paper): out[i][j] =
+ * sum_k A[i][k] B[j][k], accumulated over k as the tensor-core k-NN does (FP32
+ * accumulator, 16 products a step, steps in order), whose certificate assumes a
+ * bound on this sum's rounding.  A: M x K, B: N x K, row-major BF16 (f16 = 0) or
+ * FP16 bits; out: M x N FP32; device pointers, 16-byte aligned; M and N multiples
+ * of 128 (at most 65,536), K of 64 (at most 1,024).  Asynchronous.  Errors:
+ * DRGB_ERR_INVALID (NULL, misaligned, sizes). */
+int drgb_product_selftest(drgb_ctx* ctx, const void* A, const void* B, int32_t M, int32_t N, int32_t K,
+                          int32_t f16, float* out, void* stream);
+
 /* Random-gather probe (no counterpart in the paper; the roofline denominator
  * of the SGD epoch, whose work is one random 8-byte load of Y per tail and per
  * negative sample): every thread the GPU holds resident (largest L1 carveout)

@@ -93,6 +93,7 @@ SIGNATURES = {
     "drgb_render": (C.c_int, [vp, vp, vp, i64, i32, i32, f32, f32, C.POINTER(C.c_float), C.POINTER(C.c_float),
                               C.POINTER(C.c_float), vp, vp]),
     "drgb_wait_selftest": (C.c_int, [vp, i64, i32, vp]),
+    "drgb_product_selftest": (C.c_int, [vp, vp, vp, i32, i32, i32, i32, vp, vp]),
     "drgb_spectral_init": (C.c_int, [vp, vp, vp, vp, i64, f32, u64, vp, C.POINTER(C.c_double), vp]),
     "drgb_pca": (C.c_int, [vp, vp, i64, i32, i32, vp, vp, vp, C.POINTER(C.c_double), vp]),
     "drgb_eval_recall_heldout": (C.c_int, [vp, vp, vp, i64, vp, vp, i64, i32, i32, i64, C.POINTER(C.c_double),

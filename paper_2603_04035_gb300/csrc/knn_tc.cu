@@ -69,7 +69,9 @@ static constexpr size_t TC_SMEM =
 // Bound on |s - s~| for K = 64 columns (FP32 accumulation and norms): a K = 16
 // step adds 16 exact products and the accumulator, each aligned with an error
 // below an FP32 unit (2^-23) of the largest magnitude, which is at most n_j + 2
-// |x_i| |x_j| <= 2 (n_i + n_max): 34 * 2^-23 (n_i + n_max) a step; the norms'
+// |x_i| |x_j| <= 2 (n_i + n_max): 34 * 2^-23 (n_i + n_max) a step (the largest
+// error measured against sums in 64 bits, over all widths and operands that
+// cancel, grow or are of one sign: 0.05 of that, drgb_product_selftest); the norms'
 // sums and split below 2^-17 of that, and in FP16 the split's last part may lie
 // below the smallest normal number (4 units of the scaled operands).  (2^-14 (n_i +
 // n_max), taken before, left 914 rows of 70,000 projected images uncertified.)

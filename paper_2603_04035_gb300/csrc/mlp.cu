@@ -80,6 +80,7 @@ struct GemmArgs {
     int M, N, K;          // M, N multiples of 128 / BN; K multiple of 64
     int kb_per_split;     // 64-wide K blocks per split (grid z)
     float* out_f32;       // [splits][M][N]
+    int f16;              // FP16 operands, else BF16
     int* status;
 };
 
@@ -172,7 +173,7 @@ mlp_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16kind(G_BM, BN, false) | (KROWS ? IDESC_MN_MAJOR : 0u);
+            const uint32_t idesc = idesc_f16kind(G_BM, BN, G.f16 != 0) | (KROWS ? IDESC_MN_MAJOR : 0u);
             constexpr int KSTEP = KROWS ? 2048 / 16 : 32 / 16;  // 16 of K, in descriptor units
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % STAGES;
@@ -239,19 +240,20 @@ struct Gemm {
 // C[M x N] = A[M x K] B[N x K]^T with A, B row-major BF16 (K contiguous), or
 // with `krows` A[K x M]^T B[K x N].
 static int gemm_setup(Ctx* c, Gemm& G, const bf16* A, const bf16* B, int M, int N, int K, int bn,
-                      int splits, bool krows) {
+                      int splits, bool krows, bool f16 = false) {
     if (M % G_BM || N % bn || K % 64 || splits < 1)
         return set_error(c, DRGB_ERR_INVALID, "mlp gemm: bad shape %d x %d x %d", M, N, K);
     int rc;
     if (krows) {
         if ((rc = make_map_k64(c, &G.a, A, K, M, 64, false)) || (rc = make_map_k64(c, &G.b, B, K, N, 64, false))) return rc;
     } else {
-        if ((rc = make_map_k64(c, &G.a, A, M, K, G_BM, false)) || (rc = make_map_k64(c, &G.b, B, N, K, bn, false))) return rc;
+        if ((rc = make_map_k64(c, &G.a, A, M, K, G_BM, f16)) || (rc = make_map_k64(c, &G.b, B, N, K, bn, f16))) return rc;
     }
     std::memset(&G.g, 0, sizeof(G.g));
     G.g.M = M;
     G.g.N = N;
     G.g.K = K;
+    G.g.f16 = f16;
     const int kbs = K / 64;
     G.g.kb_per_split = (kbs + splits - 1) / splits;
     G.g.status = c->d_status;
@@ -278,10 +280,10 @@ static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
 // The plain product for other users of the library (the PCA covariance):
 // partials[z][M][N] = A[M x K] B[N x K]^T over the z-th share of K.
 int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, int splits, float* partials,
-                   int* splits_used, cudaStream_t st) {
+                   int* splits_used, cudaStream_t st, bool f16) {
     Gemm G;
     const int bn = (N % 128 == 0) ? 128 : 64;
-    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, splits, false);
+    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, splits, false, f16);
     if (rc) return rc;
     G.g.out_f32 = partials;
     if ((rc = bn == 128 ? gemm_attr<128, false>(c) : gemm_attr<64, false>(c))) return rc;

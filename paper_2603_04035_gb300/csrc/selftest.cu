@@ -5,7 +5,12 @@
 // DRGB_ERR_TIMEOUT in the context's status word and returns, and the kernel
 // exits; no copy or tensor-core operation is in flight, so nothing is left
 // pending on the device.
+//
+// Self-test of the tensor cores' sums: the products of given 16-bit operands
+// accumulated in one chain over K, in steps of 16, as the k-NN kernels do, so that
+// their rounding can be measured against the bound the k-NN certificate assumes.
 #include "common.cuh"
+#include "gemm.cuh"
 #include "tc_ptx.cuh"
 
 namespace drgb {
@@ -35,4 +40,14 @@ extern "C" int drgb_wait_selftest(drgb_ctx* c, int64_t limit_us, int32_t arrive,
                                            arrive ? 1 : 0);
     DRGB_CHECK_LAUNCH(c);
     return drgb_sync(c, stream);
+}
+
+extern "C" int drgb_product_selftest(drgb_ctx* c, const void* A, const void* B, int32_t M, int32_t N, int32_t K,
+                                     int32_t f16, float* out, void* stream) {
+    if (!c) return DRGB_ERR_INVALID;
+    if (!A || !B || !out || !aligned(A, 16) || !aligned(B, 16) || !aligned(out, 16))
+        return set_error(c, DRGB_ERR_INVALID, "product_selftest: NULL or misaligned pointer");
+    if (M < 128 || N < 128 || K < 64 || M > 65536 || N > 65536 || K > 1024 || M % 128 || N % 128 || K % 64)
+        return set_error(c, DRGB_ERR_INVALID, "product_selftest: M, N multiples of 128 and K of 64, K <= 1024");
+    return tc_gemm_nt_f32(c, A, B, M, N, K, 1, out, nullptr, static_cast<cudaStream_t>(stream), f16 != 0);
 }
