@@ -121,13 +121,8 @@ __device__ __forceinline__ float pow_pos(float d, float b) { return hw_ex2(b * h
 static constexpr unsigned FULL = 0xffffffffu;
 
 // Read of one point of Y^(t).  (Read-only-path and L1 evict-last loads were
-// measured and made no difference.)  L2: through L2 only, for a kernel that
-// runs several epochs (its L1 may hold an older epoch's line).
-template <bool L2 = false>
-__device__ __forceinline__ float2 load_y(const float2* p) {
-    if constexpr (L2) return __ldcg(p);
-    return *p;
-}
+// measured and made no difference; epoch_loop_kernel must not take the former.)
+__device__ __forceinline__ float2 load_y(const float2* p) { return *p; }
 
 // Instance-local view of a row: rows [off, off + n) with entries from eoff on,
 // negatives drawn under Philox key (k0, k1).  A single instance has off = 0,
@@ -219,20 +214,20 @@ __device__ __forceinline__ void draw_entry(const EpochArgs& A, const EpochStep& 
     }
 }
 
-template <int NEG, bool L2 = false>
+template <int NEG>
 __device__ __forceinline__ void gather_entry(const EpochStep& S, const RowInst& R, const EntryPlan<NEG>& pl,
                                              EntryInputs<NEG>& in) {
     in.ok = pl.ok;
     in.e = pl.e;
     in.i = pl.i;
-    in.yi = load_y<L2>(S.Y_in + pl.ii);
-    in.yj = load_y<L2>(S.Y_in + pl.jj);
+    in.yi = load_y(S.Y_in + pl.ii);
+    in.yj = load_y(S.Y_in + pl.jj);
     const float2* Yb = S.Y_in + R.off;
 #pragma unroll
-    for (int w = 0; w < EntryInputs<NEG>::NP; ++w) in.ym[w] = load_y<L2>(Yb + pl.m[w]);
+    for (int w = 0; w < EntryInputs<NEG>::NP; ++w) in.ym[w] = load_y(Yb + pl.m[w]);
 }
 
-template <int NEG, bool BATCHED, bool L2 = false>
+template <int NEG, bool BATCHED>
 __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep& S, const RowInst& R,
                                              const EntryInputs<NEG>& in, float two_ab, float two_b) {
     constexpr int NP = EntryInputs<NEG>::NP;
@@ -274,7 +269,7 @@ __device__ __forceinline__ float2 entry_math(const EpochArgs& A, const EpochStep
             for (int w = 0; w < 4; ++w) {
                 const uint32_t m = __umulhi(v[w], n32);
                 const bool ok = (g * 4 + w < neg) && (m != i32);
-                yg[w] = ok ? load_y<L2>(Yb + m) : yi;
+                yg[w] = ok ? load_y(Yb + m) : yi;
             }
 #pragma unroll
             for (int w = 0; w < 4; ++w) repel(yg[w]);
@@ -811,7 +806,12 @@ __global__ void __launch_bounds__(LOOP_WARPS * 32, loop_ctas_per_sm(LOOP_WARPS))
         for (int b = 0; b < LOOP_CHUNKS; ++b) qv[b] = e0 + 32 * b < ee ? A.q[e0 + 32 * b] : 0u;  // 0 never fires
     };
     if (n_mine > 0) load_round(s_win[0].es, s_win[0].ee);
-    // every CTA has finished the previous epoch (bounded; false: give up)
+    // Every CTA has finished the previous epoch (bounded; false: give up).  A CTA's
+    // barrier and its first thread's release order the epoch's writes of Y before
+    // the count; the acquire here and the barrier after it order the count before the
+    // other threads' reads, plain loads included (the acquire drops the L1's older
+    // lines).  Loads that are not coherent (ld.global.nc, __restrict__) would not be
+    // ordered.
     auto wait_epoch = [&]() -> bool {
         if (tid == 0 && arrivals) {
             const unsigned target = arrivals * ctas;

@@ -4,23 +4,6 @@
 
 namespace drgb {
 
-// Insert (d, j) into a list D[0..K) sorted ascending by d, dropping the last
-// entry; precondition d < D[K-1].  Equal values keep their arrival order.
-template <int K>
-__device__ __forceinline__ void topk_insert(float (&D)[K], int32_t (&I)[K], float d, int32_t j) {
-#pragma unroll
-    for (int s = K - 1; s > 0; --s) {
-        const bool shift = d < D[s - 1];
-        const bool place = !shift && d < D[s];
-        D[s] = shift ? D[s - 1] : (place ? d : D[s]);
-        I[s] = shift ? I[s - 1] : (place ? j : I[s]);
-    }
-    if (d < D[0]) {
-        D[0] = d;
-        I[0] = j;
-    }
-}
-
 int check_knn_args(Ctx* c, const float* X, int64_t n, int d, int k, const void* idx_out,
                    const void* dist_out);
 // Exact FP32 k-NN scan: query p is row rows[p] (null: p) of Q; `separate`: Q is

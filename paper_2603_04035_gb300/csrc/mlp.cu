@@ -273,7 +273,7 @@ static int gemm_attr(Ctx* c) {
 static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
     auto go = [&](auto kernel, size_t smem) { return launch_dep(c, kernel, G.grid, G_THREADS, smem, dep, st, G.a, G.b, G.g); };
     if (G.bn == 128) return go(G.krows ? mlp_gemm_kernel<128, true> : mlp_gemm_kernel<128, false>, GemmSmem<128>::TOTAL);
-    if (G.bn == 64) return go(G.krows ? mlp_gemm_kernel<64, true> : mlp_gemm_kernel<64, false>, GemmSmem<64>::TOTAL);
+    if (G.bn == 64 && G.krows) return go(mlp_gemm_kernel<64, true>, GemmSmem<64>::TOTAL);
     return set_error(c, DRGB_ERR_INVALID, "mlp gemm: unsupported tile");
 }
 
@@ -282,11 +282,10 @@ static int gemm_launch(Ctx* c, const Gemm& G, bool dep, cudaStream_t st) {
 int tc_gemm_nt_f32(Ctx* c, const void* A, const void* B, int M, int N, int K, int splits, float* partials,
                    int* splits_used, cudaStream_t st, bool f16) {
     Gemm G;
-    const int bn = (N % 128 == 0) ? 128 : 64;
-    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, bn, splits, false, f16);
+    int rc = gemm_setup(c, G, static_cast<const bf16*>(A), static_cast<const bf16*>(B), M, N, K, 128, splits, false, f16);
     if (rc) return rc;
     G.g.out_f32 = partials;
-    if ((rc = bn == 128 ? gemm_attr<128, false>(c) : gemm_attr<64, false>(c))) return rc;
+    if ((rc = gemm_attr<128, false>(c))) return rc;
     if (splits_used) *splits_used = int(G.grid.z);
     return gemm_launch(c, G, false, st);
 }
@@ -1206,7 +1205,7 @@ struct MlpBuffers {
     float* grad;
     MlpWeights W;
     uint32_t* step;
-    int s_split, n_chunks;
+    int n_chunks;
 };
 
 static constexpr int MLP_SPLITS = 32;
@@ -1234,7 +1233,6 @@ static MlpBuffers mlp_carve(void* base, int M) {
     const size_t m = size_t(M);
     b.M = M;
     b.n_chunks = int((m + MLP_CHUNK - 1) / MLP_CHUNK);
-    b.s_split = MLP_SPLITS;
     b.rows = cv.take<int32_t>(m);
     b.Xb = cv.take<bf16>(m * MLP_IN);
     b.H1b = cv.take<bf16>(m * MLP_H);
