@@ -187,9 +187,11 @@ static int launch_fuzzy_rows(Ctx* c, const int32_t* idx, const float* dist, int6
                              float* w_dir, int32_t* out_col, float* out_w, float* rho, float* sigma, int32_t* in_cnt,
                              int32_t* slot, cudaStream_t st) {
     const float target = float(std::log2(double(k)));
-    const size_t smem = size_t(4) * FR_THREADS * (k | 1) * 4;
+    const auto bytes = [](int list) { return size_t(4) * FR_THREADS * (list | 1) * 4; };
+    const size_t smem = bytes(k);
     auto kernel = k <= 8 ? fuzzy_rows_kernel<8> : (k <= 16 ? fuzzy_rows_kernel<16> : fuzzy_rows_kernel<32>);
-    DRGB_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    // (the same for every call: a setting of the process, read by other threads' launches)
+    DRGB_CUDA(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes(DRGB_MAX_K))));
     kernel<<<grid_for(n, FR_THREADS, c->num_sms * 16), FR_THREADS, smem, st>>>(
         idx, dist, n, k, target, w_dir, out_col, out_w, rho, sigma, c->d_status, db_n, in_cnt, slot);
     DRGB_CHECK_LAUNCH(c);

@@ -83,6 +83,10 @@ static size_t scan_smem(int d, int k, bool ranks) {
            size_t(SC_Q) * kl * 8 + (SC_Q * 4) + (ranks ? size_t(SC_Q) * kl * 4 : 0);
 }
 
+// The most a scan may take.  The limit is a setting of the process: each call sets
+// the same value, so that none is lowered before another thread's launch.
+static int scan_smem_max(bool ranks) { return int(scan_smem(2 * SC_DC, DRGB_MAX_K, ranks)); }
+
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     uint64_t r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -629,7 +633,8 @@ template <int MODE>
 static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
     A.chunk = scan_chunk(A.n, C);
     const size_t smem = scan_smem(A.d, A.k, MODE == SCAN_RANKS);
-    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      scan_smem_max(MODE == SCAN_RANKS)));
     const dim3 grid(unsigned((A.n_rows + SC_Q - 1) / SC_Q), unsigned((A.n + A.chunk - 1) / A.chunk));
     scan_kernel<MODE><<<grid, SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
@@ -757,7 +762,8 @@ int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, 
     A.partial = true;
     A.cells = CellScan{rows, perm, K, cell_beg, chunk_beg, cell_cnt, cell_rows};
     const size_t smem = scan_smem(d, k, false);
-    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<SCAN_CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_kernel<SCAN_CELLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      scan_smem_max(false)));
     scan_kernel<SCAN_CELLS><<<dim3(unsigned((cnt + SC_Q - 1) / SC_Q), unsigned(nchunk)), SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
     *done = true;
@@ -799,7 +805,7 @@ int launch_knn_exact_listed(Ctx* c, const float* Q, bool separate, const int64_t
     A.part_bytes = part_bytes;
     A.slots = 2 * int64_t(c->num_sms);
     const size_t smem = scan_smem(d, k, false);
-    DRGB_CUDA(c, cudaFuncSetAttribute(scan_listed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    DRGB_CUDA(c, cudaFuncSetAttribute(scan_listed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, scan_smem_max(false)));
     scan_listed_kernel<<<int(A.slots), SC_THREADS, smem, st>>>(A);
     DRGB_CHECK_LAUNCH(c);
     const int mb = c->num_sms * 4;

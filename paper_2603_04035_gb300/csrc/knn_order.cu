@@ -271,7 +271,6 @@ int knn_order(Ctx* c, const float* X, int64_t n, int d, int K, int32_t* perm, in
     gather_rows_kernel<<<grid_for(int64_t(K) * d, 256, c->num_sms), 256, 0, st>>>(X, d, pivots, K, centre);
     DRGB_CHECK_LAUNCH(c);
     const size_t asm_bytes = size_t(K) * ORD_DMAX * 4;
-    DRGB_CUDA(c, cudaFuncSetAttribute(cell_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(asm_bytes)));
     cell_assign_kernel<<<unsigned((n + 255) / 256), 256, asm_bytes, st>>>(X, n, d, centre, K, cell, cdist);
     DRGB_CHECK_LAUNCH(c);
     int rc = DRGB_OK;

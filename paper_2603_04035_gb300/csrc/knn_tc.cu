@@ -776,6 +776,7 @@ static constexpr int RR_WARPS = 4;
 // d (rows read as float pairs): twice an odd number of pairs, which keeps the
 // 64-bit reads of a half-warp on distinct bank pairs.
 static inline int rr_pitch(int d) { return (d & 1) ? d : 2 * ((d >> 1) | 1); }
+// At most 33 KB: no call has to raise the limit, which is a setting of the process.
 static inline size_t rr_smem(int d) { return size_t(RR_WARPS) * (32 * rr_pitch(d) + 64) * 4; }
 
 __device__ __forceinline__ void cp_async8(float* dst, const float* src) {
@@ -1016,7 +1017,6 @@ static int knn_tc_impl(Ctx* c, const float* X, int64_t n, int d, int k, int32_t*
 
     {
         auto rr = (d & 1) ? tc_rerank_kernel<F16, false> : tc_rerank_kernel<F16, true>;
-        DRGB_CUDA(c, cudaFuncSetAttribute(rr, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rr_smem(d))));
         rr<<<grid_for(n, RR_WARPS, c->num_sms * 8), RR_WARPS * 32, rr_smem(d), st>>>(
             Xp, perm, n, d, k, cand_idx, cand_s, norm, resid, maxbits, lbstop, idx_out, dist_out,
             defer_rows ? defer_rows : fail_rows, defer_count ? defer_count : fail_count);

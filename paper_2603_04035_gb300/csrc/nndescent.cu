@@ -298,7 +298,8 @@ int nnd_run(Ctx* c, const float* X, int64_t n, int d, int k, uint64_t seed, doub
     const size_t smem = size_t(wpb) * L.bytes;
     auto kern = pairs ? (rev ? nnd_iter_kernel<true, true> : nnd_iter_kernel<true, false>)
                       : (rev ? nnd_iter_kernel<false, true> : nnd_iter_kernel<false, false>);
-    DRGB_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    // (the same for every call: a setting of the process, read by other threads' launches)
+    DRGB_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(NND_SMEM_CAP)));
     int per_sm = 0;
     DRGB_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, wpb * 32, smem));
     const int64_t need = (n + wpb - 1) / wpb;
