@@ -164,6 +164,8 @@ int64_t drgb_launch_count(const drgb_ctx* ctx);
  *                             flight, 24 warps per SM), 0 flat (one group, 40
  *                             warps per SM); until it is set, single instances
  *                             of 200,000 to 9 million rows take the flat form
+ * They are the settings of a launch an epoch; loops of epochs over small graphs
+ * run in one launch (see drgb_embed_epochs), which has none.
  * Returns DRGB_ERR_INVALID for an unknown parameter or value. */
 #define DRGB_TUNE_EPOCH_WARPS 1
 #define DRGB_TUNE_EPOCH_PIPE 2
@@ -424,13 +426,18 @@ int drgb_embed_epoch(drgb_ctx* ctx, const float* Y_in, float* Y_out, const int32
                      int32_t neg, int32_t epoch, uint64_t seed, void* stream);
 
 /* Epochs t_begin .. t_end-1 of a T = n_epochs schedule, lr_t = lr0 (1 - t/T),
- * as one captured CUDA graph replayed on `stream`.  Y (n x 2) holds Y^(t_begin)
- * on entry and Y^(t_end) on return; Y_tmp (n x 2) is ping-pong scratch.
+ * Y (n x 2) holds Y^(t_begin) on entry and Y^(t_end) on return; Y_tmp (n x 2) is
+ * ping-pong scratch.  A small graph (its entries in 512s, and one more per instance
+ * of a batch, at most 11 for every SM) runs all epochs in one cooperative launch
+ * whose blocks meet after each epoch, a wait of at most 2 s (DRGB_ERR_TIMEOUT in
+ * the status word); a larger one, or one that the stream's SMs do not hold at
+ * once, as one captured CUDA graph with a launch an epoch, replayed on `stream`.
  * Because the schedule and the negatives are pure functions of (t, seed),
  * running [0, t1) then [t1, T) gives bit-identical results to [0, T).
  * Like drgb_embed_epoch it reads row_ptr[n] back first.
  * Errors: as drgb_embed_epoch (Y is scanned on entry), plus DRGB_ERR_INVALID
- * if 0 <= t_begin <= t_end <= n_epochs does not hold. */
+ * if 0 <= t_begin <= t_end <= n_epochs does not hold; DRGB_ERR_TIMEOUT as above,
+ * reported by the next synchronising call. */
 int drgb_embed_epochs(drgb_ctx* ctx, float* Y, float* Y_tmp, const int32_t* row_ptr,
                       const int32_t* col, const uint32_t* q, int64_t n, float a, float b,
                       float lr0, int32_t neg, int32_t t_begin, int32_t t_end, int32_t n_epochs,
@@ -459,9 +466,10 @@ int drgb_fit_transform(drgb_ctx* ctx, const float* X, int64_t n, int32_t d,
  * array of count + 1 int64 with offsets[0] = 0; seeds_init / seeds_neg are
  * optional HOST arrays of per-instance Philox keys (NULL: every instance uses
  * p->seed_init / p->seed_neg).  Each instance's k-NN graph is computed on its
- * own rows, the fuzzy graph of all instances is built in one pass, and each
- * of the p->n_epochs epochs is one force and one update launch over all rows
- * (the loop is one captured CUDA graph).  Instance b's result is bit-identical to
+ * own rows, the fuzzy graph of all instances is built in one pass, and the
+ * p->n_epochs epochs run over all rows at once (as drgb_embed_epochs: one
+ * cooperative launch, or one captured CUDA graph with a launch an epoch; the
+ * settings that DRGB_FLAG_AUTOTUNE times and stores are the latter's).  Instance b's result is bit-identical to
  * drgb_fit_transform of its rows alone with the same parameters and seeds.
  * Synchronous.  Errors: DRGB_ERR_INVALID (an instance with fewer than k + 1
  * rows, bad offsets or parameters), plus those of drgb_fit_transform. */
@@ -538,7 +546,7 @@ int drgb_mlp_train(drgb_ctx* ctx, const float* X, int64_t n, int32_t d, const in
                    float* losses, void* stream);
 
 /* Embed n new points: Y (n x 2 FP32, device) = MLP(X) for X (n x d FP32,
- * device), in chunks of 65536 rows on the tensor cores.  Asynchronous. */
+ * device), in one kernel on the tensor cores.  Asynchronous. */
 int drgb_mlp_embed(drgb_ctx* ctx, const float* params, const float* X, int64_t n, int32_t d, float* Y,
                    void* stream);
 
@@ -614,7 +622,7 @@ int drgb_eval_trust(drgb_ctx* ctx, const float* X, const float* Y, int64_t n, in
  * training points X_train (n x d) to X_new[p], and N_Y(p) the k nearest of
  * the training embedding Y_train (n x 2) to Y_new[p] (n_new x 2): for the
  * plain transform Y_train is the fitted embedding, for the learned embedder
- * its own image of the training set.  Exact FP32 scans, ties by index.
+ * its own image of the training set.  Exact FP32 neighbours, ties by index.
  * Query points: all if n_query <= 0 or n_query >= n_new, else the evenly
  * strided p_r = floor(r n_new / n_query).  Device pointers, caller-owned;
  * X rows 4-byte and Y rows 8-byte aligned.  Errors: DRGB_ERR_INVALID (NULL,

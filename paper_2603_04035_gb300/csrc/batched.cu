@@ -10,7 +10,7 @@
 // negative ranges and Philox keys.  Every arithmetic step of a row is the one a
 // single-instance fit performs, so each instance's embedding is bit-identical
 // to fitting it alone with the same seeds.  The epoch loop of all instances is
-// one captured CUDA graph.
+// one captured CUDA graph, or for few rows one cooperative launch.
 //
 // Also here: the epoch autotuner's entry point, which times every supported
 // force-kernel setting (width 4 or 8 warps per CTA, pipelined or flat form)

@@ -1204,7 +1204,8 @@ static int run_epoch_loop(Ctx* c, float2* Y, float2* Y_tmp, EpochArgs& A, float 
 }
 
 // Epochs [t_begin, t_end) of a T-epoch schedule, ping-ponging between Y and
-// Y_tmp; the result is left in Y.  The launches are captured into a CUDA
+// Y_tmp; the result is left in Y.  A small graph's run in one launch.  Else, and
+// where that launch is refused, the launches are captured into a CUDA
 // graph (on a private stream) and the graph is launched on `st`.  Building an
 // executable graph of hundreds of nodes costs milliseconds of host time, so
 // the context keeps the last one and refreshes it in place

@@ -70,8 +70,8 @@ int launch_epoch(Ctx* c, const EpochArgs& A, int warps, cudaStream_t st, bool af
 int launch_init(Ctx* c, float2* Y, int64_t n, float range, uint64_t seed, cudaStream_t st);
 
 // Epochs [t_begin, t_end) of a T-epoch schedule, ping-ponging between Y and
-// Y_tmp (the result is left in Y), captured as one CUDA graph.  `scratch`
-// holds epoch_scratch_bytes(n, nnz_cap, count) bytes.
+// Y_tmp (the result is left in Y): one cooperative launch for small graphs, else
+// one captured CUDA graph.  `scratch` holds epoch_scratch_bytes(n, nnz_cap, count) bytes.
 int run_epochs(Ctx* c, float2* Y, float2* Y_tmp, const int32_t* rp, const int32_t* col, const uint32_t* q,
                int64_t n, float a, float b, float lr0, int neg, int t_begin, int t_end, int T, uint64_t seed,
                cudaStream_t st, int64_t nnz_cap, void* scratch, int count = 0, const int64_t* inst_off = nullptr,

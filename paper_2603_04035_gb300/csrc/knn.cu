@@ -941,10 +941,12 @@ namespace drgb {
 int knn_resolve_mode(int64_t n, int d, int k, int mode) {
     if (mode != 0) return mode;
     // The cell-ordered product (knn_tc) spends about 150 us on the order and its
-    // bounds, and wins from about 16,000 rows on where clusters are few (10 in 50
-    // dimensions, wide / cells us: 8,000 rows 184 / 294, 16,000 306 / 312, 20,000
-    // 403 / 343, 30,000 633 / 466; 100 clusters, more than cells at these sizes: 308 /
-    // 417 at 16,000, 933 / 1,266 at 40,000).
+    // bounds, and wins from between 16,000 and 20,000 rows on where the data has fewer
+    // clusters than the order has cells (n / 2,048, at least 16): 10 clusters in 50
+    // dimensions, wide / cells us: 8,000 rows 148 / 258, 16,000 265 / 301, 20,000
+    // 366 / 322, 30,000 591 / 471.  With 100 clusters the bounds rule out little and
+    // it loses (268 / 459 at 16,000, 886 / 1,278 at 40,000).  The clusters are not
+    // known before the search, so the line is drawn by n for data of few.
     if (knn_tc_preferred(n, d, k) && (n > 16000 || !knn_wide_preferred(n, n, d, k))) return 3;
     return knn_wide_preferred(n, n, d, k) ? KNN_WIDE : 1;
 }

@@ -571,11 +571,12 @@ size_t knn_wide_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d) {
            8192;
 }
 
-// Against the FP32 scan (the line lies where they cross, measured for a graph of
-// X on itself): 1.5e8 pairs x dimensions, 1,100 x 50 144 and 144 us, 2,000 x 50
-// 113 and 168 us, 4,096 x 50 126 and 427 us, 2,000 x 784 (some rows re-scanned)
-// 493 and 682 us.  Rows of fewer than 16 dimensions are often denser than the
-// operands' rounding, and would mostly be re-scanned.
+// Against the FP32 scan, at 1.5e8 pairs x dimensions and above (graphs of X on
+// itself, product / scan us): 1,733 x 50 91 / 106, 2,000 x 50 85 / 124, 3,100 x 16
+// 93 / 135, 4,096 x 50 97 / 210, 2,000 x 784 (5 rows re-scanned) 496 / 627.  (The
+// line was drawn where they crossed while the host read the number of uncertified
+// rows back: 144 / 144 at 1,100 x 50.)  Rows of fewer than 16 dimensions are often denser
+// than the operands' rounding, and would mostly be re-scanned.
 bool knn_wide_preferred(int64_t nq, int64_t n, int d, int k) {
     return d >= 16 && d <= WD_MAX_D && k < TC_KP && n >= 1024 && double(nq) * double(n) * d >= 1.5e8;
 }
