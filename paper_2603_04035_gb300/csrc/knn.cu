@@ -1,7 +1,7 @@
 // Exact k-NN by an FP32 scan (SIMT), and the FP32 rank counts used by the
 // trustworthiness metric.
 //
-// Both are one kernel: a CTA takes 64 query rows and streams a chunk of the
+// Both are one kernel (but for small databases, scan_small_kernel): a CTA takes 64 query rows and streams a chunk of the
 // database through shared memory, 128 points by 32 dimensions at a time
 // (transposed, two buffers filled by cp.async), and each of its 256 threads
 // accumulates the squared distances of 4 queries to 8 points in registers as
@@ -112,6 +112,41 @@ __device__ __forceinline__ void cmp_swap(float& d, int32_t& i, int st, bool keep
     if (!same && less == keep_min) {
         d = od;
         i = oi;
+    }
+}
+
+// The 32 smallest, by (distance, index), of a sorted list and 32 candidates, one of
+// each a lane: sort the candidates, pair them with the list reversed, merge.
+__device__ __forceinline__ void sorted_insert(float cd, int32_t ci, int lane, float& D, int32_t& I) {
+#pragma unroll
+    for (int kk = 2; kk <= 32; kk <<= 1) {
+#pragma unroll
+        for (int st = kk >> 1; st > 0; st >>= 1) cmp_swap(cd, ci, st, ((lane & kk) == 0) == ((lane & st) == 0));
+    }
+    const float od = __shfl_sync(0xffffffffu, cd, 31 - lane);
+    const int32_t oi = __shfl_sync(0xffffffffu, ci, 31 - lane);
+    if (od < D || (od == D && oi < I)) {
+        D = od;
+        I = oi;
+    }
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1) cmp_swap(D, I, st, (lane & st) == 0);
+}
+
+// One candidate into a sorted list of which the first k count.
+__device__ __forceinline__ void list_insert(float cd, int32_t ci, int k, int lane, float& D, int32_t& I) {
+    const bool less = D < cd || (D == cd && I < ci);
+    const int pos = __popc(__ballot_sync(0xffffffffu, less));
+    if (pos >= k) return;  // overtaken by other candidates
+    const float Du = __shfl_up_sync(0xffffffffu, D, 1);
+    const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
+    if (lane > pos) {
+        D = Du;
+        I = Iu;
+    }
+    if (lane == pos) {
+        D = cd;
+        I = ci;
     }
 }
 
@@ -379,19 +414,7 @@ __device__ __forceinline__ void scan_block(const ScanArgs& A, const unsigned bx,
                                     ci = INT32_MAX;
                                 }
                             }
-#pragma unroll
-                            for (int kk = 2; kk <= 32; kk <<= 1) {
-#pragma unroll
-                                for (int st = kk >> 1; st > 0; st >>= 1) cmp_swap(cd, ci, st, ((lane & kk) == 0) == ((lane & st) == 0));
-                            }
-                            const float od = __shfl_sync(0xffffffffu, cd, 31 - lane);
-                            const int32_t oi = __shfl_sync(0xffffffffu, ci, 31 - lane);
-                            if (od < D || (od == D && oi < I)) {
-                                D = od;
-                                I = oi;
-                            }
-#pragma unroll
-                            for (int st = 16; st > 0; st >>= 1) cmp_swap(D, I, st, (lane & st) == 0);
+                            sorted_insert(cd, ci, lane, D, I);
                             todo = 0;
                         }
                         while (todo) {
@@ -403,19 +426,7 @@ __device__ __forceinline__ void scan_block(const ScanArgs& A, const unsigned bx,
                                 ci = A.cells.perm[ci];
                                 if (ci == s_qi[q]) continue;
                             }
-                            const bool less = D < cd || (D == cd && I < ci);
-                            const int pos = __popc(__ballot_sync(0xffffffffu, less));
-                            if (pos >= k) continue;  // overtaken by this tile's other points
-                            const float Du = __shfl_up_sync(0xffffffffu, D, 1);
-                            const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
-                            if (lane > pos) {
-                                D = Du;
-                                I = Iu;
-                            }
-                            if (lane == pos) {
-                                D = cd;
-                                I = ci;
-                            }
+                            list_insert(cd, ci, k, lane, D, I);
                         }
                     }
                     if (lane < kl) {
@@ -457,6 +468,70 @@ __device__ __forceinline__ void scan_block(const ScanArgs& A, const unsigned bx,
 template <int MODE>
 __global__ void __launch_bounds__(SC_THREADS, 2) scan_kernel(const ScanArgs A) {
     scan_block<MODE>(A, blockIdx.x, blockIdx.y);
+}
+
+// The k nearest of every query row in a small database: a warp a query, a point a
+// lane, the list one entry a lane.
+//
+// Why: the tiled scan gives a CTA 64 queries, and a warp selects eight of them one
+// after the other; with a few hundred points that is a chain on a few SMs.  This
+// is a chain over the tiles of 32 points.  Measured (graphs, us a call, tiled / this):
+// 40 x 8 46 / 15, 200 x 50 66 / 19, 512 x 50 89 / 39, 1,000 x 61 111 / 68, 1,500 x
+// 61 116 / 101 (89 / 95 with 5 neighbours), 200 x 300 148 / 63, 512 x 784 323 / 351.  With
+// many queries the tiles' sharing of the points tells: 20,000 queries of 1,000 x 61 and
+// all that follows 578 / 512, 60,000 865 / 1,165; of 300 x 200 4,000 queries 325 / 249,
+// 8,000 326 / 367.
+static bool scan_is_small(int64_t n_rows, int64_t n, int d) {
+    return d <= 64 ? n <= 1200 && n_rows <= 20000 : n <= 400 && n_rows <= 2000;
+}
+static constexpr int SS_WARPS = 4, SS_DC = 64, SS_PITCH = SS_DC + 1;
+
+__global__ void __launch_bounds__(SS_WARPS * 32) scan_small_kernel(const ScanArgs A) {
+    __shared__ float s_x[32 * SS_PITCH];          // 32 points' dimensions of a step
+    __shared__ float s_q[SS_WARPS][SS_DC];
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int d = A.d, k = A.k, n = int(A.n);
+    const int64_t p = int64_t(blockIdx.x) * SS_WARPS + w;  // (the last CTA's spare warps repeat its last query)
+    const int64_t r = p < A.n_rows ? p : A.n_rows - 1, q = A.rows ? A.rows[r] : r;
+    const int self = A.separate ? -1 : int(q);
+    float D = INFINITY;
+    int32_t I = INT32_MAX;
+    for (int p0 = 0; p0 < n; p0 += 32) {
+        const int pts = n - p0 < 32 ? n - p0 : 32;
+        float a = 0.f;
+        for (int c0 = 0; c0 < d; c0 += SS_DC) {
+            const int cc = d - c0 < SS_DC ? d - c0 : SS_DC;
+            __syncthreads();  // the previous step has been read
+            for (int t = tid; t < pts * SS_DC; t += SS_WARPS * 32) {
+                const int u = t / SS_DC, c = t % SS_DC;
+                if (c < cc) s_x[u * SS_PITCH + c] = A.X[int64_t(p0 + u) * d + c0 + c];
+            }
+            if (d > SS_DC || p0 == 0)
+                for (int c = lane; c < cc; c += 32) s_q[w][c] = A.Q[q * d + c0 + c];
+            __syncthreads();
+#pragma unroll 8
+            for (int c = 0; c < cc; ++c) {
+                const float df = s_x[lane * SS_PITCH + c] - s_q[w][c];
+                a = fmaf(df, df, a);
+            }
+        }
+        const float thr = __shfl_sync(0xffffffffu, D, k - 1);
+        const bool in = lane < pts && p0 + lane != self && a < thr;
+        unsigned todo = __ballot_sync(0xffffffffu, in);
+        if (__popc(todo) > SC_BULK) {
+            sorted_insert(in ? a : INFINITY, in ? p0 + lane : INT32_MAX, lane, D, I);
+            continue;
+        }
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            list_insert(__shfl_sync(0xffffffffu, a, src), p0 + src, k, lane, D, I);
+        }
+    }
+    if (p < A.n_rows && lane < k) {
+        A.idx[p * k + lane] = I == INT32_MAX ? -1 : I;
+        A.dist[p * k + lane] = sqrtf(D);
+    }
 }
 
 // Database chunks of a scan: enough (row block, chunk) CTAs for one to four
@@ -624,7 +699,8 @@ static int scan_chunks(const Ctx* c, int64_t n_rows, int64_t n, int k, size_t pa
     return scan_split(2 * int64_t(c->num_sms), n_rows, n, k, part_bytes, lists);
 }
 
-size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k) {
+size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int d, int k) {
+    if (scan_is_small(n_rows, n, d)) return 0;
     const int C = scan_chunks(c, n_rows, n, k, ~size_t(0) >> 1, true);
     return C > 1 ? 2 * (size_t(n_rows) * C * k * 4 + 512) + size_t(n_rows) * 4 + 512 : 0;
 }
@@ -646,6 +722,13 @@ static int scan_launch(Ctx* c, ScanArgs& A, int C, cudaStream_t st) {
 static int scan_nearest(Ctx* c, ScanArgs& A, int32_t* idx_out, float* dist_out, void* part, size_t part_bytes,
                         int32_t none, cudaStream_t st) {
     if (A.n_rows <= 0) return DRGB_OK;
+    if (scan_is_small(A.n_rows, A.n, A.d) && !A.ub && !A.list) {
+        A.idx = idx_out;
+        A.dist = dist_out;
+        scan_small_kernel<<<unsigned((A.n_rows + SS_WARPS - 1) / SS_WARPS), SS_WARPS * 32, 0, st>>>(A);
+        DRGB_CHECK_LAUNCH(c);
+        return DRGB_OK;
+    }
     const int C = scan_chunks(c, A.n_rows, A.n, A.k, part ? part_bytes : 0, true);
     if (C <= 1) {
         A.idx = idx_out;
@@ -842,7 +925,7 @@ int launch_knn_scan(Ctx* c, const float* Q, int64_t nq, bool separate, const int
 }
 
 size_t knn_queries_scratch_bytes(const Ctx* c, int64_t nq, int64_t n, int d, int k) {
-    return knn_wide_preferred(nq, n, d, k) ? knn_wide_scratch_bytes(c, nq, n, d) : knn_scan_scratch_bytes(c, nq, n, k);
+    return knn_wide_preferred(nq, n, d, k) ? knn_wide_scratch_bytes(c, nq, n, d) : knn_scan_scratch_bytes(c, nq, n, d, k);
 }
 
 int knn_queries(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
@@ -955,7 +1038,7 @@ size_t knn_scratch_bytes(const Ctx* c, int64_t n, int d, int k, int mode, size_t
     const int m = knn_resolve_mode(n, d, k, mode);
     const bool cells = m == 2 || m == 3 || (m == KNN_WIDE && knn_tc_preferred(n, d, k));
     const size_t tb = cells ? knn_tc_scratch_bytes(n, d) : 0;
-    const size_t b = m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : (m == 1 ? knn_scan_scratch_bytes(c, n, n, k) : 0);
+    const size_t b = m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : (m == 1 ? knn_scan_scratch_bytes(c, n, n, d, k) : 0);
     if (least) *least = tb;
     return b > tb ? b : tb;
 }
@@ -997,7 +1080,7 @@ extern "C" int drgb_knn_graph(drgb_ctx* c, const float* X, int64_t n, int32_t d,
     // the context's scratch, and other searches, on another.  A captured call
     // scans unsplit (its graph may outlive the buffer); so does one that the scratch
     // limit or the device leaves no room for.
-    const size_t want = captured ? 0 : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, k));
+    const size_t want = captured ? 0 : (m == KNN_WIDE ? knn_wide_scratch_bytes(c, n, n, d) : knn_scan_scratch_bytes(c, n, n, d, k));
     KnnBuf* buf = nullptr;
     if (want && (rc = take_knn_buf(c, want, st, &buf))) return rc;
     if (!buf) return cells ? by_cells(3) : knn_run(c, X, n, d, k, 1, idx_out, dist_out, st, nullptr, 0);

@@ -13,7 +13,7 @@ int check_knn_args(Ctx* c, const float* X, int64_t n, int d, int k, const void* 
 // lists, and take it whole when it is null or too small; the results are the same.
 int launch_knn_scan(Ctx* c, const float* Q, int64_t nq, bool separate, const int64_t* rows, const float* X, int64_t n,
                     int d, int k, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part, size_t part_bytes);
-size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int k);
+size_t knn_scan_scratch_bytes(const Ctx* c, int64_t n_rows, int64_t n, int d, int k);
 // Exact FP32 scan of the rows listed in rows32[0 .. cnt).  On entry each listed
 // row of idx_out/dist_out must already hold k
 // distinct points other than the row in ascending order of their FP32
