@@ -1143,6 +1143,13 @@ static void fill_args(EpochArgs& A, const int32_t* rp, const int32_t* col, const
 // 10.9 / 11.5, 30,000 11.8 / 14.2, 35,000 14.5 / 14.5, 40,000 15.1 / 14.7, 50,000
 // 19.0 / 15.9 (35,000 rows are 11.5 windows an SM).
 static constexpr int64_t LOOP_MAX_WINDOWS_PER_SM = 11;
+// A short loop over more than a few windows an SM takes launches too: the graph's
+// launches are prepared while the device works on the call's tables, and the loop's
+// CTAs take their windows in turn (us a call, loop / launches: 20,000 rows 3
+// epochs 75 / 66, 6 103 / 100, 10 139 / 148; with 20 negatives 108 / 94, 167 / 166, 251 /
+// 265; 10,000 rows, 3 windows an SM, 60 / 66 and 72 / 93).
+static constexpr int64_t LOOP_FEW_WINDOWS_PER_SM = 4;
+static constexpr int LOOP_MIN_EPOCHS = 8;
 static constexpr int LOOP_MAX_EPOCHS = 1000000;  // the barrier counts epochs x CTAs in 32 bits
 
 // *done is false, and no epoch has run, where the device, or the part of it that
@@ -1219,7 +1226,8 @@ int run_epochs(Ctx* c, float2* Y, float2* Y_tmp, const int32_t* rp, const int32_
     EpochScratch es;
     int rc = epoch_prepare(c, rp, n, row_begin, nnz_cap, count, inst_off, scratch, &es, st);
     if (rc) return rc;
-    if (t_end - t_begin > 1 && t_end - t_begin <= LOOP_MAX_EPOCHS &&
+    const int few = es.win_cap <= LOOP_FEW_WINDOWS_PER_SM * c->num_sms ? 2 : LOOP_MIN_EPOCHS;
+    if (t_end - t_begin >= few && t_end - t_begin <= LOOP_MAX_EPOCHS &&
         es.win_cap <= LOOP_MAX_WINDOWS_PER_SM * c->num_sms) {
         EpochArgs A;
         fill_args(A, rp, col, q, n, a, b, neg, seed, c->d_status, es, count, inst_off, inst_seed, row_begin, neg_n);
