@@ -804,6 +804,12 @@ __global__ void cell_reach_kernel(const float* __restrict__ X, int d, int k, con
     }
 }
 
+// Below this the five short kernels cost more than scanning all points for the
+// uncertified rows does (us a call with that re-scan / this one, about a tenth of
+// the rows uncertified: 4,096 x 3 263 / 325, 9,000 x 15 330 / 379, 16,500 x 61 554 / 605,
+// 20,000 x 3 660 / 654, 30,000 x 2 1,122 / 965).
+static constexpr int64_t CELLS_MIN_ROWS = 16384;
+
 int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, int k, const int32_t* rows,
                      int64_t cnt, int K, const int32_t* perm, const int32_t* cell_beg, const float* cell_c,
                      const float* cell_r, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,
@@ -813,7 +819,7 @@ int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, 
     // scratch holds (at most n / CH + K chunks in all)
     const size_t fixed = 3 * Carve::round(size_t(K + 1) * 4) + Carve::round(size_t(K) * cnt * 4) + 4096;
     const size_t per_list = size_t(cnt) * k * 8;
-    if (K <= 1 || fixed >= part_bytes) return DRGB_OK;
+    if (K <= 1 || n < CELLS_MIN_ROWS || fixed >= part_bytes) return DRGB_OK;
     const int64_t max_lists = int64_t((part_bytes - fixed) / per_list) - K;
     if (max_lists <= 0) return DRGB_OK;
     int64_t CH = CELL_CHUNK;

@@ -26,8 +26,8 @@ int launch_knn_exact_rows_n(Ctx* c, const float* X, int64_t n, int d, int k, con
 // The same over the cells that each listed row can reach: Xp holds the points
 // in cell order (cell C: positions [cell_beg[C], cell_beg[C+1]), in the sphere
 // (cell_c[C], cell_r[C]); position p holds point perm[p]; indices ascend within
-// a cell).  *done is false, and nothing was enqueued, when there is one cell or
-// part_bytes do not hold the lists.
+// a cell).  *done is false, and nothing was enqueued, when there is one cell, the
+// points are few or part_bytes do not hold the lists.
 int launch_knn_cells(Ctx* c, const float* X, const float* Xp, int64_t n, int d, int k, const int32_t* rows,
                      int64_t cnt, int K, const int32_t* perm, const int32_t* cell_beg, const float* cell_c,
                      const float* cell_r, int32_t* idx_out, float* dist_out, cudaStream_t st, void* part,

@@ -60,3 +60,17 @@ def test_graph_of_a_matrix_off_the_boundary(drgb, d, shift):
     X = _points(4100, d, 3, "clusters", shift)
     got, want = drgb.knn_graph(X, 15), drgb.knn_graph(X, 15, mode=1)
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("n", [16383, 16384, 20001])
+@pytest.mark.parametrize("d,k", [(3, 15), (16, 30), (61, 5)])
+def test_uncertified_rows_on_both_sides_of_the_cells_line(drgb, n, d, k):
+    # many copies of a point leave rows uncertified: scanned over all points, or
+    # over the cells they reach
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(n + d)
+    X = torch.randn(n // 20, d, generator=g, device="cuda")[torch.randint(0, n // 20, (n,), generator=g, device="cuda")]
+    got = drgb.knn_graph(X, k, mode=3)
+    assert drgb.knn_uncertified() > 0
+    want = drgb.knn_graph(X, k, mode=1)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
