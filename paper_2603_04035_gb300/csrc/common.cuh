@@ -198,9 +198,9 @@ __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol
 // one before drains and waits in dep_enter, before its first access to memory
 // that an earlier one writes.  Only then may the next one start, so at most two
 // kernels of the chain are resident, and whatever came before the previous one is
-// complete when a kernel starts.  What such a kernel reads is being written while it
-// runs, so its parameters are not `const __restrict__`, which would promise the
-// opposite and let the compiler load before the wait.
+// complete when a kernel starts.  What the kernel before writes is being written while
+// such a kernel runs, so its parameters are not `const __restrict__`, which would
+// promise the opposite and let the compiler load before the wait; that of older data may be.
 __device__ __forceinline__ void dep_enter() {
     grid_dep_wait();
     grid_dep_launch();

@@ -637,12 +637,13 @@ __global__ void mlp_gather_kernel(const float* __restrict__ X, int d, const int3
 // 101 us.)
 static constexpr int HEAD_ROWS = 4;
 
-__global__ void __launch_bounds__(256) mlp_head_loss_kernel(const bf16* H2, const float* W3f,
-                                                            const float* P, const int32_t* rows,
+__global__ void __launch_bounds__(256) mlp_head_loss_kernel(const bf16* H2, const float* __restrict__ W3f,
+                                                            const float* __restrict__ P, const int32_t* __restrict__ rows,
                                                             int B, int neg, float a, float b, float* __restrict__ dz,
                                                             float* __restrict__ loss_part, uint32_t* __restrict__ step_dev) {
     const int lane = threadIdx.x & 31;
-    // (the weights are older than the kernel before)
+    // (the weights and the rows are older than the kernel before, so they are read
+    // before the wait, and qualified)
     float w0[MLP_H / 32], w1[MLP_H / 32];
 #pragma unroll
     for (int i = 0; i < MLP_H / 32; ++i) {
@@ -736,7 +737,7 @@ static constexpr int MC_PITCH = MLP_CHUNK * 4 + 4;  // floats per float4 column:
 static constexpr size_t L3_SMEM = size_t(8) * MC_PITCH * 4 + MLP_CHUNK * 8;
 
 __global__ void __launch_bounds__(MC_THREADS, 3)
-mlp_l3back_kernel(const float* dz, const float* W3f, const float* dgelu2, int M,
+mlp_l3back_kernel(const float* dz, const float* __restrict__ W3f, const float* __restrict__ dgelu2, int M,
                   bf16* __restrict__ D, float* __restrict__ pb2) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]: dpre2, float4 columns
     float2* s_z = reinterpret_cast<float2*>(s_v + 8 * MC_PITCH);  // [MLP_CHUNK]: dz
@@ -744,7 +745,10 @@ mlp_l3back_kernel(const float* dz, const float* W3f, const float* dgelu2, int M,
     const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;  // a multiple of 128
     float wx[4], wy[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {  // (the weights are older than the kernel before)
+    // (the weights and GELU' are older than the kernel before: qualified, so that their
+    // first loads may be issued before the wait; unqualified, a step of 4096 edges took 6 us
+    // more where the process had used 8 streams)
+    for (int j = 0; j < 4; ++j) {
         wx[j] = W3f[c0 + 4 * warp + j];
         wy[j] = W3f[MLP_H + c0 + 4 * warp + j];
     }
@@ -790,7 +794,7 @@ mlp_l3back_kernel(const float* dz, const float* W3f, const float* dgelu2, int M,
 
 // Over the chunk: dW3[o] = sum dz[.][o] H2 and db3[o] = sum dz[.][o].
 __global__ void __launch_bounds__(MC_THREADS)
-mlp_w3grad_kernel(const float* dz, const bf16* H2, int M, float* __restrict__ pw3) {
+mlp_w3grad_kernel(const float* __restrict__ dz, const bf16* __restrict__ H2, int M, float* __restrict__ pw3) {
     __shared__ __align__(16) bf16 s_h[MLP_CHUNK * 32];  // H2
     __shared__ float2 s_z[MLP_CHUNK];                   // dz
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -823,7 +827,7 @@ mlp_w3grad_kernel(const float* dz, const bf16* H2, int M, float* __restrict__ pw
 static constexpr size_t CS_SMEM = size_t(8) * MC_PITCH * 4;
 
 __global__ void __launch_bounds__(MC_THREADS, 3)
-mlp_colsum_kernel(const float* A, int M, float* __restrict__ part) {
+mlp_colsum_kernel(const float* __restrict__ A, int M, float* __restrict__ part) {
     extern __shared__ __align__(16) float s_v[];  // [8][MC_PITCH]
     const int r0 = blockIdx.x * MLP_CHUNK, c0 = blockIdx.y * 32, tid = threadIdx.x;
     const int rows = M - r0 < MLP_CHUNK ? M - r0 : MLP_CHUNK;
