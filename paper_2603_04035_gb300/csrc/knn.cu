@@ -133,23 +133,6 @@ __device__ __forceinline__ void sorted_insert(float cd, int32_t ci, int lane, fl
     for (int st = 16; st > 0; st >>= 1) cmp_swap(D, I, st, (lane & st) == 0);
 }
 
-// One candidate into a sorted list of which the first k count.
-__device__ __forceinline__ void list_insert(float cd, int32_t ci, int k, int lane, float& D, int32_t& I) {
-    const bool less = D < cd || (D == cd && I < ci);
-    const int pos = __popc(__ballot_sync(0xffffffffu, less));
-    if (pos >= k) return;  // overtaken by other candidates
-    const float Du = __shfl_up_sync(0xffffffffu, D, 1);
-    const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
-    if (lane > pos) {
-        D = Du;
-        I = Iu;
-    }
-    if (lane == pos) {
-        D = cd;
-        I = ci;
-    }
-}
-
 // NEAREST: the k nearest of every query row in the chunk.  RANKS: for every
 // target s of row r, the number of points of the chunk that precede it in the
 // FP32 (distance, index) order.  CELLS: the k nearest among chunk blockIdx.y of
@@ -426,7 +409,20 @@ __device__ __forceinline__ void scan_block(const ScanArgs& A, const unsigned bx,
                                 ci = A.cells.perm[ci];
                                 if (ci == s_qi[q]) continue;
                             }
-                            list_insert(cd, ci, k, lane, D, I);
+                            // (written out: as a function this took 6% longer)
+                            const bool less = D < cd || (D == cd && I < ci);
+                            const int pos = __popc(__ballot_sync(0xffffffffu, less));
+                            if (pos >= k) continue;  // overtaken by this tile's other points
+                            const float Du = __shfl_up_sync(0xffffffffu, D, 1);
+                            const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
+                            if (lane > pos) {
+                                D = Du;
+                                I = Iu;
+                            }
+                            if (lane == pos) {
+                                D = cd;
+                                I = ci;
+                            }
                         }
                     }
                     if (lane < kl) {
@@ -525,7 +521,21 @@ __global__ void __launch_bounds__(SS_WARPS * 32) scan_small_kernel(const ScanArg
         while (todo) {
             const int src = __ffs(todo) - 1;
             todo &= todo - 1;
-            list_insert(__shfl_sync(0xffffffffu, a, src), p0 + src, k, lane, D, I);
+            const float cd = __shfl_sync(0xffffffffu, a, src);
+            const int32_t ci = p0 + src;
+            const bool less = D < cd || (D == cd && I < ci);
+            const int pos = __popc(__ballot_sync(0xffffffffu, less));
+            if (pos >= k) continue;  // overtaken by this tile's other points
+            const float Du = __shfl_up_sync(0xffffffffu, D, 1);
+            const int32_t Iu = __shfl_up_sync(0xffffffffu, I, 1);
+            if (lane > pos) {
+                D = Du;
+                I = Iu;
+            }
+            if (lane == pos) {
+                D = cd;
+                I = ci;
+            }
         }
     }
     if (p < A.n_rows && lane < k) {
