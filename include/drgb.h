@@ -427,11 +427,13 @@ int drgb_embed_epoch(drgb_ctx* ctx, const float* Y_in, float* Y_out, const int32
 
 /* Epochs t_begin .. t_end-1 of a T = n_epochs schedule, lr_t = lr0 (1 - t/T),
  * Y (n x 2) holds Y^(t_begin) on entry and Y^(t_end) on return; Y_tmp (n x 2) is
- * ping-pong scratch.  A small graph (its entries in 512s, and one more per instance
- * of a batch, at most 11 for every SM) runs all epochs in one cooperative launch
- * whose blocks meet after each epoch, a wait of at most 2 s (DRGB_ERR_TIMEOUT in
- * the status word); a larger one, or one that the stream's SMs do not hold at
- * once, as one captured CUDA graph with a launch an epoch, replayed on `stream`.
+ * ping-pong scratch.  On a small graph (its entries in 512s, and one more per
+ * instance of a batch, at most 11 for every SM) 8 epochs or more (2 or more where
+ * they are at most 4 for every SM) run in one cooperative launch, which starts when
+ * the stream's SMs have room for all its blocks; they meet after each epoch, a
+ * wait of at most 2 s (DRGB_ERR_TIMEOUT in the status word).  Otherwise, and where
+ * the SMs can never hold the blocks at once, the epochs run as one captured CUDA
+ * graph with a launch an epoch, replayed on `stream`.
  * Because the schedule and the negatives are pure functions of (t, seed),
  * running [0, t1) then [t1, T) gives bit-identical results to [0, T).
  * Like drgb_embed_epoch it reads row_ptr[n] back first.
