@@ -96,6 +96,9 @@ int release_knn_bufs(Ctx* c);
 // records its end (KnnBuf::ev) on `st` when it has enqueued its work.
 int take_knn_buf(Ctx* c, size_t bytes, cudaStream_t st, KnnBuf** out);
 
+// Wait for `st` and for the searches that use k-NN buffers, on whichever stream.
+int wait_for_searches(Ctx* c, cudaStream_t st);
+
 // Ensure the context holds at least `bytes` of scratch.  Growing synchronises
 // `stream` first, so that work still using the old buffer has finished.
 int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream);

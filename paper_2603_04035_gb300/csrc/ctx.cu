@@ -102,6 +102,13 @@ int take_knn_buf(Ctx* c, size_t bytes, cudaStream_t st, KnnBuf** out) {
     return DRGB_OK;
 }
 
+int wait_for_searches(Ctx* c, cudaStream_t st) {
+    DRGB_CUDA(c, cudaStreamSynchronize(st));
+    for (KnnBuf& b : c->knn_bufs)
+        if (b.ev) DRGB_CUDA(c, cudaEventSynchronize(b.ev));
+    return DRGB_OK;
+}
+
 int ensure_scratch(Ctx* c, size_t bytes, cudaStream_t stream) {
     if (bytes <= c->scratch_bytes) return DRGB_OK;
     if (c->scratch_limit && bytes > c->scratch_limit)

@@ -1056,7 +1056,8 @@ int knn_tc(Ctx* c, const float* X, int64_t n, int d, int k, bool f16, int32_t* i
 extern "C" int drgb_knn_tiles(drgb_ctx* c, int64_t* done, int64_t* total, void* stream) {
     if (!c || !done || !total) return DRGB_ERR_INVALID;
     unsigned long long v = 0;
-    DRGB_CUDA(c, cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
+    int rc = wait_for_searches(c, static_cast<cudaStream_t>(stream));
+    if (rc) return rc;
     DRGB_CUDA(c, cudaMemcpy(&v, c->d_counter + 4, sizeof(v), cudaMemcpyDeviceToHost));
     *done = int64_t(v);
     *total = c->knn_tiles_total;
@@ -1066,7 +1067,8 @@ extern "C" int drgb_knn_tiles(drgb_ctx* c, int64_t* done, int64_t* total, void* 
 extern "C" int drgb_knn_uncertified(drgb_ctx* c, int64_t* count, void* stream) {
     if (!c || !count) return DRGB_ERR_INVALID;
     int32_t v = 0;
-    DRGB_CUDA(c, cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
+    int rc = wait_for_searches(c, static_cast<cudaStream_t>(stream));
+    if (rc) return rc;
     DRGB_CUDA(c, cudaMemcpy(&v, c->d_counter, sizeof(int32_t), cudaMemcpyDeviceToHost));
     *count = v;
     return DRGB_OK;

@@ -143,6 +143,23 @@ def test_searches_on_two_streams_do_not_wait_for_each_other(drgb, n, d, mode):
             assert torch.equal(r[0], want[0]) and torch.equal(r[1], want[1])
 
 
+def test_counters_wait_for_the_search(drgb):
+    # asked on another stream than the search's, which is still behind other work
+    import torch
+    X = _points(3000, 200)
+    X[100:200] = X[:1]  # copies: more than the candidate lists hold
+    drgb.knn_graph(X, 15)
+    want = (drgb.knn_uncertified(), drgb.knn_tiles())
+    assert want[0] >= 100
+    drgb.knn_graph(_points(2000, 50), 15)
+    assert (drgb.knn_uncertified(), drgb.knn_tiles()) != want
+    s1 = torch.cuda.Stream()
+    _busy(s1)
+    with torch.cuda.stream(s1):
+        drgb.knn_graph(X, 15)
+    assert (drgb.knn_uncertified(), drgb.knn_tiles()) == want
+
+
 def test_searches_on_many_streams_with_growth(drgb):
     # more streams than the context keeps buffers, sizes that grow in between
     import torch
